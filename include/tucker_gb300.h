@@ -60,7 +60,12 @@ typedef enum { TUCKER_F32 = 0, TUCKER_F64 = 1 } tucker_dtype;
  * up to ~1.5e-10 ||X||^2 on the discarded subspace, too close to the
  * threshold eps^2 ||X||^2 / N below that.  The result reports the kernel of
  * every step.
- *   FP64   : products and sums in FP64 (any input dtype); core in FP64.
+ *   FP64   : products and sums in FP64 (any input dtype); core in FP64.  Large
+ *            Grams (I_n >= 64) and TTMs form them on the tensor cores from
+ *            exact integer digits: each value as a 55-bit fixed-point number
+ *            of its row (rounding 2^-55 of the row's largest magnitude), every
+ *            digit product and sum exact, one rounding to FP64 at the end; an
+ *            operand with NaN, Inf or a row below 2^-958 takes the FP64 pipe.
  *   FP32   : FP32 products, round-to-nearest FP32 sums over short chunks
  *            combined exactly (TwoSum) and in FP64; working tensor and core
  *            in the input dtype.
@@ -118,7 +123,7 @@ typedef struct tucker_result {
   double threshold;                  /* eps^2 ||X||^2 / N (0 when ranks were given)    */
   double discarded_sq[TUCKER_MAX_MODES]; /* sum of discarded eigenvalues per mode      */
   int jacobi_sweeps[TUCKER_MAX_MODES];
-  int gram_kernel[TUCKER_MAX_MODES]; /* kernel that ran: 0 SIMT FP64, 1 SIMT FP32, 2 tcgen05
+  int gram_kernel[TUCKER_MAX_MODES]; /* kernel that ran: 0 FP64, 1 SIMT FP32, 2 tcgen05
                                         (rounded split), 3 small-mode FP64, 4 FP32 with
                                         exact block sums, 5 / 6 tcgen05 on exact three- /
                                         two-digit products */

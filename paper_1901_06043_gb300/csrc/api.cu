@@ -298,7 +298,8 @@ int digit_gram_digits(const unsigned* rowmax_bits, int64_t I, int64_t K, double 
   return 0;
 }
 
-// Which kernel serves a Gram / TTM step: 0 SIMT FP64, 1 SIMT FP32, 2 tcgen05
+// Which kernel serves a Gram / TTM step: 0 FP64 (SIMT, or digit64.cu from a
+// size), 1 SIMT FP32, 2 tcgen05
 // (rounded FP16 split products), 3 small-mode FP64 (I < 64, every
 // precision), 4 FP32 with exact (compensated) block sums (row modes with few
 // slabs), 5 tcgen05 on exact integer digit products (MIXED, I <= 4096;
@@ -335,6 +336,22 @@ tucker_status rowmax_pass(tucker_ctx* c, const float* y, int64_t I0, int64_t nco
 tucker_status view_rowmax(tucker_ctx* c, const float* y, const SlabView& v, unsigned* rowmax) {
   if (v.L == 1 && v.I <= 8192) return rowmax_pass(c, y, v.I, v.Rt, rowmax);
   TK_CUDA(c, launch_rowmax_slab(y, v.L, v.I, v.Rt, c->num_sms, rowmax, c->stream));
+  return TUCKER_OK;
+}
+
+// Waits for an FP64 digit kernel and reads its verdict words: *bad when an
+// operand is outside its range (the caller then computes the step on the FP64
+// pipe).
+tucker_status digit64_verdict(tucker_ctx* c, const unsigned* words, const char* what, bool* bad) {
+  unsigned w[2] = {0, 0};
+  TK_CUDA(c, cudaMemcpyAsync(w, words, sizeof w, cudaMemcpyDeviceToHost, c->stream));
+  TK_TRY(sync(c));
+  if (w[1]) {
+    char m[96];
+    snprintf(m, sizeof m, "FP64 digit %s reported device error word 0x%x", what, w[1]);
+    return set_err(c, TUCKER_ERR_CUDA, m);
+  }
+  *bad = w[0] != 0;
   return TUCKER_OK;
 }
 
@@ -414,6 +431,22 @@ tucker_status gram_once(tucker_ctx* c, const void* y, tucker_dtype dt, const Sla
       TK_CUDA(c, launch_gram_f32((const float*)y, v.L, v.I, v.Rt, v.L0, pc, scratch.as<double>(),
                                  S, c->stream));
       return TUCKER_OK;
+    }
+  }
+  if (kern == 0) {
+    // FP64 products: seven exact digits on the tensor cores from the size
+    // where they beat the FP64 pipe (digit64.cu); out of their range (NaN,
+    // Inf, rows below 2^-958): the FP64 pipe
+    const GramPlan pd = plan_gram_d64(v.L, v.I, v.Rt, sms);
+    if (pd.nctas > 0) {
+      DevBuf scratch;
+      TK_TRY(dev_alloc(c, scratch, pd.scratch_bytes));
+      TK_CUDA(c, launch_gram_d64(y, dt, v.L, v.I, v.Rt, pd, c->num_sms, scratch.p,
+                                 check ? nullptr : c->d_words + 8, S, c->stream));
+      if (!check) return TUCKER_OK;
+      bool bad = false;
+      TK_TRY(digit64_verdict(c, gram_d64_verdict(pd, v.I, scratch.p), "Gram", &bad));
+      if (!bad) return TUCKER_OK;
     }
   }
   GramPlan p = plan_gram_simt(v.L, v.I, v.Rt, sms, v.L0);
@@ -512,6 +545,10 @@ size_t gram_scratch_bytes(const tucker_ctx* c, tucker_prec prec, tucker_dtype dt
   if (kern == 1 && dt == TUCKER_F32) {
     const GramPlan pc = plan_gram_f32(v.L, v.I, v.Rt, c->num_sms, v.L0);
     if (pc.ntiles > 0) return pc.scratch_bytes;
+  }
+  if (kern == 0) {
+    const GramPlan pd = plan_gram_d64(v.L, v.I, v.Rt, c->num_sms);
+    if (pd.nctas > 0) return pd.scratch_bytes;
   }
   return plan_gram_simt(v.L, v.I, v.Rt, c->num_sms, v.L0).scratch_bytes;
 }
@@ -745,6 +782,19 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
       return set_err(c, TUCKER_ERR_CUDA, m);
     }
     return TUCKER_OK;
+  }
+  // FP64: seven exact digits on the tensor cores from the size where they
+  // beat the FP64 pipe (digit64.cu); out of their range (NaN, Inf, rows below
+  // 2^-958): the FP64 pipe
+  if (prec == TUCKER_PREC_FP64 && ttm_d64_supported(v.L, v.I, v.Rt, K)) {
+    DevBuf scratch;
+    TK_TRY(dev_alloc(c, scratch, ttm_d64_scratch_bytes(v.L, v.I, v.Rt, K)));
+    TK_CUDA(c, launch_ttm_d64(y, ydt, v.L, v.I, v.Rt, A, K, lda, arow, z, zdt, zt, scratch.p,
+                              check ? nullptr : c->d_words + 9, c->num_sms, c->stream));
+    if (!check) return TUCKER_OK;
+    bool bad = false;
+    TK_TRY(digit64_verdict(c, ttm_d64_verdict(v.L, v.I, v.Rt, K, scratch.p), "TTM", &bad));
+    if (!bad) return TUCKER_OK;
   }
   // the FP32 copy of the operator pays off once the TTM spans several waves
   DevBuf a32;

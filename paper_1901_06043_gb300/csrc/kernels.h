@@ -47,6 +47,26 @@ cudaError_t launch_gram_tcx(const float* y, int64_t L, int64_t I, int64_t Rt, co
 cudaError_t launch_rowmax_slab(const float* y, int64_t L, int64_t I, int64_t Rt, int num_sms,
                                unsigned* rowmax_bits, cudaStream_t st);
 
+// ---- FP64 Gram and TTM on exact seven-digit tensor-core products
+// (digit64.cu).  plan.nctas == 0 / supported == 0 when the work is too small
+// (or I < 64, I > 8192 for the Gram).  scratch: plan.scratch_bytes /
+// ttm_d64_scratch_bytes, holding two verdict words (*_verdict): [0] nonzero when
+// an operand holds NaN, Inf or a row below 2^-958 (the output is then NaN and a
+// caller that reads the word computes the step with the SIMT kernel), [1] the
+// error word when err is NULL.
+GramPlan plan_gram_d64(int64_t L, int64_t I, int64_t Rt, int num_sms);
+const unsigned* gram_d64_verdict(const GramPlan& p, int64_t I, const void* scratch);
+cudaError_t launch_gram_d64(const void* y, tucker_dtype dt, int64_t L, int64_t I, int64_t Rt,
+                            const GramPlan& p, int num_sms, void* scratch, unsigned* err, double* S,
+                            cudaStream_t st);
+int ttm_d64_supported(int64_t L, int64_t I, int64_t Rt, int64_t K);
+size_t ttm_d64_scratch_bytes(int64_t L, int64_t I, int64_t Rt, int64_t K);
+const unsigned* ttm_d64_verdict(int64_t L, int64_t I, int64_t Rt, int64_t K, const void* scratch);
+cudaError_t launch_ttm_d64(const void* y, tucker_dtype ydt, int64_t L, int64_t I, int64_t Rt,
+                           const double* A, int64_t K, int64_t lda, int a_rowmajor, void* z,
+                           tucker_dtype zdt, bool zt, void* scratch, unsigned* err, int num_sms,
+                           cudaStream_t st);
+
 // L0: the fastest sub-index of l (the first dim of the tensor for a mode
 // n > 0); row-mode K-blocks never cross a multiple of it
 GramPlan plan_gram_simt(int64_t L, int64_t I, int64_t Rt, int num_sms, int64_t L0);
