@@ -637,7 +637,7 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   const int G = tridiag_team_size(n, c->num_sms);
   const size_t nn = (size_t)n * n;
   const size_t nwy = eig_wy_doubles(n);
-  const size_t ndbl = nn + 3 * (size_t)n + 4 * (size_t)n + 2 * (size_t)G + (size_t)n + 1 + nwy;
+  const size_t ndbl = nn + 3 * (size_t)n + 4 * (size_t)n + 2 * (size_t)G + nwy;
   DevBuf work;
   TK_TRY(dev_alloc(c, work, sizeof(double) * ndbl + sizeof(EigProblem) + 16));
   EigProblem h{};
@@ -646,8 +646,7 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   h.e = h.d + n;
   h.tau = h.e + n;
   h.xch = h.tau + n;
-  double* tail = h.xch + 4 * (size_t)n + 2 * (size_t)G;
-  h.wyT = tail + n + 1;
+  h.wyT = h.xch + 4 * (size_t)n + 2 * (size_t)G;
   EigProblem* pd = reinterpret_cast<EigProblem*>(h.wyT + nwy);
   int* info = reinterpret_cast<int*>(pd + 1);
   h.w = w;
@@ -658,10 +657,10 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   cudaStream_t st = c->stream;
   TK_CUDA(c, cudaMemcpyAsync(h.A, S, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
   TK_CUDA(c, cudaMemsetAsync(c->d_words + 32, 0, sizeof(unsigned) * 3, st));
-  TK_CUDA(c, cudaMemsetAsync(info, 0, sizeof(int), st));
+  TK_CUDA(c, cudaMemsetAsync(info, 0, 2 * sizeof(int), st));
   TK_CUDA(c, launch_tridiag(pd, &h, 1, c->d_words + 32, c->d_words + 34, st, c->barrier_polls));
   TK_CUDA(c, launch_bisect(pd, 1, n, n, c->num_sms, st));
-  TK_CUDA(c, launch_rank_cut(w, n, thr, fixed_R, c->d_i64, c->d_small + 2, tail, st));
+  TK_CUDA(c, launch_rank_cut(w, n, thr, fixed_R, c->d_i64, c->d_small + 2, st));
   int64_t R = 0;
   unsigned werr = 0;
   TK_CUDA(c, cudaMemcpyAsync(&R, c->d_i64, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -683,7 +682,6 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   h.U = U.as<double>();
   h.R = Ri;
   h.zoff = 0;
-  h.roff = 0;
   TK_CUDA(c, cudaMemcpyAsync(pd, &h, sizeof(h), cudaMemcpyHostToDevice, st));
   TK_CUDA(c, launch_invit(pd, 1, Ri, st));
   // Cholesky QR, twice (the second pass restores orthogonality to rounding
@@ -692,8 +690,7 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   const SlabView zv{1, (int64_t)Ri, (int64_t)n, 1};
   for (int pass = 0; pass < 2; ++pass) {
     TK_TRY(do_gram(c, h.z, TUCKER_F64, zv, TUCKER_PREC_FP64, h.gram, nullptr));
-    TK_CUDA(c, launch_chol(pd, 1, st));
-    TK_CUDA(c, launch_trsm_rows(pd, 1, n, st));
+    TK_CUDA(c, launch_cholqr(pd, &h, 1, pass, c->num_sms, st));
   }
   TK_CUDA(c, launch_backtransform(pd, 1, Ri, n, st));
   int hinfo = 0;
@@ -705,10 +702,7 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
 
 tucker_status do_cut(tucker_ctx* c, const double* w, int n, double thr, int fixed_R, int64_t* R,
                      double* disc) {
-  DevBuf tail;
-  TK_TRY(dev_alloc(c, tail, sizeof(double) * (n + 1)));
-  TK_CUDA(c, launch_rank_cut(w, n, thr, fixed_R, c->d_i64, c->d_small + 2, tail.as<double>(),
-                             c->stream));
+  TK_CUDA(c, launch_rank_cut(w, n, thr, fixed_R, c->d_i64, c->d_small + 2, c->stream));
   TK_CUDA(c, cudaMemcpyAsync(R, c->d_i64, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
   TK_CUDA(c, cudaMemcpyAsync(disc, c->d_small + 2, sizeof(double), cudaMemcpyDeviceToHost,
                              c->stream));
@@ -1585,13 +1579,13 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
     DevBuf work, meta;
     TK_TRY(dev_alloc(c, work, sizeof(double) * wtot));
     TK_TRY(dev_alloc(c, meta, sizeof(EigProblem) * m + sizeof(double) * m + sizeof(int64_t) * m +
-                                  sizeof(double) * m + sizeof(int) * m + sizeof(unsigned) * (m + 1)));
+                                  sizeof(double) * m + 2 * sizeof(int) * m + sizeof(unsigned) * (m + 1)));
     EigProblem* pd = meta.as<EigProblem>();
     double* thr_d = reinterpret_cast<double*>(pd + m);
     int64_t* R_d = reinterpret_cast<int64_t*>(thr_d + m);
     double* disc_d = reinterpret_cast<double*>(R_d + m);
     int* info_d = reinterpret_cast<int*>(disc_d + m);
-    unsigned* bars_d = reinterpret_cast<unsigned*>(info_d + m);   // m team barriers + error word
+    unsigned* bars_d = reinterpret_cast<unsigned*>(info_d + 2 * m);   // m team barriers + error word
     std::vector<EigProblem> h(m);
     std::vector<DevBuf> wbuf(m);
     std::vector<double> thr(m);
@@ -1609,7 +1603,7 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
       P.tau = P.e + n;
       P.xch = P.tau + n;
       P.wyT = P.xch + 4 * (size_t)n + 2 * (size_t)team[q];
-      P.info = info_d + q;
+      P.info = info_d + 2 * q;
       P.n = n;
       P.team_size = team[q];
       P.team_off = q == 0 ? 0 : h[q - 1].team_off + h[q - 1].team_size;
@@ -1624,7 +1618,7 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
     TK_TRY(join_side(c));
     tg.stop(c);
     te.start(c);
-    TK_CUDA(c, cudaMemsetAsync(info_d, 0, sizeof(int) * m + sizeof(unsigned) * (m + 1), st));
+    TK_CUDA(c, cudaMemsetAsync(info_d, 0, 2 * sizeof(int) * m + sizeof(unsigned) * (m + 1), st));
     TK_CUDA(c, cudaMemcpyAsync(thr_d, thr.data(), sizeof(double) * m, cudaMemcpyHostToDevice, st));
     TK_CUDA(c, launch_tridiag(pd, h.data(), m, bars_d, bars_d + m, st, c->barrier_polls));
     int neig = 0;
@@ -1638,7 +1632,7 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
     TK_TRY(sync(c));
     // ---- leading eigenvectors of all problems
     size_t vtot = 0;
-    int zoff = 0, roff = 0;
+    int zoff = 0;
     std::vector<size_t> vo(m);
     std::vector<DevBuf> ubuf(m);
     for (int q = 0; q < m; ++q) {
@@ -1658,26 +1652,23 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
       P.lu = P.gram + (size_t)P.R * P.R;
       P.U = ubuf[q].as<double>();
       P.zoff = zoff;
-      P.roff = roff;
       zoff += P.R;
-      roff += P.n;
     }
     TK_CUDA(c, cudaMemcpyAsync(pd, h.data(), sizeof(EigProblem) * m, cudaMemcpyHostToDevice, st));
     TK_CUDA(c, launch_invit(pd, m, zoff, st));
     for (int pass = 0; pass < 2; ++pass) {
-      TK_CUDA(c, launch_zgram_batched(pd, m, st));   // problems with R <= 64
+      TK_CUDA(c, launch_zgram_batched(pd, m, pass, st));   // problems with R <= 64
       for (int q = 0; q < m; ++q)
         if (h[q].R > zgram_batched_max_r()) {
           const SlabView zv{1, (int64_t)h[q].R, (int64_t)h[q].n, 1};
           TK_TRY(do_gram(c, h[q].z, TUCKER_F64, zv, TUCKER_PREC_FP64, h[q].gram, nullptr));
         }
-      TK_CUDA(c, launch_chol(pd, m, st));
-      TK_CUDA(c, launch_trsm_rows(pd, m, roff, st));
+      TK_CUDA(c, launch_cholqr(pd, h.data(), m, pass, c->num_sms, st));
     }
     TK_CUDA(c, launch_backtransform(pd, m, zoff, nmax, st));
-    std::vector<int> info(m);
+    std::vector<int> info(2 * m);
     unsigned berr = 0;
-    TK_CUDA(c, cudaMemcpyAsync(info.data(), info_d, sizeof(int) * m, cudaMemcpyDeviceToHost, st));
+    TK_CUDA(c, cudaMemcpyAsync(info.data(), info_d, 2 * sizeof(int) * m, cudaMemcpyDeviceToHost, st));
     TK_CUDA(c, cudaMemcpyAsync(&berr, bars_d + m, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
     TK_TRY(sync(c));
     if (berr & DEV_ERR_BARRIER_TIMEOUT)
@@ -1688,7 +1679,7 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
       int64_t Rq = R[q];
       double dq = disc[q];
       res[i]->eig_kernel[s] = 1;
-      if (info[q]) {
+      if (info[2 * q]) {
         DevBuf S2, V2, U2;
         TK_TRY(dev_alloc(c, S2, sizeof(double) * (size_t)n * n));
         TK_TRY(dev_alloc(c, V2, sizeof(double) * (size_t)n * n));

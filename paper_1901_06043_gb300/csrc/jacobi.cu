@@ -20,6 +20,7 @@
 // bounded (see GridBarrier).
 #include "common.cuh"
 #include "kernels.h"
+#include "rank_cut.cuh"
 
 namespace tk {
 
@@ -443,24 +444,11 @@ __global__ void k_eig_gather(const double* __restrict__ V, int n, int np, const 
   }
 }
 
-// Eq. Un: R = min{R in 1..n : sum_{i>=R} w_i <= thr}; the tail is
-// accumulated from the smallest eigenvalue up.  out_R[0] = R, out_d[0] = tail(R).
-// With fixed_R > 0 the rank is given (rank-specified variant) and only the
-// discarded tail is computed.
-__global__ void k_rank_cut(const double* __restrict__ w, int n, double thr, int fixed_R,
-                           int64_t* out_R, double* out_d, double* tail) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  tail[n] = 0.0;
-  for (int i = n - 1; i >= 0; --i) tail[i] = tail[i + 1] + w[i];
-  int R = n;
-  if (fixed_R > 0) {
-    R = fixed_R;
-  } else {
-    for (int r = 1; r <= n; ++r)
-      if (tail[r] <= thr) { R = r; break; }
-  }
-  out_R[0] = R;
-  out_d[0] = tail[R];
+// Eq. Un, or the discarded tail of a given rank (rank_cut.cuh).
+__global__ void __launch_bounds__(RANK_CUT_NT) k_rank_cut(const double* __restrict__ w, int n,
+                                                          double thr, int fixed_R, int64_t* out_R,
+                                                          double* out_d) {
+  rank_cut_cta(w, n, thr, fixed_R, out_R, out_d);
 }
 
 namespace {
@@ -562,8 +550,8 @@ cudaError_t launch_eig_finish(int n, double* work, const int* info_host, int* in
 }
 
 cudaError_t launch_rank_cut(const double* w, int n, double thr, int fixed_R, int64_t* out_R,
-                            double* out_d, double* tail, cudaStream_t st) {
-  k_rank_cut<<<1, 32, 0, st>>>(w, n, thr, fixed_R, out_R, out_d, tail);
+                            double* out_d, cudaStream_t st) {
+  k_rank_cut<<<1, RANK_CUT_NT, 0, st>>>(w, n, thr, fixed_R, out_R, out_d);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -133,7 +133,7 @@ cudaError_t launch_jacobi(const double* S, int n, double* work, const double* fr
 cudaError_t launch_eig_finish(int n, double* work, const int* info_host, int* info_dev,
                               double* w_out, double* V_out, cudaStream_t st);
 cudaError_t launch_rank_cut(const double* w, int n, double thr, int fixed_R, int64_t* out_R,
-                            double* out_d, double* tail, cudaStream_t st);
+                            double* out_d, cudaStream_t st);
 
 // ---- tridiagonal eigensolver (tridiag.cu): all eigenvalues, the leading R
 // eigenvectors.  One descriptor per matrix (device array of descriptors).
@@ -149,10 +149,9 @@ struct EigProblem {
   double* gram;   // R x R
   double* U;      // n x R column-major output
   double* wyT;    // eig_wy_doubles(n): T factors of the blocked back-transformation
-  int* info;      // 0 ok; 1 / 2 the Cholesky QR failed (see k_chol)
+  int* info;      // [0]: 0 ok; 1 / 2 the Cholesky QR failed; [1]: it needs its second pass
   int n, R;
   int zoff;       // first flattened vector index of this problem
-  int roff;       // first flattened row index of this problem
   int team_off;   // k_tridiag: first CTA of this problem's team
   int team_size;  // k_tridiag: CTAs of the team (xch holds 4 n + 2 team_size)
   int srows;      // k_tridiag: the team's rows live in shared memory
@@ -177,8 +176,10 @@ cudaError_t launch_rcp64_probe(const double* x, double* y, int64_t n, cudaStream
 cudaError_t launch_bisect(const EigProblem* probs_dev, int count, int nmax, int total_eigs,
                           int num_sms, cudaStream_t st);
 cudaError_t launch_invit(const EigProblem* probs_dev, int count, int total_vectors, cudaStream_t st);
-cudaError_t launch_chol(const EigProblem* probs_dev, int count, cudaStream_t st);
-cudaError_t launch_trsm_rows(const EigProblem* probs_dev, int count, int total_rows, cudaStream_t st);
+// Cholesky QR of every problem's Z with its Gram in P.gram, pass 0 or 1 (pass 1
+// does nothing where pass 0 found the Gram near the identity: info[1] == 0)
+cudaError_t launch_cholqr(const EigProblem* probs_dev, const EigProblem* probs_host, int count,
+                          int pass, int num_sms, cudaStream_t st);
 cudaError_t launch_backtransform(const EigProblem* probs_dev, int count, int total_vectors,
                                  int nmax, cudaStream_t st);
 // batched rank cut (thr[p], fixed[p] > 0 or NULL) and Z^T Z for problems with R <= 64
@@ -186,7 +187,8 @@ cudaError_t launch_rank_cut_batched(const EigProblem* probs_dev, int count, cons
                                     const int* fixed, int64_t* R_out, double* disc_out,
                                     cudaStream_t st);
 int zgram_batched_max_r();
-cudaError_t launch_zgram_batched(const EigProblem* probs_dev, int count, cudaStream_t st);
+cudaError_t launch_zgram_batched(const EigProblem* probs_dev, int count, int pass,
+                                 cudaStream_t st);
 
 // ---- pre- and post-processing of Section 3.5 (prepost.cu)
 // Statistics of every hyperslice of the slab view (Rt, I, L): stats[6 i + k]

@@ -10,7 +10,7 @@
 //   4. eigenvectors of T for the leading R eigenvalues by
 //      inverse iteration                                     (k_invit)
 //   5. their Cholesky QR in descending eigenvalue order, two passes:
-//      Gram (gram kernels), L = chol (k_chol), Z L^-T        (k_trsm_rows)
+//      Gram (gram kernels), L^-1 and Z L^-T           (k_chol_*, k_apply_*)
 //   6. back-transformation U = Q Z                           (k_backtransform)
 //
 // Every stage is FP64.  Work is ~(4/3) n^3 for stage 1 and O(n^2 R) for the
@@ -32,15 +32,17 @@
 // one pass over its own rows, applies step k's update and computes its part
 // of p_{k+1}: the update of step k and the product of step k+1 share a
 // barrier.
+#include <algorithm>
 #include <cfloat>
 
 #include "common.cuh"
 #include "kernels.h"
+#include "rank_cut.cuh"
 
 namespace tk {
 namespace {
 
-constexpr int TNT = 256;            // threads per CTA of k_tridiag / k_chol
+constexpr int TNT = 256;            // threads per CTA of k_tridiag / k_chol_*
 constexpr int TNW = TNT / 32;
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -623,58 +625,282 @@ __global__ void k_invit(const EigProblem* probs, int nprob) {
 }
 
 // ---------------------------------------------------------------- stage 5
-// Cholesky factor of the R x R Gram G = Z^T Z (lower, in place), one CTA per
-// problem, column by column.  A pivot <= 0 (info = 1) or a condition number
-// of Z above 1e6 (info = 2: inverse iteration returned nearly dependent
-// vectors, and the QR would lose orthogonality) marks the problem as failed;
-// the host then takes another solver for it.
-__global__ void __launch_bounds__(TNT) k_chol(const EigProblem* probs) {
-  const EigProblem P = probs[blockIdx.x];
-  const int R = P.R;
-  double* Gm = P.gram;
-  double lmin = INFINITY, lmax = 0.0;
-  for (int col = 0; col < R; ++col) {
-    const double piv = Gm[(int64_t)col * R + col];
-    if (!(piv > 0.0)) {
-      if (threadIdx.x == 0) *P.info = 1;
-      return;
-    }
-    const double l = sqrt(piv);
-    const double il = 1.0 / l;
-    lmin = fmin(lmin, l);
-    lmax = fmax(lmax, l);
-    __syncthreads();   // every thread has read the pivot
-    // scale the column below the pivot, then update the trailing lower part
-    for (int r = col + threadIdx.x; r < R; r += TNT)
-      Gm[(int64_t)r * R + col] = (r == col) ? l : Gm[(int64_t)r * R + col] * il;
-    __syncthreads();
-    const int m = R - col - 1;
-    for (int q = threadIdx.x; q < m * m; q += TNT) {
-      const int r = col + 1 + q / m, s = col + 1 + q % m;
-      if (s <= r)
-        Gm[(int64_t)r * R + s] = fma(-Gm[(int64_t)r * R + col], Gm[(int64_t)s * R + col],
-                                     Gm[(int64_t)r * R + s]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && lmin < 1e-6 * lmax) *P.info = 2;
+// Cholesky QR: with G = Z^T Z = L L^T, Q = Z L^-T.  Every diagonal block of 32
+// columns (64: the whole matrix, when R <= 64) is factored by one CTA as
+// W G W^T = D, W unit lower triangular, by eliminating [G | I] in shared memory:
+// a column costs one reciprocal of a pivot on the chain and one barrier, and
+// the inverse comes out with the factor, so that Q is a product (no chain of
+// divisions per row).  L^-1 = D^-1/2 W.
+//   R <= 64: k_chol_small leaves L^-1 in P.gram, k_apply_small forms Q.
+//   R > 64: per block of 32 columns k_chol_diag (L_pp^-1 into the diagonal
+// block), k_chol_panel (L_ip = G_ip L_pp^-T), k_chol_trail (G_ij -= L_ip
+// L_jp^T, lower blocks); k_apply_big substitutes block by block.
+// Measured: R = 401 of n = 1500 took 17.9 ms for the factor in one CTA and 6.3 ms
+// for the substitution in one thread per row; R = 28 of n = 200 53 and 54 us.
+//   A pivot <= 0 (info[0] = 1) or a condition number of Z above 1e6 (info[0] =
+// 2: inverse iteration returned nearly dependent vectors, and the QR would
+// lose orthogonality) marks the problem as failed; the host then takes
+// another solver for it.
+//   The second pass restores orthogonality to rounding when eigenvalues are
+// clustered.  Z's columns are unit vectors; when their Gram is the identity
+// to within 1/64 in norm (the first pass's k_chol_small / k_chol_far look), the
+// first pass's Q is orthonormal to rounding already and the second is not run
+// (info[1] stays 0: its kernels return).
+constexpr int CB = 32;                       // columns per block, R > 64
+constexpr int CS = 64;                       // largest R of the one-CTA factor
+
+// Whether an off-diagonal or diagonal entry is too far from the identity's for
+// the first pass to be enough: the sum of squares of all R^2 deviations within
+// (1/64)^2 if each is within 1 / (64 R).
+__device__ __forceinline__ bool far_from_identity(double g, bool diag, int R) {
+  const double e = fabs(diag ? g - 1.0 : g);
+  return !(e * (64.0 * R) <= 1.0);
 }
 
-// Q = Z L^-T, one thread per row of Z (forward substitution with L).
-__global__ void k_trsm_rows(const EigProblem* probs, int nprob) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  int p = 0;
-  while (p + 1 < nprob && probs[p + 1].roff <= t) ++p;
-  const EigProblem P = probs[p];
-  const int i = t - P.roff;
-  if (i < 0 || i >= P.n || *P.info) return;
+// Eliminates [G | I] of the m x m block in sm (m <= CS): on return the lower
+// triangle's diagonal holds D, and W's strict lower triangle sits transposed
+// in the upper one (W[i][j] at sm[j][i]).  256 threads: four per row.  s_r: a
+// shared word for the pivot's reciprocal.  Returns false on a pivot <= 0.
+__device__ bool eliminate(double (*sm)[CS + 1], int m, double* s_r) {
+  const int i = threadIdx.x >> 2, jg = threadIdx.x & 3;
+  if (threadIdx.x == 0) *s_r = sm[0][0] > 0.0 ? rcp64(sm[0][0]) : 0.0;
+  __syncthreads();
+  for (int c = 0; c < m; ++c) {
+    const double r = *s_r;
+    if (!(r > 0.0)) return false;              // the same word for every thread
+    const bool act = i > c && i < m;
+    const bool piv = i == c + 1 && i < m && jg == ((c + 1) & 3);
+    double f = 0.0, rn = 0.0;
+    if (act) {
+      f = sm[i][c] * r;
+      if (piv) {                               // the next pivot first: its reciprocal is the chain
+        const double p = fma(-f, sm[i][c], sm[i][i]);
+        sm[i][i] = p;
+        rn = p > 0.0 ? rcp64(p) : 0.0;
+      }
+      for (int j = jg; j < c; j += 4) sm[j][i] = fma(-f, sm[j][c], sm[j][i]);      // W[i][j] -= f W[c][j]
+      for (int j = c + 1 + ((jg - c - 1) & 3); j <= i; j += 4)
+        if (!(piv && j == i)) sm[i][j] = fma(-f, sm[j][c], sm[i][j]);
+    }
+    __syncthreads();                           // column c and the reciprocal are read
+    if (act && jg == (c & 3)) sm[c][i] = -f;   // W[i][c] (over nothing: column c of G is used up)
+    if (piv) *s_r = rn;
+    __syncthreads();
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(TNT) k_chol_small(const EigProblem* probs, int pass) {
+  const EigProblem P = probs[blockIdx.x];
   const int R = P.R;
-  double* z = P.z + (int64_t)i * R;
-  const double* L = P.gram;
-  for (int c = 0; c < R; ++c) {
-    double s = z[c];
-    for (int q = 0; q < c; ++q) s = fma(-L[(int64_t)c * R + q], z[q], s);
-    z[c] = s / L[(int64_t)c * R + c];
+  if (R > CS || P.info[0] || (pass > 0 && !P.info[1])) return;
+  __shared__ double sm[CS][CS + 1];
+  __shared__ double s_r, isq[CS];
+  double* Gm = P.gram;
+  bool far = false;
+  for (int e = threadIdx.x; e < R * R; e += TNT) {
+    const int i = e / R, j = e - i * R;
+    const double g = Gm[e];
+    sm[i][j] = j <= i ? g : 0.0;
+    far |= far_from_identity(g, i == j, R);
+  }
+  if (pass == 0 && __syncthreads_or(far) && threadIdx.x == 0) P.info[1] = 1;
+  __syncthreads();
+  if (!eliminate(sm, R, &s_r)) {
+    if (threadIdx.x == 0) P.info[0] = 1;
+    return;
+  }
+  if (threadIdx.x < R) isq[threadIdx.x] = 1.0 / sqrt(sm[threadIdx.x][threadIdx.x]);
+  __syncthreads();
+  for (int e = threadIdx.x; e < R * R; e += TNT) {
+    const int i = e / R, j = e - i * R;
+    Gm[e] = j > i ? 0.0 : (j == i ? isq[i] : isq[i] * sm[j][i]);
+  }
+  if (threadIdx.x < 32) {
+    double lo = INFINITY, hi = 0.0;            // of the pivots' 1 / sqrt
+    for (int c = threadIdx.x; c < R; c += 32) { lo = fmin(lo, isq[c]); hi = fmax(hi, isq[c]); }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if (threadIdx.x == 0 && lo < 1e-6 * hi) P.info[0] = 2;
+  }
+}
+
+// Q = Z L^-T, eight rows of Z per CTA (x) and problem (y), R <= 64.
+constexpr int AR = 8;
+__global__ void __launch_bounds__(TNT) k_apply_small(const EigProblem* probs, int pass) {
+  const EigProblem P = probs[blockIdx.y];
+  const int R = P.R, i0 = blockIdx.x * AR;
+  if (R > CS || i0 >= P.n || P.info[0] || (pass > 0 && !P.info[1])) return;
+  __shared__ double ws[CS][CS + 1], zs[AR][CS + 1];
+  for (int e = threadIdx.x; e < R * R; e += TNT) ws[e / R][e % R] = P.gram[e];
+  const int nr = min(AR, P.n - i0);
+  for (int e = threadIdx.x; e < nr * R; e += TNT) zs[e / R][e % R] = P.z[(int64_t)i0 * R + e];
+  __syncthreads();
+  const int r = threadIdx.x >> 5;
+  if (r >= nr) return;
+  for (int c = threadIdx.x & 31; c < R; c += 32) {
+    double s0 = 0.0, s1 = 0.0;
+    int k = 0;
+    for (; k + 1 <= c; k += 2) {
+      s0 = fma(zs[r][k], ws[c][k], s0);
+      s1 = fma(zs[r][k + 1], ws[c][k + 1], s1);
+    }
+    if (k <= c) s0 = fma(zs[r][k], ws[c][k], s0);
+    P.z[(int64_t)(i0 + r) * R + c] = s0 + s1;
+  }
+}
+
+// R > 64: is G far from the identity (first pass)?
+__global__ void __launch_bounds__(TNT) k_chol_far(const EigProblem* P_) {
+  const EigProblem P = *P_;
+  const int64_t R = P.R;
+  bool far = false;
+  for (int64_t e = (int64_t)blockIdx.x * TNT + threadIdx.x; e < R * R; e += (int64_t)gridDim.x * TNT)
+    far |= far_from_identity(P.gram[e], e / R == e % R, (int)R);
+  if (__syncthreads_or(far) && threadIdx.x == 0) P.info[1] = 1;
+}
+
+// Diagonal block p: L_pp^-1 in place (lower); its pivots' 1 / sqrt into P.lu (free
+// by now); the last block checks the condition.
+__global__ void __launch_bounds__(TNT) k_chol_diag(const EigProblem* P_, int p, int pass) {
+  const EigProblem P = *P_;
+  if (P.info[0] || (pass > 0 && !P.info[1])) return;
+  __shared__ double sm[CS][CS + 1];
+  __shared__ double s_r, isq[CB], red[2][TNW];
+  const int R = P.R, c0 = p * CB, m = min(CB, R - c0);
+  for (int e = threadIdx.x; e < m * m; e += TNT) {
+    const int i = e / m, j = e - i * m;
+    sm[i][j] = j <= i ? P.gram[(int64_t)(c0 + i) * R + c0 + j] : 0.0;
+  }
+  __syncthreads();
+  if (!eliminate(sm, m, &s_r)) {
+    if (threadIdx.x == 0) P.info[0] = 1;
+    return;
+  }
+  if (threadIdx.x < m) {
+    isq[threadIdx.x] = 1.0 / sqrt(sm[threadIdx.x][threadIdx.x]);
+    P.lu[c0 + threadIdx.x] = isq[threadIdx.x];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < m * m; e += TNT) {
+    const int i = e / m, j = e - i * m;
+    P.gram[(int64_t)(c0 + i) * R + c0 + j] = j > i ? 0.0 : (j == i ? isq[i] : isq[i] * sm[j][i]);
+  }
+  if (c0 + m < R) return;
+  double lo = INFINITY, hi = 0.0;
+  for (int c = threadIdx.x; c < R; c += TNT) {
+    const double v = c < c0 ? P.lu[c] : isq[c - c0];
+    lo = fmin(lo, v);
+    hi = fmax(hi, v);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = lo; red[1][threadIdx.x >> 5] = hi; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < TNW; ++w) { lo = fmin(lo, red[0][w]); hi = fmax(hi, red[1][w]); }
+    if (lo < 1e-6 * hi) P.info[0] = 2;
+  }
+}
+
+// acc[q] += sum_k a[row][k] b[col][k], a thread's 4 outputs of a 32 x 32 tile:
+// row = threadIdx.x / 8, columns threadIdx.x % 8 + 8 q.
+__device__ __forceinline__ void tile_dot(const double (*a)[CB + 1], const double (*b)[CB + 1],
+                                         double (&acc)[4]) {
+  const int row = threadIdx.x >> 3, col = threadIdx.x & 7;
+#pragma unroll 8
+  for (int k = 0; k < CB; ++k) {
+    const double v = a[row][k];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = fma(v, b[col + 8 * q][k], acc[q]);
+  }
+}
+// Loads the 32 x 32 tile at (r0, c0) of the R x R matrix (zero outside).
+__device__ __forceinline__ void tile_load(const double* G, int64_t R, int64_t r0, int64_t c0,
+                                          double (*t)[CB + 1]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int row = (threadIdx.x >> 5) + 8 * q, col = threadIdx.x & 31;
+    t[row][col] = (r0 + row < R && c0 + col < R) ? G[(r0 + row) * R + c0 + col] : 0.0;
+  }
+}
+
+// L_ip = G_ip L_pp^-T, block i = p + 1 + blockIdx.x.
+__global__ void __launch_bounds__(TNT) k_chol_panel(const EigProblem* P_, int p, int pass) {
+  const EigProblem P = *P_;
+  if (P.info[0] || (pass > 0 && !P.info[1])) return;
+  __shared__ double a[CB][CB + 1], b[CB][CB + 1];
+  const int64_t R = P.R, r0 = (int64_t)(p + 1 + blockIdx.x) * CB, c0 = (int64_t)p * CB;
+  tile_load(P.gram, R, r0, c0, a);
+  tile_load(P.gram, R, c0, c0, b);
+  __syncthreads();
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  tile_dot(a, b, acc);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int64_t row = r0 + (threadIdx.x >> 3), col = c0 + (threadIdx.x & 7) + 8 * q;
+    if (row < R && col < R) P.gram[row * R + col] = acc[q];
+  }
+}
+
+// G_ij -= L_ip L_jp^T, blocks i >= j > p (blockIdx.x: the lower triangle in row order).
+__global__ void __launch_bounds__(TNT) k_chol_trail(const EigProblem* P_, int p, int pass) {
+  const EigProblem P = *P_;
+  if (P.info[0] || (pass > 0 && !P.info[1])) return;
+  __shared__ double a[CB][CB + 1], b[CB][CB + 1];
+  const int t = (int)blockIdx.x;
+  int bi = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+  while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
+  while (bi * (bi + 1) / 2 > t) --bi;
+  const int bj = t - bi * (bi + 1) / 2;
+  const int64_t R = P.R, r0 = (int64_t)(p + 1 + bi) * CB, q0 = (int64_t)(p + 1 + bj) * CB;
+  tile_load(P.gram, R, r0, (int64_t)p * CB, a);
+  tile_load(P.gram, R, q0, (int64_t)p * CB, b);
+  __syncthreads();
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  tile_dot(a, b, acc);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int64_t row = r0 + (threadIdx.x >> 3), col = q0 + (threadIdx.x & 7) + 8 * q;
+    if (row < R && col < R) P.gram[row * R + col] -= acc[q];
+  }
+}
+
+// Q = Z L^-T by blocks of columns, blockDim.x / 32 rows of Z per CTA: Q_p = (Z_p -
+// sum_{q < p} Q_q L_pq^T) L_pp^-T.  A thread owns one row and one column of the block.
+__global__ void __launch_bounds__(512) k_apply_big(const EigProblem* P_, int pass) {
+  const EigProblem P = *P_;
+  if (P.info[0] || (pass > 0 && !P.info[1])) return;
+  __shared__ double ls[CB][CB + 1], zs[16][CB + 1];
+  const int64_t R = P.R;
+  const int nr = blockDim.x >> 5, r = threadIdx.x >> 5, c = threadIdx.x & 31;
+  const int64_t i = (int64_t)blockIdx.x * nr + r;
+  double* z = P.z + (i < P.n ? i : 0) * R;
+  for (int64_t c0 = 0; c0 < R; c0 += CB) {
+    double acc = (i < P.n && c0 + c < R) ? z[c0 + c] : 0.0;
+    for (int64_t q0 = 0; q0 <= c0; q0 += CB) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < CB * CB; e += blockDim.x) {
+        const int64_t row = c0 + e / CB, col = q0 + e % CB;
+        ls[e / CB][e % CB] = (row < R && col < R) ? P.gram[row * R + col] : 0.0;
+      }
+      zs[r][c] = q0 < c0 ? (i < P.n ? z[q0 + c] : 0.0) : acc;   // (blocks q0 < c0 are whole)
+      __syncthreads();
+      double s = 0.0, t = 0.0;
+#pragma unroll
+      for (int k = 0; k < CB; k += 2) {
+        s = fma(zs[r][k], ls[c][k], s);
+        t = fma(zs[r][k + 1], ls[c][k + 1], t);
+      }
+      acc = q0 < c0 ? acc - (s + t) : s + t;
+    }
+    if (i < P.n && c0 + c < R) z[c0 + c] = acc;
   }
 }
 
@@ -741,7 +967,7 @@ __global__ void __launch_bounds__(256) k_backtransform(const EigProblem* probs, 
   while (p + 1 < nprob && probs[p + 1].zoff <= t) ++p;
   const EigProblem P = probs[p];
   const int j = t - P.zoff;
-  if (j < 0 || j >= P.R || *P.info) return;
+  if (j < 0 || j >= P.R || P.info[0]) return;
   const int n = P.n, R = P.R;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const double* A = P.A;
@@ -783,35 +1009,23 @@ __global__ void __launch_bounds__(256) k_backtransform(const EigProblem* probs, 
 }
 
 // ---------------------------------------------------------------- batched helpers
-// Rank cut of Eq. Un for each problem (one thread each): R = min{R in 1..n :
-// tail(R) <= thr}, tail accumulated from the smallest eigenvalue up (the same
-// order as k_rank_cut), or R = fixed when fixed > 0; disc = tail(R).
-__global__ void k_rank_cut_batched(const EigProblem* probs, int count, const double* thr,
-                                   const int* fixed, int64_t* R_out, double* disc_out) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= count) return;
-  const EigProblem P = probs[p];
-  const int n = P.n;
-  const int fr = fixed ? fixed[p] : 0;
-  double tail = 0.0, best_tail = 0.0;
-  int best = n;
-  for (int R = n - 1; R >= 1; --R) {
-    tail += P.w[R];
-    if (fr > 0 ? (R == fr) : (tail <= thr[p])) { best = R; best_tail = tail; }
-  }
-  if (fr > 0 && fr == n) { best = n; best_tail = 0.0; }
-  R_out[p] = best;
-  disc_out[p] = best_tail;
+// Rank cut of Eq. Un (or the given rank) for each problem, one CTA each.
+__global__ void __launch_bounds__(RANK_CUT_NT) k_rank_cut_batched(const EigProblem* probs,
+                                                                  const double* thr,
+                                                                  const int* fixed, int64_t* R_out,
+                                                                  double* disc_out) {
+  const int p = blockIdx.x;
+  rank_cut_cta(probs[p].w, probs[p].n, thr[p], fixed ? fixed[p] : 0, R_out + p, disc_out + p);
 }
 
 // G = Z^T Z (R x R, full) for each problem with R <= 64, one CTA each: rows of
 // Z staged 16 at a time in shared memory, one thread per lower-triangle entry
 // (several when R(R+1)/2 > 256), FP64 sums in row order.
 constexpr int ZG_MAXR = 64, ZG_ROWS = 16, ZG_PPT = (ZG_MAXR * (ZG_MAXR + 1) / 2 + TNT - 1) / TNT;
-__global__ void __launch_bounds__(TNT) k_zgram_batched(const EigProblem* probs) {
+__global__ void __launch_bounds__(TNT) k_zgram_batched(const EigProblem* probs, int pass) {
   const EigProblem P = probs[blockIdx.x];
   const int n = P.n, R = P.R;
-  if (R > ZG_MAXR || *P.info) return;
+  if (R > ZG_MAXR || P.info[0] || (pass > 0 && !P.info[1])) return;
   __shared__ double zs[ZG_ROWS][ZG_MAXR + 1];
   const int npair = R * (R + 1) / 2;
   int pa[ZG_PPT], pb[ZG_PPT];
@@ -854,16 +1068,16 @@ __global__ void __launch_bounds__(TNT) k_zgram_batched(const EigProblem* probs) 
 cudaError_t launch_rank_cut_batched(const EigProblem* probs_dev, int count, const double* thr,
                                     const int* fixed, int64_t* R_out, double* disc_out,
                                     cudaStream_t st) {
-  k_rank_cut_batched<<<(count + 127) / 128, 128, 0, st>>>(probs_dev, count, thr, fixed, R_out,
-                                                           disc_out);
+  k_rank_cut_batched<<<count, RANK_CUT_NT, 0, st>>>(probs_dev, thr, fixed, R_out, disc_out);
   count_launches(1);
   return cudaGetLastError();
 }
 
 int zgram_batched_max_r() { return ZG_MAXR; }
 
-cudaError_t launch_zgram_batched(const EigProblem* probs_dev, int count, cudaStream_t st) {
-  k_zgram_batched<<<count, TNT, 0, st>>>(probs_dev);
+cudaError_t launch_zgram_batched(const EigProblem* probs_dev, int count, int pass,
+                                 cudaStream_t st) {
+  k_zgram_batched<<<count, TNT, 0, st>>>(probs_dev, pass);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -951,16 +1165,39 @@ cudaError_t launch_invit(const EigProblem* probs_dev, int count, int total_vecto
   return cudaGetLastError();
 }
 
-cudaError_t launch_chol(const EigProblem* probs_dev, int count, cudaStream_t st) {
-  k_chol<<<count, TNT, 0, st>>>(probs_dev);
-  count_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_trsm_rows(const EigProblem* probs_dev, int count, int total_rows, cudaStream_t st) {
-  if (total_rows < 1) return cudaSuccess;
-  k_trsm_rows<<<(total_rows + 127) / 128, 128, 0, st>>>(probs_dev, count);
-  count_launches(1);
+cudaError_t launch_cholqr(const EigProblem* probs_dev, const EigProblem* probs_host, int count,
+                          int pass, int num_sms, cudaStream_t st) {
+  int nmax = 0;
+  for (int p = 0; p < count; ++p)
+    if (probs_host[p].R <= CS) nmax = probs_host[p].n > nmax ? probs_host[p].n : nmax;
+  if (nmax > 0) {
+    k_chol_small<<<count, TNT, 0, st>>>(probs_dev, pass);
+    k_apply_small<<<dim3((nmax + AR - 1) / AR, count), TNT, 0, st>>>(probs_dev, pass);
+    count_launches(2);
+  }
+  for (int p = 0; p < count; ++p) {
+    const int R = probs_host[p].R, n = probs_host[p].n;
+    if (R <= CS) continue;
+    const EigProblem* pd = probs_dev + p;
+    if (pass == 0) {
+      k_chol_far<<<(int)std::min<int64_t>(((int64_t)R * R + TNT - 1) / TNT, num_sms), TNT, 0, st>>>(pd);
+      count_launches(1);
+    }
+    const int nb = (R + CB - 1) / CB;
+    for (int b = 0; b < nb; ++b) {
+      const int rest = nb - 1 - b;
+      k_chol_diag<<<1, TNT, 0, st>>>(pd, b, pass);
+      if (rest > 0) {
+        k_chol_panel<<<rest, TNT, 0, st>>>(pd, b, pass);
+        k_chol_trail<<<rest * (rest + 1) / 2, TNT, 0, st>>>(pd, b, pass);
+      }
+      count_launches(rest > 0 ? 3 : 1);
+    }
+    // one wave of CTAs where that leaves at most 16 rows each
+    const int rows = std::max(4, std::min(16, (n + num_sms - 1) / num_sms));
+    k_apply_big<<<(n + rows - 1) / rows, 32 * rows, 0, st>>>(pd, pass);
+    count_launches(1);
+  }
   return cudaGetLastError();
 }
 

@@ -1,0 +1,51 @@
+"""The truncated eigensolve's Cholesky QR at the edges of its blocks (one CTA
+up to 64 vectors, then blocks of 32), with well separated eigenvalues (one
+pass) and with clusters (two passes): orthonormal vectors and small residuals."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1901_06043_gb300 import tucker
+    c = tucker.Context()
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("clustered", [False, True])
+@pytest.mark.parametrize("n,R", [(5, 1), (33, 31), (40, 32), (70, 33), (100, 63), (100, 64),
+                                 (100, 65), (200, 96), (200, 97), (300, 161), (257, 257)])
+def test_vectors_are_orthonormal_eigenvectors(ctx, n, R, clustered):
+    import torch
+    rng = np.random.default_rng(n + R)
+    Q, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    lam = np.sort(10.0 ** np.linspace(0, -6, n))[::-1]
+    if clustered:                       # runs of three within 1e-9 of each other
+        lam = lam[(np.arange(n) // 3) * 3] * (1 + 1e-9 * (np.arange(n) % 3))
+        lam = np.sort(lam)[::-1]
+    S = (Q * lam) @ Q.T
+    S = (S + S.T) / 2
+    w, U, k, _ = ctx.eig_trunc(torch.from_numpy(S).cuda(), R=R)
+    w, U = w.cpu().numpy(), U.cpu().numpy()
+    assert k == R and np.abs(w - lam).max() <= 1e-13 * n
+    assert np.abs(U.T @ U - np.eye(R)).max() <= 1e-13 * n
+    assert np.abs(S @ U - U * w[:R]).max() <= 1e-13 * n
+
+
+@pytest.mark.parametrize("n", [1, 2, 127, 128, 129, 1023, 1024, 1025, 2500])
+def test_rank_cut_sums_in_order(ctx, n):
+    """Bitwise the sequential sum from the smallest value up, also across the
+    kernel's chunks of 1024."""
+    import torch
+    rng = np.random.default_rng(n)
+    w = np.sort(10.0 ** rng.uniform(-12, 0, n))[::-1] * np.where(np.arange(n) > n // 2, -1.0, 1.0)
+    tail = np.zeros(n + 1)
+    for i in range(n - 1, -1, -1):
+        tail[i] = tail[i + 1] + w[i]
+    for thr in (0.0, abs(tail[n // 3]), 1e-6, 10.0 * n):
+        R, d = ctx.rank_cut(torch.from_numpy(w).cuda(), thr)
+        want = next(r for r in range(1, n + 1) if tail[r] <= thr)
+        assert (R, d) == (want, tail[want])
