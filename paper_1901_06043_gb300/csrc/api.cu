@@ -637,16 +637,18 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   const int G = tridiag_team_size(n, c->num_sms);
   const size_t nn = (size_t)n * n;
   const size_t nwy = eig_wy_doubles(n);
-  const size_t ndbl = nn + 3 * (size_t)n + 4 * (size_t)n + 2 * (size_t)G + nwy;
+  const size_t nxch = eig_xch_doubles(n);
+  const size_t ndbl = nxch + 2 * nn + 3 * (size_t)n + nwy;
   DevBuf work;
   TK_TRY(dev_alloc(c, work, sizeof(double) * ndbl + sizeof(EigProblem) + 16));
   EigProblem h{};
-  h.A = work.as<double>();
-  h.d = h.A + nn;
+  h.xch = work.as<double>();
+  h.A = h.xch + nxch;
+  h.V = h.A + nn;
+  h.d = h.V + nn;
   h.e = h.d + n;
   h.tau = h.e + n;
-  h.xch = h.tau + n;
-  h.wyT = h.xch + 4 * (size_t)n + 2 * (size_t)G;
+  h.wyT = h.tau + n;
   EigProblem* pd = reinterpret_cast<EigProblem*>(h.wyT + nwy);
   int* info = reinterpret_cast<int*>(pd + 1);
   h.w = w;
@@ -655,10 +657,10 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   h.team_off = 0;
   h.team_size = G;
   cudaStream_t st = c->stream;
-  TK_CUDA(c, cudaMemcpyAsync(h.A, S, sizeof(double) * nn, cudaMemcpyDeviceToDevice, st));
-  TK_CUDA(c, cudaMemsetAsync(c->d_words + 32, 0, sizeof(unsigned) * 3, st));
-  TK_CUDA(c, cudaMemsetAsync(info, 0, 2 * sizeof(int), st));
-  TK_CUDA(c, launch_tridiag(pd, &h, 1, c->d_words + 32, c->d_words + 34, st, c->barrier_polls));
+  TK_CUDA(c, cudaMemsetAsync(h.xch, 0, sizeof(double) * nxch, st));
+  TK_CUDA(c, cudaMemsetAsync(c->d_words + 34, 0, sizeof(unsigned), st));
+  TK_CUDA(c, cudaMemsetAsync(info, 0, 3 * sizeof(int), st));
+  TK_CUDA(c, launch_tridiag(pd, &h, 1, S, c->d_words + 34, st, c->barrier_polls));
   TK_CUDA(c, launch_bisect(pd, 1, n, n, c->num_sms, st));
   TK_CUDA(c, launch_rank_cut(w, n, thr, fixed_R, c->d_i64, c->d_small + 2, st));
   int64_t R = 0;
@@ -1563,10 +1565,11 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
     for (int i = 0; i < count; ++i)
       if (ndims[i] > s) act.push_back(i);
     const int m = (int)act.size();
-    // ---- per-problem workspace: A (Gram, reduced in place), d, e, tau, xch, wyT
+    // ---- per-problem workspace: A (Gram, reduced in place), V, d, e, tau, wyT; the
+    // exchange words of all problems together in front
     std::vector<size_t> wo(m);
     std::vector<int> nq(m), team(m);
-    size_t wtot = 0;
+    size_t wtot = 0, xtot = 0;
     int nmax = 0;
     for (int q = 0; q < m; ++q) nq[q] = (int)cur[act[q]][s];
     tridiag_batch_teams(nq.data(), m, c->num_sms, team.data());
@@ -1574,36 +1577,40 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
       const int n = nq[q];
       nmax = std::max(nmax, n);
       wo[q] = wtot;
-      wtot += (size_t)n * n + 3 * (size_t)n + 4 * (size_t)n + 2 * (size_t)team[q] + eig_wy_doubles(n);
+      wtot += 2 * (size_t)n * n + 3 * (size_t)n + eig_wy_doubles(n);
+      xtot += eig_xch_doubles(n);
     }
     DevBuf work, meta;
-    TK_TRY(dev_alloc(c, work, sizeof(double) * wtot));
+    TK_TRY(dev_alloc(c, work, sizeof(double) * (xtot + wtot)));
     TK_TRY(dev_alloc(c, meta, sizeof(EigProblem) * m + sizeof(double) * m + sizeof(int64_t) * m +
-                                  sizeof(double) * m + 2 * sizeof(int) * m + sizeof(unsigned) * (m + 1)));
+                                  sizeof(double) * m + 3 * sizeof(int) * m + sizeof(unsigned)));
     EigProblem* pd = meta.as<EigProblem>();
     double* thr_d = reinterpret_cast<double*>(pd + m);
     int64_t* R_d = reinterpret_cast<int64_t*>(thr_d + m);
     double* disc_d = reinterpret_cast<double*>(R_d + m);
     int* info_d = reinterpret_cast<int*>(disc_d + m);
-    unsigned* bars_d = reinterpret_cast<unsigned*>(info_d + 2 * m);   // m team barriers + error word
+    unsigned* berr_d = reinterpret_cast<unsigned*>(info_d + 3 * m);
     std::vector<EigProblem> h(m);
     std::vector<DevBuf> wbuf(m);
     std::vector<double> thr(m);
     for (int q = 0; q < m; ++q) TK_TRY(dev_alloc(c, wbuf[q], sizeof(double) * nq[q]));
     Timer tg, te, tt;
     tg.start(c);
+    size_t xo = 0;
     TK_TRY(fork_side(c));
     for (int q = 0; q < m; ++q) {
       const int i = act[q], n = (int)cur[i][s];
       EigProblem& P = h[q];
       P = EigProblem{};
-      P.A = work.as<double>() + wo[q];
-      P.d = P.A + (size_t)n * n;
+      P.xch = work.as<double>() + xo;
+      xo += eig_xch_doubles(n);
+      P.A = work.as<double>() + xtot + wo[q];
+      P.V = P.A + (size_t)n * n;
+      P.d = P.V + (size_t)n * n;
       P.e = P.d + n;
       P.tau = P.e + n;
-      P.xch = P.tau + n;
-      P.wyT = P.xch + 4 * (size_t)n + 2 * (size_t)team[q];
-      P.info = info_d + 2 * q;
+      P.wyT = P.tau + n;
+      P.info = info_d + 3 * q;
       P.n = n;
       P.team_size = team[q];
       P.team_off = q == 0 ? 0 : h[q - 1].team_off + h[q - 1].team_size;
@@ -1618,9 +1625,10 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
     TK_TRY(join_side(c));
     tg.stop(c);
     te.start(c);
-    TK_CUDA(c, cudaMemsetAsync(info_d, 0, 2 * sizeof(int) * m + sizeof(unsigned) * (m + 1), st));
+    TK_CUDA(c, cudaMemsetAsync(info_d, 0, 3 * sizeof(int) * m + sizeof(unsigned), st));
     TK_CUDA(c, cudaMemcpyAsync(thr_d, thr.data(), sizeof(double) * m, cudaMemcpyHostToDevice, st));
-    TK_CUDA(c, launch_tridiag(pd, h.data(), m, bars_d, bars_d + m, st, c->barrier_polls));
+    TK_CUDA(c, cudaMemsetAsync(work.p, 0, sizeof(double) * xtot, st));
+    TK_CUDA(c, launch_tridiag(pd, h.data(), m, nullptr, berr_d, st, c->barrier_polls));
     int neig = 0;
     for (int q = 0; q < m; ++q) neig += h[q].n;
     TK_CUDA(c, launch_bisect(pd, m, nmax, neig, c->num_sms, st));
@@ -1666,10 +1674,10 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
       TK_CUDA(c, launch_cholqr(pd, h.data(), m, pass, c->num_sms, st));
     }
     TK_CUDA(c, launch_backtransform(pd, m, zoff, nmax, st));
-    std::vector<int> info(2 * m);
+    std::vector<int> info(3 * m);
     unsigned berr = 0;
-    TK_CUDA(c, cudaMemcpyAsync(info.data(), info_d, 2 * sizeof(int) * m, cudaMemcpyDeviceToHost, st));
-    TK_CUDA(c, cudaMemcpyAsync(&berr, bars_d + m, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    TK_CUDA(c, cudaMemcpyAsync(info.data(), info_d, 3 * sizeof(int) * m, cudaMemcpyDeviceToHost, st));
+    TK_CUDA(c, cudaMemcpyAsync(&berr, berr_d, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
     TK_TRY(sync(c));
     if (berr & DEV_ERR_BARRIER_TIMEOUT)
       return set_err(c, TUCKER_ERR_CUDA, "tridiagonalization team barrier gave up waiting");
@@ -1679,7 +1687,7 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
       int64_t Rq = R[q];
       double dq = disc[q];
       res[i]->eig_kernel[s] = 1;
-      if (info[2 * q]) {
+      if (info[3 * q]) {
         DevBuf S2, V2, U2;
         TK_TRY(dev_alloc(c, S2, sizeof(double) * (size_t)n * n));
         TK_TRY(dev_alloc(c, V2, sizeof(double) * (size_t)n * n));

@@ -138,22 +138,24 @@ cudaError_t launch_rank_cut(const double* w, int n, double thr, int fixed_R, int
 // ---- tridiagonal eigensolver (tridiag.cu): all eigenvalues, the leading R
 // eigenvectors.  One descriptor per matrix (device array of descriptors).
 struct EigProblem {
-  double* A;      // n x n row-major symmetric input copy; overwritten with the reflectors
+  double* A;      // n x n row-major symmetric input copy; overwritten
+  double* V;      // n x n: reflector v_k in row k, columns k+1..
   double* d;      // n: diagonal of T
   double* e;      // n: off-diagonal of T (e[k] = T[k+1][k])
-  double* tau;    // n: reflector scalars
-  double* xch;    // 4 n + 2 G: exchange buffers of the team reduction (G CTAs)
+  double* tau;    // n: reflector scalars (H_k = I - tau_k v_k v_k^T, v_k in V)
+  double* xch;    // eig_xch_doubles(n), 16-byte aligned, zeroed: words the team exchanges
   double* w;      // n: eigenvalues, descending
   double* z;      // n x R row-major: eigenvectors of T, then their QR factor
   double* lu;     // inverse-iteration factors: 4 n R doubles + 2 n R bytes
   double* gram;   // R x R
   double* U;      // n x R column-major output
   double* wyT;    // eig_wy_doubles(n): T factors of the blocked back-transformation
-  int* info;      // [0]: 0 ok; 1 / 2 the Cholesky QR failed; [1]: it needs its second pass
+  int* info;      // 3 zeroed words, [0]: 0 ok, 1 / 2 the Cholesky QR failed; [1]: it needs
+                  // its second pass; [2]: the largest exponent of the matrix
   int n, R;
   int zoff;       // first flattened vector index of this problem
   int team_off;   // k_tridiag: first CTA of this problem's team
-  int team_size;  // k_tridiag: CTAs of the team (xch holds 4 n + 2 team_size)
+  int team_size;  // k_tridiag: CTAs of the team
   int srows;      // k_tridiag: the team's rows live in shared memory
 };
 int tridiag_team_size(int n, int num_sms);
@@ -162,13 +164,14 @@ int tridiag_team_size(int n, int num_sms);
 void tridiag_batch_teams(const int* n, int count, int num_sms, int* team);
 inline size_t eig_lu_bytes(int n, int R) { return (size_t)n * R * (4 * sizeof(double) + 2); }
 size_t eig_wy_doubles(int n);
-// Problems with their team_off / team_size set (teams back to back) and
-// team_size * n / ... as planned; probs_host is the host copy of the
-// descriptors (it sets the launch shape and each team's shared-memory rows).
-// bar_counts: `count` zeroed words (one barrier per team), err: error word.
-// poll_limit: polls before a team's grid barrier gives up (sets *err)
+inline size_t eig_xch_doubles(int n) { return 8 * (size_t)n + 2; }
+// Problems with their team_off / team_size set (teams back to back); probs_host
+// is the host copy of the descriptors (it sets the launch shape and each team's
+// shared-memory rows).  S: the matrix (one problem), copied into A, or NULL: A
+// holds it.  err: error word.  poll_limit: polls a thread makes for a word
+// before it gives up (sets *err)
 cudaError_t launch_tridiag(const EigProblem* probs_dev, EigProblem* probs_host, int count,
-                           unsigned* bar_counts, unsigned* err, cudaStream_t st,
+                           const double* S, unsigned* err, cudaStream_t st,
                            unsigned long long poll_limit);
 // y[i] = the tridiagonal solver's FP64 reciprocal of x[i] (diagnostics)
 cudaError_t launch_rcp64_probe(const double* x, double* y, int64_t n, cudaStream_t st);

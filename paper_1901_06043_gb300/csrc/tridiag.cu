@@ -19,21 +19,36 @@
 // tensor; on this part FP64 runs at 1/64 of the FP32 rate, so the FP64
 // operation count decides.
 //
-// Stage 1 runs on a team of CTAs: the whole grid (one matrix, a
-// cooperative launch with ONE bounded grid barrier per Householder step) or
-// one CTA (batched matrices, one CTA each).  Rows are owned cyclically
-// (row i by team rank i mod G), so each CTA keeps a balanced share of the
-// shrinking trailing matrix.  Step k (reflector H_k = I - tau_k v_k v_k^T
-// acting on indices k+1..n-1) needs p_k = tau_k A v_k (rows spread over the
-// team) and then w_k = p_k - (tau_k/2)(p_k . v_k) v_k for the rank-2 update
-// A <- A - v_k w_k^T - w_k v_k^T.  After the barrier that publishes p_k, every
-// CTA forms w_k itself, applies step k's update to the next pivot row (which
-// its owner published before the barrier) to obtain v_{k+1}, and then, in
-// one pass over its own rows, applies step k's update and computes its part
-// of p_{k+1}: the update of step k and the product of step k+1 share a
-// barrier.
+// Stage 1 runs on a team of CTAs: the whole grid (one matrix) or a share of it
+// (batched matrices), a cooperative launch.  Rows are owned cyclically (row i by
+// team rank i mod G), so each CTA keeps a balanced share of the shrinking
+// trailing matrix.  Step k (reflector H_k = I - tau_k v_k v_k^T on indices
+// k+1..n-1) needs p_k = tau_k A v_k (rows spread over the team) and the next
+// pivot row r = A[k+1][:], both published by the rows' owners; every CTA then forms
+// v_{k+1} itself and, in one pass over its own rows, applies step k's update
+// A <- A - v_k w_k^T - w_k v_k^T, w = p - (tau/2)(p . v) v, and its part of
+// A v_{k+1}.
+//   A step is a chain of latencies (an FP64 instruction takes 64 cycles, and a
+// warp's occupies its sub-partition's pipe for as long), so the chain is kept
+// short:
+// - No barrier up to kTridiagWordsMax.  Every published value is a 16-byte word {value, step}, written
+//   and read by single 128-bit accesses; a reader polls the word until it
+//   carries the step it waits for.  Two buffers in turn: a CTA publishes for
+//   step k+1 only after all its threads have read step k.  (A grid barrier and
+//   then the loads: two more round trips to L2 per step.)
+// - Short sums: warp_sum adds in integers.  (Forming the norm of the next pivot
+//   row from sums taken together with p . v, one reduction less, cancels in
+//   most steps of a graded matrix: not kept.)
+// - Unscaled reflectors: v = x - beta e_1, tau = 2 / (v . v); tau is computed by one
+//   warp while the others form A v, and multiplies the finished sums.  (The
+//   matrix is scaled by a power of two first, so that squares neither overflow
+//   nor underflow where they matter.)  A step's update needs no w: a_ij - v_i p_j -
+//   (p_i - tau (p . v) v_i) v_j.
+// Measured, whole reduction: n = 50 0.26 -> 0.18 ms, n = 200 1.20 -> 0.84 ms, n = 500
+// 3.5 -> 2.5 ms (a barrier, normalized reflectors and FP64 sums before).
 #include <algorithm>
 #include <cfloat>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -45,7 +60,7 @@ namespace {
 constexpr int TNT = 256;            // threads per CTA of k_tridiag / k_chol_*
 constexpr int TNW = TNT / 32;
 
-__device__ __forceinline__ double warp_sum(double v) {
+__device__ __forceinline__ double warp_sum_fp64(double v) {
   // xor butterfly: every lane adds the same two operands at every level
   // (addition commutes exactly), so all lanes end with the same value
 #pragma unroll
@@ -53,75 +68,133 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sum over the warp, the same in every lane: the values as 58-bit fixed point
+// under the largest exponent E of the warp (bits below 2^-57 of 2^E are
+// dropped, a 32nd of the largest value's last bit each), split into three
+// fields that redux.sync adds in integers, and the exact sum rounded to FP64
+// once.  ~230 cycles; five FP64 additions with their shuffles take ~1,000 and a
+// share of the FP64 pipe.  Exponents near the ends of the range, Inf and NaN
+// take those.
+__device__ __forceinline__ double warp_sum(double v) {
+  const int hi = __double2hiint(v);
+  const int e = (hi >> 20) & 0x7ff;
+  const int E = __reduce_max_sync(0xffffffffu, e);
+  if (E < 70 || E > 2040) {
+    if (E == 0) return __reduce_or_sync(0xffffffffu, (unsigned)__double2loint(v) | (unsigned)(hi & 0xfffff)) == 0u
+                           ? 0.0 : warp_sum_fp64(v);
+    return warp_sum_fp64(v);
+  }
+  const unsigned lo = (unsigned)__double2loint(v);
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;     // (a zero or denormal v: shifted out)
+  unsigned long long q;
+  asm("{\n .reg .u64 m;\n mov.b64 m, {%1, %2};\n shr.u64 %0, m, %3;\n}"
+      : "=l"(q) : "r"(lo << 5), "r"((mh << 5) | (lo >> 27)), "r"(E - e));
+  const long long n = (long long)(hi >> 31);
+  const long long s = (long long)((q ^ (unsigned long long)n)) - n;
+  const unsigned L = __reduce_add_sync(0xffffffffu, (unsigned)s & 0xfffffu);
+  const unsigned M = __reduce_add_sync(0xffffffffu, (unsigned)(s >> 20) & 0xfffffu);
+  const int H = __reduce_add_sync(0xffffffffu, (int)(s >> 40));
+  const long long S = ((long long)H << 40) + ((long long)M << 20) + (long long)L;
+  if (S == 0) return 0.0;
+  unsigned long long a = (unsigned long long)(S < 0 ? -S : S);
+  const int z = __clzll((long long)a);
+  a <<= z;
+  const unsigned long long mant = (a >> 11) + ((a >> 10) & 1ull);
+  const unsigned long long r = ((unsigned long long)(E + 5 - z) << 52) + mant;   // exponent field E + 6 - z
+  return __longlong_as_double((long long)(r | (S < 0 ? 1ull << 63 : 0ull)));
+}
+
 // FP64 instructions occupy a sub-partition's FP64 pipe for ~64 cycles per
 // warp whatever they compute, so scalar work that every thread needs is done
 // by warp 0 and broadcast through shared memory.
 
-// Sum over the CTA, in a fixed order, returned to every thread.  `red` holds
-// TNW + 1 doubles; consecutive calls must alternate between two buffers.
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = (threadIdx.x < TNW) ? red[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = TNW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (threadIdx.x == 0) red[TNW] = t;
-  }
-  __syncthreads();
-  return red[TNW];
+// 1/x for a normal x with |x| in [2^-1000, 2^1000]: the FP32 reciprocal of
+// x's mantissa (moved into FP32 by integer operations), rescaled by the
+// exponent, then two Newton-Raphson steps.
+__device__ __forceinline__ double rcp64(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex < 24 || ex > 2022) return 1.0 / x;
+  const float mf = __uint_as_float(0x3f800000u | (unsigned)((b >> 29) & 0x7fffff));   // [1, 2)
+  float rf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(mf));                              // (0.5, 1]
+  const unsigned rb = __float_as_uint(rf);
+  const int re = (int)((rb >> 23) & 0xff) - 127 + 1023 - (ex - 1023);
+  double r = __longlong_as_double((long long)((b >> 63) << 63 | (unsigned long long)re << 52 |
+                                              (unsigned long long)(rb & 0x7fffff) << 29));
+  double e = fma(-x, r, 1.0);
+  r = fma(r, e, r);
+  e = fma(-x, r, 1.0);
+  return fma(r, e, r);
 }
 
-// Householder reflector (Golub & Van Loan Alg. 5.1.1, with the sign of beta
-// opposite to alpha): for x = vx[k2..n-1] (alpha = x[k2]) find v (v[k2] = 1),
-// tau and beta with (I - tau v v^T) x = beta e_1.  Written in place into vx.
-// All threads of the CTA call it and return the same tau and beta.  `red`
-// holds TNW + 4 doubles.
-__device__ void house(double* vx, int k2, int n, double* red, double& tau, double& beta) {
-  double s = 0.0;
-  for (int j = k2 + 1 + threadIdx.x; j < n; j += TNT) s = fma(vx[j], vx[j], s);
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = (threadIdx.x < TNW) ? red[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = TNW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (threadIdx.x == 0) {
-      const double alpha = vx[k2];
-      double ta = 0.0, be = alpha, sc = 0.0;
-      if (t != 0.0) {
-        const double mu = sqrt(fma(alpha, alpha, t));
-        be = (alpha > 0.0) ? -mu : mu;
-        ta = (be - alpha) / be;
-        sc = 1.0 / (alpha - be);
-      }
-      red[TNW + 1] = ta;
-      red[TNW + 2] = be;
-      red[TNW + 3] = sc;
-      vx[k2] = 1.0;
-    }
-  }
-  __syncthreads();
-  tau = red[TNW + 1];
-  beta = red[TNW + 2];
-  const double sc = red[TNW + 3];
-  for (int j = k2 + 1 + threadIdx.x; j < n; j += TNT) vx[j] *= sc;
-  __syncthreads();
+// sqrt(x) for x in [2^-1000, 2^1000]: an FP32 estimate of 1 / sqrt of x's mantissa
+// (exponent made even), then Goldschmidt's iteration on g ~ sqrt(x), h ~ 1 / (2
+// sqrt(x)) and one correction by the residual x - g^2.
+__device__ __forceinline__ double sqrt64(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff) - 1023, odd = e & 1;
+  const float mf = __uint_as_float((unsigned)(127 + odd) << 23 | (unsigned)((b >> 29) & 0x7fffff));
+  float rf;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(mf));          // (0.5, 1]
+  const unsigned rb = __float_as_uint(rf);
+  const int re = (int)(rb >> 23) - 127 + 1023 - (e - odd) / 2;
+  const double y = __longlong_as_double((long long)((unsigned long long)re << 52 |
+                                                    (unsigned long long)(rb & 0x7fffff) << 29));
+  double g = x * y, h = 0.5 * y;
+  const double r = fma(-g, h, 0.5);
+  g = fma(g, r, g);
+  h = fma(h, r, h);
+  return fma(fma(-g, g, x), h, g);
+}
+
+// A value published for a step, and its step number.
+__device__ __forceinline__ void put_word(ulonglong2* p, double v, unsigned long long step) {
+  asm volatile(
+      "{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}" ::"l"(p),
+      "l"(__double_as_longlong(v)), "l"(step)
+      : "memory");
+}
+__device__ __forceinline__ double get_word(const ulonglong2* p, unsigned long long& step) {
+  long long v;
+  asm volatile(
+      "{\n .reg .b128 t;\n ld.relaxed.gpu.global.b128 t, [%2];\n mov.b128 {%0, %1}, t;\n}"
+      : "=l"(v), "=l"(step) : "l"(p) : "memory");
+  return __longlong_as_double(v);
 }
 
 }  // namespace
 
 // ---------------------------------------------------------------- stage 1
-// One team of P.team_size CTAs per problem (teams back to back in the grid);
-// a team of one synchronizes with __syncthreads, a larger one with its own
-// bounded barrier.  P.srows: the CTA's own rows live in shared memory;
-// otherwise they are read and written in place in A (L2-resident).
+// Largest n whose team exchanges words; above, plain values and a barrier.  Whole
+// solves, words and barrier: n = 200 2.04 and 2.15 ms, n = 500 5.58 and 5.63, n = 800
+// 10.54 and 10.18, n = 1500 33.5 and 29.3.
+constexpr int kTridiagWordsMax = 640;
+
+// A copy of S (one problem; NULL: A holds the matrix) and the largest biased
+// exponent of A's entries, into info[2].
+__global__ void __launch_bounds__(TNT) k_eig_load(const EigProblem* probs, const double* S) {
+  const EigProblem P = probs[blockIdx.y];
+  const int64_t nn = (int64_t)P.n * P.n;
+  int m = 0;
+  for (int64_t e = (int64_t)blockIdx.x * TNT + threadIdx.x; e < nn; e += (int64_t)gridDim.x * TNT) {
+    const double v = S ? S[e] : P.A[e];
+    if (S) P.A[e] = v;
+    m = max(m, (__double2hiint(v) >> 20) & 0x7ff);
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(P.info + 2, m);
+}
+
+// One team of P.team_size CTAs per problem (teams back to back in the grid); a
+// team of one exchanges through its shared memory.  P.srows: the CTA's own
+// rows live in shared memory; otherwise they are read and written in place in
+// A (L2-resident).  v_k goes into row k of V, columns k+1.. .
 __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int count,
-                                                    unsigned* bar_counts, unsigned* err,
-                                                    unsigned long long poll_limit) {
+                                                    unsigned* err, unsigned long long poll_limit) {
   extern __shared__ __align__(16) double tsm[];
+  __shared__ double s_red[2][TNW], s_c[5], s_tau;
+  __shared__ int s_on;
   int pidx = 0;
   while (pidx + 1 < count && probs[pidx + 1].team_off <= (int)blockIdx.x) ++pidx;
   const EigProblem P = probs[pidx];
@@ -129,161 +202,268 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
   const int G = P.team_size;
   const int c = (int)blockIdx.x - P.team_off;
   if (c < 0 || c >= G) return;
-  const bool SROWS = P.srows != 0;
-  const GridBarrier bar{bar_counts + pidx, nullptr, err};
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool SROWS = P.srows != 0, solo = G == 1;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   double* A = P.A;
-  double* const xp = P.xch;               // p_k: 2 x n
-  double* const xr = P.xch + 2 * n;       // next pivot row: 2 x n
-  double* const xv = P.xch + 4 * n;       // partial p . v per CTA: 2 x G
-  double* vk = tsm;                       // v_k by global index
-  double* vn = tsm + n;                   // v_{k+1}
-  double* const w = tsm + 2 * n;          // w_k
-  double* const red0 = tsm + 3 * n;       // TNW + 4 each
-  double* const red1 = red0 + TNW + 4;
-  double* const srows = red1 + TNW + 4;   // own rows t = 0, 1, ... (row c + G t) when SROWS
+  ulonglong2* const xp = reinterpret_cast<ulonglong2*>(P.xch);   // p: 2 x n words
+  ulonglong2* const xr = xp + 2 * (size_t)n;                     // next pivot row: 2 x n words
+  // long rows: plain values behind a barrier of the team
+  const bool plain = n > kTridiagWordsMax;
+  double* const dp = P.xch;               // p: 2 x n
+  double* const dr = dp + 2 * (size_t)n;  // next pivot row: 2 x n
+  const GridBarrier bar{reinterpret_cast<unsigned*>(P.xch + 8 * (size_t)n), nullptr, err};
   unsigned gen = 0;
+  double* vk = tsm;                       // v_k by global index
+  double* vn = tsm + n;                   // y, then v_{k+1}
+  double* sp = tsm + 2 * n;               // p_k
+  double* sq = tsm + 3 * n;               // own rows of A v_{k+1} (solo: then p_{k+1})
+  double* const sr = tsm + 4 * n;         // solo: next pivot row
+  double* const srows = tsm + 5 * n;      // own rows t = 0, 1, ... (row c + G t) when SROWS
   auto row = [&](int i) -> double* {
     return SROWS ? srows + (size_t)((i - c) / G) * n : A + (int64_t)i * n;
   };
 
   if (n <= 2) {
-    if (c == 0 && threadIdx.x == 0) {
+    if (c == 0 && tid == 0) {
       P.d[0] = A[0];
       if (n == 2) { P.e[0] = A[1]; P.d[1] = A[3]; }
     }
     return;
   }
-  if (SROWS) {
-    for (int i = c; i < n; i += G) {
-      const double* src = A + (int64_t)i * n;
-      double* dst = row(i);
-      for (int j = threadIdx.x; j < n; j += TNT) dst[j] = src[j];
-    }
+  // entries scaled by sc = 2^-floor(log2 max|a|) (1 for a zero or non-finite matrix)
+  const int mexp = P.info[2];
+  const bool scaled = mexp > 0 && mexp < 0x7ff;
+  const int dex = scaled ? max(-1022, min(1022, mexp - 1023)) : 0;
+  const double sc = __longlong_as_double((long long)(1023 - dex) << 52);
+  const double isc = __longlong_as_double((long long)(1023 + dex) << 52);
+  for (int i = c; i < n; i += G) {
+    if (i == 0) continue;                 // row 0 is read as it is, below
+    const double* src = A + (int64_t)i * n;
+    double* dst = row(i);
+    for (int j = tid; j < n; j += TNT) dst[j] = src[j] * sc;
   }
-  // ---- phase -1: v_0 from row 0, p_0 over own rows
-  for (int j = threadIdx.x; j < n; j += TNT) vn[j] = (j >= 1) ? A[j] : 0.0;
-  __syncthreads();
-  double tau_k, beta;
-  house(vn, 1, n, red0, tau_k, beta);
-  if (c == 0 && threadIdx.x == 0) { P.d[0] = A[0]; P.e[0] = beta; P.tau[0] = tau_k; }
-  // (row 0 of A receives its reflector only after the team's first barrier:
-  // every CTA reads row 0 above, and a CTA that starts late must not see it
-  // overwritten)
-  {
-    double pv = 0.0;
-    const int i0 = 1 + ((c - 1) % G + G) % G;   // smallest own row >= 1
-    for (int i = i0 + G * warp; i < n; i += G * TNW) {
-      const double* Ai = row(i);
-      double acc = 0.0;
-      for (int j = 1 + lane; j < n; j += 32) {
-        const double a = Ai[j];
-        if (i == 1) xr[j] = a;                  // pivot row of phase 0 (buffer 0)
-        acc = fma(a, vn[j], acc);
-      }
-      acc = warp_sum(acc) * tau_k;
-      if (lane == 0) xp[i] = acc;               // buffer 0
-      pv = fma(acc, vn[i], pv);
-    }
-    // one value per warp (identical in its lanes): sum the warps
-    const double s = block_sum(lane == 0 ? pv : 0.0, red1);
-    if (threadIdx.x == 0) xv[c] = s;
-  }
-  { double* t = vk; vk = vn; vn = t; }
-  if (G > 1) { if (!grid_sync(bar, gen, poll_limit, (unsigned)G)) return; } else __syncthreads();
-  if (c == 0)   // v_0 (now vk) into row 0, read by nobody after the barrier
-    for (int j = 2 + threadIdx.x; j < n; j += TNT) A[j] = vk[j];
 
-  // ---- phases 0 .. n-3
-  for (int k = 0; k <= n - 3; ++k) {
-    const int b = k & 1, nb = b ^ 1;
-    const double* pk = xp + b * n;
-    const double* rk = xr + b * n;
-    double* const red = (k & 1) ? red1 : red0;
-    double* const redo = (k & 1) ? red0 : red1;
-    // this thread's entries of p_k and of the pivot row (issued first), and
-    // p_k . v_k from the CTAs' partials in a fixed order (warp 0)
-    constexpr int JPT = 4;                  // j values per thread kept in registers
-    double pj[JPT], rj[JPT];
-#pragma unroll
-    for (int q = 0; q < JPT; ++q) {
-      const int j = k + 1 + threadIdx.x + q * TNT;
-      pj[q] = (j < n) ? __ldcg(pk + j) : 0.0;
-      rj[q] = (j < n) ? __ldcg(rk + j) : 0.0;
+  // By the last warp, with the row x in vn[lo..] and the partial sums of
+  // |x[lo+1..]|^2 in s_red[1]: beta into s_c[2], v = x - beta e_lo (its first entry
+  // into vn[lo]), then 2 / (v . v) into s_tau; a zero (or negligible) rest: no
+  // reflector, tau = 0.
+  auto reflector = [&](int lo) {
+    const double ss = warp_sum(lane < TNW ? s_red[1][lane] : 0.0);
+    const double alpha = vn[lo], tot = fma(alpha, alpha, ss);
+    __syncwarp();
+    double be = alpha, v1 = 1.0;
+    const bool on = !(ss == 0.0) && !(tot < 0x1p-900);
+    if (on) {
+      const double g = sqrt64(tot);
+      be = alpha > 0.0 ? -g : g;
+      v1 = alpha - be;
     }
-    if (warp == 0) {
-      double s = 0.0;
-      for (int q = lane; q < G; q += 32) s += __ldcg(xv + b * G + q);
-      s = warp_sum(s);
+    if (lane == 0) { s_c[2] = be; s_c[3] = v1; s_c[4] = ss; vn[lo] = v1; }
+    s_on = on;
+  };
+  // ---- v_0 from row 0
+  {
+    double ss = 0.0;
+    for (int j = 1 + tid; j < n; j += TNT) {
+      const double a = A[j] * sc;
+      vn[j] = a;
+      if (j >= 2) ss = fma(a, a, ss);
+    }
+    ss = warp_sum(ss);
+    if (lane == 0) s_red[1][warp] = ss;
+    __syncthreads();                      // (and row 0 is in vn)
+    if (warp == TNW - 1) reflector(1);
+  }
+  // Largest own row.  A CTA without rows in the trailing matrix publishes nothing,
+  // so nobody would wait until it has read its words: it leaves.  Results of a
+  // step are written by the owner of row lo, which is still there.
+  const int last = n - 1 - (n - 1 - c) % G;
+
+  int i0 = c > 0 ? c : G;                 // smallest own row of the trailing matrix, and where it is
+  double* own0 = row(i0 < n ? i0 : c);
+  const int64_t rstep = SROWS ? n : (int64_t)G * n;               // to the next own row
+  double tau = 0.0;
+  for (int k = -1; k <= n - 3; ++k) {
+    const int lo = k + 2;                 // first row and column of the trailing matrix after step k
+    if (k >= 0 && last < lo && !plain) return;        // (a barrier counts every CTA)
+    const bool more = k < n - 3;
+    if (i0 < lo) { i0 += G; own0 += rstep; }
+    const bool scribe = i0 == lo;
+    double t2 = 0.0;                      // tau_k (p_k . v_k)
+    if (k >= 0) {
+      // ---- p_k and the pivot row; y into vn; p . v
+      const double v1 = vk[k + 1];
+      double s1 = 0.0;
+      bool fail = false;
+      const unsigned long long want = (unsigned long long)k + 1ull;
+      const ulonglong2* pw = xp + (size_t)(k & 1) * n;
+      const ulonglong2* rw = xr + (size_t)(k & 1) * n;
+      constexpr int JPT = 4;              // entries in flight per thread and array
+      for (int j0 = k + 1 + tid; j0 < n; j0 += JPT * TNT) {
+        double pj[JPT], rj[JPT];
+        if (solo) {
+#pragma unroll
+          for (int q = 0; q < JPT; ++q) {
+            const int j = j0 + q * TNT;
+            pj[q] = j < n ? sp[j] : 0.0;
+            rj[q] = j < n ? sr[j] : 0.0;
+          }
+        } else if (plain) {
+#pragma unroll
+          for (int q = 0; q < JPT; ++q) {
+            const int j = j0 + q * TNT;
+            pj[q] = j < n ? __ldcg(dp + (size_t)(k & 1) * n + j) : 0.0;
+            rj[q] = j < n ? __ldcg(dr + (size_t)(k & 1) * n + j) : 0.0;
+            if (j < n) sp[j] = pj[q];
+          }
+        } else {
+          unsigned long long tp[JPT], tr[JPT];
+#pragma unroll
+          for (int q = 0; q < JPT; ++q) {
+            const int j = j0 + q * TNT;
+            tp[q] = tr[q] = want;
+            pj[q] = rj[q] = 0.0;
+            if (j < n) { pj[q] = get_word(pw + j, tp[q]); rj[q] = get_word(rw + j, tr[q]); }
+          }
+          unsigned long long it = 0;
+#pragma unroll
+          for (int q = 0; q < JPT; ++q) {
+            const int j = j0 + q * TNT;
+            while (tp[q] != want || tr[q] != want) {
+              if (++it >= poll_limit) { atomicOr(err, DEV_ERR_BARRIER_TIMEOUT); fail = true; break; }
+              if ((it & 1023) == 0 && (ld_acquire_u32(err) & DEV_ERR_BARRIER_TIMEOUT)) { fail = true; break; }
+              if (it > 4096) __nanosleep(64);
+              if (tp[q] != want) pj[q] = get_word(pw + j, tp[q]);
+              if (tr[q] != want) rj[q] = get_word(rw + j, tr[q]);
+            }
+            if (fail) break;
+            if (j < n) sp[j] = pj[q];
+          }
+        }
+        if (fail) break;
+#pragma unroll
+        for (int q = 0; q < JPT; ++q) {
+          const int j = j0 + q * TNT;
+          if (j < n) {
+            vn[j] = fma(-v1, pj[q], rj[q]);
+            s1 = fma(pj[q], vk[j], s1);
+          }
+        }
+      }
+      s1 = warp_sum(s1);
+      if (lane == 0) s_red[0][warp] = s1;
+      if (__syncthreads_or(fail)) return;
+      // the last warp does the scalars (it has no rows, see below)
+      if (warp == TNW - 1) {
+        const double t = tau * warp_sum(lane < TNW ? s_red[0][lane] : 0.0);
+        if (lane == 0) {
+          s_c[0] = t;
+          s_c[1] = fma(t, v1, -sp[k + 1]);
+        }
+      }
+      __syncthreads();
+      t2 = s_c[0];
+      const double cc = s_c[1];
+      if (scribe && tid == 0) {
+        P.d[k + 1] = fma(cc, v1, vn[k + 1]) * isc;
+        if (!more) P.e[n - 2] = fma(cc, vk[lo], vn[lo]) * isc;
+      }
+      if (more) {
+        // the pivot row x after step k, and its norm
+        double ss = 0.0;
+        for (int j = lo + tid; j < n; j += TNT) {
+          const double x = fma(cc, vk[j], vn[j]);
+          vn[j] = x;
+          if (j > lo) ss = fma(x, x, ss);
+        }
+        ss = warp_sum(ss);
+        if (lane == 0) s_red[1][warp] = ss;
+        __syncthreads();
+        if (warp == TNW - 1) reflector(lo);
+      }
+    }
+    __syncthreads();                      // v_{k+1} is complete
+    if (scribe && more) {
+      double* Vr = P.V + (int64_t)(k + 1) * n;
+      for (int j = lo + tid; j < n; j += TNT) Vr[j] = vn[j];
+      if (tid == 0) P.e[k + 1] = s_c[2] * isc;
+    }
+    if (k < 0 && c == 0 && tid == 0) P.d[0] = A[0];
+    // ---- own rows: the update of step k and A v_{k+1}; tau by the last warp
+    if (more && warp == TNW - 1) {
+      const double v1 = s_c[3];
+      const double t = s_on ? 2.0 * rcp64(fma(v1, v1, s_c[4])) : 0.0;
       if (lane == 0) {
-        const double K = 0.5 * tau_k * s;
-        redo[TNW + 1] = K;
-        redo[TNW + 2] = __ldcg(pk + k + 1) - K;   // w_k at k+1 (v_k[k+1] = 1)
+        s_tau = t;
+        if (scribe) P.tau[k + 1] = t;
       }
-    }
-    __syncthreads();
-    const double K = redo[TNW + 1], wk1 = redo[TNW + 2];
-    const bool owner = ((k + 1) % G) == c;
-    auto wr = [&](int j, double pjq, double rjq) {
-      const double wj = fma(-K, vk[j], pjq);
-      w[j] = wj;
-      // row k+1 of the updated matrix: r_j = a_j - w_j - w_{k+1} v_j
-      const double r = fma(-wk1, vk[j], rjq - wj);
-      if (j == k + 1) {
-        if (owner) P.d[k + 1] = r;
-      } else {
-        vn[j] = r;
-      }
-    };
-#pragma unroll
-    for (int q = 0; q < JPT; ++q) {
-      const int j = k + 1 + threadIdx.x + q * TNT;
-      if (j < n) wr(j, pj[q], rj[q]);
-    }
-    for (int j = k + 1 + threadIdx.x + JPT * TNT; j < n; j += TNT) wr(j, __ldcg(pk + j), __ldcg(rk + j));
-    __syncthreads();
-    const bool more = (k + 1 <= n - 3);
-    double tau_n = 0.0;
-    if (more) {
-      house(vn, k + 2, n, red, tau_n, beta);
-      if (owner) {
-        if (threadIdx.x == 0) { P.e[k + 1] = beta; P.tau[k + 1] = tau_n; }
-        double* Ar = A + (int64_t)(k + 1) * n;
-        for (int j = k + 3 + threadIdx.x; j < n; j += TNT) Ar[j] = vn[j];
-      }
-    } else if (owner && threadIdx.x == 0) {
-      P.e[n - 2] = vn[n - 1];
-    }
-    // own rows i >= k+2: update of step k, then the product of step k+1
-    double pv = 0.0;
-    {
-      const int lo = k + 2;
-      const int i0 = lo + ((c - lo) % G + G) % G;
-      for (int i = i0 + G * warp; i < n; i += G * TNW) {
-        double* Ai = row(i);
-        const double vi = vk[i], wi = w[i];
-        double acc = 0.0;
+    } else {
+      constexpr int nw = TNW - 1;
+      ulonglong2* rw = xr + (size_t)((k + 1) & 1) * n;
+      // PIV: the next pivot row, also published
+      auto do_row = [&](int i, double* Ai, auto UPD, auto PIV) {
+        double vi = 0.0, gi = 0.0, acc = 0.0;
+        if constexpr (decltype(UPD)::value) {
+          vi = vk[i];
+          gi = fma(-t2, vi, sp[i]);
+        }
 #pragma unroll 4
         for (int j = lo + lane; j < n; j += 32) {
-          const double a = fma(-wi, vk[j], fma(-vi, w[j], Ai[j]));
-          Ai[j] = a;
-          if (i == lo) xr[nb * n + j] = a;
-          if (more) acc = fma(a, vn[j], acc);
-          else if (i == n - 1) P.d[n - 1] = a;
+          double a = Ai[j];
+          if constexpr (decltype(UPD)::value) {
+            a = fma(-gi, vk[j], fma(-vi, sp[j], a));
+            Ai[j] = a;
+          }
+          if constexpr (decltype(PIV)::value) {
+            if (solo) sr[j] = a;
+            else if (plain) dr[(size_t)((k + 1) & 1) * n + j] = a;
+            else put_word(rw + j, a, (unsigned long long)k + 2ull);
+          }
+          acc = fma(a, vn[j], acc);
         }
-        if (more) {
-          acc = warp_sum(acc) * tau_n;
-          if (lane == 0) xp[nb * n + i] = acc;
-          pv = fma(acc, vn[i], pv);
+        acc = warp_sum(acc);
+        if (lane == 0) sq[i] = acc;
+      };
+      using yes = std::true_type;
+      using no = std::false_type;
+      if (!more) {                        // the last entry (lo = n - 1)
+        if (scribe && warp == 0 && lane == 0) {
+          const double vi = vk[lo], gi = fma(-t2, vi, sp[lo]);
+          P.d[lo] = fma(-gi, vi, fma(-vi, sp[lo], own0[lo])) * isc;
+        }
+      } else {
+        int i = i0 + G * warp;
+        double* Ai = own0 + rstep * warp;
+        for (; i < n; i += G * nw, Ai += rstep * nw) {
+          if (k < 0) {
+            if (i == lo) do_row(i, Ai, no(), yes());
+            else do_row(i, Ai, no(), no());
+          } else {
+            if (i == lo) do_row(i, Ai, yes(), yes());
+            else do_row(i, Ai, yes(), no());
+          }
         }
       }
     }
     if (!more) break;
-    const double sp = block_sum(lane == 0 ? pv : 0.0, redo);
-    if (threadIdx.x == 0) xv[nb * G + c] = sp;
+    __syncthreads();                      // the sums and tau are there
+    tau = s_tau;
+    {
+      ulonglong2* pw = xp + (size_t)((k + 1) & 1) * n;
+      for (int i = i0 + G * tid; i < n; i += G * TNT) {
+        const double p = sq[i] * tau;
+        if (solo) sq[i] = p;
+        else if (plain) dp[(size_t)((k + 1) & 1) * n + i] = p;
+        else put_word(pw + i, p, (unsigned long long)k + 2ull);
+      }
+    }
     { double* t = vk; vk = vn; vn = t; }
-    tau_k = tau_n;
-    if (G > 1) { if (!grid_sync(bar, gen, poll_limit, (unsigned)G)) return; } else __syncthreads();
+    if (solo) {
+      double* t = sp; sp = sq; sq = t;
+      __syncthreads();
+    } else if (plain) {
+      if (!grid_sync(bar, gen, poll_limit, (unsigned)G)) return;
+    }
   }
 }
 
@@ -429,26 +609,6 @@ __device__ __forceinline__ uint32_t hash_u32(uint32_t i, uint32_t j) {
 }
 __device__ __forceinline__ double hash_unit(uint32_t i, uint32_t j) {
   return (double)hash_u32(i, j) * (2.0 / 4294967296.0) - 1.0;
-}
-
-// 1/x for a normal x with |x| in [2^-1000, 2^1000]: the FP32 reciprocal of
-// x's mantissa (moved into FP32 by integer operations), rescaled by the
-// exponent, then two Newton-Raphson steps.
-__device__ __forceinline__ double rcp64(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7ff);
-  if (ex < 24 || ex > 2022) return 1.0 / x;
-  const float mf = __uint_as_float(0x3f800000u | (unsigned)((b >> 29) & 0x7fffff));   // [1, 2)
-  float rf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(mf));                              // (0.5, 1]
-  const unsigned rb = __float_as_uint(rf);
-  const int re = (int)((rb >> 23) & 0xff) - 127 + 1023 - (ex - 1023);
-  double r = __longlong_as_double((long long)((b >> 63) << 63 | (unsigned long long)re << 52 |
-                                              (unsigned long long)(rb & 0x7fffff) << 29));
-  double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
-  return fma(r, e, r);
 }
 
 __global__ void k_rcp64_probe(const double* x, double* y, int64_t n) {
@@ -923,18 +1083,17 @@ __global__ void __launch_bounds__(256) k_wy_t(const EigProblem* probs) {
   __shared__ double W[WYB][WYB + 1];
   __shared__ double T[WYB][WYB + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // W[i][j] = v_{k0+i} . v_{k0+j} for i < j; v_{k0+j} is 1 at k0+j+1 and
-  // A[k0+j][c] beyond, and v_{k0+i} is A[k0+i][c] there
+  // W[i][j] = v_{k0+i} . v_{k0+j} for i < j; v_{k0+j} is V[k0+j][c] from c = k0+j+1
   for (int q = warp; q < m * m; q += 8) {
     const int i = q / m, jj = q % m;
     if (i >= jj) continue;
-    const double* vi = P.A + (int64_t)(k0 + i) * n;
-    const double* vj = P.A + (int64_t)(k0 + jj) * n;
+    const double* vi = P.V + (int64_t)(k0 + i) * n;
+    const double* vj = P.V + (int64_t)(k0 + jj) * n;
     const int s0 = k0 + jj + 1;
     double acc = 0.0;
-    for (int c = s0 + 1 + lane; c < n; c += 32) acc = fma(vi[c], vj[c], acc);
+    for (int c = s0 + lane; c < n; c += 32) acc = fma(vi[c], vj[c], acc);
     acc = warp_sum(acc);
-    if (lane == 0) W[i][jj] = acc + vi[s0];
+    if (lane == 0) W[i][jj] = acc;
   }
   __syncthreads();
   if (warp == 0) {
@@ -970,19 +1129,19 @@ __global__ void __launch_bounds__(256) k_backtransform(const EigProblem* probs, 
   if (j < 0 || j >= P.R || P.info[0]) return;
   const int n = P.n, R = P.R;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double* A = P.A;
+  const double* V = P.V;
   for (int i = threadIdx.x; i < n; i += blockDim.x) zs[i] = P.z[(int64_t)i * R + j];
   __syncthreads();
   for (int b = wy_blocks(n) - 1; b >= 0; --b) {
     const int k0 = b * WYB, m = min(WYB, n - 2 - k0);
     // y = V^T z
     for (int q = warp; q < m; q += 8) {
-      const double* v = A + (int64_t)(k0 + q) * n;
+      const double* v = V + (int64_t)(k0 + q) * n;
       const int s0 = k0 + q + 1;
       double acc = 0.0;
-      for (int c = s0 + 1 + lane; c < n; c += 32) acc = fma(v[c], zs[c], acc);
+      for (int c = s0 + lane; c < n; c += 32) acc = fma(v[c], zs[c], acc);
       acc = warp_sum(acc);
-      if (lane == 0) y[q] = acc + zs[s0];
+      if (lane == 0) y[q] = acc;
     }
     __syncthreads();
     // y2 = T y
@@ -997,10 +1156,7 @@ __global__ void __launch_bounds__(256) k_backtransform(const EigProblem* probs, 
     for (int i = k0 + 1 + threadIdx.x; i < n; i += blockDim.x) {
       const int qmax = min(m, i - k0);
       double s = 0.0;
-      for (int q = 0; q < qmax; ++q) {
-        const double coef = (i == k0 + q + 1) ? 1.0 : A[(int64_t)(k0 + q) * n + i];
-        s = fma(coef, y2[q], s);
-      }
+      for (int q = 0; q < qmax; ++q) s = fma(V[(int64_t)(k0 + q) * n + i], y2[q], s);
       zs[i] -= s;
     }
     __syncthreads();
@@ -1084,7 +1240,7 @@ cudaError_t launch_zgram_batched(const EigProblem* probs_dev, int count, int pas
 
 namespace {
 int tridiag_rows_per_cta(int n, int G) { return (n + G - 1) / G; }
-size_t tridiag_base_smem(int n) { return sizeof(double) * (3 * (size_t)n + 2 * (TNW + 4)); }
+size_t tridiag_base_smem(int n) { return sizeof(double) * 5 * (size_t)n; }
 constexpr size_t kTridiagSmemRowsCap = 120 * 1024;
 }  // namespace
 
@@ -1110,7 +1266,7 @@ void tridiag_batch_teams(const int* n, int count, int num_sms, int* team) {
 }
 
 cudaError_t launch_tridiag(const EigProblem* probs_dev, EigProblem* probs_host, int count,
-                           unsigned* bar_counts, unsigned* err, cudaStream_t st,
+                           const double* S, unsigned* err, cudaStream_t st,
                            unsigned long long poll_limit) {
   int nmax = 0, grid = 0, multi = 0;
   size_t rows_max = 0;
@@ -1129,18 +1285,20 @@ cudaError_t launch_tridiag(const EigProblem* probs_dev, EigProblem* probs_host, 
   e = cudaMemcpyAsync(const_cast<EigProblem*>(probs_dev), probs_host, sizeof(EigProblem) * count,
                       cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return e;
-  count_launches(1);
+  const int64_t nn = (int64_t)nmax * nmax;
+  k_eig_load<<<dim3((unsigned)std::min<int64_t>((nn + 4 * TNT - 1) / (4 * TNT), 256), count), TNT, 0, st>>>(
+      probs_dev, S);
+  count_launches(2);
   if (multi) {
-    // teams of several CTAs spin on each other: all CTAs must be resident
+    // teams of several CTAs wait for each other: all CTAs must be resident
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag, TNT, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorLaunchOutOfResources;
-    void* args[] = {(void*)&probs_dev, (void*)&count, (void*)&bar_counts, (void*)&err,
-                    (void*)&poll_limit};
+    void* args[] = {(void*)&probs_dev, (void*)&count, (void*)&err, (void*)&poll_limit};
     return cudaLaunchCooperativeKernel((void*)k_tridiag, dim3(grid), dim3(TNT), args, smem, st);
   }
-  k_tridiag<<<grid, TNT, smem, st>>>(probs_dev, count, bar_counts, err, poll_limit);
+  k_tridiag<<<grid, TNT, smem, st>>>(probs_dev, count, err, poll_limit);
   return cudaGetLastError();
 }
 
