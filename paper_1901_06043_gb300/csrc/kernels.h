@@ -142,7 +142,8 @@ struct EigProblem {
   double* V;      // n x n: reflector v_k in row k, columns k+1..
   double* d;      // n: diagonal of T
   double* e;      // n: off-diagonal of T (e[k] = T[k+1][k])
-  double* tau;    // n: reflector scalars (H_k = I - tau_k v_k v_k^T, v_k in V)
+  double* tau;    // n: reflector scalars (H_k = I - tau_k v_k v_k^T, v_k in V); tau[n - 1]
+                  // holds ||T|| after the bisection
   double* xch;    // eig_xch_doubles(n), 16-byte aligned, zeroed: words the team exchanges
   double* w;      // n: eigenvalues, descending
   double* z;      // n x R row-major: eigenvectors of T, then their QR factor

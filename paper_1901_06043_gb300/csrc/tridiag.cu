@@ -472,143 +472,209 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
 // changes in the leading principal minors p_0 = 1, p_1, ..., p_n of T - x I,
 // from the three-term recurrence p_i = (d_{i-1} - x) p_{i-1} -
 // e_{i-2}^2 p_{i-2} (Wilkinson, The Algebraic Eigenvalue Problem, Ch. 5: the
-// computed signs are exact for a matrix within a few ulps of T).  No
-// division: three FP64 operations a step (a division costs ~7 FMAs here).
-// T arrives scaled by a power of two to entries of magnitude <= 1, so the
-// minors grow by at most ~3 per step: both are rescaled by a power of two
-// when their exponents leave [-256, 256], tested every 8 steps.  An exact
-// zero minor becomes -sign(previous) 2^-600 (integer operations only), the
-// counterpart of the -pivmin safeguard of the ratio form; with e_i != 0 the
-// count is then the same as with the zero counted either way.
+// computed signs are exact for a matrix within a few ulps of T).  The FP64 pipe
+// takes 64 cycles per warp instruction, so the recurrence is scaled to two of
+// them a step: with q_i = p_i / c_i, c_i = e_{i-2}^2 c_{i-2}, it reads
+// q_i = (d_{i-1} - x) r_i q_{i-1} - q_{i-2}, r_i = c_{i-1} / c_i, and (d - x) r is one FMA
+// of d r and r.  c_i > 0, so the signs are those of p_i, and each coefficient
+// is off by a few ulps, as rounding does to T's entries.
+//   The c start at 1 every SB = 8 steps.  T arrives scaled by a power of two to
+// entries of magnitude <= 1, and e_i^2 below 2^-112 counts as 2^-112 (e_i = 2^-56:
+// below the rounding of entries of magnitude 1), so c >= 2^-448.  In 8 steps the
+// larger of two neighbouring |p| grows by at most 3^8 and, solving the
+// recurrence for p_{i-2}, falls by at most (3 2^112)^8 < 2^909; it is set to about
+// 1 (a power of two) at the end of the 8, so nothing overflows or vanishes.  One
+// of the pair may be 0, exactly or by underflow: the next q is then minus the one
+// before it, and one sign change is counted whichever sign the zero has.
+//   Per step: one shared load, two FMAs and a shift of the sign into a register,
+// whose changes are counted by 8 at the block's end; ~210 cycles a step, of which
+// the FP64 pipe 160 (the block's rescale included).  n = 200 397 -> 203 us,
+// n = 1500 4.97 -> 2.62 ms against (d - x) p - e^2 p with a test for zero and a sign
+// count in each step.
+constexpr int SB = 8;
 __device__ __forceinline__ int exp_bits(double v) {
   return (int)((__double_as_longlong(v) >> 52) & 0x7ff);
 }
-__device__ __forceinline__ double nonzero_or_tiny(double pn, double pc) {
-  const long long b = __double_as_longlong(pn);
-  if ((b << 1) != 0) return pn;
-  // -sign(pc) * 2^-600
-  const long long t = (~__double_as_longlong(pc) & (long long)0x8000000000000000ull) |
-                      ((long long)(1023 - 600) << 52);
-  return __longlong_as_double(t);
-}
-__device__ __forceinline__ int sturm_count(const double* d, const double* e2, int n, double x) {
-  double pm = 1.0;          // p_{i-1}
-  double pc = nonzero_or_tiny(d[0] - x, 1.0);
-  int cnt = (int)((unsigned long long)__double_as_longlong(pc) >> 63);
-  int i = 1;
-  while (i < n) {
-    const int iend = min(n, i + 8);
-#pragma unroll 8
-    for (; i < iend; ++i) {
-      const double pn = nonzero_or_tiny(fma(d[i] - x, pc, -e2[i - 1] * pm), pc);
-      cnt += (int)(((unsigned long long)(__double_as_longlong(pn) ^ __double_as_longlong(pc))) >> 63);
-      pm = pc;
-      pc = pn;
-    }
-    const int em = max(exp_bits(pc), exp_bits(pm));
-    if (em > 1023 + 256 || em < 1023 - 256) {
-      const double f = __longlong_as_double((long long)(2046 - em) << 52);   // 2^(1023 - em)
-      pc *= f;
-      pm *= f;
-    }
+// t[i] = {d_i r_{i+1}, r_{i+1}}, c[b] = the last two c of block b of SB steps
+__device__ __forceinline__ int sturm_count(const double2* t, const double2* c, int n, double x) {
+  double pm = 0.0, pc = 1.0;          // q_{i-1}, q_i
+  unsigned sg = 0;                    // signs of the q, the last in bit 0
+  int cnt = 0;
+  // a step ahead: the coefficient, two steps ahead: the table (both padded)
+  double a = fma(-x, t[0].y, t[0].x);
+  double2 v = t[1];
+  auto step = [&](int i) {
+    const double pn = fma(a, pc, -pm);
+    a = fma(-x, v.y, v.x);
+    v = t[i + 2];
+    sg = __funnelshift_l((unsigned)__double2hiint(pn), sg, 1);
+    pm = pc;
+    pc = pn;
+  };
+  int i = 0;
+  for (; i + SB <= n; i += SB) {
+#pragma unroll
+    for (int q = 0; q < SB; ++q) step(i + q);
+    cnt += __popc((sg ^ (sg >> 1)) & ((1u << SB) - 1u));
+    const double2 cb = c[i / SB];
+    pm *= cb.x;
+    pc *= cb.y;
+    const int em = min(max(max(exp_bits(pc), exp_bits(pm)), 1), 2045);
+    const double f = __longlong_as_double((long long)(2046 - em) << 52);     // 2^(1023 - em)
+    pc *= f;
+    pm *= f;
   }
-  return cnt;
+  const int rest = n - i;
+  for (; i < n; ++i) step(i);
+  return cnt + __popc((sg ^ (sg >> 1)) & ((1u << rest) - 1u));
 }
 
-// Bisection by multisection: L lanes (1 <= L <= 32, a power of two) work on
-// one eigenvalue, each round counting at L interior points of [lo, hi] and
-// keeping the sub-interval that holds eigenvalue number a (ascending), until
-// its width is below 2 eps ||T|| (the accuracy of the counts).  A warp issues
-// one FP64 instruction per step whatever its lanes do, so L trades rounds
-// (53 / log2(L + 1)) against warps: wide L for a few eigenvalues, narrow L for
-// many.  CTA = BNW warps of one problem.
+// Doubles as integers of the same order, and back.
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
+}
+__device__ __forceinline__ double from_key(long long k) {
+  return __longlong_as_double(k ^ (long long)((unsigned long long)(k >> 63) >> 1));
+}
+
+// Bisection by multisection: L lanes (a power of two up to 128: up to four
+// warps) work on one eigenvalue, each round counting at L interior points of
+// [lo, hi] and keeping the sub-interval that holds eigenvalue number a
+// (ascending), until its width is below 2 eps ||T|| (the accuracy of the
+// counts).  A warp issues one FP64 instruction per step whatever its lanes do, so
+// L trades rounds (53 / log2(L + 1)) against warps: wide L for a few
+// eigenvalues, narrow L for many.  CTA = BNW warps of one problem.
 constexpr int BNW = 4;
 __global__ void __launch_bounds__(BNW * 32) k_bisect(const EigProblem* probs, int L) {
   extern __shared__ __align__(16) double bsm[];
   const EigProblem P = probs[blockIdx.y];
   const int n = P.n;
-  const int per_warp = 32 / L;
-  const int per_cta = BNW * per_warp;
+  const int per_cta = BNW * 32 / L;
   if ((int)blockIdx.x * per_cta >= n) return;
-  double* d = bsm;
-  double* e2 = bsm + n;
-  __shared__ double s_lo[BNW * 32], s_hi[BNW * 32];
-  double glo = INFINITY, ghi = -INFINITY;
+  double2* t = reinterpret_cast<double2*>(bsm);        // {d r, r}
+  double2* tc = t + n + 2;                             // the last two c per SB steps
+  if (threadIdx.x < 2) t[n + threadIdx.x] = make_double2(0.0, 0.0);
+  __shared__ long long s_lo[BNW], s_hi[BNW];
+  __shared__ int s_first[BNW];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // Gershgorin's bounds
+  long long klo = 0x7fffffffffffffffll, khi = -0x7fffffffffffffffll;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const double di = P.d[i];
-    const double el = (i > 0) ? fabs(P.e[i - 1]) : 0.0;
-    const double er = (i < n - 1) ? fabs(P.e[i]) : 0.0;
-    glo = fmin(glo, di - el - er);
-    ghi = fmax(ghi, di + el + er);
+    const double r = (i > 0 ? fabs(P.e[i - 1]) : 0.0) + (i < n - 1 ? fabs(P.e[i]) : 0.0);
+    klo = min(klo, order_key(di - r));
+    khi = max(khi, order_key(di + r));
   }
-  s_lo[threadIdx.x] = glo;
-  s_hi[threadIdx.x] = ghi;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    klo = min(klo, __shfl_xor_sync(0xffffffffu, klo, o));
+    khi = max(khi, __shfl_xor_sync(0xffffffffu, khi, o));
+  }
+  if (lane == 0) { s_lo[warp] = klo; s_hi[warp] = khi; }
   __syncthreads();
-  for (int i = 0; i < BNW * 32; ++i) {
-    glo = fmin(glo, s_lo[i]);
-    ghi = fmax(ghi, s_hi[i]);
-  }
+  for (int w = 0; w < BNW; ++w) { klo = min(klo, s_lo[w]); khi = max(khi, s_hi[w]); }
+  double glo = from_key(klo), ghi = from_key(khi);
   const double tnorm = fmax(fabs(glo), fabs(ghi));
   // scale by 2^-ex (exact) so that ||T|| / 2^ex is in [0.5, 1)
   const int ex = (tnorm > 0.0) ? exp_bits(tnorm) - 1022 : 0;
   const double sc = __longlong_as_double((long long)(1023 - ex) << 52);
   const double isc = __longlong_as_double((long long)(1023 + ex) << 52);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    d[i] = P.d[i] * sc;
-    if (i < n - 1) { const double ei = P.e[i] * sc; e2[i] = ei * ei; }
+  for (int b0 = threadIdx.x * SB; b0 < n; b0 += blockDim.x * SB) {
+    double ca = 1.0, cb = 1.0;                         // c_{i-2}, c_{i-1}
+#pragma unroll
+    for (int q = 0; q < SB; ++q) {
+      const int i = b0 + q;
+      if (i < n) {
+        const double ei = i > 0 ? P.e[i - 1] * sc : 1.0;
+        const double e2 = ei * ei;
+        const double c = ca * (e2 > 0x1p-112 ? e2 : 0x1p-112);
+        const double r = cb * rcp64(c);
+        t[i] = make_double2(P.d[i] * sc * r, r);
+        ca = cb;
+        cb = c;
+      }
+    }
+    tc[b0 / SB] = make_double2(ca, cb);
   }
   __syncthreads();
   const double tn = tnorm * sc;
   const double atol = 2.0 * DBL_EPSILON * tn + DBL_MIN;
   glo = glo * sc - (2.0 * DBL_EPSILON * tn * n + DBL_MIN);
   ghi = ghi * sc + (2.0 * DBL_EPSILON * tn * n + DBL_MIN);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane / L, l = lane % L;                         // group, lane in group
-  const int j = blockIdx.x * per_cta + warp * per_warp + g;     // descending index
+  const int g = threadIdx.x / L, l = threadIdx.x % L;           // group, lane in group
+  const int j = blockIdx.x * per_cta + g;                       // descending index
   const bool valid = j < n;
   const int a = n - 1 - (valid ? j : n - 1);                    // ascending index
-  const unsigned gmask = (L == 32) ? 0xffffffffu : (((1u << L) - 1u) << (g * L));
+  const double part = 1.0 / (double)(L + 1);
   double lo = glo, hi = ghi;
-  for (int round = 0; round < 64; ++round) {
-    const bool active = valid && (hi - lo > atol);
-    if (!__any_sync(0xffffffffu, active)) break;
-    const double x = lo + (hi - lo) * ((double)(l + 1) / (double)(L + 1));
-    const int cnt = active ? sturm_count(d, e2, n, x) : 0;
-    const unsigned above = __ballot_sync(0xffffffffu, active && cnt > a) & gmask;
-    const int m = above ? (__ffs(above) - 1 - g * L) : L;      // first point above, in group
-    const double xm = __shfl_sync(0xffffffffu, x, g * L + (m < L ? m : L - 1));
-    const double xl = __shfl_sync(0xffffffffu, x, g * L + (m > 0 ? m - 1 : 0));
-    if (active) {
-      if (m < L) hi = xm;
-      if (m > 0) lo = xl;
+  auto point = [&](int m) { return fma(hi - lo, (double)(m + 1) * part, lo); };
+  if (L <= 32) {
+    const int base = lane & ~(L - 1);
+    const unsigned gmask = (L == 32) ? 0xffffffffu : (((1u << L) - 1u) << base);
+    for (int round = 0; round < 64; ++round) {
+      const bool active = valid && (hi - lo > atol);
+      if (!__any_sync(0xffffffffu, active)) break;
+      const int cnt = active ? sturm_count(t, tc, n, point(l)) : 0;
+      const unsigned above = __ballot_sync(0xffffffffu, active && cnt > a) & gmask;
+      const int m = above ? (__ffs(above) - 1 - base) : L;       // first point above, in group
+      if (active) {
+        const double xm = point(m), xl = point(m - 1);
+        if (m < L) hi = xm;
+        if (m > 0) lo = xl;
+      }
+    }
+  } else {
+    const int wpg = L / 32, w0 = warp - warp % wpg;
+    for (int round = 0; round < 64; ++round) {
+      const bool active = valid && (hi - lo > atol);
+      if (!__syncthreads_or(active)) break;
+      const int cnt = active ? sturm_count(t, tc, n, point(l)) : 0;
+      const unsigned above = __ballot_sync(0xffffffffu, active && cnt > a);
+      if (lane == 0) s_first[warp] = above ? __ffs(above) - 1 : 32;
+      __syncthreads();
+      int m = L;
+      for (int w = wpg - 1; w >= 0; --w)
+        if (s_first[w0 + w] < 32) m = 32 * w + s_first[w0 + w];
+      if (active) {
+        const double xm = point(m), xl = point(m - 1);
+        if (m < L) hi = xm;
+        if (m > 0) lo = xl;
+      }
     }
   }
   if (valid && l == 0) P.w[j] = 0.5 * (lo + hi) * isc;
+  if (blockIdx.x == 0 && threadIdx.x == 0) P.tau[n - 1] = tnorm;      // for k_invit
 }
 
 // ---------------------------------------------------------------- stage 4
-// Inverse iteration, one thread per wanted eigenvector: Gaussian elimination
-// with partial pivoting of T - lambda I (a tridiagonal; U gets a second
-// superdiagonal from the row swaps), then two solves, the first from a
-// pseudo-random right-hand side, each followed by normalization.  Pivots
-// below eps ||T|| are raised to that size (the shift is an eigenvalue, so
-// one pivot is ~0); a running power-of-two rescale (|z| <= 2^400, so the
-// sum of squares stays finite) keeps the back substitution finite.  Output
-// column j of Z (n x R, row-major: Z[i*R + j]).
-//
-// The factorization runs fused with the first forward elimination, and the
-// pivots are stored as reciprocals, so the only reciprocal on the dependent
-// chain is the factorization's; it is an FP32 seed refined by two
-// Newton-Raphson steps r <- r (2 - x r) in FP64 (quadratic convergence:
-// 2^-23 -> 2^-46 -> below FP64 rounding), ~5 dependent FP64 operations
-// against ~7 for a full division.
+// Inverse iteration: Gaussian elimination with partial pivoting of T - lambda I,
+// then two solves, the first from a pseudo-random right-hand side.  Two lanes
+// per wanted eigenvector: one eliminates from the first row down, the other
+// from the last row up ("burning at both ends"), the 2 x 2 system where they
+// meet gives the two middle entries, and both substitute back outwards, so the
+// dependent chain is n / 2 steps long.  In local indices (s = 0 at the lane's end)
+// both lanes run the same code; a row swap gives U a second superdiagonal.
+// Pivots below eps ||T|| are raised to that size (the shift is an eigenvalue, so
+// one pivot is ~0); a running power-of-two rescale (|z| <= 2^400, so the sum of
+// squares stays finite) keeps the back substitution finite.  Output column j
+// of Z (n x R, row-major: Z[i*R + j]), a unit vector.
+//   The FP64 pipe is the limit (a warp instruction takes 64 cycles of it whatever
+// its lanes do), so what need not be FP64 is not: the right-hand side's bits
+// are hashed directly, pivots are compared as integers, nothing is scaled
+// that need not be.  18 FP64 instructions a step, n / 2 steps: 186 us at n = 200, 489 us at
+// n = 500 (34 and n with one lane per vector: 371 and 975 us).  The factorization runs
+// fused with the first forward elimination, and the pivots are stored as
+// reciprocals (rcp64), so the only reciprocal on the chain is the factorization's.
 __device__ __forceinline__ uint32_t hash_u32(uint32_t i, uint32_t j) {
   uint32_t h = i * 0x9E3779B1u ^ (j + 0x7F4A7C15u) * 0x85EBCA77u;
   h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
   return h;
 }
+// +-[1, 2)
 __device__ __forceinline__ double hash_unit(uint32_t i, uint32_t j) {
-  return (double)hash_u32(i, j) * (2.0 / 4294967296.0) - 1.0;
+  const uint32_t h = hash_u32(i, j);
+  return __hiloint2double((int)(0x3ff00000u | (h & 0x800fffffu)), (int)(h * 0x9E3779B1u));
 }
 
 __global__ void k_rcp64_probe(const double* x, double* y, int64_t n) {
@@ -616,172 +682,217 @@ __global__ void k_rcp64_probe(const double* x, double* y, int64_t n) {
   if (i < n) y[i] = rcp64(x[i]);
 }
 
-__global__ void k_invit(const EigProblem* probs, int nprob) {
-  // flattened (problem, vector): probs[p].zoff is the first thread of p
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32) k_invit(const EigProblem* probs, int nprob, int total) {
+  // flattened (problem, vector): probs[p].zoff is the first vector of p; lanes
+  // 0-15 from the top, 16-31 from the bottom (past the last vector: no rows)
+  const bool up = threadIdx.x >= 16;
+  const int tv = (int)(blockIdx.x * 16 + (threadIdx.x & 15)), t = min(tv, total - 1);
   int p = 0;
   while (p + 1 < nprob && probs[p + 1].zoff <= t) ++p;
   const EigProblem P = probs[p];
   const int j = t - P.zoff;
-  if (j < 0 || j >= P.R) return;
   const int n = P.n, R = P.R;
+  const int len = tv >= total ? 0 : (up ? n / 2 : n - n / 2);      // rows of this lane
   const double lam = P.w[j];
-  const double* __restrict__ d = P.d;
-  const double* __restrict__ e = P.e;
-  double* __restrict__ RI = P.lu;                        // 1 / pivot
+  const double* __restrict__ d = P.d + (up ? n - 1 : 0);
+  const double* __restrict__ e = P.e + (up ? n - 2 : 0);
+  const int dir = up ? -1 : 1;
+  const int64_t o0 = (int64_t)(up ? n - 1 : 0) * R + j, step = (int64_t)dir * R;
+  double* __restrict__ RI = P.lu + o0;                   // 1 / pivot
   double* __restrict__ U1 = RI + (int64_t)n * R;
   double* __restrict__ U2 = U1 + (int64_t)n * R;
   double* __restrict__ M = U2 + (int64_t)n * R;
-  unsigned char* __restrict__ flag = reinterpret_cast<unsigned char*>(M + (int64_t)n * R);
+  unsigned char* __restrict__ flag = reinterpret_cast<unsigned char*>(P.lu + 4 * (int64_t)n * R) + o0;
   unsigned char* __restrict__ scnt = flag + (int64_t)n * R;
-  double* __restrict__ Z = P.z;
-  auto at = [&](int k) { return (int64_t)k * R + j; };
-  // ||T||_1 bound for the pivot floor
-  double tn = 0.0;
-  for (int i = 0; i < n; ++i) {
-    const double r = fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i < n - 1 ? fabs(e[i]) : 0.0);
-    tn = fmax(tn, r);
-  }
-  const double ptol = fmax(DBL_EPSILON * tn, 0x1p-990);
+  double* __restrict__ Z = P.z + o0;
+  auto at = [&](int s) { return s * step; };
+  const double ptol = fmax(DBL_EPSILON * P.tau[n - 1], 0x1p-990);      // tau[n - 1]: ||T|| (k_bisect)
   const unsigned long long ptol_bits = (unsigned long long)__double_as_longlong(ptol);
   auto absb = [](double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
   };
-  // factorization fused with the forward elimination of b (random); y -> Z
-  double p0 = d[0] - lam, p1 = (n > 1) ? e[0] : 0.0;
-  double pb = hash_unit(0, j);
-  for (int k = 0; k + 1 < n; ++k) {
-    const double ek = e[k];
-    const double a1 = d[k + 1] - lam;
-    const double e1 = (k + 2 < n) ? e[k + 1] : 0.0;
-    const double bk1 = hash_unit(k + 1, j);
-    const bool swap = absb(ek) > absb(p0);
-    if (!swap && absb(p0) < ptol_bits) p0 = (p0 < 0.0) ? -ptol : ptol;
-    const double piv = swap ? ek : p0;
-    const double r = rcp64(piv);
-    const double m = (swap ? p0 : ek) * r;
-    RI[at(k)] = r;
-    U1[at(k)] = swap ? a1 : p1;
-    U2[at(k)] = swap ? e1 : 0.0;
-    M[at(k)] = m;
-    flag[at(k)] = swap ? 1 : 0;
-    double yk;
+  auto floored = [&](double v) { return absb(v) < ptol_bits ? (v < 0.0 ? -ptol : ptol) : v; };
+  // factorization fused with the forward elimination of b (random); y -> Z.
+  // The pending row is p0 z(s) + p1 z(s + 1) = pb.
+  double p0 = 1.0, p1 = 0.0, pb = 0.0;
+  if (len > 0) {
+    p0 = d[0] - lam;
+    p1 = n > 1 ? e[0] : 0.0;
+    pb = hash_unit(up ? n - 1 : 0, j);
+  }
+  for (int s = 0; s + 1 < len; ++s) {
+    const double es = e[dir * s];
+    const double a1 = d[dir * (s + 1)] - lam;
+    // (local s + 1 couples to s + 2, at the end to the other lane's last row)
+    const int ie = up ? n - 2 - (s + 1) : s + 1;
+    const double e1 = ie >= 0 && ie < n - 1 ? e[dir * (s + 1)] : 0.0;
+    const double bs1 = hash_unit(up ? n - 2 - s : s + 1, j);
+    const bool swap = absb(es) > absb(p0);
+    if (!swap) p0 = floored(p0);
+    const double r = rcp64(swap ? es : p0);
+    const double m = (swap ? p0 : es) * r;
+    RI[at(s)] = r;
+    U1[at(s)] = swap ? a1 : p1;
+    U2[at(s)] = swap ? e1 : 0.0;
+    M[at(s)] = m;
+    flag[at(s)] = swap ? 1 : 0;
+    double ys;
     if (swap) {
-      yk = bk1;
-      pb = fma(-m, bk1, pb);
+      ys = bs1;
+      pb = fma(-m, bs1, pb);
       p0 = fma(-m, a1, p1);
       p1 = -m * e1;
     } else {
-      yk = pb;
-      pb = fma(-m, pb, bk1);
+      ys = pb;
+      pb = fma(-m, pb, bs1);
       p0 = fma(-m, p1, a1);
       p1 = e1;
     }
-    Z[at(k)] = yk;
+    Z[at(s)] = ys;
   }
-  if (absb(p0) < ptol_bits) p0 = (p0 < 0.0) ? -ptol : ptol;
-  RI[at(n - 1)] = rcp64(p0);
-  U1[at(n - 1)] = 0.0;
-  U2[at(n - 1)] = 0.0;
-  Z[at(n - 1)] = pb;
+  // The 2 x 2 system of the two pending rows, unknowns (top's last, bottom's
+  // last), factored once, the same in both lanes.
+  double t0, t1, b0, b1;
+  {
+    const double q0 = __shfl_xor_sync(0xffffffffu, p0, 16), q1 = __shfl_xor_sync(0xffffffffu, p1, 16);
+    t0 = up ? q0 : p0;  t1 = up ? q1 : p1;                // top's row
+    b0 = up ? p1 : q1;  b1 = up ? p0 : q0;                // bottom's row, same unknowns
+    if (n == 1) { t1 = 0.0; b0 = 0.0; b1 = 1.0; }
+  }
+  const bool mswap = absb(b0) > absb(t0);
+  const double piv = floored(mswap ? b0 : t0), piv_x = mswap ? b1 : t1;
+  const double rp = rcp64(piv), mm = (mswap ? t0 : b0) * rp;
+  const double rq = rcp64(floored(fma(-mm, piv_x, mswap ? t1 : b1)));
   const double SMALL = 0x1p-400;
-  double bscale = 1.0;
+  // (1 / pivot may be near overflow: the first solution is scaled to about 1)
+  const bool tiny = P.tau[n - 1] < 0x1p-400;
+  double ss = 0.0;
+  int nres = 0;
   // the passes below prefetch the operands of the next PF steps into
   // registers before working through the current ones, which keeps the L2
   // latency off the dependent chain (each step stores into Z, so the
   // compiler cannot move the next loads ahead by itself)
   constexpr int PF = 8;
   for (int it = 0; it < 2; ++it) {
-    if (it == 1) {
-      // forward elimination of the previous solution (times bscale)
-      double pv = Z[at(0)] * bscale;
+    if (it == 1 && len > 0) {
+      // forward elimination of the previous solution
+      double pv = Z[at(0)];
       double nb_[PF], nm_[PF];
       unsigned char nf_[PF];
-      auto load_f = [&](int k0) {
+      auto load_f = [&](int s0) {
 #pragma unroll
         for (int q = 0; q < PF; ++q) {
-          const int k = k0 + q;
-          const bool ok = k + 1 < n;
-          nb_[q] = ok ? Z[at(k + 1)] : 0.0;
-          nm_[q] = ok ? M[at(k)] : 0.0;
-          nf_[q] = ok ? flag[at(k)] : 0;
+          const int s = s0 + q;
+          const bool ok = s + 1 < len;
+          nb_[q] = ok ? Z[at(s + 1)] : 0.0;
+          nm_[q] = ok ? M[at(s)] : 0.0;
+          nf_[q] = ok ? flag[at(s)] : 0;
         }
       };
       load_f(0);
-      for (int k0 = 0; k0 + 1 < n; k0 += PF) {
+      for (int s0 = 0; s0 + 1 < len; s0 += PF) {
         double cb[PF], cm[PF];
         unsigned char cf[PF];
 #pragma unroll
         for (int q = 0; q < PF; ++q) { cb[q] = nb_[q]; cm[q] = nm_[q]; cf[q] = nf_[q]; }
-        if (k0 + PF + 1 < n) load_f(k0 + PF);
+        if (s0 + PF + 1 < len) load_f(s0 + PF);
 #pragma unroll
         for (int q = 0; q < PF; ++q) {
-          const int k = k0 + q;
-          if (k + 1 < n) {
-            const double bk1 = cb[q] * bscale;
-            double yk;
-            if (cf[q] == 0) { yk = pv; pv = fma(-cm[q], pv, bk1); }
-            else { yk = bk1; pv = fma(-cm[q], bk1, pv); }
-            Z[at(k)] = yk;
+          const int s = s0 + q;
+          if (s + 1 < len) {
+            const double ys = cf[q] ? cb[q] : pv;
+            pv = cf[q] ? fma(-cm[q], cb[q], pv) : fma(-cm[q], pv, cb[q]);
+            Z[at(s)] = ys;
           }
         }
       }
-      Z[at(n - 1)] = pv;
+      pb = pv;
     }
-    // back substitution with rescaling; scnt[i] = rescales before z_i was
+    // the middle entries: z1 this lane's last, z2 the other's
+    double z1, z2;
+    {
+      const double o = __shfl_xor_sync(0xffffffffu, pb, 16);
+      const double bt = up ? o : pb, bb = n == 1 ? 0.0 : (up ? pb : o);
+      const double rhs = mswap ? bb : bt;
+      const double zb = fma(-mm, rhs, mswap ? bt : bb) * rq;          // bottom's last
+      const double zt = fma(-piv_x, zb, rhs) * rp;                    // top's last
+      z1 = up ? zb : zt;
+      z2 = up ? zt : zb;
+    }
+    // back substitution with rescaling; scnt[s] = rescales before z(s) was
     // stored; the sum of squares is kept at the running scale
-    int nres = 0;
+    nres = 0;
     double sc = 1.0;             // 2^(-400 nres): the scale of z1, z2 and zk
-    double z1 = 0.0, z2 = 0.0;   // z_{k+1}, z_{k+2} at the current scale
-    double ss = 0.0;
+    ss = 0.0;
+    if (len > 0) {
+      for (int q = 0; q < 3 && max(absb(z1), absb(z2)) > 0x58F0000000000000ull; ++q) {   // > 2^400
+        z1 *= SMALL; z2 *= SMALL; sc *= SMALL;
+        ++nres;
+      }
+      Z[at(len - 1)] = z1;
+      scnt[at(len - 1)] = (unsigned char)nres;
+      ss = z1 * z1;
+    }
     double ny[PF], n1[PF], n2[PF], nr[PF];
-    auto load_b = [&](int k0) {   // steps k0, k0 - 1, ..., k0 - PF + 1
+    auto load_b = [&](int s0) {   // steps s0, s0 - 1, ..., s0 - PF + 1
 #pragma unroll
       for (int q = 0; q < PF; ++q) {
-        const int k = k0 - q;
-        const bool ok = k >= 0;
-        ny[q] = ok ? Z[at(k)] : 0.0;
-        n1[q] = ok ? U1[at(k)] : 0.0;
-        n2[q] = ok ? U2[at(k)] : 0.0;
-        nr[q] = ok ? RI[at(k)] : 0.0;
+        const int s = s0 - q;
+        const bool ok = s >= 0;
+        ny[q] = ok ? Z[at(s)] : 0.0;
+        n1[q] = ok ? U1[at(s)] : 0.0;
+        n2[q] = ok ? U2[at(s)] : 0.0;
+        nr[q] = ok ? RI[at(s)] : 0.0;
       }
     };
-    load_b(n - 1);
-    for (int k0 = n - 1; k0 >= 0; k0 -= PF) {
+    load_b(len - 2);
+    for (int s0 = len - 2; s0 >= 0; s0 -= PF) {
       double cy[PF], c1[PF], c2[PF], cr[PF];
 #pragma unroll
       for (int q = 0; q < PF; ++q) { cy[q] = ny[q]; c1[q] = n1[q]; c2[q] = n2[q]; cr[q] = nr[q]; }
-      if (k0 - PF >= 0) load_b(k0 - PF);
+      if (s0 - PF >= 0) load_b(s0 - PF);
 #pragma unroll
       for (int q = 0; q < PF; ++q) {
-        const int k = k0 - q;
-        if (k >= 0) {
-          double rr = cy[q] * sc;
-          rr = fma(-c2[q], z2, rr);     // U2 and U1 are 0 past the end
+        const int s = s0 - q;
+        if (s >= 0) {
+          double rr = cy[q];
+          if (nres) rr *= sc;
+          if (absb(c2[q]) != 0) rr = fma(-c2[q], z2, rr);
           rr = fma(-c1[q], z1, rr);
           double zk = rr * cr[q];
           if (absb(zk) > 0x58F0000000000000ull) {   // |zk| > 2^400: rescale by 2^-400
             zk *= SMALL; z1 *= SMALL; z2 *= SMALL; sc *= SMALL; ss *= 0x1p-800;
             ++nres;
           }
-          Z[at(k)] = zk;
-          scnt[at(k)] = (unsigned char)(nres > 255 ? 255 : nres);
-          ss = fma(zk, zk, ss);
+          Z[at(s)] = zk;
+          scnt[at(s)] = (unsigned char)(nres > 255 ? 255 : nres);
+          if (it == 1) ss = fma(zk, zk, ss);
           z2 = z1;
           z1 = zk;
         }
       }
     }
-    if (nres > 0) {
-      for (int k = 0; k < n; ++k) {
-        double zk = Z[at(k)];
-        for (int q = scnt[at(k)]; q < nres; ++q) zk *= SMALL;
-        Z[at(k)] = zk;
+    // one scale for both ends
+    const int nmax = max(nres, __shfl_xor_sync(0xffffffffu, nres, 16));
+    if (nmax > 0) {
+      for (int s = 0; s < len; ++s) {
+        double zk = Z[at(s)];
+        for (int q = scnt[at(s)]; q < nmax; ++q) zk *= SMALL;
+        Z[at(s)] = zk;
       }
+      for (int q = nres; q < nmax; ++q) ss *= 0x1p-800;
     }
-    bscale = (ss > 0.0) ? rcp64(sqrt(ss)) : 1.0;
+    if (it == 0 && __any_sync(0xffffffffu, tiny)) {
+      unsigned long long mx = 1ull << 52;
+      for (int s = 0; s < len; ++s) mx = max(mx, absb(Z[at(s)]));
+      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+      const double f = __longlong_as_double((long long)(2046 - min((int)(mx >> 52), 2045)) << 52);
+      for (int s = 0; s < len; ++s) Z[at(s)] *= f;
+    }
   }
-  for (int k = 0; k < n; ++k) Z[at(k)] *= bscale;
+  ss += __shfl_xor_sync(0xffffffffu, ss, 16);
+  const double bscale = (ss > 0.0) ? rcp64(sqrt(ss)) : 1.0;
+  for (int s = 0; s < len; ++s) Z[at(s)] *= bscale;
 }
 
 // ---------------------------------------------------------------- stage 5
@@ -1075,6 +1186,7 @@ constexpr int WYB = 32;
 __host__ __device__ __forceinline__ int wy_blocks(int n) { return n > 2 ? (n - 2 + WYB - 1) / WYB : 0; }
 
 // One CTA per block of reflectors: the T factor into wyT (WYB x WYB, row-major).
+// probs NULL: the problem `one`.
 __global__ void __launch_bounds__(256) k_wy_t(const EigProblem* probs) {
   const EigProblem P = probs[blockIdx.y];
   const int n = P.n, b = blockIdx.x;
@@ -1305,12 +1417,12 @@ cudaError_t launch_tridiag(const EigProblem* probs_dev, EigProblem* probs_host, 
 cudaError_t launch_bisect(const EigProblem* probs_dev, int count, int nmax, int total_eigs,
                           int num_sms, cudaStream_t st) {
   // lanes per eigenvalue: about one warp per SM sub-partition in total
-  int L = 32;
+  int L = 32 * BNW;
   while (L > 1 && (int64_t)total_eigs * L > (int64_t)num_sms * 4 * 32) L >>= 1;
-  const size_t smem = sizeof(double) * 2 * (size_t)nmax;
+  const size_t smem = sizeof(double2) * (size_t)(nmax + 2 + (nmax + SB - 1) / SB);
   cudaError_t e = allow_max_dyn_smem((const void*)k_bisect);
   if (e != cudaSuccess) return e;
-  const int per_cta = BNW * (32 / L);
+  const int per_cta = BNW * 32 / L;
   k_bisect<<<dim3((nmax + per_cta - 1) / per_cta, count), BNW * 32, smem, st>>>(probs_dev, L);
   count_launches(1);
   return cudaGetLastError();
@@ -1318,7 +1430,7 @@ cudaError_t launch_bisect(const EigProblem* probs_dev, int count, int nmax, int 
 
 cudaError_t launch_invit(const EigProblem* probs_dev, int count, int total_vectors, cudaStream_t st) {
   if (total_vectors < 1) return cudaSuccess;
-  k_invit<<<(total_vectors + 63) / 64, 64, 0, st>>>(probs_dev, count);
+  k_invit<<<(total_vectors + 15) / 16, 32, 0, st>>>(probs_dev, count, total_vectors);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -49,3 +49,31 @@ def test_rank_cut_sums_in_order(ctx, n):
         R, d = ctx.rank_cut(torch.from_numpy(w).cuda(), thr)
         want = next(r for r in range(1, n + 1) if tail[r] <= thr)
         assert (R, d) == (want, tail[want])
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 16, 17, 31, 47, 64, 129, 153, 304, 305, 610])
+@pytest.mark.parametrize("kind", ["dense", "diagonal", "split", "tiny", "huge"])
+def test_eigenvalues_and_vectors_over_sizes(ctx, n, kind):
+    """Every width of the multisection (one to four warps per eigenvalue, down
+    to one lane in batches), the two-ended inverse iteration at odd and even
+    sizes, exact zeros on T's off-diagonal and matrices near the ends of the
+    exponent range."""
+    import torch
+    rng = np.random.default_rng(n)
+    S = rng.standard_normal((n, n)) * 10.0 ** rng.uniform(-3, 0, n)
+    S = S @ S.T
+    if kind == "diagonal":
+        S = np.diag(10.0 ** rng.uniform(-9, 0, n))
+    elif kind == "split":
+        h = n // 2
+        S[h:, :h] = S[:h, h:] = 0.0
+    scale = {"tiny": 2.0 ** -480, "huge": 2.0 ** 480}.get(kind, 1.0)
+    lam, _ = np.linalg.eigh(S)
+    lam = lam[::-1]
+    R = max(1, n // 3)
+    w, U, k, _ = ctx.eig_trunc(torch.from_numpy(S * scale).cuda(), R=R)
+    w, U = w.cpu().numpy() / scale, U.cpu().numpy()
+    top = abs(lam).max()
+    assert np.abs(w - lam).max() <= 1e-14 * n * top + 1e-15 * top
+    assert np.abs(U.T @ U - np.eye(R)).max() <= 1e-13 * n
+    assert np.abs(S @ U - U * w[:R]).max() <= 1e-13 * n * top
