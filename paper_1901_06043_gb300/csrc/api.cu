@@ -175,6 +175,29 @@ tucker_status join_side(tucker_ctx* c) {
   }
   return TUCKER_OK;
 }
+// Work on side stream 0 beside the context stream: begin() lets it start after
+// everything enqueued so far, join() (or the destructor, on any way out) lets
+// the context stream go on after it; so buffers freed on the context stream
+// outlive the work.
+struct SideWork {
+  tucker_ctx* c;
+  bool open = false;
+  explicit SideWork(tucker_ctx* cc) : c(cc) {}
+  cudaError_t begin() {
+    cudaError_t e = cudaEventRecord(c->fork_ev, c->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side[0], c->fork_ev, 0);
+    open = e == cudaSuccess;
+    return e;
+  }
+  cudaError_t join() {
+    if (!open) return cudaSuccess;
+    open = false;
+    cudaError_t e = cudaEventRecord(c->side_ev[0], c->side[0]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->side_ev[0], 0);
+    return e;
+  }
+  ~SideWork() { join(); }
+};
 struct StreamSwap {
   tucker_ctx* c;
   cudaStream_t main;
@@ -661,6 +684,11 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   TK_CUDA(c, cudaMemsetAsync(c->d_words + 34, 0, sizeof(unsigned), st));
   TK_CUDA(c, cudaMemsetAsync(info, 0, 3 * sizeof(int), st));
   TK_CUDA(c, launch_tridiag(pd, &h, 1, S, c->d_words + 34, st, c->barrier_polls));
+  // the back-transformation's T factors beside the eigenvalues and vectors of T,
+  // which leave most of the GPU idle
+  SideWork wy(c);
+  TK_CUDA(c, wy.begin());
+  TK_CUDA(c, launch_wy(nullptr, &h, 1, n, c->side[0]));
   TK_CUDA(c, launch_bisect(pd, 1, n, n, c->num_sms, st));
   TK_CUDA(c, launch_rank_cut(w, n, thr, fixed_R, c->d_i64, c->d_small + 2, st));
   int64_t R = 0;
@@ -694,6 +722,7 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
     TK_TRY(do_gram(c, h.z, TUCKER_F64, zv, TUCKER_PREC_FP64, h.gram, nullptr));
     TK_CUDA(c, launch_cholqr(pd, &h, 1, pass, c->num_sms, st));
   }
+  TK_CUDA(c, wy.join());
   TK_CUDA(c, launch_backtransform(pd, 1, Ri, n, st));
   int hinfo = 0;
   TK_CUDA(c, cudaMemcpyAsync(&hinfo, info, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1673,6 +1702,7 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
         }
       TK_CUDA(c, launch_cholqr(pd, h.data(), m, pass, c->num_sms, st));
     }
+    TK_CUDA(c, launch_wy(pd, nullptr, m, nmax, st));
     TK_CUDA(c, launch_backtransform(pd, m, zoff, nmax, st));
     std::vector<int> info(3 * m);
     unsigned berr = 0;

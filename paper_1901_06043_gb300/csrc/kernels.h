@@ -184,6 +184,10 @@ cudaError_t launch_invit(const EigProblem* probs_dev, int count, int total_vecto
 // does nothing where pass 0 found the Gram near the identity: info[1] == 0)
 cudaError_t launch_cholqr(const EigProblem* probs_dev, const EigProblem* probs_host, int count,
                           int pass, int num_sms, cudaStream_t st);
+// T factors of the blocked back-transformation (after launch_tridiag; needed by
+// launch_backtransform): of the `count` problems, or of `one` (host) alone
+cudaError_t launch_wy(const EigProblem* probs_dev, const EigProblem* one, int count, int nmax,
+                      cudaStream_t st);
 cudaError_t launch_backtransform(const EigProblem* probs_dev, int count, int total_vectors,
                                  int nmax, cudaStream_t st);
 // batched rank cut (thr[p], fixed[p] > 0 or NULL) and Z^T Z for problems with R <= 64

@@ -1187,8 +1187,8 @@ __host__ __device__ __forceinline__ int wy_blocks(int n) { return n > 2 ? (n - 2
 
 // One CTA per block of reflectors: the T factor into wyT (WYB x WYB, row-major).
 // probs NULL: the problem `one`.
-__global__ void __launch_bounds__(256) k_wy_t(const EigProblem* probs) {
-  const EigProblem P = probs[blockIdx.y];
+__global__ void __launch_bounds__(256) k_wy_t(const EigProblem* probs, const EigProblem one) {
+  const EigProblem P = probs ? probs[blockIdx.y] : one;
   const int n = P.n, b = blockIdx.x;
   if (b >= wy_blocks(n)) return;
   const int k0 = b * WYB, m = min(WYB, n - 2 - k0);
@@ -1473,14 +1473,19 @@ cudaError_t launch_cholqr(const EigProblem* probs_dev, const EigProblem* probs_h
 
 size_t eig_wy_doubles(int n) { return (size_t)wy_blocks(n) * WYB * WYB; }
 
+cudaError_t launch_wy(const EigProblem* probs_dev, const EigProblem* one, int count, int nmax,
+                      cudaStream_t st) {
+  const int nb = wy_blocks(nmax);
+  if (nb > 0) {
+    k_wy_t<<<dim3(nb, count), 256, 0, st>>>(one ? nullptr : probs_dev, one ? *one : EigProblem{});
+    count_launches(1);
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t launch_backtransform(const EigProblem* probs_dev, int count, int total_vectors,
                                  int nmax, cudaStream_t st) {
   if (total_vectors < 1) return cudaSuccess;
-  const int nb = wy_blocks(nmax);
-  if (nb > 0) {
-    k_wy_t<<<dim3(nb, count), 256, 0, st>>>(probs_dev);
-    count_launches(1);
-  }
   const size_t smem = sizeof(double) * (size_t)nmax;
   cudaError_t e = allow_max_dyn_smem((const void*)k_backtransform);
   if (e != cudaSuccess) return e;
