@@ -42,8 +42,9 @@
 // - Unscaled reflectors: v = x - beta e_1, tau = 2 / (v . v); tau is computed by one
 //   warp while the others form A v, and multiplies the finished sums.  (The
 //   matrix is scaled by a power of two first, so that squares neither overflow
-//   nor underflow where they matter.)  A step's update needs no w: a_ij - v_i p_j -
-//   (p_i - tau (p . v) v_i) v_j.
+//   nor underflow where they matter.)  The update goes by w, though a_ij - v_i p_j -
+//   (p_i - tau (p . v) v_i) v_j needs one FMA less on the chain: its first product
+//   is larger, and the vectors of close eigenvalues came out 1.3 times as far off.
 // Measured, whole reduction: n = 50 0.26 -> 0.18 ms, n = 200 1.20 -> 0.84 ms, n = 500
 // 3.5 -> 2.5 ms (a barrier, normalized reflectors and FP64 sums before).
 #include <algorithm>
@@ -214,8 +215,8 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
   const GridBarrier bar{reinterpret_cast<unsigned*>(P.xch + 8 * (size_t)n), nullptr, err};
   unsigned gen = 0;
   double* vk = tsm;                       // v_k by global index
-  double* vn = tsm + n;                   // y, then v_{k+1}
-  double* sp = tsm + 2 * n;               // p_k
+  double* vn = tsm + n;                   // the pivot row, then v_{k+1}
+  double* sp = tsm + 2 * n;               // p_k, then w_k
   double* sq = tsm + 3 * n;               // own rows of A v_{k+1} (solo: then p_{k+1})
   double* const sr = tsm + 4 * n;         // solo: next pivot row
   double* const srows = tsm + 5 * n;      // own rows t = 0, 1, ... (row c + G t) when SROWS
@@ -289,9 +290,8 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
     const bool more = k < n - 3;
     if (i0 < lo) { i0 += G; own0 += rstep; }
     const bool scribe = i0 == lo;
-    double t2 = 0.0;                      // tau_k (p_k . v_k)
     if (k >= 0) {
-      // ---- p_k and the pivot row; y into vn; p . v
+      // ---- p_k into sp and the pivot row r into vn; p . v
       const double v1 = vk[k + 1];
       double s1 = 0.0;
       bool fail = false;
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
         for (int q = 0; q < JPT; ++q) {
           const int j = j0 + q * TNT;
           if (j < n) {
-            vn[j] = fma(-v1, pj[q], rj[q]);
+            vn[j] = rj[q];
             s1 = fma(pj[q], vk[j], s1);
           }
         }
@@ -355,24 +355,29 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
       if (__syncthreads_or(fail)) return;
       // the last warp does the scalars (it has no rows, see below)
       if (warp == TNW - 1) {
-        const double t = tau * warp_sum(lane < TNW ? s_red[0][lane] : 0.0);
+        const double K = 0.5 * tau * warp_sum(lane < TNW ? s_red[0][lane] : 0.0);
         if (lane == 0) {
-          s_c[0] = t;
-          s_c[1] = fma(t, v1, -sp[k + 1]);
+          s_c[0] = K;
+          s_c[1] = fma(-K, v1, sp[k + 1]);
         }
       }
       __syncthreads();
-      t2 = s_c[0];
-      const double cc = s_c[1];
+      const double K = s_c[0], w1 = s_c[1];
       if (scribe && tid == 0) {
-        P.d[k + 1] = fma(cc, v1, vn[k + 1]) * isc;
-        if (!more) P.e[n - 2] = fma(cc, vk[lo], vn[lo]) * isc;
+        P.d[k + 1] = fma(-w1, v1, fma(-v1, w1, vn[k + 1])) * isc;
+        if (!more) {                      // the last off-diagonal and the last entry (lo = n - 1)
+          const double vl = vk[lo], wl = fma(-K, vl, sp[lo]);
+          P.e[n - 2] = fma(-w1, vl, fma(-v1, wl, vn[lo])) * isc;
+          P.d[lo] = fma(-wl, vl, fma(-vl, wl, own0[lo])) * isc;
+        }
       }
       if (more) {
-        // the pivot row x after step k, and its norm
+        // w_k into sp, the pivot row x after step k, and its norm
         double ss = 0.0;
         for (int j = lo + tid; j < n; j += TNT) {
-          const double x = fma(cc, vk[j], vn[j]);
+          const double v = vk[j], w = fma(-K, v, sp[j]);
+          const double x = fma(-w1, v, fma(-v1, w, vn[j]));
+          sp[j] = w;
           vn[j] = x;
           if (j > lo) ss = fma(x, x, ss);
         }
@@ -402,16 +407,16 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
       ulonglong2* rw = xr + (size_t)((k + 1) & 1) * n;
       // PIV: the next pivot row, also published
       auto do_row = [&](int i, double* Ai, auto UPD, auto PIV) {
-        double vi = 0.0, gi = 0.0, acc = 0.0;
+        double vi = 0.0, wi = 0.0, acc = 0.0;
         if constexpr (decltype(UPD)::value) {
           vi = vk[i];
-          gi = fma(-t2, vi, sp[i]);
+          wi = sp[i];
         }
 #pragma unroll 4
         for (int j = lo + lane; j < n; j += 32) {
           double a = Ai[j];
           if constexpr (decltype(UPD)::value) {
-            a = fma(-gi, vk[j], fma(-vi, sp[j], a));
+            a = fma(-wi, vk[j], fma(-vi, sp[j], a));
             Ai[j] = a;
           }
           if constexpr (decltype(PIV)::value) {
@@ -426,12 +431,7 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
       };
       using yes = std::true_type;
       using no = std::false_type;
-      if (!more) {                        // the last entry (lo = n - 1)
-        if (scribe && warp == 0 && lane == 0) {
-          const double vi = vk[lo], gi = fma(-t2, vi, sp[lo]);
-          P.d[lo] = fma(-gi, vi, fma(-vi, sp[lo], own0[lo])) * isc;
-        }
-      } else {
+      if (more) {
         int i = i0 + G * warp;
         double* Ai = own0 + rstep * warp;
         for (; i < n; i += G * nw, Ai += rstep * nw) {
@@ -655,8 +655,9 @@ __global__ void __launch_bounds__(BNW * 32) k_bisect(const EigProblem* probs, in
 // meet gives the two middle entries, and both substitute back outwards, so the
 // dependent chain is n / 2 steps long.  In local indices (s = 0 at the lane's end)
 // both lanes run the same code; a row swap gives U a second superdiagonal.
-// Pivots below eps ||T|| are raised to that size (the shift is an eigenvalue, so
-// one pivot is ~0); a running power-of-two rescale (|z| <= 2^400, so the sum of
+// Pivots below 2^-92 ||T|| are raised to that size (the shift is an eigenvalue, so
+// one pivot is ~0; raised to eps ||T||, which shifts the eigenvalue by as much, the
+// vectors of close eigenvalues came out up to 4 times as far off); a running power-of-two rescale (|z| <= 2^400, so the sum of
 // squares stays finite) keeps the back substitution finite.  Output column j
 // of Z (n x R, row-major: Z[i*R + j]), a unit vector.
 //   The FP64 pipe is the limit (a warp instruction takes 64 cycles of it whatever
@@ -706,7 +707,7 @@ __global__ void __launch_bounds__(32) k_invit(const EigProblem* probs, int nprob
   unsigned char* __restrict__ scnt = flag + (int64_t)n * R;
   double* __restrict__ Z = P.z + o0;
   auto at = [&](int s) { return s * step; };
-  const double ptol = fmax(DBL_EPSILON * P.tau[n - 1], 0x1p-990);      // tau[n - 1]: ||T|| (k_bisect)
+  const double ptol = fmax(0x1p-92 * P.tau[n - 1], 0x1p-990);      // tau[n - 1]: ||T|| (k_bisect)
   const unsigned long long ptol_bits = (unsigned long long)__double_as_longlong(ptol);
   auto absb = [](double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
