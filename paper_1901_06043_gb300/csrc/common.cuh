@@ -89,4 +89,12 @@ __device__ __forceinline__ bool grid_sync(const GridBarrier& b, unsigned& my_gen
   return s_ok != 0;
 }
 
+// Packed FP32 pair arithmetic (f32x2), each lane rounded to nearest.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {    // a - b, one rounding
+  return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+}
+
 }  // namespace tk

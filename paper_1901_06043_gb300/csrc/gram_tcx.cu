@@ -158,14 +158,6 @@ __device__ __forceinline__ float4 ld_nl1(const float4* p) {
   return v;
 }
 
-// Packed FP32 pair arithmetic (f32x2), each lane rounded to nearest.
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {    // a - b, one rounding
-  return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
-}
-
 // Per-row sums a diagonal tile's producers keep for its diagonal entries,
 // two rows per float2 (FP32, exact or short; moved into FP64 every 32
 // stages): r2 = sum r^2 (r the last rounding's remainder, in units of the

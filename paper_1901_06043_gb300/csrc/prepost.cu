@@ -19,10 +19,12 @@
 // FP32 data is reduced and transformed on the FP32 pipe with error-free
 // transformations: each sum is an FP32 pair (hi, lo) grown by TwoSum (a new
 // term may exceed the running sum, so never the cheaper Fast2Sum), squares are exact
-// (TwoProduct by FMA).  Every 16 elements of a thread the pair is merged
+// (TwoProduct by FMA).  Every 16 terms the pair is merged
 // exactly into a second-level pair that is renormalised (|lo| <= ulp(hi) / 2,
-// so its later roundings stay at 2^-48 of hi), and every 1024 elements that
-// pair moves into FP64; the result is the FP64 sum to ~1e-14 of sum |x|.  The
+// so its later roundings stay at 2^-48 of hi), and every 1024 terms that
+// pair moves into FP64; the result is the FP64 sum to ~1e-14 of sum |x|.  A
+// thread sums two streams in the halves of packed f32x2 registers: ~30 FP32
+// operations an element set the pace otherwise, not HBM.  The
 // standard deviation takes a second pass over the data, sum (x - mean)^2 with
 // the mean as an FP32 pair and x - mean_hi exact by TwoSum, which avoids the
 // cancellation of sum x^2 - count mean^2.  The transform evaluates
@@ -33,6 +35,8 @@
 // bitwise reproducible from run to run.
 #include "common.cuh"
 #include "kernels.h"
+
+#include <type_traits>
 
 namespace tk {
 namespace {
@@ -67,105 +71,152 @@ __device__ __forceinline__ void two_sum(float& h, float& l, float v) {
 template <typename T, int PASS> struct Part;
 
 template <int PASS> struct Part<double, PASS> {
-  double s, s2, sa, c2, mx, mn, mean;
+  double s, s2, sa, c2, mean;
+  long long mx, mn;                       // ordered bits: an FP64 comparison takes as
+                                          // long as an FMA, an integer one does not
   __device__ void init(double m) {
     s = s2 = sa = c2 = 0.0;
-    mx = -INFINITY;
-    mn = INFINITY;
+    mx = ordered(-INFINITY);
+    mn = ordered(INFINITY);
     mean = m;
   }
-  __device__ __forceinline__ void add(double v) {
+  __device__ __forceinline__ void add1(double v) {
     if (PASS == 0) {
       s += v;
       s2 = fma(v, v, s2);
       sa += fabs(v);
-      mx = fmax(mx, v);
-      mn = fmin(mn, v);
+      const long long k = ordered(v);
+      mx = max(mx, k);
+      mn = min(mn, k);
     } else {
       const double d = v - mean;
       c2 = fma(d, d, c2);
     }
   }
+  __device__ __forceinline__ void add2(double v, double w) { add1(v); add1(w); }
+  __device__ __forceinline__ void tick(int) {}
   __device__ void flush() {}
 };
 
+// (h, l) += v exactly in both halves
+__device__ __forceinline__ void two_sum2(float2& h, float2& l, float2 v) {
+  const float2 s = add2(h, v);
+  const float2 bb = sub2(s, h);
+  const float2 err = add2(sub2(h, sub2(s, bb)), sub2(v, bb));
+  h = s;
+  l = add2(l, err);
+}
+
 template <int PASS> struct Part<float, PASS> {
-  double s, s2, sa, c2, mx, mn;           // FP64 totals
-  float sh, sl, qh, ql, ah, al;           // level 1: FP32 pairs of the current group
-  float SH, SL, QH, QL, AH, AL;           // level 2: renormalised pairs of the groups
-  float mh, ml;                           // the mean as an FP32 pair (PASS 1)
+  double s, s2, sa, c2;                    // FP64 totals
+  long long mx, mn;
+  // two streams, one per half
+  float2 sh, sl, qh, ql, ah, al;           // level 1: FP32 pairs of the current group
+  float2 SH, SL, QH, QL, AH, AL;           // level 2: renormalised pairs of the groups
+  float mh, ml;                            // the mean as an FP32 pair (PASS 1)
   float fmx, fmn;
   int n, g;
   __device__ void init(double m) {
     s = s2 = sa = c2 = 0.0;
-    mx = -INFINITY;
-    mn = INFINITY;
-    sh = sl = qh = ql = ah = al = 0.f;
-    SH = SL = QH = QL = AH = AL = 0.f;
+    const float2 z = make_float2(0.f, 0.f);
+    sh = sl = qh = ql = ah = al = z;
+    SH = SL = QH = QL = AH = AL = z;
+    mx = ordered(-INFINITY);
+    mn = ordered(INFINITY);
     fmx = -INFINITY;
     fmn = INFINITY;
     mh = (float)m;
     ml = (float)(m - (double)mh);
     n = g = 0;
   }
-  __device__ __forceinline__ void add(float v) {
+  __device__ __forceinline__ void add2(float v, float w) {
+    const float2 x = make_float2(v, w);
     if (PASS == 0) {
-      two_sum(sh, sl, v);
+      two_sum2(sh, sl, x);
+      const float2 p = mul2(x, x);
+      const float2 pe = fma2(x, x, make_float2(-p.x, -p.y));   // x^2 = p + pe exactly
+      two_sum2(qh, ql, p);
+      ql = tk::add2(ql, pe);
+      two_sum2(ah, al, make_float2(fabsf(v), fabsf(w)));
+      fmx = fmaxf(fmx, fmaxf(v, w));
+      fmn = fminf(fmn, fminf(v, w));
+    } else {
+      // d = x - mean = (s + e) - ml with s + e = x - mh exactly
+      float2 s_ = x, e = make_float2(0.f, 0.f);
+      two_sum2(s_, e, make_float2(-mh, -mh));
+      const float2 t = tk::add2(e, make_float2(-ml, -ml));
+      const float2 p = mul2(s_, s_);
+      const float2 pe = fma2(s_, s_, make_float2(-p.x, -p.y));
+      // d^2 = p + pe + t (2 s + t); |t| can be a sizeable part of |s| when
+      // the slice varies little around its mean, so t^2 stays
+      two_sum2(qh, ql, p);
+      ql = tk::add2(ql, fma2(fma2(s_, make_float2(2.f, 2.f), t), t, pe));
+    }
+  }
+  // one element, into the first half
+  __device__ __forceinline__ void add1(float v) {
+    if (PASS == 0) {
+      two_sum(sh.x, sl.x, v);
       const float p = __fmul_rn(v, v);
-      const float pe = __fmaf_rn(v, v, -p);            // v^2 = p + pe exactly
-      two_sum(qh, ql, p);
-      ql = __fadd_rn(ql, pe);
-      two_sum(ah, al, fabsf(v));
+      const float pe = __fmaf_rn(v, v, -p);
+      two_sum(qh.x, ql.x, p);
+      ql.x = __fadd_rn(ql.x, pe);
+      two_sum(ah.x, al.x, fabsf(v));
       fmx = fmaxf(fmx, v);
       fmn = fminf(fmn, v);
     } else {
-      // d = v - mean = (s + e) - ml with s + e = v - mh exactly
       float s_ = v, e = 0.f;
       two_sum(s_, e, -mh);
       const float t = __fsub_rn(e, ml);
       const float p = __fmul_rn(s_, s_);
       const float pe = __fmaf_rn(s_, s_, -p);
-      // d^2 = p + pe + t (2 s + t); |t| can be a sizeable part of |s| when
-      // the slice varies little around its mean, so t^2 stays
-      two_sum(qh, ql, p);
-      ql = __fadd_rn(ql, __fmaf_rn(__fadd_rn(2.f * s_, t), t, pe));
+      two_sum(qh.x, ql.x, p);
+      ql.x = __fadd_rn(ql.x, __fmaf_rn(__fmaf_rn(2.f, s_, t), t, pe));
     }
-    if (++n == kGroup) merge();
+  }
+  // after every k <= 8 terms of a half: merge before a group exceeds kGroup
+  __device__ __forceinline__ void tick(int k) {
+    n += k;
+    if (n > kGroup - 8) merge();
   }
   // (H, L) += (h, l) exactly up to the rounding of L, then renormalised so
   // that |L| <= ulp(H) / 2 (its later roundings stay at 2^-48 of H)
-  __device__ __forceinline__ static void merge_pair(float& H, float& L, float h, float l) {
-    two_sum(H, L, h);
-    L = __fadd_rn(L, l);
-    float t = H, e = 0.f;                       // (t, e) = H + L exactly (TwoSum)
-    two_sum(t, e, L);
+  __device__ __forceinline__ static void merge_pair(float2& H, float2& L, float2 h, float2 l) {
+    two_sum2(H, L, h);
+    L = tk::add2(L, l);
+    float2 t = H, e = make_float2(0.f, 0.f);    // (t, e) = H + L exactly (TwoSum)
+    two_sum2(t, e, L);
     H = t;
     L = e;
   }
-  // level 1 -> level 2 every kGroup elements; level 2 -> FP64 every
-  // kGroups groups
+  // level 1 -> level 2 every kGroup terms; level 2 -> FP64 every kGroups groups
   __device__ void merge() {
+    const float2 z = make_float2(0.f, 0.f);
     if (PASS == 0) {
       merge_pair(SH, SL, sh, sl);
       merge_pair(QH, QL, qh, ql);
       merge_pair(AH, AL, ah, al);
-      sh = sl = qh = ql = ah = al = 0.f;
+      sh = sl = qh = ql = ah = al = z;
     } else {
       merge_pair(QH, QL, qh, ql);
-      qh = ql = 0.f;
+      qh = ql = z;
     }
     n = 0;
     if (++g == kGroups) flush_groups();
   }
+  __device__ static double total(float2 H, float2 L) {
+    return ((double)H.x + (double)L.x) + ((double)H.y + (double)L.y);
+  }
   __device__ void flush_groups() {
+    const float2 z = make_float2(0.f, 0.f);
     if (PASS == 0) {
-      s += (double)SH + (double)SL;
-      s2 += (double)QH + (double)QL;
-      sa += (double)AH + (double)AL;
-      SH = SL = QH = QL = AH = AL = 0.f;
+      s += total(SH, SL);
+      s2 += total(QH, QL);
+      sa += total(AH, AL);
+      SH = SL = QH = QL = AH = AL = z;
     } else {
-      c2 += (double)QH + (double)QL;
-      QH = QL = 0.f;
+      c2 += total(QH, QL);
+      QH = QL = z;
     }
     g = 0;
   }
@@ -173,8 +224,8 @@ template <int PASS> struct Part<float, PASS> {
   __device__ void flush() {
     merge();
     flush_groups();
-    mx = fmax(mx, (double)fmx);
-    mn = fmin(mn, (double)fmn);
+    mx = max(mx, ordered((double)fmx));
+    mn = min(mn, ordered((double)fmn));
     fmx = -INFINITY;
     fmn = INFINITY;
   }
@@ -187,8 +238,8 @@ __device__ void to_global(double* acc, int64_t i, const Part<T, PASS>& p) {
     atomicAdd(a + 0, p.s);
     atomicAdd(a + 1, p.s2);
     atomicAdd(a + 2, p.sa);
-    atomicMax(reinterpret_cast<long long*>(a + 3), ordered(p.mx));
-    atomicMin(reinterpret_cast<long long*>(a + 4), ordered(p.mn));
+    atomicMax(reinterpret_cast<long long*>(a + 3), p.mx);
+    atomicMin(reinterpret_cast<long long*>(a + 4), p.mn);
   } else {
     atomicAdd(a + 5, p.c2);
   }
@@ -197,7 +248,8 @@ __device__ void to_global(double* acc, int64_t i, const Part<T, PASS>& p) {
 // Block reduction of the FP64 totals into thread 0 (all threads call it).
 template <typename T, int PASS>
 __device__ void block_reduce(Part<T, PASS>& p) {
-  __shared__ double sh[6][kThreads / 32];
+  __shared__ double sh[4][kThreads / 32];
+  __shared__ long long sm[2][kThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -205,22 +257,22 @@ __device__ void block_reduce(Part<T, PASS>& p) {
       p.s += __shfl_xor_sync(0xffffffffu, p.s, o);
       p.s2 += __shfl_xor_sync(0xffffffffu, p.s2, o);
       p.sa += __shfl_xor_sync(0xffffffffu, p.sa, o);
-      p.mx = fmax(p.mx, __shfl_xor_sync(0xffffffffu, p.mx, o));
-      p.mn = fmin(p.mn, __shfl_xor_sync(0xffffffffu, p.mn, o));
+      p.mx = max(p.mx, __shfl_xor_sync(0xffffffffu, p.mx, o));
+      p.mn = min(p.mn, __shfl_xor_sync(0xffffffffu, p.mn, o));
     } else {
       p.c2 += __shfl_xor_sync(0xffffffffu, p.c2, o);
     }
   }
   __syncthreads();
   if (lane == 0) {
-    sh[0][w] = p.s; sh[1][w] = p.s2; sh[2][w] = p.sa;
-    sh[3][w] = p.mx; sh[4][w] = p.mn; sh[5][w] = p.c2;
+    sh[0][w] = p.s; sh[1][w] = p.s2; sh[2][w] = p.sa; sh[3][w] = p.c2;
+    sm[0][w] = p.mx; sm[1][w] = p.mn;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int k = 1; k < kThreads / 32; ++k) {
-      p.s += sh[0][k]; p.s2 += sh[1][k]; p.sa += sh[2][k];
-      p.mx = fmax(p.mx, sh[3][k]); p.mn = fmin(p.mn, sh[4][k]); p.c2 += sh[5][k];
+      p.s += sh[0][k]; p.s2 += sh[1][k]; p.sa += sh[2][k]; p.c2 += sh[3][k];
+      p.mx = max(p.mx, sm[0][k]); p.mn = min(p.mn, sm[1][k]);
     }
   }
 }
@@ -247,19 +299,30 @@ __global__ void __launch_bounds__(kThreads) k_stats_rows(const T* __restrict__ x
   for (; r + 3 * C < r1; r += 4 * C, ptr += 4 * step) {   // four loads in flight
     const T a = __ldg(ptr), b = __ldg(ptr + step), d = __ldg(ptr + 2 * step),
             e = __ldg(ptr + 3 * step);
-    p.add(a);
-    p.add(b);
-    p.add(d);
-    p.add(e);
+    p.add2(a, b);
+    p.add2(d, e);
+    p.tick(2);
   }
-  for (; r < r1; r += C, ptr += step) p.add(__ldg(ptr));
+  for (; r < r1; r += C, ptr += step) {
+    p.add1(__ldg(ptr));
+    p.tick(1);
+  }
   p.flush();
   if (r1 > r0) to_global(acc, i, p);
 }
 
+// CTAs per SM in the grids of the runs kernels: several waves, as the SMs' shares
+// of the bandwidth differ.  250^3 x 11 x 4 FP32 (2.75 GB), map / stats passes 0 and
+// 1: one wave 945 / 744 / 554 us, these 820 / 744 / 512 us; at 6.77 TB/s the bytes
+// take 812 / 406 / 406 us.  Pass 0 is bound by its FP32 operations (993 us
+// unpacked, pass 1 822).
+constexpr int kStatsCtas = 20;
+constexpr int kApplyCtas = 128;
+
 // runs regime (L >= 4096): units (i, r, chunk) in i-major order, a
-// contiguous range of units per CTA, walked without divisions.
-template <typename T, int PASS>
+// contiguous range of units per CTA, walked without divisions.  VEC: every run
+// starts on 16 bytes.
+template <typename T, int PASS, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_stats_runs(const T* __restrict__ x, int64_t L,
                                                           int64_t I, int64_t Rt,
                                                           const double* __restrict__ mean,
@@ -282,16 +345,40 @@ __global__ void __launch_bounds__(kThreads) k_stats_runs(const T* __restrict__ x
     }
     const int64_t l0 = ch * kChunk, l1 = min(L, l0 + kChunk);
     const T* run = x + L * (i + I * r);
-    int64_t l = l0 + threadIdx.x;
-    for (; l + 3 * kThreads < l1; l += 4 * kThreads) {
-      const T a = __ldg(run + l), b = __ldg(run + l + kThreads),
-              d = __ldg(run + l + 2 * kThreads), e = __ldg(run + l + 3 * kThreads);
-      p.add(a);
-      p.add(b);
-      p.add(d);
-      p.add(e);
+    constexpr int V = 16 / sizeof(T);
+    // four 16-byte loads in flight where the run allows them
+    if (VEC && l1 - l0 == kChunk) {
+      constexpr int U = 4;
+      for (int64_t l = l0 + V * (int64_t)threadIdx.x; l < l1; l += U * V * kThreads) {
+        if constexpr (sizeof(T) == 4) {
+          float4 q[U];
+#pragma unroll
+          for (int k = 0; k < U; ++k) q[k] = __ldg(reinterpret_cast<const float4*>(run + l + k * V * kThreads));
+#pragma unroll
+          for (int k = 0; k < U; ++k) { p.add2(q[k].x, q[k].y); p.add2(q[k].z, q[k].w); }
+          p.tick(2 * U);
+        } else {
+          double2 q[U];
+#pragma unroll
+          for (int k = 0; k < U; ++k) q[k] = __ldg(reinterpret_cast<const double2*>(run + l + k * V * kThreads));
+#pragma unroll
+          for (int k = 0; k < U; ++k) p.add2(q[k].x, q[k].y);
+        }
+      }
+    } else {
+      int64_t l = l0 + threadIdx.x;
+      for (; l + 3 * kThreads < l1; l += 4 * kThreads) {
+        const T a = __ldg(run + l), b = __ldg(run + l + kThreads),
+                d = __ldg(run + l + 2 * kThreads), e = __ldg(run + l + 3 * kThreads);
+        p.add2(a, b);
+        p.add2(d, e);
+        p.tick(2);
+      }
+      for (; l < l1; l += kThreads) {
+        p.add1(__ldg(run + l));
+        p.tick(1);
+      }
     }
-    for (; l < l1; l += kThreads) p.add(__ldg(run + l));
     if (++ch == nch) {
       ch = 0;
       if (++r == Rt) { r = 0; ++i; }
@@ -403,40 +490,59 @@ __global__ void __launch_bounds__(kThreads) k_apply_rows(const T* x, int64_t L, 
   for (; r < r1; r += C, o += step) y[o] = f(x[o]);
 }
 
-// runs regime: a unit is (run j = i + I r, chunk); VEC: 16-byte accesses
-// (L and both pointers aligned so that every run starts on 16 bytes)
+// runs regime: a unit is (run j = i + I r, chunk), a contiguous range of units
+// per CTA, so the map (its FP64 division and conversions cost as much as
+// hundreds of elements) is made once per run; VEC: 16-byte accesses (L and
+// both pointers aligned so that every run starts on 16 bytes), four in flight.
+// x may be y, so a thread loads and stores the same elements.
 template <typename T, bool INV, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_apply_runs(const T* x, int64_t L, int64_t I,
                                                           int64_t Rt,
                                                           const double* __restrict__ shift,
                                                           const double* __restrict__ scale, T* y) {
-  constexpr int V = 16 / sizeof(T);
+  constexpr int V = 16 / sizeof(T), U = 4;
   const int64_t nch = (L + kChunk - 1) / kChunk;
   const int64_t units = I * Rt * nch;
-  for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
-    const int64_t j = u / nch, ch = u % nch;
-    const int64_t i = j % I;
-    const Map<T, INV> f(shift[i], scale[i]);
+  const int64_t u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
+  if (u0 >= u1) return;
+  int64_t j = u0 / nch, ch = u0 % nch, i = j % I;
+  Map<T, INV> f(shift[i], scale[i]);
+  for (int64_t u = u0; u < u1; ++u) {
     const int64_t l0 = ch * kChunk, l1 = min(L, l0 + kChunk);
-    const int64_t base = L * j;
+    const T* xr = x + L * j;
+    T* yr = y + L * j;
     if (VEC) {
-      for (int64_t l = l0 + (int64_t)threadIdx.x * V; l < l1; l += (int64_t)kThreads * V) {
+      using T4 = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+      auto map4 = [&](T4 v) {
+        v.x = f(v.x);
+        v.y = f(v.y);
         if constexpr (sizeof(T) == 4) {
-          float4 v = *reinterpret_cast<const float4*>(x + base + l);
-          v.x = f(v.x);
-          v.y = f(v.y);
           v.z = f(v.z);
           v.w = f(v.w);
-          *reinterpret_cast<float4*>(y + base + l) = v;
-        } else {
-          double2 v = *reinterpret_cast<const double2*>(x + base + l);
-          v.x = f(v.x);
-          v.y = f(v.y);
-          *reinterpret_cast<double2*>(y + base + l) = v;
         }
+        return v;
+      };
+      int64_t l = l0 + (int64_t)threadIdx.x * V;
+      if (l1 - l0 == kChunk) {
+        for (; l < l1; l += U * V * kThreads) {
+          T4 q[U];
+#pragma unroll
+          for (int k = 0; k < U; ++k) q[k] = *reinterpret_cast<const T4*>(xr + l + k * V * kThreads);
+#pragma unroll
+          for (int k = 0; k < U; ++k) *reinterpret_cast<T4*>(yr + l + k * V * kThreads) = map4(q[k]);
+        }
+      } else {
+        for (; l < l1; l += V * kThreads)
+          *reinterpret_cast<T4*>(yr + l) = map4(*reinterpret_cast<const T4*>(xr + l));
       }
     } else {
-      for (int64_t l = l0 + threadIdx.x; l < l1; l += kThreads) y[base + l] = f(x[base + l]);
+      for (int64_t l = l0 + threadIdx.x; l < l1; l += kThreads) yr[l] = f(xr[l]);
+    }
+    if (++ch == nch) {
+      ch = 0;
+      ++j;
+      if (++i == I) i = 0;
+      if (u + 1 < u1) f = Map<T, INV>(shift[i], scale[i]);
     }
   }
 }
@@ -480,9 +586,12 @@ void stats_pass(const T* x, int64_t L, int64_t I, int64_t Rt, const double* mean
                                                                         acc);
   } else {
     const int64_t units = I * Rt * ((L + kChunk - 1) / kChunk);
-    int64_t g = (int64_t)num_sms * 8;
+    int64_t g = (int64_t)num_sms * kStatsCtas;
     if (g > units) g = units;
-    k_stats_runs<T, PASS><<<(unsigned)g, kThreads, 0, st>>>(x, L, I, Rt, mean, acc);
+    if (L % (16 / (int64_t)sizeof(T)) == 0 && ((uintptr_t)x & 15) == 0)
+      k_stats_runs<T, PASS, true><<<(unsigned)g, kThreads, 0, st>>>(x, L, I, Rt, mean, acc);
+    else
+      k_stats_runs<T, PASS, false><<<(unsigned)g, kThreads, 0, st>>>(x, L, I, Rt, mean, acc);
   }
 }
 
@@ -515,7 +624,7 @@ void apply_t(const T* x, int64_t L, int64_t I, int64_t Rt, const double* shift,
     return;
   }
   const int64_t units = I * Rt * ((L + kChunk - 1) / kChunk);
-  int64_t g = (int64_t)num_sms * 16;
+  int64_t g = (int64_t)num_sms * kApplyCtas;
   if (g > units) g = units;
   const bool vec = (L % (16 / (int64_t)sizeof(T))) == 0 && ((uintptr_t)x & 15) == 0 &&
                    ((uintptr_t)y & 15) == 0;

@@ -226,3 +226,33 @@ def test_sthosvd_in_the_flop_optimal_order(ctx):
         dims, res.ranks, range(4))
     r0.close()
     res.close()
+
+
+# runs of exactly one chunk, of chunks and a remainder, of odd length, and a tensor that
+# starts one element past a 16-byte boundary; more runs than blocks, runs across blocks
+@pytest.mark.parametrize("dims,mode", [((4096, 5, 3), 1), ((64, 64, 3000), 2), ((9000, 3, 7), 1),
+                                       ((8191, 2, 3), 1), ((4100, 1, 2), 1), ((3000000, 2), 1)])
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+def test_long_runs(ctx, dims, mode, off, dt):
+    n = oracle.linear_size(dims)
+    buf = torch.empty(n + off, device="cuda", dtype=dt)
+    t = buf[off:]
+    t.copy_(torch.from_numpy(_data(dims, mode, 5 * sum(dims) + mode)))
+    xs = host(t)
+    want = oracle.slice_stats(xs, dims, mode)
+    got = host(ctx.slice_stats(t, dims, mode))
+    for k in (0, 4, 5):
+        assert np.allclose(got[:, k], want[:, k], rtol=1e-12, atol=1e-13 * np.abs(want[:, k]).max())
+    sd_tol = 1e-12 * np.maximum(want[:, 1], 1e-3 * np.abs(want[:, 0]))
+    assert np.all(np.abs(got[:, 1] - want[:, 1]) <= sd_tol + 1e-300)
+    assert np.array_equal(got[:, 2:4], want[:, 2:4])
+    sh, sc = oracle.standardize_params(want)
+    for inverse in (False, True):
+        src = host(t)
+        ref = oracle.slice_transform(src, dims, mode, sh, sc, inverse=inverse)
+        ctx.slice_transform(t, dims, mode, dev(sh), dev(sc), inverse=inverse, out=t)
+        if dt == torch.float64:
+            assert np.allclose(host(t), ref, rtol=4e-16 * 8, atol=1e-15 * np.abs(ref).max())
+        else:
+            assert np.all(np.abs(host(t) - ref) <= np.spacing(np.abs(ref).astype(np.float32)))
