@@ -338,19 +338,12 @@ int gram_kernel_for(tucker_prec prec, tucker_dtype dt, const SlabView& v, int sm
 }
 
 // Row maxima of the column-major mode-0 view (as FP32 bits) for the digit
-// scales of the exact tensor-core Gram; own scratch, so it may run on a side
-// stream.  Also gives the sum of squares, unused here.
+// scales of the exact tensor-core Gram.
 tucker_status rowmax_pass(tucker_ctx* c, const float* y, int64_t I0, int64_t ncols,
                           unsigned* rowmax) {
-  const int nb = c->num_sms * 4;
-  DevBuf scr;
-  TK_TRY(dev_alloc(c, scr, sizeof(double) * (2 * (size_t)nb + 2) + sizeof(unsigned)));
-  double* part = scr.as<double>();
-  double* out = part + 2 * nb;
-  unsigned* bad = reinterpret_cast<unsigned*>(out + 2);
-  TK_CUDA(c, cudaMemsetAsync(bad, 0, sizeof(unsigned), c->stream));
   TK_CUDA(c, cudaMemsetAsync(rowmax, 0, sizeof(unsigned) * I0, c->stream));
-  TK_CUDA(c, launch_sumsq_rowmax(y, I0, ncols, part, nb, bad, rowmax, out, c->stream));
+  TK_CUDA(c, launch_sumsq_rowmax(y, I0, ncols, nullptr, c->num_sms * 4, nullptr, rowmax, nullptr,
+                                 c->stream));
   return TUCKER_OK;
 }
 

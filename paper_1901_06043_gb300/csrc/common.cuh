@@ -97,4 +97,16 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {    // a - b, one ro
   return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
 }
 
+// A running 64-bit maximum by 32-bit comparisons: the 64-bit minimum and maximum
+// run at the rate of the FP64 pipe (as long as an FMA each).
+struct Max64 {
+  unsigned hi = 0, lo = 0;
+  __device__ __forceinline__ void add(unsigned h, unsigned l) {
+    lo = h > hi ? l : (h == hi ? max(lo, l) : lo);
+    hi = max(hi, h);
+  }
+  __device__ __forceinline__ void add(unsigned long long v) { add((unsigned)(v >> 32), (unsigned)v); }
+  __device__ __forceinline__ unsigned long long get() const { return (unsigned long long)hi << 32 | lo; }
+};
+
 }  // namespace tk

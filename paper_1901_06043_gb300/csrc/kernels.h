@@ -16,7 +16,7 @@ cudaError_t launch_sumsq(const void* y, tucker_dtype dt, int64_t n, double* part
 // The same over the column-major I0 x ncols mode-0 view, also recording each
 // row's max |x| as FP32 bits (atomicMax into the zeroed rowmax_bits[I0]);
 // I0 <= 8192, 4-byte aligned y (16-byte loads when I0 % 4 == 0 and y is
-// 16-byte aligned)
+// 16-byte aligned); out NULL: the row maxima alone
 cudaError_t launch_sumsq_rowmax(const float* y, int64_t I0, int64_t ncols, double* partial,
                                 int nblocks, unsigned* nonfinite, unsigned* rowmax_bits, double* out,
                                 cudaStream_t st);

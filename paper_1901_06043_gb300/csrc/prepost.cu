@@ -72,12 +72,14 @@ template <typename T, int PASS> struct Part;
 
 template <int PASS> struct Part<double, PASS> {
   double s, s2, sa, c2, mean;
-  long long mx, mn;                       // ordered bits: an FP64 comparison takes as
-                                          // long as an FMA, an integer one does not
+  long long mx, mn;                       // ordered bits
+  Max64 up, dn;                           // running maxima of the bits, biased, and of their
+                                          // complement: an FP64 comparison takes as long as an FMA
   __device__ void init(double m) {
     s = s2 = sa = c2 = 0.0;
     mx = ordered(-INFINITY);
     mn = ordered(INFINITY);
+    up = dn = Max64();
     mean = m;
   }
   __device__ __forceinline__ void add1(double v) {
@@ -85,9 +87,10 @@ template <int PASS> struct Part<double, PASS> {
       s += v;
       s2 = fma(v, v, s2);
       sa += fabs(v);
-      const long long k = ordered(v);
-      mx = max(mx, k);
-      mn = min(mn, k);
+      const unsigned f = (unsigned)(__double2hiint(v) >> 31);      // all ones: negative
+      const unsigned h = (unsigned)__double2hiint(v) ^ (f | 0x80000000u), l = (unsigned)__double2loint(v) ^ f;
+      up.add(h, l);
+      dn.add(~h, ~l);
     } else {
       const double d = v - mean;
       c2 = fma(d, d, c2);
@@ -95,7 +98,12 @@ template <int PASS> struct Part<double, PASS> {
   }
   __device__ __forceinline__ void add2(double v, double w) { add1(v); add1(w); }
   __device__ __forceinline__ void tick(int) {}
-  __device__ void flush() {}
+  __device__ void flush() {
+    if (PASS == 0 && (up.hi | dn.hi)) {
+      mx = max(mx, (long long)(up.get() ^ 0x8000000000000000ull));
+      mn = min(mn, (long long)(~dn.get() ^ 0x8000000000000000ull));
+    }
+  }
 };
 
 // (h, l) += v exactly in both halves
