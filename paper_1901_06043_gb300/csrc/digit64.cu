@@ -33,7 +33,8 @@
 //   NaN, Inf, or a row whose largest magnitude is below 2^-958 (its exponents
 // would need the denormal range): the exponent pass sets *bad and the caller
 // computes the step on the FP64 pipe (the host reads the flag with the error
-// word); a caller that does not wait gets NaN.
+// word); a caller that does not wait gets NaN for NaN and Inf, and small rows in
+// units of 2^-1013.
 //
 // Tile and roles.  One CTA owns a 128 x 64 tile (M x N): eight classes of 64
 // columns are all 512 tensor-memory columns.  The digit planes of the 64-row
@@ -120,12 +121,15 @@ __device__ __forceinline__ int mag_bits(double x) {
   return (__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0 ? 1 : 0);
 }
 __device__ __forceinline__ int mag_bits(float x) { return (int)(__float_as_uint(x) & 0x7fffffffu); }
-// MIN_EXP for a row of zeros; BAD_EXP for NaN, Inf and rows below MIN_EXP
-__device__ __forceinline__ int row_exp(int m, double) {
+// MIN_EXP for a row of zeros; BAD_EXP for NaN, Inf and rows below MIN_EXP.  A
+// caller that does not wait for the verdict (small = false) has such rows at
+// MIN_EXP: their entries are then off by up to 2^-1013 each, below the rounding of a
+// Gram's or a TTM's norm.
+__device__ __forceinline__ int row_exp(int m, double, int small) {
   const int e = m >> 20;
-  return m == 0 ? MIN_EXP : (e < MIN_EXP ? BAD_EXP : e);
+  return m == 0 ? MIN_EXP : (e < MIN_EXP ? (small ? BAD_EXP : MIN_EXP) : e);
 }
-__device__ __forceinline__ int row_exp(int m, float) {
+__device__ __forceinline__ int row_exp(int m, float, int) {
   const int e = m >> 23;
   return e == 0xff ? BAD_EXP : (e < 1 ? 1 : e) + 896;
 }
@@ -753,10 +757,11 @@ __global__ void __launch_bounds__(256) k_rowexp_runs(const T* __restrict__ x, in
 
 // Row maxima (magnitude bits) to exponents, in place.
 template <typename T>
-__global__ void k_rowexp_final(unsigned* __restrict__ rexp, int64_t I, unsigned* __restrict__ bad) {
+__global__ void k_rowexp_final(unsigned* __restrict__ rexp, int64_t I, int small,
+                               unsigned* __restrict__ bad) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= I) return;
-  const int e = row_exp((int)rexp[i], T());
+  const int e = row_exp((int)rexp[i], T(), small);
   rexp[i] = (unsigned)e;
   if (e == BAD_EXP) atomicOr(bad, 1u);
 }
@@ -786,7 +791,7 @@ GramPlan plan_gram_d64(int64_t L, int64_t I, int64_t Rt, int num_sms) {
 
 template <typename T>
 static cudaError_t launch_rowexp(const T* x, int64_t L, int64_t I, int64_t Rt, int num_sms,
-                                 unsigned* rexp, unsigned* bad, cudaStream_t st) {
+                                 int small, unsigned* rexp, unsigned* bad, cudaStream_t st) {
   // rexp[I], rexp[I + 1]: the verdict words
   cudaError_t e = cudaMemsetAsync(rexp, 0, sizeof(unsigned) * (size_t)(I + 2), st);
   if (e != cudaSuccess) return e;
@@ -803,7 +808,7 @@ static cudaError_t launch_rowexp(const T* x, int64_t L, int64_t I, int64_t Rt, i
     const int64_t warps = I * nck;
     k_rowexp_runs<T><<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(x, L, I, Rt, (int)nck, rexp);
   }
-  k_rowexp_final<T><<<(unsigned)((I + 255) / 256), 256, 0, st>>>(rexp, I, bad);
+  k_rowexp_final<T><<<(unsigned)((I + 255) / 256), 256, 0, st>>>(rexp, I, small, bad);
   count_launches(2);
   return cudaGetLastError();
 }
@@ -823,7 +828,7 @@ static cudaError_t gram_d64(const T* y, int64_t L, int64_t I, int64_t Rt, const 
   double* part = static_cast<double*>(scratch);
   unsigned* rexp = reinterpret_cast<unsigned*>(part + (size_t)p.nctas * TILE_ELEMS);
   unsigned* bad = rexp + I;
-  cudaError_t e = launch_rowexp(y, L, I, Rt, num_sms, rexp, bad, st);
+  cudaError_t e = launch_rowexp(y, L, I, Rt, num_sms, err == nullptr, rexp, bad, st);
   if (e != cudaSuccess) return e;
   Args a{};
   a.x = y;
@@ -869,7 +874,8 @@ cudaError_t launch_gram_d64(const void* y, tucker_dtype dt, int64_t L, int64_t I
 // m when the m are contiguous (L > 1) ...
 template <typename T>
 __global__ void __launch_bounds__(256) k_mexp_rows(const T* __restrict__ y, int64_t L, int64_t I,
-                                                   int64_t M, uint16_t* __restrict__ mexp,
+                                                   int64_t M, int small,
+                                                   uint16_t* __restrict__ mexp,
                                                    unsigned* __restrict__ bad) {
   const int64_t m = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (m >= M) return;
@@ -885,7 +891,7 @@ __global__ void __launch_bounds__(256) k_mexp_rows(const T* __restrict__ y, int6
     for (int u = 0; u < 8; ++u) b = max(b, mag_bits(v[u]));
   }
   for (; i < I; ++i) b = max(b, mag_bits(__ldg(p + L * i)));
-  const int e = row_exp(b, T());
+  const int e = row_exp(b, T(), small);
   mexp[m] = (uint16_t)e;
   if (e == BAD_EXP) atomicOr(bad, 1u);
 }
@@ -893,7 +899,7 @@ __global__ void __launch_bounds__(256) k_mexp_rows(const T* __restrict__ y, int6
 // ... and a warp per m (four at a time) when the contraction is (L == 1).
 template <typename T>
 __global__ void __launch_bounds__(256) k_mexp_cols(const T* __restrict__ y, int64_t I, int64_t M,
-                                                   uint16_t* __restrict__ mexp,
+                                                   int small, uint16_t* __restrict__ mexp,
                                                    unsigned* __restrict__ bad) {
   const int64_t m0 = 4 * (((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
@@ -915,7 +921,7 @@ __global__ void __launch_bounds__(256) k_mexp_cols(const T* __restrict__ y, int6
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) e[j] = max(e[j], __shfl_xor_sync(0xffffffffu, e[j], o));
     if (lane == 0 && m0 + j < M) {
-      const int x = row_exp(e[j], T());
+      const int x = row_exp(e[j], T(), small);
       mexp[m0 + j] = (uint16_t)x;
       if (x == BAD_EXP) atomicOr(bad, 1u);
     }
@@ -926,7 +932,7 @@ __global__ void __launch_bounds__(256) k_mexp_cols(const T* __restrict__ y, int6
 // planes of rows k = 64 nt.., columns i = 32 ks.. (zero outside K x I) in the
 // 64-row operand's layout; kexp[64 nt + row] = the row's exponent.
 __global__ void __launch_bounds__(256) k_digit64_prep(const double* __restrict__ A, int K,
-                                                      int64_t I, int64_t lda, int arow,
+                                                      int64_t I, int64_t lda, int arow, int small,
                                                       uint8_t* __restrict__ img,
                                                       unsigned* __restrict__ kexp,
                                                       unsigned* __restrict__ bad) {
@@ -953,7 +959,7 @@ __global__ void __launch_bounds__(256) k_digit64_prep(const double* __restrict__
     atomicMax(&eb[row], e);
   }
   __syncthreads();
-  if (threadIdx.x < NT) eb[threadIdx.x] = row_exp(eb[threadIdx.x], 0.0);
+  if (threadIdx.x < NT) eb[threadIdx.x] = row_exp(eb[threadIdx.x], 0.0, small);
   __syncthreads();
   if (ks == 0 && threadIdx.x < NT) {
     kexp[nt * NT + threadIdx.x] = (unsigned)eb[threadIdx.x];
@@ -1036,12 +1042,13 @@ static cudaError_t ttm_d64(const T* y, int64_t L, int64_t I, int64_t Rt, const d
   a.kexp = kexp;
   a.z = z;
   a.zt = zt ? 1 : 0;
+  const int small = err == nullptr;                      // the caller reads the verdict
   k_digit64_prep<<<dim3((unsigned)a.nks, (unsigned)a.ntn), 256, 0, st>>>(A, (int)K, I, lda, arow,
-                                                                        scr + lay.img, kexp, bad);
+                                                                        small, scr + lay.img, kexp, bad);
   if (L > 1)
-    k_mexp_rows<T><<<(unsigned)((a.M + 255) / 256), 256, 0, st>>>(y, L, I, a.M, mexp, bad);
+    k_mexp_rows<T><<<(unsigned)((a.M + 255) / 256), 256, 0, st>>>(y, L, I, a.M, small, mexp, bad);
   else
-    k_mexp_cols<T><<<(unsigned)((a.M + 31) / 32), 256, 0, st>>>(y, I, a.M, mexp, bad);
+    k_mexp_cols<T><<<(unsigned)((a.M + 31) / 32), 256, 0, st>>>(y, I, a.M, small, mexp, bad);
   const unsigned grid = (unsigned)std::min<int64_t>(a.nitems, num_sms);
   const bool vec = L > 1 && L % 4 == 0 && ((uintptr_t)y & 15) == 0;
   auto go = [&](auto kern) -> cudaError_t {

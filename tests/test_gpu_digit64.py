@@ -134,3 +134,24 @@ def test_fp64_digits_out_of_range_take_the_fp64_pipe(ctx, what):
             assert np.array_equal(np.isnan(got), np.isnan(want))
             assert np.array_equal(got[np.isinf(want)], want[np.isinf(want)])
             assert (np.abs(got - want)[fin] <= 1400 * 2.0 ** -52 * scale[fin] + 1e-322).all()
+
+
+def test_batched_tensors_with_tiny_slices(ctx):
+    """A batch does not wait for the verdict on each step; a slice below the digits' range
+    (here 1e-295 of the others) is as good as zero there, as it is in the norm."""
+    from paper_1901_06043_gb300 import synth
+    import torch
+    dims = (70, 80, 90)
+    x, _ = synth.tucker_numpy(dims, (9, 8, 7), decay=0.2, eta=1e-6, seed=3)
+    x = np.asarray(x, dtype=np.float64).reshape(dims, order="F")
+    x[5] *= 1e-295
+    x[:, 7] *= 1e-295
+    xs = torch.from_numpy(x.reshape(-1, order="F").copy()).cuda()
+    one = ctx.sthosvd(xs, dims, eps=1e-4, prec="fp64")
+    many = ctx.sthosvd_batched([xs, xs], [dims, dims], eps=1e-4, prec="fp64")
+    whole = one.reconstruct().cpu().numpy()
+    for r in many:
+        assert r.ranks == one.ranks
+        # both are within eps of x; between them, the last kept vectors turn by rounding
+        # over their gap: 1e-9 as for single steps of this size
+        assert np.linalg.norm(r.reconstruct().cpu().numpy() - whole) <= 1e-9 * np.linalg.norm(whole)
