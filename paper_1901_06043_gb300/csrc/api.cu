@@ -430,6 +430,22 @@ tucker_status gram_once(tucker_ctx* c, const void* y, tucker_dtype dt, const Sla
     }
     return TUCKER_OK;
   }
+  if (kern == 0 || kern == 3) {
+    // FP64 products: seven exact digits on the tensor cores from the size
+    // where they beat the FP64 pipe (digit64.cu); out of their range (NaN,
+    // Inf, rows below 2^-958): the FP64 pipe
+    const GramPlan pd = plan_gram_d64(v.L, v.I, v.Rt, sms);
+    if (pd.nctas > 0) {
+      DevBuf scratch;
+      TK_TRY(dev_alloc(c, scratch, pd.scratch_bytes));
+      TK_CUDA(c, launch_gram_d64(y, dt, v.L, v.I, v.Rt, pd, c->num_sms, scratch.p,
+                                 check ? nullptr : c->d_words + 8, S, c->stream));
+      if (!check) return TUCKER_OK;
+      bool bad = false;
+      TK_TRY(digit64_verdict(c, gram_d64_verdict(pd, v.I, scratch.p), "Gram", &bad));
+      if (!bad) return TUCKER_OK;
+    }
+  }
   if (kern == 3) {
     const GramPlan ps = plan_gram_small(v.L, v.I, v.Rt, sms, v.L0);
     DevBuf scratch;
@@ -447,22 +463,6 @@ tucker_status gram_once(tucker_ctx* c, const void* y, tucker_dtype dt, const Sla
       TK_CUDA(c, launch_gram_f32((const float*)y, v.L, v.I, v.Rt, v.L0, pc, scratch.as<double>(),
                                  S, c->stream));
       return TUCKER_OK;
-    }
-  }
-  if (kern == 0) {
-    // FP64 products: seven exact digits on the tensor cores from the size
-    // where they beat the FP64 pipe (digit64.cu); out of their range (NaN,
-    // Inf, rows below 2^-958): the FP64 pipe
-    const GramPlan pd = plan_gram_d64(v.L, v.I, v.Rt, sms);
-    if (pd.nctas > 0) {
-      DevBuf scratch;
-      TK_TRY(dev_alloc(c, scratch, pd.scratch_bytes));
-      TK_CUDA(c, launch_gram_d64(y, dt, v.L, v.I, v.Rt, pd, c->num_sms, scratch.p,
-                                 check ? nullptr : c->d_words + 8, S, c->stream));
-      if (!check) return TUCKER_OK;
-      bool bad = false;
-      TK_TRY(digit64_verdict(c, gram_d64_verdict(pd, v.I, scratch.p), "Gram", &bad));
-      if (!bad) return TUCKER_OK;
     }
   }
   GramPlan p = plan_gram_simt(v.L, v.I, v.Rt, sms, v.L0);
@@ -557,7 +557,9 @@ size_t gram_scratch_bytes(const tucker_ctx* c, tucker_prec prec, tucker_dtype dt
   const int kern = gram_kernel_for(prec, dt, v, c->num_sms);
   if (kern == 5) return plan_gram_tcx(v.L, v.I, v.Rt, c->num_sms).scratch_bytes + 8 * (size_t)v.I;
   if (kern == 2) return plan_gram_tc(v.L, v.I, v.Rt, c->num_sms).scratch_bytes;
-  if (kern == 3) return plan_gram_small(v.L, v.I, v.Rt, c->num_sms, v.L0).scratch_bytes;
+  if (kern == 3)
+    return std::max(plan_gram_small(v.L, v.I, v.Rt, c->num_sms, v.L0).scratch_bytes,
+                    plan_gram_d64(v.L, v.I, v.Rt, c->num_sms).scratch_bytes);
   if (kern == 1 && dt == TUCKER_F32) {
     const GramPlan pc = plan_gram_f32(v.L, v.I, v.Rt, c->num_sms, v.L0);
     if (pc.ntiles > 0) return pc.scratch_bytes;

@@ -103,6 +103,11 @@ constexpr int OUT_EXP = -2 * 1022 - 70;        // an entry is its sum times 2^(e
 // I = 60), or 2 K I M >= 4e7 (I = 26: 95 and 87 us; 64 and 87 us at 2e7).
 constexpr double kDigit64MinGram = 2e7, kDigit64MinTtm = 4e7;
 constexpr int kDigit64MinTtmI = 64;
+// Modes below 64 (gram_small.cu otherwise, ~I^2 / 2 FP64 instructions per 32 k;
+// here ~0.6 ns a k whatever I, one padded tile): K (I^2 - 565) >= 6.5e7.  Whole calls
+// there and here: I = 28, K = 4e5 342 and 332 us (2e5 197 and 220); I = 40, 5e4 122 and
+// 125 (1e5 193 and 155); I = 63, 2e4 136 and 113 (1e6 3.44 and 0.71 ms).
+constexpr double kDigit64SmallII = 565, kDigit64SmallGram = 6.5e7;
 
 // Byte offset of (mn, k) in plane 0 of an operand region with k-group stride kg.
 __device__ __forceinline__ uint32_t mn_off(int mn, int k, uint32_t kg) {
@@ -770,9 +775,9 @@ __global__ void k_rowexp_final(unsigned* __restrict__ rexp, int64_t I, int small
 
 GramPlan plan_gram_d64(int64_t L, int64_t I, int64_t Rt, int num_sms) {
   GramPlan p;
-  if (I < 64 || I > 8192 || L < 1 || Rt < 1 || L * I >= ((int64_t)1 << 31)) return p;
-  const double K = (double)L * (double)Rt;
-  if ((double)I * (double)I * K < kDigit64MinGram) return p;
+  if (I < 1 || I > 8192 || L < 1 || Rt < 1 || L * I >= ((int64_t)1 << 31)) return p;
+  const double K = (double)L * (double)Rt, II = (double)I * (double)I;
+  if (I < 64 ? (II - kDigit64SmallII) * K < kDigit64SmallGram : II * K < kDigit64MinGram) return p;
   const int64_t stages = (L * Rt + BK - 1) / BK;
   const int TA = (int)((I + MT - 1) / MT), TB = (int)((I + NT - 1) / NT);
   int ntiles = 0;

@@ -10,7 +10,8 @@
 // threshold on a 256x256x256x11x32 tensor.  The work is I(I+1)/2 FP64 FMAs
 // per K element (products of FP32 inputs are exact in FP64), which for
 // I < 64 is a small fraction of the mode's reads even at this part's FP64
-// rate.
+// rate.  (From the size where it is not, the same products run on exact integer
+// digits, digit64.cu.)
 //
 // Layout: one thread per entry (i <= j) of the lower triangle (several per
 // thread when I(I+1)/2 > 256); a CTA stages K-blocks of 64 (the K geometry of

@@ -57,7 +57,9 @@ GRAMS = [  # dims, mode, shift
     ((128, 1300), 0, 1), ((129, 1217), 0, 0), ((192, 16, 37), 0, 0), ((200, 129, 7), 0, 0),
     ((500, 128), 0, 0), ((513, 100), 0, 0),
     ((2, 130, 700), 1, 0), ((3, 64, 1700), 1, 1), ((5, 7, 150, 31), 2, 0), ((33, 200, 19), 1, 0),
-    ((1700, 129), 1, 0), ((16, 257, 33), 1, 0)]
+    ((1700, 129), 1, 0), ((16, 257, 33), 1, 0),
+    # modes below 64, where K (I^2 - 565) reaches 6.5e7: one padded tile
+    ((63, 22000), 0, 0), ((48, 45100), 0, 1), ((130, 60, 199), 1, 0), ((3, 50, 13000), 1, 1)]
 
 
 @pytest.mark.parametrize("dtype,spread", [("f8", False), ("f8", True), ("f4", False)])
