@@ -591,10 +591,287 @@ cudaError_t launch_gram_simt(const void* y, tucker_dtype dt, bool fp64, int64_t 
 }
 
 // ------------------------------------------------------------------- TTM
+//
+// Z (K x M) = A (K x I) * Y (I x M), M = the (l, r) pairs of the slab view, l
+// fastest.  A block of four warps owns MT m and KT outputs, KT = 8, 16, 24 or 32, the
+// smallest that divides K into tiles of at most 32 (few outputs are what a
+// truncation leaves).  WK warps share the outputs and 4 / WK the m; a thread owns MM
+// m (lane + 32 j) and KK = KT / WK outputs of each.  The sums run over i in order.
+//   Stages of 32 i, two in turn, through registers a quarter at a time between the
+// products (16-byte accesses where the view allows).  L > 1: Y as it lies, m fastest.
+// L == 1: a row of 32 i per m, padded by 16 bytes, so that 16-byte reads of one m per
+// lane do not conflict; zt writes Z transposed (z[m + M k]), else the block's Z
+// goes through shared memory, k being fastest.
+//   Bound: instructions (FP64: its pipe).  FP32 products go two outputs at a time
+// (f32x2); addresses advance by additions, bounds are tested only in tiles that need
+// it (64-bit comparisons run at the FP64 pipe's rate); four blocks per SM (two
+// blocks of 256 m took 1.2 times as long).  Measured, with one 64 x 64 tile per block
+// before: I = 301, M = 287,000, K = 20 (345 MB) 540 -> 183 us; I = 200, M = 56,000 82 -> 31;
+// row view 3.5e6 x 32 to 10 638 -> 226; I = 54, M = 32,000 to 502 106 -> 81; FP64 I = 40,
+// M = 1500, K = 5 55 -> 17.
+constexpr int TNT = 128;                  // threads
+constexpr int TIC = 32;                   // i per stage
+
+// round to nearest by integer operations (a conversion takes the FP64 pipe's 64
+// cycles per warp); out of FP32's normal range: the conversion
+__device__ __forceinline__ float f64_to_f32(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u >= 253u) return (float)v;             // 2^-126 <= |v| < 2^127 below
+  const unsigned m = __funnelshift_l(lo, hi, 3);     // low 20 + 3 mantissa bits, exponent above
+  const unsigned rest = lo << 3;                     // the 29 bits dropped, at the top
+  unsigned r = ((e - 896u) << 23) | (m & 0x7fffffu);
+  r += (rest > 0x80000000u || (rest == 0x80000000u && (r & 1u))) ? 1u : 0u;
+  return __uint_as_float((hi & 0x80000000u) | r);
+}
+
+// dynamic shared memory: two stages of Y, then (L == 1) the block's Z
+template <typename TIn, typename TC, int KT, int MT, bool COL>
+constexpr size_t ttm_smem() {
+  return COL ? std::max(2 * (size_t)MT * (TIC * sizeof(TIn) + 16), (size_t)MT * (KT + 1) * sizeof(TC))
+             : 2 * (size_t)MT * TIC * sizeof(TIn);
+}
+
+template <typename TIn, typename TOut, typename TC, int KT, int WK, int MM, bool COL>
+__global__ void __launch_bounds__(TNT, sizeof(TC) == 4 ? 4 : 2)
+    k_ttm(const TIn* __restrict__ y, int64_t L, int64_t I,
+                                             int64_t M, const double* __restrict__ A, int64_t K,
+                                             int64_t lda, int a_rowmajor,
+                                             const float* __restrict__ A32, TOut* __restrict__ z,
+                                             int zt) {
+  constexpr int NW = TNT / 32, MT = NW / WK * 32 * MM, KK = KT / WK;
+  constexpr int KP = KT + 16 / (int)sizeof(TC);                     // padded, 16-byte rows
+  constexpr int VY = 16 / (int)sizeof(TIn), YP = TIC + VY;
+  __shared__ __align__(16) TC As[2][TIC][KP];
+  extern __shared__ __align__(16) unsigned char ttm_sm[];
+  TIn* Ys = reinterpret_cast<TIn*>(ttm_sm);                         // COL: [2][MT][YP], else [2][TIC][MT]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t m0 = (int64_t)blockIdx.x * MT, k0 = (int64_t)blockIdx.y * KT;
+  const int nk = (int)min((int64_t)KT, K - k0);
+
+  // entries of A for i0..: threads along whichever index is contiguous
+  constexpr int AE = TIC * KT / TNT;
+  const bool ifast = A32 || a_rowmajor;
+  auto load_a = [&](double (&v)[AE], int64_t i0) {
+#pragma unroll
+    for (int e = 0; e < AE; ++e) {
+      const int idx = tid + TNT * e;
+      const int ii = ifast ? idx % TIC : idx / KT, kk = ifast ? idx / TIC : idx % KT;
+      const int64_t i = i0 + ii, k = k0 + kk;
+      v[e] = 0.0;
+      if (kk < nk && i < I) {
+        if (sizeof(TC) == 4 && A32) v[e] = __hiloint2double(0, __float_as_int(A32[k * I + i]));   // bits
+        else v[e] = a_rowmajor ? A[k * lda + i] : A[k + lda * i];
+      }
+    }
+  };
+  auto store_a = [&](const double (&v)[AE], int b) {
+#pragma unroll
+    for (int e = 0; e < AE; ++e) {
+      const int idx = tid + TNT * e;
+      const int ii = ifast ? idx % TIC : idx / KT, kk = ifast ? idx / TIC : idx % KT;
+      if constexpr (sizeof(TC) == 4) As[b][ii][kk] = A32 ? __int_as_float(__double2loint(v[e])) : f64_to_f32(v[e]);
+      else As[b][ii][kk] = v[e];
+    }
+  };
+  // a stage of Y in four parts of PB values per thread; 16-byte accesses: chunk c of
+  // the stage, CPR per row of it, by thread c % TNT
+  constexpr int PB = MT * TIC / TNT / 4, CPR = (COL ? TIC : MT) / VY, ME = MT / TNT;
+  const bool y16 = (COL ? I : L) % VY == 0 && ((uintptr_t)y & 15) == 0;
+  const int cq = y16 ? tid % CPR * VY : (COL ? lane : tid);         // first column
+  int64_t yo[COL ? 1 : ME];                                         // ROW: offsets of this thread's m
+  if constexpr (!COL) {
+#pragma unroll
+    for (int e = 0; e < ME; ++e) {
+      const int64_t m = m0 + cq + (y16 ? 0 : TNT * e), r = m / L;
+      yo[e] = m < M ? m - r * L + L * I * r : -1;
+    }
+  }
+  auto row16 = [&](int q, int e) { return (q * (PB / VY) + e) * (TNT / CPR) + tid / CPR; };
+  using V16 = typename std::conditional<sizeof(TIn) == 4, float4, double2>::type;
+  const bool mfull = m0 + MT <= M;
+  const int64_t step = COL ? I * (y16 ? TNT / CPR : NW) : L * (y16 ? TNT / CPR : 1);   // per row copied
+  auto load_y = [&](TIn* v, int q, int64_t i0) {
+    const bool full = mfull && i0 + TIC <= I;             // else every access is tested
+    if (y16) {
+      const int r0 = row16(q, 0);
+      const TIn* p = COL ? y + I * (m0 + r0) + i0 + cq : y + yo[0] + L * (i0 + r0);
+#pragma unroll
+      for (int e = 0; e < PB / VY; ++e, p += step) {
+        const int r = r0 + e * (TNT / CPR);
+        const bool ok = full || (COL ? (i0 + cq < I && m0 + r < M) : (i0 + r < I && yo[0] >= 0));
+        *reinterpret_cast<V16*>(v + VY * e) = ok ? __ldg(reinterpret_cast<const V16*>(p)) : V16{};
+      }
+    } else {
+      const int r0 = COL ? warp + NW * q * PB : q * PB / ME;
+      const TIn* p[COL ? 1 : ME];
+#pragma unroll
+      for (int c = 0; c < (COL ? 1 : ME); ++c)
+        p[c] = COL ? y + I * (m0 + r0) + i0 + cq : y + yo[c] + L * (i0 + r0);
+      if (full) {
+#pragma unroll
+        for (int e = 0; e < PB; ++e) {
+          v[e] = __ldg(p[COL ? 0 : e % ME]);
+          p[COL ? 0 : e % ME] += step;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < PB; ++e) {
+          const int r = COL ? r0 + NW * e : r0 + e / ME;
+          const bool ok = COL ? (i0 + cq < I && m0 + r < M) : (i0 + r < I && yo[e % ME] >= 0);
+          v[e] = ok ? __ldg(p[COL ? 0 : e % ME]) : (TIn)0;
+          p[COL ? 0 : e % ME] += step;
+        }
+      }
+    }
+  };
+  auto store_y = [&](const TIn* v, int q, int b) {
+    TIn* d = Ys + (size_t)b * (COL ? MT * YP : MT * TIC) + cq;
+    constexpr int P = COL ? YP : MT;
+    if (y16) {
+#pragma unroll
+      for (int e = 0; e < PB / VY; ++e)
+        *reinterpret_cast<V16*>(d + row16(q, e) * P) = *reinterpret_cast<const V16*>(v + VY * e);
+    } else {
+#pragma unroll
+      for (int e = 0; e < PB; ++e) {
+        const int r = COL ? warp + NW * (q * PB + e) : (q * PB + e) / ME;
+        d[r * P + (COL ? 0 : TNT * (e % ME))] = v[e];
+      }
+    }
+  };
+
+  // this thread's outputs kq.. and m (within the block) mq + 32 j
+  const int kq = warp % WK * KK, mq = warp / WK * 32 * MM + lane;
+  TC acc[MM][KK];
+#pragma unroll
+  for (int j = 0; j < MM; ++j)
+#pragma unroll
+    for (int k = 0; k < KK; ++k) acc[j][k] = (TC)0;
+  auto mac = [&](const TC* a, const TC (&v)[MM]) {
+    __align__(16) TC av[KK];
+    constexpr int VB = KK * sizeof(TC) % 16 == 0 ? 16 : 8;
+#pragma unroll
+    for (int k = 0; k < KK; k += VB / (int)sizeof(TC)) {
+      if constexpr (VB == 16) *reinterpret_cast<float4*>(av + k) = *reinterpret_cast<const float4*>(a + k);
+      else *reinterpret_cast<float2*>(av + k) = *reinterpret_cast<const float2*>(a + k);
+    }
+#pragma unroll
+    for (int j = 0; j < MM; ++j) {
+      if constexpr (sizeof(TC) == 4) {
+#pragma unroll
+        for (int k = 0; k < KK; k += 2) {
+          const float2 r = fma2(make_float2(av[k], av[k + 1]), make_float2(v[j], v[j]),
+                                make_float2(acc[j][k], acc[j][k + 1]));
+          acc[j][k] = r.x;
+          acc[j][k + 1] = r.y;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < KK; ++k) acc[j][k] = fma(av[k], v[j], acc[j][k]);
+      }
+    }
+  };
+
+  const int64_t nst = (I + TIC - 1) / TIC;
+  {
+    __align__(16) TIn v[2][PB];
+    double av[AE];
+    load_y(v[0], 0, 0);
+    load_y(v[1], 1, 0);
+    load_a(av, 0);
+    store_y(v[0], 0, 0);
+    store_y(v[1], 1, 0);
+    load_y(v[0], 2, 0);
+    load_y(v[1], 3, 0);
+    store_a(av, 0);
+    store_y(v[0], 2, 0);
+    store_y(v[1], 3, 0);
+  }
+  for (int64_t s = 0; s < nst; ++s) {
+    const int b = (int)(s & 1);
+    const int ni = (int)min((int64_t)TIC, I - s * TIC);             // (past I: zeros)
+    const bool more = s + 1 < nst;
+    __syncthreads();                      // stage s is there, stage s - 1 is used up
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+      __align__(16) TIn nv[PB];
+      double av[AE];
+      if (more) {
+        load_y(nv, q, (s + 1) * TIC);
+        if (q == 0) load_a(av, (s + 1) * TIC);
+      }
+      constexpr int QI = TIC / 4;
+      if (QI * q < ni) {
+        if constexpr (COL) {
+          const TIn* ys = Ys + ((size_t)b * MT + mq) * YP + QI * q;
+#pragma unroll 1
+          for (int i = 0; i < QI; i += VY) {
+            __align__(16) TIn x[MM][VY];
+#pragma unroll
+            for (int j = 0; j < MM; ++j)
+              *reinterpret_cast<V16*>(x[j]) = *reinterpret_cast<const V16*>(ys + 32 * j * YP + i);
+#pragma unroll
+            for (int w = 0; w < VY; ++w) {
+              TC v[MM];
+#pragma unroll
+              for (int j = 0; j < MM; ++j) v[j] = (TC)x[j][w];
+              mac(&As[b][QI * q + i + w][kq], v);
+            }
+          }
+        } else {
+          const TIn* ys = Ys + (size_t)b * MT * TIC + QI * q * MT + mq;
+#pragma unroll 4
+          for (int i = 0; i < QI; ++i) {
+            TC v[MM];
+#pragma unroll
+            for (int j = 0; j < MM; ++j) v[j] = (TC)ys[i * MT + 32 * j];
+            mac(&As[b][QI * q + i][kq], v);
+          }
+        }
+      }
+      if (more) {
+        store_y(nv, q, b ^ 1);
+        if (q == 0) store_a(av, b ^ 1);
+      }
+    }
+  }
+  if (COL && !zt) __syncthreads();
+
+  if (COL && !zt) {
+    // z[k + K m]: through shared memory, lanes along k
+    TC* zs = reinterpret_cast<TC*>(ttm_sm);                         // [MT][KT + 1]
+    constexpr int ZP = KT + 1;
+#pragma unroll
+    for (int j = 0; j < MM; ++j)
+#pragma unroll
+      for (int k = 0; k < KK; ++k) zs[(mq + 32 * j) * ZP + kq + k] = acc[j][k];
+    __syncthreads();
+    constexpr int RPW = KT >= 24 ? 1 : 32 / KT;                     // rows of m per warp
+    const int k = KT >= 24 ? lane : lane % KT, sub = KT >= 24 ? 0 : lane / KT;
+    const int mc = (int)min((int64_t)MT, M - m0);
+    if (k < nk) {
+      TOut* zr = z + K * m0 + k0 + k;
+      for (int m = warp * RPW + sub; m < mc; m += NW * RPW) zr[K * m] = (TOut)zs[m * ZP + k];
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < MM; ++j) {
+      const int64_t m = m0 + mq + 32 * j;
+      if (m >= M) continue;
+      const int64_t r = COL ? 0 : m / L;
+      TOut* zr = z + (m - r * L) + (COL ? 0 : L * K * r) + (COL ? M : L) * (k0 + kq);
+#pragma unroll
+      for (int k = 0; k < KK; ++k)
+        if (kq + k < nk) zr[(COL ? M : L) * k] = (TOut)acc[j][k];
+    }
+  }
+}
 
 constexpr int TT = 64;    // output tile (k and m)
 constexpr int TBI = 16;   // contraction step
 
+// FP32 arithmetic on FP64 input or output (a 64 x 64 tile per block).
 // Z (K x M) = A (K x I) * Y (I x M), M = the (r, l) pairs of the slab view.
 // Row mode (L > 1): an m-tile is 64 consecutive l of one slab.  Column mode
 // (L == 1): an m-tile is 64 consecutive slabs; zt writes Z transposed
@@ -710,16 +987,36 @@ __global__ void k_ttm_a32(const double* __restrict__ A, int64_t K, int64_t I, in
   }
 }
 
-template <typename TIn, typename TOut>
-static void ttm_dispatch_c(bool fp64, dim3 grid, cudaStream_t st, const void* y, int64_t L, int64_t I,
-                           int64_t Rt, int64_t nLT, const double* A, int64_t K, int64_t lda,
-                           int arow, const float* A32, void* z, int zt) {
-  if (fp64)
-    k_ttm_simt<TIn, TOut, double><<<grid, 256, 0, st>>>((const TIn*)y, L, I, Rt, nLT, A, K, lda, arow,
-                                                        nullptr, (TOut*)z, zt);
-  else
-    k_ttm_simt<TIn, TOut, float><<<grid, 256, 0, st>>>((const TIn*)y, L, I, Rt, nLT, A, K, lda, arow,
-                                                       A32, (TOut*)z, zt);
+template <typename TIn, typename TOut, typename TC, int KT, bool COL>
+static cudaError_t ttm_tile(const TIn* y, int64_t L, int64_t I, int64_t M, const double* A, int64_t K,
+                            int64_t lda, int arow, const float* A32, TOut* z, int zt,
+                            cudaStream_t st) {
+  constexpr int WK = KT == 8 ? 2 : 4, MM = WK, MT = TNT;
+  const int64_t gx = (M + MT - 1) / MT;
+  if (gx > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+  auto kern = k_ttm<TIn, TOut, TC, KT, WK, MM, COL>;
+  cudaError_t e = allow_max_dyn_smem((const void*)kern);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3((unsigned)gx, (unsigned)((K + KT - 1) / KT)), TNT, ttm_smem<TIn, TC, KT, MT, COL>(), st>>>(
+      y, L, I, M, A, K, lda, arow, A32, z, zt);
+  return cudaGetLastError();
+}
+
+template <typename TIn, typename TOut, typename TC>
+static cudaError_t ttm_new(const void* y, int64_t L, int64_t I, int64_t Rt, const double* A, int64_t K,
+                           int64_t lda, int arow, const float* A32, void* z, int zt,
+                           cudaStream_t st) {
+  const int64_t nt = (K + 31) / 32, per = (K + nt - 1) / nt;       // outputs per tile
+  auto tile = [&](auto KT) {
+    return L == 1 ? ttm_tile<TIn, TOut, TC, decltype(KT)::value, true>(
+                        (const TIn*)y, L, I, Rt, A, K, lda, arow, A32, (TOut*)z, zt, st)
+                  : ttm_tile<TIn, TOut, TC, decltype(KT)::value, false>(
+                        (const TIn*)y, L, I, L * Rt, A, K, lda, arow, A32, (TOut*)z, zt, st);
+  };
+  if (per <= 8) return tile(std::integral_constant<int, 8>());
+  if (per <= 16) return tile(std::integral_constant<int, 16>());
+  if (per <= 24) return tile(std::integral_constant<int, 24>());
+  return tile(std::integral_constant<int, 32>());
 }
 
 cudaError_t launch_ttm_simt(const void* y, tucker_dtype ydt, bool fp64, int64_t L, int64_t I,
@@ -727,12 +1024,7 @@ cudaError_t launch_ttm_simt(const void* y, tucker_dtype ydt, bool fp64, int64_t 
                             float* a32_scratch, void* z, tucker_dtype zdt, cudaStream_t st,
                             bool zt) {
   if (zt && L != 1) return cudaErrorInvalidValue;
-  int64_t nLT = 1, nMT;
-  if (L == 1) nMT = (Rt + TT - 1) / TT;
-  else { nLT = (L + TT - 1) / TT; nMT = Rt * nLT; }
-  if (nMT <= 0 || K <= 0) return cudaSuccess;
-  if (nMT > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-  dim3 grid((unsigned)nMT, (unsigned)((K + TT - 1) / TT));
+  if (L * Rt <= 0 || K <= 0) return cudaSuccess;
   const float* A32 = nullptr;
   if (!fp64 && a32_scratch) {
     const int64_t n = K * I;
@@ -742,13 +1034,23 @@ cudaError_t launch_ttm_simt(const void* y, tucker_dtype ydt, bool fp64, int64_t 
     A32 = a32_scratch;
   }
   count_launches(1);
-  if (ydt == TUCKER_F64) {
-    if (zdt == TUCKER_F64) ttm_dispatch_c<double, double>(fp64, grid, st, y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, z, zt);
-    else ttm_dispatch_c<double, float>(fp64, grid, st, y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, z, zt);
-  } else {
-    if (zdt == TUCKER_F64) ttm_dispatch_c<float, double>(fp64, grid, st, y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, z, zt);
-    else ttm_dispatch_c<float, float>(fp64, grid, st, y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, z, zt);
+  const bool yd = ydt == TUCKER_F64, zd = zdt == TUCKER_F64;
+  if (fp64) {
+    if (yd) return zd ? ttm_new<double, double, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st)
+                      : ttm_new<double, float, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st);
+    return zd ? ttm_new<float, double, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st)
+              : ttm_new<float, float, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st);
   }
+  if (!yd && !zd) return ttm_new<float, float, float>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st);
+  const int64_t nLT = L == 1 ? 1 : (L + TT - 1) / TT, nMT = L == 1 ? (Rt + TT - 1) / TT : Rt * nLT;
+  if (nMT > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+  const dim3 grid((unsigned)nMT, (unsigned)((K + TT - 1) / TT));
+  if (yd && zd)
+    k_ttm_simt<double, double, float><<<grid, 256, 0, st>>>((const double*)y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, (double*)z, zt);
+  else if (yd)
+    k_ttm_simt<double, float, float><<<grid, 256, 0, st>>>((const double*)y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, (float*)z, zt);
+  else
+    k_ttm_simt<float, double, float><<<grid, 256, 0, st>>>((const float*)y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, (double*)z, zt);
   return cudaGetLastError();
 }
 

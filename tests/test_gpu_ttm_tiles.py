@@ -1,0 +1,55 @@
+"""The TTM on the FP32 and FP64 pipes at the edges of its tiles: outputs around the tile
+widths (8, 16, 24, 32 and several tiles), products below and above a block's m and
+above the size from which a thread takes several, contraction lengths around a
+stage of 32, column views (L = 1) and row views, unaligned inputs.
+
+Bound per entry: the sum of I products in order, I u sum |a||y| with u = 2^-24 (FP32:
+and both operands rounded once, 2 u) or 2^-53, and one rounding of an FP32 result.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1901_06043_gb300 import tucker
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    c = tucker.Context()
+    yield c
+    c.close()
+
+
+VIEWS = [  # dims, mode
+    ((1, 1), 0), ((5, 127), 0), ((31, 129), 0), ((32, 40), 0), ((33, 700), 0), ((47, 90000), 0),
+    ((3, 5), 1), ((128, 31), 1), ((7, 33, 19), 1), ((129, 40, 1), 1), ((11, 13, 32), 2),
+    ((301, 9, 120), 1), ((400, 33, 300), 1)]
+
+
+@pytest.mark.parametrize("dims,mode", VIEWS)
+@pytest.mark.parametrize("K", [1, 8, 9, 17, 24, 25, 32, 33, 70])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_ttm_tiles(ctx, dims, mode, K, prec):
+    from paper_1901_06043_gb300 import tucker
+    rng = np.random.default_rng(K + dims[0])
+    x = rng.standard_normal(int(np.prod(dims)))
+    A = rng.standard_normal((K, dims[mode]))
+    U = np.moveaxis(x.reshape(dims, order="F"), mode, 0).reshape(dims[mode], -1)
+    scale = np.abs(A) @ np.abs(U)
+    want = A @ U
+    zd = list(dims)
+    zd[mode] = K
+    buf = torch.empty(x.size + 1, device="cuda", dtype=torch.float32 if prec == "fp32" else torch.float64)
+    t = buf[1:]
+    t.copy_(torch.from_numpy(x))
+    I = dims[mode]
+    for arow in (True, False):
+        At = torch.from_numpy(A).cuda() if arow else torch.from_numpy(A.T.copy()).cuda().t()
+        for out in (tucker.F32, tucker.F64):
+            z = ctx.ttm(t, dims, mode, At, prec=prec, out_dtype=out).double().cpu().numpy()
+            z = np.moveaxis(z.reshape(zd, order="F"), mode, 0).reshape(K, -1)
+            u = 2.0 ** -24 if prec == "fp32" else 2.0 ** -53
+            bound = (I + 3) * u * scale + (2.0 ** -24 * np.abs(want) if out == tucker.F32 else 0.0)
+            assert (np.abs(z - want) <= bound).all()
