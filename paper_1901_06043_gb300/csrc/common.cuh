@@ -109,4 +109,17 @@ struct Max64 {
   __device__ __forceinline__ unsigned long long get() const { return (unsigned long long)hi << 32 | lo; }
 };
 
+// FP64 to FP32, to nearest, by integer operations (a conversion takes the FP64
+// pipe's 64 cycles per warp); out of FP32's normal range: the conversion.
+__device__ __forceinline__ float f64_to_f32(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u >= 253u) return (float)v;             // 2^-126 <= |v| < 2^127 below
+  const unsigned m = __funnelshift_l(lo, hi, 3);     // low 20 + 3 mantissa bits, exponent above
+  const unsigned rest = lo << 3;                     // the 29 bits dropped, at the top
+  unsigned r = ((e - 896u) << 23) | (m & 0x7fffffu);
+  r += (rest > 0x80000000u || (rest == 0x80000000u && (r & 1u))) ? 1u : 0u;
+  return __uint_as_float((hi & 0x80000000u) | r);
+}
+
 }  // namespace tk

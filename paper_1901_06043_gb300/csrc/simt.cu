@@ -612,19 +612,6 @@ cudaError_t launch_gram_simt(const void* y, tucker_dtype dt, bool fp64, int64_t 
 constexpr int TNT = 128;                  // threads
 constexpr int TIC = 32;                   // i per stage
 
-// round to nearest by integer operations (a conversion takes the FP64 pipe's 64
-// cycles per warp); out of FP32's normal range: the conversion
-__device__ __forceinline__ float f64_to_f32(double v) {
-  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-  const unsigned e = (hi >> 20) & 0x7ffu;
-  if (e - 897u >= 253u) return (float)v;             // 2^-126 <= |v| < 2^127 below
-  const unsigned m = __funnelshift_l(lo, hi, 3);     // low 20 + 3 mantissa bits, exponent above
-  const unsigned rest = lo << 3;                     // the 29 bits dropped, at the top
-  unsigned r = ((e - 896u) << 23) | (m & 0x7fffffu);
-  r += (rest > 0x80000000u || (rest == 0x80000000u && (r & 1u))) ? 1u : 0u;
-  return __uint_as_float((hi & 0x80000000u) | r);
-}
-
 // dynamic shared memory: two stages of Y, then (L == 1) the block's Z
 template <typename TIn, typename TC, int KT, int MT, bool COL>
 constexpr size_t ttm_smem() {
@@ -679,7 +666,7 @@ __global__ void __launch_bounds__(TNT, sizeof(TC) == 4 ? 4 : 2)
   constexpr int PB = MT * TIC / TNT / 4, CPR = (COL ? TIC : MT) / VY, ME = MT / TNT;
   const bool y16 = (COL ? I : L) % VY == 0 && ((uintptr_t)y & 15) == 0;
   const int cq = y16 ? tid % CPR * VY : (COL ? lane : tid);         // first column
-  int64_t yo[COL ? 1 : ME];                                         // ROW: offsets of this thread's m
+  int64_t yo[COL ? 1 : ME] = {};                                    // ROW: offsets of this thread's m
   if constexpr (!COL) {
 #pragma unroll
     for (int e = 0; e < ME; ++e) {

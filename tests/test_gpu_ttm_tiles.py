@@ -53,3 +53,34 @@ def test_ttm_tiles(ctx, dims, mode, K, prec):
             u = 2.0 ** -24 if prec == "fp32" else 2.0 ** -53
             bound = (I + 3) * u * scale + (2.0 ** -24 * np.abs(want) if out == tucker.F32 else 0.0)
             assert (np.abs(z - want) <= bound).all()
+
+
+@pytest.mark.parametrize("dims,mode,K", [((40, 128), 0, 17), ((500, 384), 0, 100), ((16, 33, 7), 1, 300),
+                                         ((132, 54, 3), 1, 513), ((128, 5, 2), 1, 1)])
+@pytest.mark.parametrize("scale", [1e-25, 1.0, 1e12])
+@pytest.mark.parametrize("arow", [True, False])
+def test_mixed_operator_images(ctx, dims, mode, K, scale, arow):
+    """The tensor-core TTM's operator images at any scale of the operator, rows of very
+    different size, and a NaN that leaves the other outputs alone.  Both operands are
+    rounded to 22 bits of their largest value and three of the four products kept:
+    1e-5 of sum |a|max |y| covers I <= 500 products and the FP32 accumulation."""
+    from paper_1901_06043_gb300 import tucker
+    rng = np.random.default_rng(K)
+    x = rng.standard_normal(int(np.prod(dims))).astype(np.float32)
+    A = rng.standard_normal((K, dims[mode])) * scale * 10.0 ** rng.uniform(-8, 0, (K, 1))
+    U = np.moveaxis(x.astype(np.float64).reshape(dims, order="F"), mode, 0).reshape(dims[mode], -1)
+    bound = 1e-5 * np.abs(A).max() * np.abs(U).sum(0)
+    zd = list(dims)
+    zd[mode] = K
+    for nan in (False, True):
+        B = A.copy()
+        if nan:
+            B[K // 2, 3] = np.nan
+        want = B @ U
+        At = torch.from_numpy(B).cuda() if arow else torch.from_numpy(B.T.copy()).cuda().t()
+        z = ctx.ttm(torch.from_numpy(x).cuda(), dims, mode, At, prec="mixed", out_dtype=tucker.F32)
+        z = z.double().cpu().numpy().reshape(zd, order="F")
+        z = np.moveaxis(z, mode, 0).reshape(K, -1)
+        fin = np.isfinite(want)
+        assert np.array_equal(np.isfinite(z), fin)
+        assert (np.abs(z - want)[fin] <= np.broadcast_to(bound, want.shape)[fin]).all()
