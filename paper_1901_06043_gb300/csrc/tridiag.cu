@@ -39,8 +39,9 @@
 // - Short sums: warp_sum adds in integers.  (Forming the norm of the next pivot
 //   row from sums taken together with p . v, one reduction less, cancels in
 //   most steps of a graded matrix: not kept.)
-// - Unscaled reflectors: v = x - beta e_1, tau = 2 / (v . v); tau is computed by one
-//   warp while the others form A v, and multiplies the finished sums.  (The
+// - Unscaled reflectors: v = x - beta e_1, tau = 2 / (v . v).  One warp computes beta,
+//   v's first entry and tau while the others form A x without its first column;
+//   p = tau (the sums + v_1 the first column) follows.  (The
 //   matrix is scaled by a power of two first, so that squares neither overflow
 //   nor underflow where they matter.)  The update goes by w, though a_ij - v_i p_j -
 //   (p_i - tau (p . v) v_i) v_j needs one FMA less on the chain: its first product
@@ -194,8 +195,7 @@ __global__ void __launch_bounds__(TNT) k_eig_load(const EigProblem* probs, const
 __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int count,
                                                     unsigned* err, unsigned long long poll_limit) {
   extern __shared__ __align__(16) double tsm[];
-  __shared__ double s_red[2][TNW], s_c[5], s_tau;
-  __shared__ int s_on;
+  __shared__ double s_red[2][TNW], s_c[4], s_tau;
   int pidx = 0;
   while (pidx + 1 < count && probs[pidx + 1].team_off <= (int)blockIdx.x) ++pidx;
   const EigProblem P = probs[pidx];
@@ -217,9 +217,13 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
   double* vk = tsm;                       // v_k by global index
   double* vn = tsm + n;                   // the pivot row, then v_{k+1}
   double* sp = tsm + 2 * n;               // p_k, then w_k
-  double* sq = tsm + 3 * n;               // own rows of A v_{k+1} (solo: then p_{k+1})
-  double* const sr = tsm + 4 * n;         // solo: next pivot row
-  double* const srows = tsm + 5 * n;      // own rows t = 0, 1, ... (row c + G t) when SROWS
+  // own rows t = 0, 1, ... (row c + G t): A x without the first column (solo: then
+  // p_{k+1}), the first column
+  const int nown = (n + G - 1) / G;
+  double* sq = tsm + 3 * n;
+  double* const sa = sq + nown;
+  double* const sr = sa + nown;           // solo: next pivot row
+  double* const srows = sr + (solo ? n : 0);   // the own rows when SROWS
   auto row = [&](int i) -> double* {
     return SROWS ? srows + (size_t)((i - c) / G) * n : A + (int64_t)i * n;
   };
@@ -246,7 +250,7 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
 
   // By the last warp, with the row x in vn[lo..] and the partial sums of
   // |x[lo+1..]|^2 in s_red[1]: beta into s_c[2], v = x - beta e_lo (its first entry
-  // into vn[lo]), then 2 / (v . v) into s_tau; a zero (or negligible) rest: no
+  // into vn[lo] and s_c[3]), 2 / (v . v) into s_tau; a zero (or negligible) rest: no
   // reflector, tau = 0.
   auto reflector = [&](int lo) {
     const double ss = warp_sum(lane < TNW ? s_red[1][lane] : 0.0);
@@ -259,8 +263,8 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
       be = alpha > 0.0 ? -g : g;
       v1 = alpha - be;
     }
-    if (lane == 0) { s_c[2] = be; s_c[3] = v1; s_c[4] = ss; vn[lo] = v1; }
-    s_on = on;
+    const double t = on ? 2.0 * rcp64(fma(v1, v1, ss)) : 0.0;
+    if (lane == 0) { s_c[2] = be; s_c[3] = v1; s_tau = t; vn[lo] = v1; }
   };
   // ---- v_0 from row 0
   {
@@ -272,15 +276,13 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
     }
     ss = warp_sum(ss);
     if (lane == 0) s_red[1][warp] = ss;
-    __syncthreads();                      // (and row 0 is in vn)
-    if (warp == TNW - 1) reflector(1);
   }
   // Largest own row.  A CTA without rows in the trailing matrix publishes nothing,
   // so nobody would wait until it has read its words: it leaves.  Results of a
   // step are written by the owner of row lo, which is still there.
   const int last = n - 1 - (n - 1 - c) % G;
 
-  int i0 = c > 0 ? c : G;                 // smallest own row of the trailing matrix, and where it is
+  int i0 = c > 0 ? c : G, t0 = c > 0 ? 0 : 1;   // smallest own row of the trailing matrix, and where it is
   double* own0 = row(i0 < n ? i0 : c);
   const int64_t rstep = SROWS ? n : (int64_t)G * n;               // to the next own row
   double tau = 0.0;
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
     const int lo = k + 2;                 // first row and column of the trailing matrix after step k
     if (k >= 0 && last < lo && !plain) return;        // (a barrier counts every CTA)
     const bool more = k < n - 3;
-    if (i0 < lo) { i0 += G; own0 += rstep; }
+    if (i0 < lo) { i0 += G; ++t0; own0 += rstep; }
     const bool scribe = i0 == lo;
     if (k >= 0) {
       // ---- p_k into sp and the pivot row r into vn; p . v
@@ -383,31 +385,21 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
         }
         ss = warp_sum(ss);
         if (lane == 0) s_red[1][warp] = ss;
-        __syncthreads();
-        if (warp == TNW - 1) reflector(lo);
       }
     }
-    __syncthreads();                      // v_{k+1} is complete
-    if (scribe && more) {
-      double* Vr = P.V + (int64_t)(k + 1) * n;
-      for (int j = lo + tid; j < n; j += TNT) Vr[j] = vn[j];
-      if (tid == 0) P.e[k + 1] = s_c[2] * isc;
-    }
+    if (!more) break;
+    __syncthreads();                      // x is complete
     if (k < 0 && c == 0 && tid == 0) P.d[0] = A[0];
-    // ---- own rows: the update of step k and A v_{k+1}; tau by the last warp
-    if (more && warp == TNW - 1) {
-      const double v1 = s_c[3];
-      const double t = s_on ? 2.0 * rcp64(fma(v1, v1, s_c[4])) : 0.0;
-      if (lane == 0) {
-        s_tau = t;
-        if (scribe) P.tau[k + 1] = t;
-      }
+    // ---- own rows: the update of step k and A x without its first column; v and tau
+    // by the last warp meanwhile
+    if (warp == TNW - 1) {
+      reflector(lo);
     } else {
       constexpr int nw = TNW - 1;
       ulonglong2* rw = xr + (size_t)((k + 1) & 1) * n;
       // PIV: the next pivot row, also published
-      auto do_row = [&](int i, double* Ai, auto UPD, auto PIV) {
-        double vi = 0.0, wi = 0.0, acc = 0.0;
+      auto do_row = [&](int i, int t, double* Ai, auto UPD, auto PIV) {
+        double vi = 0.0, wi = 0.0, acc = 0.0, alo = 0.0;
         if constexpr (decltype(UPD)::value) {
           vi = vk[i];
           wi = sp[i];
@@ -424,38 +416,42 @@ __global__ void __launch_bounds__(TNT, 1) k_tridiag(const EigProblem* probs, int
             else if (plain) dr[(size_t)((k + 1) & 1) * n + j] = a;
             else put_word(rw + j, a, (unsigned long long)k + 2ull);
           }
-          acc = fma(a, vn[j], acc);
+          if (j == lo) alo = a;
+          acc = fma(a, j == lo ? 0.0 : vn[j], acc);       // (vn[lo] is being replaced)
         }
         acc = warp_sum(acc);
-        if (lane == 0) sq[i] = acc;
+        if (lane == 0) { sq[t] = acc; sa[t] = alo; }
       };
       using yes = std::true_type;
       using no = std::false_type;
-      if (more) {
-        int i = i0 + G * warp;
-        double* Ai = own0 + rstep * warp;
-        for (; i < n; i += G * nw, Ai += rstep * nw) {
-          if (k < 0) {
-            if (i == lo) do_row(i, Ai, no(), yes());
-            else do_row(i, Ai, no(), no());
-          } else {
-            if (i == lo) do_row(i, Ai, yes(), yes());
-            else do_row(i, Ai, yes(), no());
-          }
+      int i = i0 + G * warp, t = t0 + warp;
+      double* Ai = own0 + rstep * warp;
+      for (; i < n; i += G * nw, t += nw, Ai += rstep * nw) {
+        if (k < 0) {
+          if (i == lo) do_row(i, t, Ai, no(), yes());
+          else do_row(i, t, Ai, no(), no());
+        } else {
+          if (i == lo) do_row(i, t, Ai, yes(), yes());
+          else do_row(i, t, Ai, yes(), no());
         }
       }
     }
-    if (!more) break;
-    __syncthreads();                      // the sums and tau are there
+    __syncthreads();                      // the sums, v and tau are there
     tau = s_tau;
     {
+      const double v1 = s_c[3];
       ulonglong2* pw = xp + (size_t)((k + 1) & 1) * n;
-      for (int i = i0 + G * tid; i < n; i += G * TNT) {
-        const double p = sq[i] * tau;
-        if (solo) sq[i] = p;
+      for (int i = i0 + G * tid, t = t0 + tid; i < n; i += G * TNT, t += TNT) {
+        const double p = fma(sa[t], v1, sq[t]) * tau;
+        if (solo) sq[t] = p;
         else if (plain) dp[(size_t)((k + 1) & 1) * n + i] = p;
         else put_word(pw + i, p, (unsigned long long)k + 2ull);
       }
+    }
+    if (scribe) {
+      double* Vr = P.V + (int64_t)(k + 1) * n;
+      for (int j = lo + tid; j < n; j += TNT) Vr[j] = vn[j];
+      if (tid == 0) { P.e[k + 1] = s_c[2] * isc; P.tau[k + 1] = tau; }
     }
     { double* t = vk; vk = vn; vn = t; }
     if (solo) {
@@ -1353,7 +1349,9 @@ cudaError_t launch_zgram_batched(const EigProblem* probs_dev, int count, int pas
 
 namespace {
 int tridiag_rows_per_cta(int n, int G) { return (n + G - 1) / G; }
-size_t tridiag_base_smem(int n) { return sizeof(double) * 5 * (size_t)n; }
+size_t tridiag_base_smem(int n, int G) {
+  return sizeof(double) * (3 * (size_t)n + 2 * (size_t)tridiag_rows_per_cta(n, G) + (G == 1 ? n : 0));
+}
 constexpr size_t kTridiagSmemRowsCap = 120 * 1024;
 }  // namespace
 
@@ -1382,17 +1380,18 @@ cudaError_t launch_tridiag(const EigProblem* probs_dev, EigProblem* probs_host, 
                            const double* S, unsigned* err, cudaStream_t st,
                            unsigned long long poll_limit) {
   int nmax = 0, grid = 0, multi = 0;
-  size_t rows_max = 0;
+  size_t rows_max = 0, base = 0;
   for (int p = 0; p < count; ++p) {
     EigProblem& P = probs_host[p];
     nmax = P.n > nmax ? P.n : nmax;
     const size_t rb = sizeof(double) * (size_t)tridiag_rows_per_cta(P.n, P.team_size) * P.n;
     P.srows = rb <= kTridiagSmemRowsCap;
     if (P.srows && rb > rows_max) rows_max = rb;
+    base = std::max(base, tridiag_base_smem(P.n, P.team_size));
     grid += P.team_size;
     multi |= P.team_size > 1;
   }
-  const size_t smem = tridiag_base_smem(nmax) + rows_max;
+  const size_t smem = base + rows_max;
   cudaError_t e = allow_max_dyn_smem((const void*)k_tridiag);
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(const_cast<EigProblem*>(probs_dev), probs_host, sizeof(EigProblem) * count,
