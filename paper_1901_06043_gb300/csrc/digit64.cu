@@ -471,7 +471,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_digit64(const Args g) {
     // the next load of each quad: its address, and how many of this tile's
     // (Gram: this CTA's) loads are left; row views also the l of its k
     int cA = 0, cB = 0;
-    int64_t lA = 0, lB = 0;
+    int lA = 0, lB = 0;                                    // (L I < 2^31; 64-bit comparisons run on the FP64 pipe)
+    const int Li = (int)g.L;
     int64_t item = blockIdx.x;
     int ks = 0;
     int mrel[4] = {0, 0, 0, 0};                            // TTM: offsets of the quad's m
@@ -488,8 +489,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_digit64(const Args g) {
       }
       const int64_t ka = s0 * BK + kA, kb = (s0 + (warp >> 3)) * BK + kB;
       const int64_t rA = ka / g.L, rB = kb / g.L;
-      lA = ka - rA * g.L;
-      lB = kb - rB * g.L;
+      lA = (int)(ka - rA * g.L);
+      lB = (int)(kb - rB * g.L);
       pA = x + (maskA ? rowA * g.L : 0) + lA + LI * rA;
       pB = x + (maskB ? rowB * g.L : 0) + lB + LI * rB;
       const int64_t na = (g.nk - ka + BK - 1) / BK, nb = (g.nk - kb + 2 * BK - 1) / (2 * BK);
@@ -539,7 +540,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_digit64(const Args g) {
         pA += stepA;
         if (!TTM && !MNC) {
           lA += BK;
-          while (lA >= g.L) { lA -= g.L; pA += LI - g.L; }
+          while (lA >= Li) { lA -= Li; pA += LI - g.L; }
         }
         if (!TTM && myB) {
           load4(smem_u32(raw) + NRAW * RAW_A + rb, pB, cB > 0 ? maskB : 0u);
@@ -547,7 +548,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_digit64(const Args g) {
           pB += 2 * stepA;
           if (!MNC) {
             lB += 2 * BK;
-            while (lB >= g.L) { lB -= g.L; pB += LI - g.L; }
+            while (lB >= Li) { lB -= Li; pB += LI - g.L; }
           }
         }
         if (TTM) {

@@ -370,7 +370,8 @@ __device__ __forceinline__ void produce(const GramTcxArgs& g, uint8_t* smem, uin
   unsigned rmask[NOPS];
   int64_t rl = 0;
   int lbl = 0;
-  const int64_t LI = g.L * g.I;
+  const int64_t LI = g.L * g.I;                  // (ROW: below 2^31)
+  const int Li = (int)g.L;
   if (ROW) {
 #pragma unroll
     for (int o = 0; o < NOPS; ++o) {
@@ -393,7 +394,7 @@ __device__ __forceinline__ void produce(const GramTcxArgs& g, uint8_t* smem, uin
   }
   auto load_next = [&](float4 (&v)[NOPS]) {
     if (ROW) {
-      const bool lok = ls < nst && 16 * lbl + kcol < g.L;
+      const bool lok = ls < nst && 16 * lbl + kcol < Li;
       const int64_t off = rl * LI + 16 * lbl;
 #pragma unroll
       for (int o = 0; o < NOPS; ++o) {

@@ -9,7 +9,7 @@
 namespace tk {
 namespace tc {
 
-constexpr unsigned long long WAIT_LIMIT = 1ull << 22;
+constexpr unsigned WAIT_LIMIT = 1u << 22;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -33,7 +33,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 }
 // Bounded wait for the phase with the given parity to complete.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned* err) {
-  for (unsigned long long it = 0; it < WAIT_LIMIT; ++it) {
+  for (unsigned it = 0; it < WAIT_LIMIT; ++it) {      // (32 bits: 64-bit comparisons run on the FP64 pipe)
     uint32_t done;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"

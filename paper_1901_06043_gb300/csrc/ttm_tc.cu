@@ -212,21 +212,21 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base_sh;
-  const int64_t my_tiles =
-      (g.ntiles > (int64_t)blockIdx.x) ? (g.ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-  const int64_t nstages = my_tiles * g.nks;
+  // (loop counters of 32 bits: 64-bit comparisons run on the FP64 pipe)
+  const int my_tiles =
+      (g.ntiles > (int64_t)blockIdx.x) ? (int)((g.ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
+  const int nstages = my_tiles * g.nks;
 
   if (warp == LOAD_WARP) {
     // ---------------- loader: Y boxes -> raw slots (TMA)
     if (lane == 0) {
-      for (int64_t gs = 0; gs < nstages; ++gs) {
+      for (int gs = 0; gs < nstages; ++gs) {
         const int r = (int)(gs % NRAW);
         if (gs >= NRAW &&
             !mbar_wait(smem_u32(&raw_empty[r]), (uint32_t)(((gs / NRAW) - 1) & 1), g.err))
           break;
-        const int64_t j = gs / g.nks;
-        const int ks = (int)(gs - j * g.nks);
-        const int64_t m0 = ((int64_t)blockIdx.x + j * gridDim.x) * TN;
+        const int j = gs / g.nks, ks = gs - j * g.nks;
+        const int64_t m0 = ((int64_t)blockIdx.x + (int64_t)j * gridDim.x) * TN;
         mbar_arrive_expect_tx(smem_u32(&raw_full[r]), RAW_BYTES);
         tma_load_2d(smem_u32(raw + (size_t)r * RAW_BYTES), &ymap, ks * SK, (int)m0,
                     smem_u32(&raw_full[r]));
@@ -236,11 +236,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   } else if (warp <= NCONV) {
     // ---------------- converters: raw FP32 -> FP16 hi/lo B operand; A chunk
     const int ct = threadIdx.x - 32;   // 0..255
-    for (int64_t gs = 0; gs < nstages; ++gs) {
+    int ks = 0;
+    for (int gs = 0; gs < nstages; ++gs, ks = ks + 1 == g.nks ? 0 : ks + 1) {
       const int r = (int)(gs % NRAW), o = (int)(gs % NOP);
-      const int64_t j = gs / g.nks;
-      const int ks = (int)(gs - j * g.nks);
-      const int64_t m0 = ((int64_t)blockIdx.x + j * gridDim.x) * TN;
       if (!mbar_wait(smem_u32(&raw_full[r]), (uint32_t)((gs / NRAW) & 1), g.err)) break;
       if (gs >= NOP &&
           !mbar_wait(smem_u32(&op_empty[o]), (uint32_t)(((gs / NOP) - 1) & 1), g.err))
@@ -256,10 +254,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
       for (int e = 0; e < CV4; ++e) {
         const int c = ct + NCONV * 32 * e;
-        const int m = c >> 4, q = c & 15;
-        const bool ok = (m0 + m < g.Rt) && ((int64_t)ks * SK + 4 * q < g.I);
-        v[e] = ok ? *reinterpret_cast<const float4*>(src + (size_t)m * (SK * 4) + 16 * q)
-                  : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int m = c >> 4, q = c & 15;           // (zeros outside the view, by the TMA)
+        v[e] = *reinterpret_cast<const float4*>(src + (size_t)m * (SK * 4) + 16 * q);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&raw_empty[r]));   // raw slot read
@@ -284,11 +280,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const uint32_t idesc = instr_desc_kk(M, TN);
       const uint32_t sbase = smem_u32(smem);
       bool ok = true;
-      for (int64_t j = 0; j < my_tiles && ok; ++j) {
+      for (int j = 0; j < my_tiles && ok; ++j) {
         const int buf = (int)(j & 1);
         if (j >= 2) ok = mbar_wait(smem_u32(&bar_acce[buf]), (uint32_t)(((j / 2) - 1) & 1), g.err);
         for (int ks = 0; ks < g.nks && ok; ++ks) {
-          const int64_t gs = j * g.nks + ks;
+          const int gs = j * g.nks + ks;
           const int o = (int)(gs % NOP);
           ok = mbar_wait(smem_u32(&op_full[o]), (uint32_t)((gs / NOP) & 1), g.err);
           if (!ok) break;
@@ -323,41 +319,37 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int r = C::RPQ * q + lane;
     const bool rl = lane < C::RPQ;
     const float inv = (float)(1.0 / ((double)g.sy * (double)*g.sa));   // powers of two: exact
-    for (int64_t j = 0; j < my_tiles; ++j) {
+    for (int j = 0; j < my_tiles; ++j) {
       const int buf = (int)(j & 1);
       if (!mbar_wait(smem_u32(&bar_accf[buf]), (uint32_t)((j / 2) & 1), g.err)) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const int64_t m0 = ((int64_t)blockIdx.x + j * gridDim.x) * TN;
+      const int64_t m0 = ((int64_t)blockIdx.x + (int64_t)j * gridDim.x) * TN;
+      const int nm = (int)(g.Rt - m0 < TN ? g.Rt - m0 : TN);      // slabs of this tile
+      float* zl = g.zt ? g.z + (int64_t)r * g.Rt + m0 : g.z + m0 * g.K + r;
       if (C::RPQ * q < g.K) {
         for (int c0 = 0; c0 < TN; c0 += 32) {
           uint32_t rr[32];
           tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)buf * (uint32_t)TN + (uint32_t)c0, rr);
           if (rl && r < g.K) {
             if (!g.zt) {
+              float* zk = zl + (int64_t)c0 * g.K;
 #pragma unroll
-              for (int jj = 0; jj < 32; ++jj) {
-                const int64_t slab = m0 + c0 + jj;
-                if (slab < g.Rt) g.z[slab * g.K + r] = __uint_as_float(rr[jj]) * inv;
-              }
+              for (int jj = 0; jj < 32; ++jj, zk += g.K)
+                if (c0 + jj < nm) *zk = __uint_as_float(rr[jj]) * inv;
             } else if ((g.Rt & 3) == 0) {
               // transposed: this lane's 32 slabs are contiguous in its row of
               // Z; 16-byte stores (Rt % 4 == 0: the row starts are aligned)
-              float* zr = g.z + (int64_t)r * g.Rt;
 #pragma unroll
               for (int jj = 0; jj < 32; jj += 4) {
-                const int64_t slab = m0 + c0 + jj;
-                if (slab < g.Rt)
-                  *reinterpret_cast<float4*>(zr + slab) =
+                if (c0 + jj < nm)
+                  *reinterpret_cast<float4*>(zl + c0 + jj) =
                       make_float4(__uint_as_float(rr[jj]) * inv, __uint_as_float(rr[jj + 1]) * inv,
                                   __uint_as_float(rr[jj + 2]) * inv, __uint_as_float(rr[jj + 3]) * inv);
               }
             } else {
-              float* zr = g.z + (int64_t)r * g.Rt;
 #pragma unroll
-              for (int jj = 0; jj < 32; ++jj) {
-                const int64_t slab = m0 + c0 + jj;
-                if (slab < g.Rt) zr[slab] = __uint_as_float(rr[jj]) * inv;
-              }
+              for (int jj = 0; jj < 32; ++jj)
+                if (c0 + jj < nm) zl[c0 + jj] = __uint_as_float(rr[jj]) * inv;
             }
           }
         }
@@ -502,14 +494,14 @@ __global__ void __launch_bounds__(RNTHREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base_sh;
-  const int64_t my_items = (g.nitems > c0) ? (g.nitems - 1 - c0) / cstep + 1 : 0;
+  const int my_items = (g.nitems > c0) ? (int)((g.nitems - 1 - c0) / cstep) + 1 : 0;
 
   if (warp == LOAD_WARP) {
     // ---------------- loader: B images once, then Y boxes -> raw slots (TMA)
     if (lane == 0) {
       mbar_arrive_expect_tx(smem_u32(&bar_b), 2 * RB_BYTES);   // bar_b counts this one arrival
       bulk_g2s(smem_u32(bimg), g.bprep + (size_t)nt * 2 * RB_BYTES, 2 * RB_BYTES, smem_u32(&bar_b));
-      for (int64_t j = 0; j < my_items; ++j) {
+      for (int j = 0; j < my_items; ++j) {
         const int r = (int)(j % RNRAW);
         if (j >= RNRAW &&
             !mbar_wait(smem_u32(&raw_empty[r]), (uint32_t)(((j / RNRAW) - 1) & 1), g.err))
@@ -525,7 +517,7 @@ __global__ void __launch_bounds__(RNTHREADS, 1)
   } else if (warp <= NCONV) {
     // ---------------- converters: raw [i][l] FP32 -> MN-major FP16 hi/lo A
     const int ct = threadIdx.x - 32;   // 0..255
-    for (int64_t j = 0; j < my_items; ++j) {
+    for (int j = 0; j < my_items; ++j) {
       const int r = (int)(j % RNRAW), o = (int)(j % RNOP);
       if (!mbar_wait(smem_u32(&raw_full[r]), (uint32_t)((j / RNRAW) & 1), g.err)) break;
       if (j >= RNOP &&
@@ -563,7 +555,7 @@ __global__ void __launch_bounds__(RNTHREADS, 1)
       bool ok = mbar_wait(smem_u32(&bar_b), 0, g.err);
       const uint64_t bh0 = smem_desc(smem_u32(bimg), 16, 1024);
       const uint64_t bl0 = smem_desc(smem_u32(bimg + RB_BYTES), 16, 1024);
-      for (int64_t j = 0; j < my_items && ok; ++j) {
+      for (int j = 0; j < my_items && ok; ++j) {
         const int buf = (int)(j & 1), o = (int)(j % RNOP);
         if (j >= 2) ok = mbar_wait(smem_u32(&bar_acce[buf]), (uint32_t)(((j / 2) - 1) & 1), g.err);
         if (ok) ok = mbar_wait(smem_u32(&op_full[o]), (uint32_t)((j / RNOP) & 1), g.err);
@@ -595,7 +587,7 @@ __global__ void __launch_bounds__(RNTHREADS, 1)
     const int half = (warp - MMA_WARP - 1) >> 2;     // columns [128 half, 128 half + 128)
     const float inv = (float)(1.0 / ((double)g.sy * (double)*g.sa));   // powers of two: exact
     const int kbase = nt * RN + 128 * half;
-    for (int64_t j = 0; j < my_items; ++j) {
+    for (int j = 0; j < my_items; ++j) {
       const int buf = (int)(j & 1);
       if (!mbar_wait(smem_u32(&bar_accf[buf]), (uint32_t)((j / 2) & 1), g.err)) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
