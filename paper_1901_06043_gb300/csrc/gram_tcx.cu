@@ -664,31 +664,49 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_gram_tcx(GramTcxArgs g) {
 }
 
 // S[i][j] = S[j][i] = (sum over the K splits of tile (ta, tb) at [col][row])
-// / (s_i s_j), i >= j, splits in order; partial tiles in cta_work's order.
-__global__ void k_gram_tcx_reduce(const double* __restrict__ part, int noff, int nkg, int T,
-                                  int nkg_diag, int64_t I, const float* __restrict__ scale,
-                                  double* __restrict__ S) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= I * I) return;
-  const int64_t i = idx / I, j = idx % I;
-  if (j > i) return;
-  const int ta = (int)(i / 128), tb = (int)(j / 128);
-  const size_t off = (size_t)(j - 128 * tb) * 128 + (size_t)(i - 128 * ta);
-  double s = 0.0;
+// / (s_i s_j), i >= j; partial tiles in cta_work's order.  A block takes 32 rows of one
+// column (consecutive in the partial tiles), a warp every eighth split, and the
+// eight sums are added in order: 150 splits of 126 rows 25 -> 10 us (one
+// thread per entry, its loads 1 KB apart and its FP64 additions one after another).
+constexpr int RED_W = 8;
+__global__ void __launch_bounds__(32 * RED_W) k_gram_tcx_reduce(
+    const double* __restrict__ part, int noff, int nkg, int T, int nkg_diag, int64_t I,
+    const float* __restrict__ scale, double* __restrict__ S) {
+  __shared__ double sm[RED_W][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int j = blockIdx.y, ib = 32 * blockIdx.x, i = ib + lane;
+  if (ib + 31 < j) return;
+  const int ta = ib / 128, tb = j / 128;
+  const bool ok = i >= j && i < I;
+  // first partial tile and the distance to the next split's
+  size_t first, step;
+  int nk = nkg;
   if (nkg == nkg_diag) {
-    const int t = ta * (ta + 1) / 2 + tb;
-    const int ntiles = T * (T + 1) / 2;
-    for (int k = 0; k < nkg; ++k) s += part[(size_t)(t + ntiles * k) * TILE_ELEMS + off];
+    first = (size_t)(ta * (ta + 1) / 2 + tb);
+    step = (size_t)(T * (T + 1) / 2);
   } else if (ta == tb) {
-    const size_t first = (size_t)noff * nkg + ta;
-    for (int k = 0; k < nkg_diag; ++k) s += part[(first + (size_t)T * k) * TILE_ELEMS + off];
+    first = (size_t)noff * nkg + ta;
+    step = (size_t)T;
+    nk = nkg_diag;
   } else {
-    const int jo = ta * (ta - 1) / 2 + tb;        // off-diagonal tile index
-    for (int k = 0; k < nkg; ++k) s += part[((size_t)jo + (size_t)noff * k) * TILE_ELEMS + off];
+    first = (size_t)(ta * (ta - 1) / 2 + tb);
+    step = (size_t)noff;
   }
-  s /= (double)scale[i] * (double)scale[j];
-  S[i * I + j] = s;
-  S[j * I + i] = s;
+  const double* p = part + first * TILE_ELEMS + (size_t)(j - 128 * tb) * 128 + (size_t)(i - 128 * ta);
+  double s = 0.0;
+  if (ok) {
+#pragma unroll 4
+    for (int k = warp; k < nk; k += RED_W) s += __ldcg(p + step * TILE_ELEMS * k);
+  }
+  sm[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && ok) {
+#pragma unroll
+    for (int w = 1; w < RED_W; ++w) s += sm[w][lane];
+    s /= (double)scale[i] * (double)scale[j];
+    S[(int64_t)i * I + j] = s;
+    S[(int64_t)j * I + i] = s;
+  }
 }
 
 // Power-of-two row scales from the row maxima (as FP32 bit patterns): the
@@ -828,8 +846,7 @@ cudaError_t launch_gram_tcx(const float* y, int64_t L, int64_t I, int64_t Rt, co
     e = ndig == 3 ? run_gram_tcx<true, 3, true>(a, p.nctas, st)
                   : run_gram_tcx<true, 2, true>(a, p.nctas, st);
   if (e != cudaSuccess) return e;
-  const int64_t tot = I * I;
-  k_gram_tcx_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(
+  k_gram_tcx_reduce<<<dim3((unsigned)((I + 31) / 32), (unsigned)I), 32 * RED_W, 0, st>>>(
       part, a.noff, p.ksplit, a.T, p.ksplit_diag, I, scale, S);
   count_launches(3);
   return cudaGetLastError();
