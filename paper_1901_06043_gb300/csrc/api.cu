@@ -237,8 +237,10 @@ struct Timer {
 // rowmax != NULL: y is FP32 with a mode-0 size I0 (n = I0 * ncols) and the
 // column-major pass also records the row maxima (for the digit scales of the
 // exact tensor-core Gram) into rowmax[I0].
-tucker_status do_norm(tucker_ctx* c, const void* y, tucker_dtype dt, int64_t n, double* out,
-                      double* maxabs = nullptr, unsigned* rowmax = nullptr, int64_t I0 = 0) {
+// Enqueues the norm: the sum of squares and max |x| into d_small[0], [1], d_words[0]
+// nonzero for NaN or Inf.
+tucker_status enqueue_norm(tucker_ctx* c, const void* y, tucker_dtype dt, int64_t n,
+                           unsigned* rowmax = nullptr, int64_t I0 = 0) {
   // four blocks per SM: 7.73 ms for the 44 GB norm pass with row maxima,
   // against 7.93 ms with eight (each thread keeps eight loads in flight)
   int nb = (int)std::min<int64_t>((n + 255) / 256, (int64_t)c->num_sms * 4);
@@ -253,6 +255,12 @@ tucker_status do_norm(tucker_ctx* c, const void* y, tucker_dtype dt, int64_t n, 
   } else {
     TK_CUDA(c, launch_sumsq(y, dt, n, part.as<double>(), nb, c->d_words, c->d_small, c->stream));
   }
+  return TUCKER_OK;
+}
+
+tucker_status do_norm(tucker_ctx* c, const void* y, tucker_dtype dt, int64_t n, double* out,
+                      double* maxabs = nullptr, unsigned* rowmax = nullptr, int64_t I0 = 0) {
+  TK_TRY(enqueue_norm(c, y, dt, n, rowmax, I0));
   double h[2] = {0.0, 0.0};
   unsigned bad = 0;
   TK_CUDA(c, cudaMemcpyAsync(h, c->d_small, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -261,6 +269,25 @@ tucker_status do_norm(tucker_ctx* c, const void* y, tucker_dtype dt, int64_t n, 
   *out = h[0];
   if (maxabs) *maxabs = h[1];
   if (bad) return set_err(c, TUCKER_ERR_NONFINITE, "tensor holds NaN or Inf");
+  return TUCKER_OK;
+}
+
+// Waits for a tensor-core TTM and reads its error word (d_words[9]) and, where its
+// data's maximum was taken on the device just before, the norm's (d_words[0]).
+tucker_status ttm_verdict(tucker_ctx* c, bool norm) {
+  unsigned w[10] = {0};
+  if (norm)
+    TK_CUDA(c, cudaMemcpyAsync(w, c->d_words, sizeof w, cudaMemcpyDeviceToHost, c->stream));
+  else
+    TK_CUDA(c, cudaMemcpyAsync(w + 9, c->d_words + 9, sizeof(unsigned), cudaMemcpyDeviceToHost,
+                               c->stream));
+  TK_TRY(sync(c));
+  if (norm && w[0]) return set_err(c, TUCKER_ERR_NONFINITE, "tensor holds NaN or Inf");
+  if (w[9]) {
+    char m[96];
+    snprintf(m, sizeof m, "tensor-core TTM reported device error word 0x%x", w[9]);
+    return set_err(c, TUCKER_ERR_CUDA, m);
+  }
   return TUCKER_OK;
 }
 
@@ -749,26 +776,15 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
                   (!zt || (((uintptr_t)z) & 15) == 0) && ttm_tc_supported(v.L, v.I, v.Rt, K);
   if (kernel_used) *kernel_used = tc ? 2 : (prec == TUCKER_PREC_FP64 ? 0 : 1);
   if (tc) {
-    if (!(ymax >= 0.0)) {
-      double nrm;
-      TK_TRY(do_norm(c, y, ydt, v.L * v.I * v.Rt, &nrm, &ymax));
-    }
+    // an unknown max|y| is found on the device and scales there
+    const double* ymax_d = ymax >= 0.0 ? nullptr : c->d_small + 1;
+    if (ymax_d) TK_TRY(enqueue_norm(c, y, ydt, v.L * v.I * v.Rt));
     DevBuf scratch;
     TK_TRY(dev_alloc(c, scratch, ttm_tc_scratch_bytes(v.I, K)));
     if (check) TK_CUDA(c, cudaMemsetAsync(c->d_words + 9, 0, sizeof(unsigned), c->stream));
-    TK_CUDA(c, launch_ttm_tc((const float*)y, v.L, v.I, v.Rt, A, K, lda, arow, split_scale(ymax),
+    TK_CUDA(c, launch_ttm_tc((const float*)y, v.L, v.I, v.Rt, A, K, lda, arow, split_scale(ymax), ymax_d,
                              (float*)z, zt, scratch.p, c->d_words + 9, c->num_sms, c->stream));
-    if (!check) return TUCKER_OK;
-    unsigned err = 0;
-    TK_CUDA(c, cudaMemcpyAsync(&err, c->d_words + 9, sizeof(unsigned), cudaMemcpyDeviceToHost,
-                               c->stream));
-    TK_TRY(sync(c));
-    if (err) {
-      char m[96];
-      snprintf(m, sizeof m, "tensor-core TTM reported device error word 0x%x", err);
-      return set_err(c, TUCKER_ERR_CUDA, m);
-    }
-    return TUCKER_OK;
+    return check ? ttm_verdict(c, ymax_d != nullptr) : TUCKER_OK;
   }
   // row-mode views with a short contraction (I <= 64: the reconstruction's
   // expansions) on the tensor cores, l as the MMA's M.  Its split scale needs
@@ -781,27 +797,15 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
                       ttm_tc_row_supported(v.L, v.I, v.Rt, K);
   if (tc_row) {
     if (kernel_used) *kernel_used = 2;
-    if (!(ymax >= 0.0)) {
-      double nrm;
-      TK_TRY(do_norm(c, y, ydt, v.L * v.I * v.Rt, &nrm, &ymax));
-    }
+    const double* ymax_d = ymax >= 0.0 ? nullptr : c->d_small + 1;
+    if (ymax_d) TK_TRY(enqueue_norm(c, y, ydt, v.L * v.I * v.Rt));
     DevBuf scratch;
     TK_TRY(dev_alloc(c, scratch, ttm_tc_row_scratch_bytes(K)));
     if (check) TK_CUDA(c, cudaMemsetAsync(c->d_words + 9, 0, sizeof(unsigned), c->stream));
     TK_CUDA(c, launch_ttm_tc_row((const float*)y, v.L, v.I, v.Rt, A, K, lda, arow,
-                                 split_scale(ymax), (float*)z, scratch.p, c->d_words + 9,
+                                 split_scale(ymax), ymax_d, (float*)z, scratch.p, c->d_words + 9,
                                  c->num_sms, c->stream));
-    if (!check) return TUCKER_OK;
-    unsigned err = 0;
-    TK_CUDA(c, cudaMemcpyAsync(&err, c->d_words + 9, sizeof(unsigned), cudaMemcpyDeviceToHost,
-                               c->stream));
-    TK_TRY(sync(c));
-    if (err) {
-      char m[96];
-      snprintf(m, sizeof m, "tensor-core TTM reported device error word 0x%x", err);
-      return set_err(c, TUCKER_ERR_CUDA, m);
-    }
-    return TUCKER_OK;
+    return check ? ttm_verdict(c, ymax_d != nullptr) : TUCKER_OK;
   }
   // FP64: seven exact digits on the tensor cores from the size where they
   // beat the FP64 pipe (digit64.cu); out of their range (NaN, Inf, rows below

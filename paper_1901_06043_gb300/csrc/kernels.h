@@ -110,10 +110,11 @@ TcGramPlan plan_gram_tc(int64_t L, int64_t I, int64_t Rt, int num_sms);
 cudaError_t launch_gram_tc(const float* y, int64_t L, int64_t I, int64_t Rt, const TcGramPlan& p,
                            float scale, double* scratch, unsigned* err, double* S, cudaStream_t st);
 // TTM of the column-major mode-0 view (L == 1, I % 4 == 0, K <= 128); sy =
-// power-of-two scale of y with max|y sy| <= 2^14
+// power-of-two scale of y with max|y sy| <= 2^14, taken from *ymax (device) instead
+// when ymax is given
 int ttm_tc_supported(int64_t L, int64_t I, int64_t Rt, int64_t K);
 cudaError_t launch_ttm_tc(const float* y, int64_t L, int64_t I, int64_t Rt, const double* A,
-                          int64_t K, int64_t lda, int a_rowmajor, float sy, float* z, bool zt,
+                          int64_t K, int64_t lda, int a_rowmajor, float sy, const double* ymax, float* z, bool zt,
                           void* scratch, unsigned* err, int num_sms, cudaStream_t st);
 size_t ttm_tc_scratch_bytes(int64_t I, int64_t K);
 // row-mode views (L > 1, L % 4 == 0, I <= 64, K <= 1024): Z(l, k, r) =
@@ -121,7 +122,7 @@ size_t ttm_tc_scratch_bytes(int64_t I, int64_t K);
 int ttm_tc_row_supported(int64_t L, int64_t I, int64_t Rt, int64_t K);
 size_t ttm_tc_row_scratch_bytes(int64_t K);
 cudaError_t launch_ttm_tc_row(const float* y, int64_t L, int64_t I, int64_t Rt, const double* A,
-                              int64_t K, int64_t lda, int a_rowmajor, float sy, float* z,
+                              int64_t K, int64_t lda, int a_rowmajor, float sy, const double* ymax, float* z,
                               void* scratch, unsigned* err, int num_sms, cudaStream_t st);
 
 // ---- Jacobi eigensolver, sort and rank cut

@@ -120,6 +120,13 @@ __device__ int prep_scale_exp(const double* __restrict__ A, int K, int64_t I, in
   // |a| < 2^(exponent field - 1022); 2^14 above
   return mx == 0u ? 0 : max(-100, min(100, 14 - ((int)(mx >> 20) - 1022)));
 }
+// The power-of-two scale s_y of Y from its largest magnitude: max|y| s_y <= 2^14 (1 for
+// zero and non-finite).
+__device__ __forceinline__ float data_scale(double ymax) {
+  const int hi = __double2hiint(ymax);
+  if (hi <= 0 || hi >= 0x7ff00000) return 1.f;       // (below 2^-1042: as far from 2^100 as zero)
+  return __int_as_float((127 + max(-100, min(100, 14 - ((hi >> 20) - 1022)))) << 23);
+}
 // a 2^e2 in FP32
 __device__ __forceinline__ float prep_value(double a, int e2) {
   const int hi = __double2hiint(a), e = ((hi >> 20) & 0x7ff) + e2;
@@ -129,14 +136,18 @@ __device__ __forceinline__ float prep_value(double a, int e2) {
 }
 
 // Per stage ks of 64 i: [A_h tile | A_l tile] as shared-memory images (K-major
-// SW128, tm rows x 64 i, zero outside K x I); *sa_out = s_a.
+// SW128, tm rows x 64 i, zero outside K x I); sc_out = {s_a, s_y}.
 __global__ void __launch_bounds__(PREP_NT) k_ttm_tc_prep(const double* __restrict__ A, int K,
                                                          int64_t I, int64_t lda, int arow, int nks,
-                                                         int tm, uint8_t* __restrict__ out,
-                                                         float* __restrict__ sa_out) {
+                                                         int tm, uint8_t* __restrict__ out, float sy,
+                                                         const double* __restrict__ ymax,
+                                                         float* __restrict__ sc_out) {
   const uint32_t a_bytes = (uint32_t)tm * SK * 2;
   const int e2 = prep_scale_exp(A, K, I, lda, arow);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *sa_out = __int_as_float((127 + e2) << 23);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    sc_out[0] = __int_as_float((127 + e2) << 23);
+    sc_out[1] = ymax ? data_scale(*ymax) : sy;
+  }
   const int per = tm * (SK / 2);                      // element pairs (i, i + 1) per stage
   for (int e = blockIdx.x * PREP_NT + threadIdx.x; e < nks * per; e += gridDim.x * PREP_NT) {
     const int ks = e / per, rem = e - ks * per;
@@ -163,9 +174,8 @@ struct TtmTcArgs {
   int K;                 // rows of A = outputs per slab (<= 128)
   int nks;               // stages per tile = ceil(I / 64)
   int64_t ntiles;        // ceil(Rt / 128)
-  float sy;              // power of two
   const uint8_t* aprep;  // nks x [A_h | A_l] images
-  const float* sa;       // the power-of-two scale of A (device)
+  const float* scales;   // the power-of-two scales of A and Y (device)
   float* z;              // K x Rt column-major, or (zt) Rt x K column-major
   int zt;                // transposed output: z[r * Rt + slab]
   unsigned* err;
@@ -236,6 +246,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   } else if (warp <= NCONV) {
     // ---------------- converters: raw FP32 -> FP16 hi/lo B operand; A chunk
     const int ct = threadIdx.x - 32;   // 0..255
+    const float sy = g.scales[1];
     int ks = 0;
     for (int gs = 0; gs < nstages; ++gs, ks = ks + 1 == g.nks ? 0 : ks + 1) {
       const int r = (int)(gs % NRAW), o = (int)(gs % NOP);
@@ -264,8 +275,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int c = ct + NCONV * 32 * e;
         const int m = c >> 4, q = c & 15;
         uint2 hp, lp;
-        split_pack(v[e].x * g.sy, v[e].y * g.sy, hp.x, lp.x);
-        split_pack(v[e].z * g.sy, v[e].w * g.sy, hp.y, lp.y);
+        split_pack(v[e].x * sy, v[e].y * sy, hp.x, lp.x);
+        split_pack(v[e].z * sy, v[e].w * sy, hp.y, lp.y);
         const uint32_t off = kmaj_off(m, 4 * q);
         *reinterpret_cast<uint2*>(st + OFF_BH + off) = hp;
         *reinterpret_cast<uint2*>(st + OFF_BL + off) = lp;
@@ -318,7 +329,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // lane; M = 64 rows 16 q + lane in lanes 0-15 of the quarter
     const int r = C::RPQ * q + lane;
     const bool rl = lane < C::RPQ;
-    const float inv = (float)(1.0 / ((double)g.sy * (double)*g.sa));   // powers of two: exact
+    const float inv = (float)(1.0 / ((double)g.scales[0] * (double)g.scales[1]));   // powers of two: exact
     for (int j = 0; j < my_tiles; ++j) {
       const int buf = (int)(j & 1);
       if (!mbar_wait(smem_u32(&bar_accf[buf]), (uint32_t)((j / 2) & 1), g.err)) break;
@@ -414,13 +425,17 @@ __device__ __forceinline__ uint32_t instr_desc_mk(int M, int N) {
 
 // B images of A^T: N-tile t holds rows k = 256 t + row (row < 256) and
 // columns i < 64 of A scaled by s_a, K-major SW128, [B_h | B_l] (64 KB per
-// tile, zero outside K x I); *sa_out = s_a.
+// tile, zero outside K x I); sc_out = {s_a, s_y}.
 __global__ void __launch_bounds__(PREP_NT) k_ttm_tc_prep_rows(const double* __restrict__ A, int K,
                                                               int64_t I, int64_t lda, int arow,
                                                               int ntile, uint8_t* __restrict__ out,
-                                                              float* __restrict__ sa_out) {
+                                                              float sy, const double* __restrict__ ymax,
+                                                              float* __restrict__ sc_out) {
   const int e2 = prep_scale_exp(A, K, I, lda, arow);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *sa_out = __int_as_float((127 + e2) << 23);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    sc_out[0] = __int_as_float((127 + e2) << 23);
+    sc_out[1] = ymax ? data_scale(*ymax) : sy;
+  }
   constexpr int PER = RN * (SK / 2);                  // element pairs (i, i + 1) per tile
   for (int e = blockIdx.x * PREP_NT + threadIdx.x; e < ntile * PER; e += gridDim.x * PREP_NT) {
     const int t = e / PER, rem = e % PER;
@@ -447,9 +462,8 @@ struct TtmTcRowArgs {
   int NT;                  // N-tiles of 256 outputs
   int64_t ntl;             // l-tiles per slab, ceil(L / 128)
   int64_t nitems;          // Rt * ntl
-  float sy;                // power of two
   const uint8_t* bprep;    // NT x [B_h | B_l]
-  const float* sa;         // the power-of-two scale of A (device)
+  const float* scales;     // the power-of-two scales of A and Y (device)
   float* z;                // z[l + L (k + K r)]
   unsigned* err;
 };
@@ -517,6 +531,7 @@ __global__ void __launch_bounds__(RNTHREADS, 1)
   } else if (warp <= NCONV) {
     // ---------------- converters: raw [i][l] FP32 -> MN-major FP16 hi/lo A
     const int ct = threadIdx.x - 32;   // 0..255
+    const float sy = g.scales[1];
     for (int j = 0; j < my_items; ++j) {
       const int r = (int)(j % RNRAW), o = (int)(j % RNOP);
       if (!mbar_wait(smem_u32(&raw_full[r]), (uint32_t)((j / RNRAW) & 1), g.err)) break;
@@ -538,8 +553,8 @@ __global__ void __launch_bounds__(RNTHREADS, 1)
         const int c = ct + NCONV * 32 * e;
         const int i = c >> 5, l = 4 * (c & 31);
         uint2 hp, lp;
-        split_pack(v[e].x * g.sy, v[e].y * g.sy, hp.x, lp.x);
-        split_pack(v[e].z * g.sy, v[e].w * g.sy, hp.y, lp.y);
+        split_pack(v[e].x * sy, v[e].y * sy, hp.x, lp.x);
+        split_pack(v[e].z * sy, v[e].w * sy, hp.y, lp.y);
         const uint32_t off = rmn_off(l, i);
         *reinterpret_cast<uint2*>(st + off) = hp;
         *reinterpret_cast<uint2*>(st + RA_BYTES + off) = lp;
@@ -585,7 +600,7 @@ __global__ void __launch_bounds__(RNTHREADS, 1)
     // ---------------- epilogue: tensor memory -> Z, coalesced along l
     const int q = warp & 3;                          // the lane quarter this warp may access
     const int half = (warp - MMA_WARP - 1) >> 2;     // columns [128 half, 128 half + 128)
-    const float inv = (float)(1.0 / ((double)g.sy * (double)*g.sa));   // powers of two: exact
+    const float inv = (float)(1.0 / ((double)g.scales[0] * (double)g.scales[1]));   // powers of two: exact
     const int kbase = nt * RN + 128 * half;
     for (int j = 0; j < my_items; ++j) {
       const int buf = (int)(j & 1);
@@ -686,7 +701,7 @@ cudaError_t run_ttm_tc_col(const TtmTcArgs& a, const CUtensorMap& ymap, int grid
 }
 
 cudaError_t launch_ttm_tc(const float* y, int64_t L, int64_t I, int64_t Rt, const double* A,
-                          int64_t K, int64_t lda, int a_rowmajor, float sy, float* z, bool zt,
+                          int64_t K, int64_t lda, int a_rowmajor, float sy, const double* ymax, float* z, bool zt,
                           void* scratch, unsigned* err, int num_sms, cudaStream_t st) {
   if (!ttm_tc_supported(L, I, Rt, K) || ((uintptr_t)y & 15) != 0) return cudaErrorInvalidValue;
   if (zt && (Rt & 3) == 0 && ((uintptr_t)z & 15) != 0) return cudaErrorInvalidValue;
@@ -694,7 +709,7 @@ cudaError_t launch_ttm_tc(const float* y, int64_t L, int64_t I, int64_t Rt, cons
   const int tm = K <= 64 ? 64 : TM;
   uint8_t* aprep = (uint8_t*)scratch;
   float* sa = (float*)(aprep + (size_t)nks * 2 * ColCfg<TM>::A_BYTES);
-  k_ttm_tc_prep<<<std::min(nks * tm * (SK / 2) / PREP_NT, PREP_CTAS), PREP_NT, 0, st>>>(A, (int)K, I, lda, a_rowmajor, nks, tm, aprep, sa);
+  k_ttm_tc_prep<<<std::min(nks * tm * (SK / 2) / PREP_NT, PREP_CTAS), PREP_NT, 0, st>>>(A, (int)K, I, lda, a_rowmajor, nks, tm, aprep, sy, ymax, sa);
   TtmTcArgs a;
   a.y = y;
   a.I = I;
@@ -702,9 +717,8 @@ cudaError_t launch_ttm_tc(const float* y, int64_t L, int64_t I, int64_t Rt, cons
   a.K = (int)K;
   a.nks = nks;
   a.ntiles = (Rt + TN - 1) / TN;
-  a.sy = sy;
   a.aprep = aprep;
-  a.sa = sa;
+  a.scales = sa;
   a.z = z;
   a.zt = zt ? 1 : 0;
   a.err = err;
@@ -738,7 +752,7 @@ size_t ttm_tc_row_scratch_bytes(int64_t K) {
 }
 
 cudaError_t launch_ttm_tc_row(const float* y, int64_t L, int64_t I, int64_t Rt, const double* A,
-                              int64_t K, int64_t lda, int a_rowmajor, float sy, float* z,
+                              int64_t K, int64_t lda, int a_rowmajor, float sy, const double* ymax, float* z,
                               void* scratch, unsigned* err, int num_sms, cudaStream_t st) {
   if (!ttm_tc_row_supported(L, I, Rt, K) || ((uintptr_t)y & 15) != 0) return cudaErrorInvalidValue;
   {
@@ -748,7 +762,7 @@ cudaError_t launch_ttm_tc_row(const float* y, int64_t L, int64_t I, int64_t Rt, 
   const int NT = (int)((K + RN - 1) / RN);
   uint8_t* bprep = (uint8_t*)scratch;
   float* sa = (float*)(bprep + (size_t)NT * 2 * RB_BYTES);
-  k_ttm_tc_prep_rows<<<std::min(NT * RN * (SK / 2) / PREP_NT, PREP_CTAS), PREP_NT, 0, st>>>(A, (int)K, I, lda, a_rowmajor, NT, bprep, sa);
+  k_ttm_tc_prep_rows<<<std::min(NT * RN * (SK / 2) / PREP_NT, PREP_CTAS), PREP_NT, 0, st>>>(A, (int)K, I, lda, a_rowmajor, NT, bprep, sy, ymax, sa);
   TtmTcRowArgs a;
   a.L = L;
   a.I = I;
@@ -757,9 +771,8 @@ cudaError_t launch_ttm_tc_row(const float* y, int64_t L, int64_t I, int64_t Rt, 
   a.NT = NT;
   a.ntl = (L + RM - 1) / RM;
   a.nitems = Rt * a.ntl;
-  a.sy = sy;
   a.bprep = bprep;
-  a.sa = sa;
+  a.scales = sa;
   a.z = z;
   a.err = err;
   // Y as a 3D tensor: x = l (contiguous), y = i, z = slab; boxes of 128 l x 64 i x 1
