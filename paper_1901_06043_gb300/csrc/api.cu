@@ -1543,24 +1543,26 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
   // ---- norms of all tensors, one synchronization
   std::vector<double> nrm2(count), xmax(count);
   {
-    std::vector<int> nb(count);
-    size_t off = 0;
+    std::vector<NormItem> items(count);
+    int64_t nmost = 1;
     for (int i = 0; i < count; ++i) {
-      const int64_t ne = numel(ndims[i], dimss[i]);
-      nb[i] = (int)std::max<int64_t>(1, std::min<int64_t>((ne + 255) / 256, (int64_t)c->num_sms * 8));
-      off += 2 * (size_t)nb[i];
+      items[i] = NormItem{xs[i], numel(ndims[i], dimss[i])};
+      nmost = std::max(nmost, items[i].n);
     }
+    // blocks per tensor: 4096 elements each in the largest one, two blocks per SM at most
+    const int nb = (int)std::min<int64_t>((nmost + 4095) / 4096, (int64_t)c->num_sms * 2);
+    constexpr int kMost = 32768;                     // tensors per launch
     DevBuf part, outb;
-    TK_TRY(dev_alloc(c, part, sizeof(double) * off));
-    TK_TRY(dev_alloc(c, outb, sizeof(double) * 2 * count + sizeof(unsigned) * count));
-    unsigned* bad_d = reinterpret_cast<unsigned*>(outb.as<double>() + 2 * count);
+    TK_TRY(dev_alloc(c, part, sizeof(double) * 2 * (size_t)nb * std::min(count, kMost)));
+    TK_TRY(dev_alloc(c, outb, (sizeof(NormItem) + sizeof(double) * 2 + sizeof(unsigned)) * (size_t)count));
+    double* out_d = outb.as<double>();
+    NormItem* items_d = reinterpret_cast<NormItem*>(out_d + 2 * (size_t)count);
+    unsigned* bad_d = reinterpret_cast<unsigned*>(items_d + count);
+    TK_CUDA(c, cudaMemcpyAsync(items_d, items.data(), sizeof(NormItem) * count, cudaMemcpyHostToDevice, st));
     TK_CUDA(c, cudaMemsetAsync(bad_d, 0, sizeof(unsigned) * count, st));
-    off = 0;
-    for (int i = 0; i < count; ++i) {
-      TK_CUDA(c, launch_sumsq(xs[i], dt, numel(ndims[i], dimss[i]), part.as<double>() + off, nb[i],
-                              bad_d + i, outb.as<double>() + 2 * i, st));
-      off += 2 * (size_t)nb[i];
-    }
+    for (int i = 0; i < count; i += kMost)
+      TK_CUDA(c, launch_sumsq_batched(items_d + i, dt, std::min(count - i, kMost), nb, part.as<double>(),
+                                      bad_d + i, out_d + 2 * (size_t)i, st));
     std::vector<double> h(2 * count);
     std::vector<unsigned> bad(count);
     TK_CUDA(c, cudaMemcpyAsync(h.data(), outb.p, sizeof(double) * 2 * count, cudaMemcpyDeviceToHost, st));

@@ -13,6 +13,15 @@ namespace tk {
 cudaError_t launch_sumsq(const void* y, tucker_dtype dt, int64_t n, double* partial, int nblocks,
                          unsigned* nonfinite, double* out, cudaStream_t st);
 
+// the same for `count` tensors, nblocks blocks each: partial 2 nblocks per tensor, out
+// two and nonfinite one (zeroed) per tensor; count <= 65535
+struct NormItem {
+  const void* y;
+  int64_t n;
+};
+cudaError_t launch_sumsq_batched(const NormItem* items_dev, tucker_dtype dt, int count, int nblocks,
+                                 double* partial, unsigned* nonfinite, double* out, cudaStream_t st);
+
 // The same over the column-major I0 x ncols mode-0 view, also recording each
 // row's max |x| as FP32 bits (atomicMax into the zeroed rowmax_bits[I0]);
 // I0 <= 8192, 4-byte aligned y (16-byte loads when I0 % 4 == 0 and y is

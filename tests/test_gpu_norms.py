@@ -55,3 +55,24 @@ def test_row_maxima_set_the_digits(ctx, I, cols):
     t = torch.from_numpy(x.reshape(-1)).to(device="cuda", dtype=torch.float32)
     got = ctx.gram(t, (I, cols), 0, prec="mixed").cpu().numpy().reshape(I, I)
     assert np.array_equal(got, x.T @ x)
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+def test_norms_of_a_batch(ctx, dt):
+    """Tensors of very different sizes, odd lengths and unaligned starts; NaN in one of them."""
+    from paper_1901_06043_gb300 import tucker
+    shapes = [(5, 3), (129, 65, 33), (7, 11, 13), (64, 50, 40), (255,), (3, 3, 3, 3)]
+    xs = []
+    for k, d in enumerate(shapes):
+        n = int(np.prod(d))
+        x = torch.zeros(n + k % 2, device="cuda", dtype=dt)[k % 2:]
+        x.copy_(torch.from_numpy(np.random.default_rng(k).standard_normal(n) * 10.0 ** (k - 3)))
+        xs.append(x)
+    for r, x in zip(ctx.sthosvd_batched(xs, shapes, eps=1e-3, prec="fp64"), xs):
+        want = float((x.double().cpu().numpy().astype(np.longdouble) ** 2).sum())
+        assert abs(r.norm_sq - want) <= 1e-13 * want
+        r.close()
+    xs[3][-1] = float("nan")
+    with pytest.raises(tucker.TuckerError) as e:
+        ctx.sthosvd_batched(xs, shapes, eps=1e-3, prec="fp64")
+    assert e.value.name == "NONFINITE"
