@@ -540,9 +540,9 @@ tucker_status do_gram(tucker_ctx* c, const void* y, tucker_dtype dt, const SlabV
     auto it = g_tune.find(key);
     if (it != g_tune.end()) best = it->second;
   }
+  DevBuf rm;                              // (outlives the call below)
   if (best == 0) {
     // the digit Gram's row maxima once, outside the timed runs
-    DevBuf rm;
     if (kern == 5 && !rowmax) {
       TK_TRY(dev_alloc(c, rm, sizeof(unsigned) * v.I));
       TK_TRY(view_rowmax(c, (const float*)y, v, rm.as<unsigned>()));
