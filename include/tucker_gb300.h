@@ -65,7 +65,8 @@ typedef enum { TUCKER_F32 = 0, TUCKER_F64 = 1 } tucker_dtype;
  *            exact integer digits: each value as a 55-bit fixed-point number
  *            of its row (rounding 2^-55 of the row's largest magnitude), every
  *            digit product and sum exact, one rounding to FP64 at the end; an
- *            operand with NaN, Inf or a row below 2^-958 takes the FP64 pipe.
+ *            operand with NaN, Inf or a row below 2^-958 takes the FP64 pipe
+ *            (in a batch, a row below 2^-958 counts in units of 2^-1013).
  *   FP32   : FP32 products, round-to-nearest FP32 sums over short chunks
  *            combined exactly (TwoSum) and in FP64; working tensor and core
  *            in the input dtype.

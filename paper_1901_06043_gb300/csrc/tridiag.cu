@@ -46,8 +46,9 @@
 //   nor underflow where they matter.)  The update goes by w, though a_ij - v_i p_j -
 //   (p_i - tau (p . v) v_i) v_j needs one FMA less on the chain: its first product
 //   is larger, and the vectors of close eigenvalues came out 1.3 times as far off.
-// Measured, whole reduction: n = 50 0.26 -> 0.18 ms, n = 200 1.20 -> 0.84 ms, n = 500
-// 3.5 -> 2.5 ms (a barrier, normalized reflectors and FP64 sums before).
+// Measured, whole reduction: n = 50 0.26 -> 0.16 ms, n = 200 1.20 -> 0.74 ms, n = 500
+// 3.48 -> 2.62 ms, n = 1500 18.2 -> 16.2 ms (a barrier, normalized reflectors and FP64
+// sums before; 0.81, 2.77 and 17.3 with the reflector ahead of A v).
 #include <algorithm>
 #include <cfloat>
 #include <type_traits>
