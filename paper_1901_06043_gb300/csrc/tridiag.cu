@@ -1381,18 +1381,19 @@ cudaError_t launch_tridiag(const EigProblem* probs_dev, EigProblem* probs_host, 
                            const double* S, unsigned* err, cudaStream_t st,
                            unsigned long long poll_limit) {
   int nmax = 0, grid = 0, multi = 0;
-  size_t rows_max = 0, base = 0;
+  // A team lays out its own vectors and rows only, so the launch takes the largest
+  // team's sum (n <= 4096: at most 3 x 4096 doubles and the rows' 120 KB, or the 6 x
+  // 4096 doubles of a team of one, which has no rows there above n = 123)
+  size_t smem = 0;
   for (int p = 0; p < count; ++p) {
     EigProblem& P = probs_host[p];
     nmax = P.n > nmax ? P.n : nmax;
     const size_t rb = sizeof(double) * (size_t)tridiag_rows_per_cta(P.n, P.team_size) * P.n;
     P.srows = rb <= kTridiagSmemRowsCap;
-    if (P.srows && rb > rows_max) rows_max = rb;
-    base = std::max(base, tridiag_base_smem(P.n, P.team_size));
+    smem = std::max(smem, tridiag_base_smem(P.n, P.team_size) + (P.srows ? rb : 0));
     grid += P.team_size;
     multi |= P.team_size > 1;
   }
-  const size_t smem = base + rows_max;
   cudaError_t e = allow_max_dyn_smem((const void*)k_tridiag);
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(const_cast<EigProblem*>(probs_dev), probs_host, sizeof(EigProblem) * count,
