@@ -60,13 +60,26 @@ typedef enum { TUCKER_F32 = 0, TUCKER_F64 = 1 } tucker_dtype;
  * up to ~1.5e-10 ||X||^2 on the discarded subspace, too close to the
  * threshold eps^2 ||X||^2 / N below that.  The result reports the kernel of
  * every step.
- *   FP64   : products and sums in FP64 (any input dtype); core in FP64.  Large
- *            Grams (I_n >= 64) and TTMs form them on the tensor cores from
- *            exact integer digits: each value as a 55-bit fixed-point number
- *            of its row (rounding 2^-55 of the row's largest magnitude), every
- *            digit product and sum exact, one rounding to FP64 at the end; an
- *            operand with NaN, Inf or a row below 2^-958 takes the FP64 pipe
- *            (in a batch, a row below 2^-958 counts in units of 2^-1013).
+ *   FP64   : products and sums in FP64 (any input dtype); core in FP64.  From
+ *            a size (csrc/digit64.cu: plan_gram_d64, ttm_d64_supported) Grams
+ *            and TTMs are formed on the tensor cores from integer digits:
+ *            each value as a 55-bit fixed-point number of its row (of a TTM:
+ *            of its fibre, and of its row of the operator), so within 2^-55
+ *            of that row's largest magnitude; digit products that weigh less
+ *            than 2^-56 of the rows' largest values are left out (15 of 49,
+ *            below 2^-63 of their product a term), the others and their sums
+ *            are exact, and a TTM's entry or a Gram's entry of one K split is
+ *            rounded to FP64 once (the splits are added in FP64).  An entry
+ *            is so within 2^-55 (|x|_max |y|_1 + |y|_max |x|_1) and a few
+ *            roundings of its value: as close as FP64 sums relative to the
+ *            norms of the two rows, but not relative to itself when the large
+ *            values of one row meet small values of the other.  TTMs with an
+ *            operator that has zeros beside other values (selections,
+ *            differences) therefore stay on the FP64 pipe, and
+ *            TUCKER_OPT_FP64_PIPE keeps every step there.  An operand with
+ *            NaN, Inf or a row below 2^-958 takes the FP64 pipe (in a batch,
+ *            a row below 2^-958 counts in units of 2^-1013, and the
+ *            operators are the factors).
  *   FP32   : FP32 products, round-to-nearest FP32 sums over short chunks
  *            combined exactly (TwoSum) and in FP64; working tensor and core
  *            in the input dtype.
@@ -185,7 +198,13 @@ const char* tucker_last_error(const tucker_ctx* ctx);
  *                          one wave.
  *   TUCKER_OPT_HOST_CHUNK  bytes per piece in which tucker_sthosvd_host copies
  *                          its input (rounded to whole mode-0 columns, four at
- *                          a time); default 2^30, at least 1. */
+ *                          a time); default 2^30, at least 1.
+ *   TUCKER_OPT_FP64_PIPE   1: every Gram and TTM of precision FP64, and the
+ *                          FP64 Grams of the others, multiplies and adds FP64
+ *                          values on the FP64 pipe whatever its size (entries
+ *                          to the rounding of FP64 sums; 3 to 30 times the
+ *                          time of large steps).  0 (default): integer digits
+ *                          from a size (see FP64). */
 #define TUCKER_OPT_TIMING 1
 #define TUCKER_OPT_MAX_SWEEPS 2
 #define TUCKER_OPT_JACOBI_TOL 3
@@ -195,6 +214,7 @@ const char* tucker_last_error(const tucker_ctx* ctx);
 #define TUCKER_OPT_GRAM_DIGITS 7
 #define TUCKER_OPT_AUTOTUNE 8
 #define TUCKER_OPT_HOST_CHUNK 9
+#define TUCKER_OPT_FP64_PIPE 10
 tucker_status tucker_set_option(tucker_ctx* ctx, int key, double value);
 
 /* Diagnostics: number of device kernels this library has launched in the

@@ -55,6 +55,7 @@ struct tucker_ctx {
   unsigned long long barrier_polls = 1ull << 24;   // grid-barrier poll limit of the eigensolvers
   double mem_limit = 0.0;        // bytes assumed available to a call (0: ask the device)
   int gram_digits = 0;           // digits of the exact-digit Gram: 0 auto, 2 or 3
+  int fp64_pipe = 0;             // 1: no FP64 step on the integer digits (digit64.cu)
   int autotune = 0;              // 1: split-K of the Gram kernels chosen by timing
   double host_chunk = 1073741824.0;   // bytes per piece of tucker_sthosvd_host's copy
   std::string err;
@@ -457,7 +458,7 @@ tucker_status gram_once(tucker_ctx* c, const void* y, tucker_dtype dt, const Sla
     }
     return TUCKER_OK;
   }
-  if (kern == 0 || kern == 3) {
+  if ((kern == 0 || kern == 3) && !c->fp64_pipe) {
     // FP64 products: seven exact digits on the tensor cores from the size
     // where they beat the FP64 pipe (digit64.cu); out of their range (NaN,
     // Inf, rows below 2^-958): the FP64 pipe
@@ -533,7 +534,7 @@ tucker_status do_gram(tucker_ctx* c, const void* y, tucker_dtype dt, const SlabV
     return gram_once(c, y, dt, v, prec, S, kernel_used, maxabs, check, rowmax, ndig, kern,
                      c->num_sms);
   const std::array<int64_t, 7> key{c->device, kern, v.L, v.I, v.Rt, (int64_t)dt,
-                                   kern == 5 ? ndig : 0};
+                                   kern == 5 ? ndig : (kern == 0 || kern == 3 ? c->fp64_pipe : 0)};
   int best = 0;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -810,7 +811,7 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
   // FP64: seven exact digits on the tensor cores from the size where they
   // beat the FP64 pipe (digit64.cu); out of their range (NaN, Inf, rows below
   // 2^-958): the FP64 pipe
-  if (prec == TUCKER_PREC_FP64 && ttm_d64_supported(v.L, v.I, v.Rt, K)) {
+  if (prec == TUCKER_PREC_FP64 && !c->fp64_pipe && ttm_d64_supported(v.L, v.I, v.Rt, K)) {
     DevBuf scratch;
     TK_TRY(dev_alloc(c, scratch, ttm_d64_scratch_bytes(v.L, v.I, v.Rt, K)));
     TK_CUDA(c, launch_ttm_d64(y, ydt, v.L, v.I, v.Rt, A, K, lda, arow, z, zdt, zt, scratch.p,
@@ -939,6 +940,10 @@ tucker_status tucker_set_option(tucker_ctx* c, int key, double value) {
       if (value != 0.0 && value != 1.0 && value != 2.0)
         return set_err(c, TUCKER_ERR_INVALID, "eigensolver must be 0 (auto), 1 or 2");
       c->eig_solver = (int)value;
+      return TUCKER_OK;
+    case TUCKER_OPT_FP64_PIPE:
+      if (value != 0.0 && value != 1.0) return set_err(c, TUCKER_ERR_INVALID, "FP64 pipe must be 0 or 1");
+      c->fp64_pipe = (int)value;
       return TUCKER_OK;
     case TUCKER_OPT_AUTOTUNE:
       if (value != 0.0 && value != 1.0) return set_err(c, TUCKER_ERR_INVALID, "autotune must be 0 or 1");

@@ -30,11 +30,19 @@
 // the classes c >= 8 left out, below 2^-63 of a product of the rows' maxima
 // per k.  So an entry is off by at most 2^-55 (|x_i|_max |x_j|_1 + |x_j|_max
 // |x_i|_1), where an FP64 sum is off by 2^-53 of each of its partial sums.
+// Against the rows' norms that is no more than an FP64 sum has; against the entry
+// itself it is more where the large values of one row meet small ones of the other
+// (a value 2^-40 of its row's largest keeps 15 bits).  Hence TUCKER_OPT_FP64_PIPE, and
+// a TTM whose operator has a zero beside other values in a row (it may be there to leave
+// out a fibre's large values: selections, differences) is computed on the FP64 pipe.
 //   NaN, Inf, or a row whose largest magnitude is below 2^-958 (its exponents
 // would need the denormal range): the exponent pass sets *bad and the caller
 // computes the step on the FP64 pipe (the host reads the flag with the error
 // word); a caller that does not wait gets NaN for NaN and Inf, and small rows in
 // units of 2^-1013.
+//   Splitting FP64 matrices into slices whose products are exact in a narrower
+// arithmetic is the error-free transformation of Ozaki, Ogita, Oishi and Rump
+// (Numerical Algorithms 59, 2012), used on integer and FP16 matrix units since.
 //
 // Tile and roles.  One CTA owns a 128 x 64 tile (M x N): eight classes of 64
 // columns are all 512 tensor-memory columns.  The digit planes of the 64-row
@@ -280,6 +288,7 @@ struct Args {
   const unsigned* kexp;     // per output (64 ntn entries)
   void* z;
   int zt;                   // L == 1: z[m + M k]
+  int waits;                // the caller reads *bad and computes the step again
 };
 
 // Gram tile t -> (ta, tb): 128-row block ta, 64-row block tb <= 2 ta + 1.
@@ -377,7 +386,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_digit64(const Args g) {
   __shared__ uint64_t bar_full[NST], bar_empty[NST], bar_accf, bar_acce, bar_done;
   __shared__ uint32_t tmem_base_sh;
   if (*g.bad) {                                          // the same for the whole grid
-    if (TTM) {
+    if (TTM && !g.waits) {
       TOut* z = static_cast<TOut*>(g.z);
       for (int64_t e = (int64_t)blockIdx.x * NTHREADS + threadIdx.x; e < g.M * g.K;
            e += (int64_t)gridDim.x * NTHREADS)
@@ -884,7 +893,7 @@ __global__ void __launch_bounds__(256) k_mexp_rows(const T* __restrict__ y, int6
                                                    uint16_t* __restrict__ mexp,
                                                    unsigned* __restrict__ bad) {
   const int64_t m = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (m >= M) return;
+  if (m >= M || *bad) return;                            // (*bad: the operator's)
   const int64_t r = m / L, l = m - r * L;
   const T* p = y + l + L * I * r;
   int b = 0;
@@ -909,7 +918,7 @@ __global__ void __launch_bounds__(256) k_mexp_cols(const T* __restrict__ y, int6
                                                    unsigned* __restrict__ bad) {
   const int64_t m0 = 4 * (((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
-  if (m0 >= M) return;
+  if (m0 >= M || __shfl_sync(0xffffffffu, *bad, 0)) return;   // (*bad: the operator's)
   int e[4] = {0, 0, 0, 0};
   const T* p = y + m0 * I;
   for (int64_t i = lane; i < I; i += 64) {
@@ -942,28 +951,43 @@ __global__ void __launch_bounds__(256) k_digit64_prep(const double* __restrict__
                                                       uint8_t* __restrict__ img,
                                                       unsigned* __restrict__ kexp,
                                                       unsigned* __restrict__ bad) {
-  __shared__ int eb[NT];
+  __shared__ int eb[NT], zeros[NT];
   const int ks = blockIdx.x, nt = blockIdx.y, nks = gridDim.x;
-  if (threadIdx.x < NT) eb[threadIdx.x] = 0;
+  if (threadIdx.x < NT) eb[threadIdx.x] = zeros[threadIdx.x] = 0;
   __syncthreads();
   auto at = [&](int k, int64_t i) { return arow ? A[(int64_t)k * lda + i] : A[k + lda * i]; };
   if (arow) {                                       // i contiguous: a warp per row
     for (int row = threadIdx.x >> 5; row < NT; row += 8) {
       const int k = nt * NT + row;
       int e = 0;
+      bool zero = false;
       if (k < K)
-        for (int64_t i = threadIdx.x & 31; i < I; i += 32) e = max(e, mag_bits(at(k, i)));
+        for (int64_t i = threadIdx.x & 31; i < I; i += 32) {
+          const int m = mag_bits(at(k, i));
+          e = max(e, m);
+          zero |= m == 0;
+        }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-      if ((threadIdx.x & 31) == 0) eb[row] = e;
+      zero = __any_sync(0xffffffffu, zero);
+      if ((threadIdx.x & 31) == 0) { eb[row] = e; zeros[row] = zero; }
     }
   } else {
     const int row = threadIdx.x & (NT - 1), k = nt * NT + row;
     int e = 0;
+    bool zero = false;
     if (k < K)
-      for (int64_t i = threadIdx.x / NT; i < I; i += 256 / NT) e = max(e, mag_bits(at(k, i)));
+      for (int64_t i = threadIdx.x / NT; i < I; i += 256 / NT) {
+        const int m = mag_bits(at(k, i));
+        e = max(e, m);
+        zero |= m == 0;
+      }
     atomicMax(&eb[row], e);
+    if (zero) zeros[row] = 1;
   }
+  __syncthreads();
+  // (a row of zeros gives zeros either way)
+  if (ks == 0 && small && threadIdx.x < NT && zeros[threadIdx.x] && eb[threadIdx.x]) atomicOr(bad, 1u);
   __syncthreads();
   if (threadIdx.x < NT) eb[threadIdx.x] = row_exp(eb[threadIdx.x], 0.0, small);
   __syncthreads();
@@ -1049,6 +1073,7 @@ static cudaError_t ttm_d64(const T* y, int64_t L, int64_t I, int64_t Rt, const d
   a.z = z;
   a.zt = zt ? 1 : 0;
   const int small = err == nullptr;                      // the caller reads the verdict
+  a.waits = small;
   k_digit64_prep<<<dim3((unsigned)a.nks, (unsigned)a.ntn), 256, 0, st>>>(A, (int)K, I, lda, arow,
                                                                         small, scr + lay.img, kexp, bad);
   if (L > 1)

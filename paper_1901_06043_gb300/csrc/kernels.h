@@ -58,11 +58,12 @@ cudaError_t launch_rowmax_slab(const float* y, int64_t L, int64_t I, int64_t Rt,
 
 // ---- FP64 Gram and TTM on exact seven-digit tensor-core products
 // (digit64.cu).  plan.nctas == 0 / supported == 0 when the work is too small
-// (or I < 64, I > 8192 for the Gram).  scratch: plan.scratch_bytes /
-// ttm_d64_scratch_bytes, holding two verdict words (*_verdict): [0] nonzero when
-// an operand holds NaN, Inf or a row below 2^-958 (the output is then NaN and a
-// caller that reads the word computes the step with the SIMT kernel), [1] the
-// error word when err is NULL.
+// (or I > 8192 for the Gram).  scratch: plan.scratch_bytes / ttm_d64_scratch_bytes,
+// holding two verdict words (*_verdict): [0] nonzero when an operand holds NaN, Inf or a
+// row below 2^-958, or (err NULL) the operator of a TTM a zero beside other values in a
+// row: err NULL, the output is then not valid and the caller, who reads the word, computes
+// the step on the FP64 pipe; else the output is NaN for NaN and Inf.  [1] the error word
+// when err is NULL.
 GramPlan plan_gram_d64(int64_t L, int64_t I, int64_t Rt, int num_sms);
 const unsigned* gram_d64_verdict(const GramPlan& p, int64_t I, const void* scratch);
 cudaError_t launch_gram_d64(const void* y, tucker_dtype dt, int64_t L, int64_t I, int64_t Rt,

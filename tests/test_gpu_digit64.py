@@ -138,6 +138,62 @@ def test_fp64_digits_out_of_range_take_the_fp64_pipe(ctx, what):
             assert (np.abs(got - want)[fin] <= 1400 * 2.0 ** -52 * scale[fin] + 1e-322).all()
 
 
+def graded(n, m, seed):
+    """Fibres whose entries fall over 40 binary digits, in an order of their own each."""
+    rng = np.random.default_rng(seed)
+    e = np.linspace(0, -40, n)
+    return np.stack([np.ldexp(rng.uniform(1, 2, n), e[rng.permutation(n)].astype(int))
+                     * rng.choice([-1.0, 1.0], n) for _ in range(m)], 1)
+
+
+@pytest.mark.parametrize("arow", [True, False])
+@pytest.mark.parametrize("what", ["identity", "selection", "difference"])
+def test_operators_with_zeros_keep_small_entries(ctx, what, arow):
+    """An operator that leaves values of a fibre out: the entries it takes are as exact as
+    in FP64 sums however large the others are."""
+    import torch
+    n, m = 96, 600
+    X = graded(n, m, 5)
+    A = np.eye(n)
+    if what == "selection":
+        A = A[3::7] * 0.75
+    elif what == "difference":
+        A = (np.eye(n) - np.eye(n, k=1))[:-1]
+    x = torch.from_numpy(np.reshape(X, -1, order="F").copy()).cuda()
+    At = torch.from_numpy(A).cuda() if arow else torch.from_numpy(A.T.copy()).cuda().t()
+    z = ctx.ttm(x, (n, m), 0, At, prec="fp64").cpu().numpy().reshape((len(A), m), order="F")
+    want = A.astype(np.longdouble) @ X.astype(np.longdouble)
+    # (two terms at most: one product rounding each and one of the sum)
+    assert (np.abs(z - want) <= 2.0 ** -52 * (np.abs(A) @ np.abs(X))).all()
+
+
+@pytest.mark.parametrize("dims,mode", [((96, 4000), 0), ((5, 96, 900), 1), ((40, 70000), 0)])
+def test_the_fp64_pipe_on_request(dims, mode):
+    """TUCKER_OPT_FP64_PIPE: entries to the rounding of FP64 sums, n 2^-53 sum |x| |y|,
+    where rows differ by 40 binary digits within themselves."""
+    import torch
+    from paper_1901_06043_gb300 import tucker
+    c = tucker.Context()
+    c.set_option(tucker.OPT_FP64_PIPE, 1)
+    I, K = dims[mode], int(np.prod(dims)) // dims[mode]
+    U = graded(K, I, 6).T                       # rows graded along the columns
+    full = np.moveaxis(U.reshape([I] + [d for k, d in enumerate(dims) if k != mode], order="F"), 0, mode)
+    x = torch.from_numpy(np.reshape(full, -1, order="F").copy()).cuda()
+    U = unfold(np.reshape(full, -1, order="F"), dims, mode)
+    S = c.gram(x, dims, mode, prec="fp64").cpu().numpy()
+    L = U.astype(np.longdouble)
+    assert (np.abs(S - L @ L.T) <= K * 2.0 ** -53 * (np.abs(U) @ np.abs(U).T)).all()
+    A = graded(I, 33, 7).T
+    z = c.ttm(x, dims, mode, torch.from_numpy(A).cuda(), prec="fp64").cpu().numpy()
+    zd = list(dims)
+    zd[mode] = 33
+    assert (np.abs(unfold(z, zd, mode) - A.astype(np.longdouble) @ L)
+            <= (I + 1) * 2.0 ** -53 * (np.abs(A) @ np.abs(U))).all()
+    with pytest.raises(tucker.TuckerError):
+        c.set_option(tucker.OPT_FP64_PIPE, 2)
+    c.close()
+
+
 def test_batched_tensors_with_tiny_slices(ctx):
     """A batch does not wait for the verdict on each step; a slice below the digits' range
     (here 1e-295 of the others) is as good as zero there, as it is in the norm."""
