@@ -22,9 +22,9 @@
 // (TwoProduct by FMA).  Every 16 terms the pair is merged
 // exactly into a second-level pair that is renormalised (|lo| <= ulp(hi) / 2,
 // so its later roundings stay at 2^-48 of hi), and every 1024 terms that
-// pair moves into FP64; the result is the FP64 sum to ~1e-14 of sum |x|.  A
-// thread sums two streams in the halves of packed f32x2 registers: ~30 FP32
-// operations an element set the pace otherwise, not HBM.  The
+// pair moves into FP64; the result is the FP64 sum to ~1e-14 of sum |x|.  In the
+// runs regime a thread sums two streams in the halves of packed f32x2 registers: ~30
+// FP32 operations an element set the pace otherwise, not HBM.  The
 // standard deviation takes a second pass over the data, sum (x - mean)^2 with
 // the mean as an FP32 pair and x - mean_hi exact by TwoSum, which avoids the
 // cancellation of sum x^2 - count mean^2.  The transform evaluates
@@ -36,6 +36,7 @@
 #include "common.cuh"
 #include "kernels.h"
 
+#include <algorithm>
 #include <type_traits>
 
 namespace tk {
@@ -58,19 +59,40 @@ __device__ __forceinline__ double unordered(long long k) {
   return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
 }
 
+// FP32 operations on one value or on the two of a packed pair, rounded to nearest.
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float vabs(float a) { return fabsf(a); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return add2(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return sub2(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return mul2(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 vabs(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
+__device__ __forceinline__ void splat(float& v, float a) { v = a; }
+__device__ __forceinline__ void splat(float2& v, float a) { v = make_float2(a, a); }
+
 // (h, l) += v exactly (TwoSum, any magnitudes); l collects the errors.
-__device__ __forceinline__ void two_sum(float& h, float& l, float v) {
-  const float s = __fadd_rn(h, v);
-  const float bb = __fsub_rn(s, h);
-  const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(v, bb));
+template <typename V>
+__device__ __forceinline__ void two_sum(V& h, V& l, V v) {
+  const V s = vadd(h, v);
+  const V bb = vsub(s, h);
+  const V err = vadd(vsub(h, vsub(s, bb)), vsub(v, bb));
   h = s;
-  l = __fadd_rn(l, err);
+  l = vadd(l, err);
 }
 // Per-thread partial sums of one hyperslice.  PASS 0: sum, sum of squares,
-// sum |x|, max, min; PASS 1: sum (x - mean)^2.
-template <typename T, int PASS> struct Part;
+// sum |x|, max, min; PASS 1: sum (x - mean)^2.  W: streams of FP32 sums per thread,
+// 2 in the halves of packed registers (runs), 1 (rows: loads are 4 bytes a thread, and
+// the second stream's registers cost resident threads; standardizing 4.2e8 elements
+// along 300 rows and back 4.50 ms with two, 4.00 with one; 2.5e7 along 512 324 and 283
+// us).
+template <typename T, int PASS, int W> struct Part;
 
-template <int PASS> struct Part<double, PASS> {
+template <int PASS, int W> struct Part<double, PASS, W> {
   double s, s2, sa, c2, mean;
   long long mx, mn;                       // ordered bits
   Max64 up, dn;                           // running maxima of the bits, biased, and of their
@@ -97,7 +119,7 @@ template <int PASS> struct Part<double, PASS> {
     }
   }
   __device__ __forceinline__ void add2(double v, double w) { add1(v); add1(w); }
-  __device__ __forceinline__ void tick(int) {}
+  template <int MOST> __device__ __forceinline__ void tick(int) {}
   __device__ void flush() {
     if (PASS == 0 && (up.hi | dn.hi)) {
       mx = max(mx, (long long)(up.get() ^ 0x8000000000000000ull));
@@ -106,29 +128,25 @@ template <int PASS> struct Part<double, PASS> {
   }
 };
 
-// (h, l) += v exactly in both halves
-__device__ __forceinline__ void two_sum2(float2& h, float2& l, float2 v) {
-  const float2 s = add2(h, v);
-  const float2 bb = sub2(s, h);
-  const float2 err = add2(sub2(h, sub2(s, bb)), sub2(v, bb));
-  h = s;
-  l = add2(l, err);
-}
-
-template <int PASS> struct Part<float, PASS> {
+template <int PASS, int W> struct Part<float, PASS, W> {
+  using V = typename std::conditional<W == 2, float2, float>::type;
   double s, s2, sa, c2;                    // FP64 totals
   long long mx, mn;
-  // two streams, one per half
-  float2 sh, sl, qh, ql, ah, al;           // level 1: FP32 pairs of the current group
-  float2 SH, SL, QH, QL, AH, AL;           // level 2: renormalised pairs of the groups
+  V sh, sl, qh, ql, ah, al;                // level 1: FP32 pairs of the current group
+  V SH, SL, QH, QL, AH, AL;                // level 2: renormalised pairs of the groups
   float mh, ml;                            // the mean as an FP32 pair (PASS 1)
   float fmx, fmn;
   int n, g;
+  __device__ __forceinline__ void clear1() {
+    splat(sh, 0.f); splat(sl, 0.f); splat(qh, 0.f); splat(ql, 0.f); splat(ah, 0.f); splat(al, 0.f);
+  }
+  __device__ __forceinline__ void clear2() {
+    splat(SH, 0.f); splat(SL, 0.f); splat(QH, 0.f); splat(QL, 0.f); splat(AH, 0.f); splat(AL, 0.f);
+  }
   __device__ void init(double m) {
     s = s2 = sa = c2 = 0.0;
-    const float2 z = make_float2(0.f, 0.f);
-    sh = sl = qh = ql = ah = al = z;
-    SH = SL = QH = QL = AH = AL = z;
+    clear1();
+    clear2();
     mx = ordered(-INFINITY);
     mn = ordered(INFINITY);
     fmx = -INFINITY;
@@ -137,95 +155,101 @@ template <int PASS> struct Part<float, PASS> {
     ml = (float)(m - (double)mh);
     n = g = 0;
   }
-  __device__ __forceinline__ void add2(float v, float w) {
-    const float2 x = make_float2(v, w);
+  // the terms of x (one value or two) into level-1 sums of the same width
+  template <typename U>
+  __device__ __forceinline__ void terms(U x, U& h0, U& l0, U& h1, U& l1, U& h2, U& l2) {
     if (PASS == 0) {
-      two_sum2(sh, sl, x);
-      const float2 p = mul2(x, x);
-      const float2 pe = fma2(x, x, make_float2(-p.x, -p.y));   // x^2 = p + pe exactly
-      two_sum2(qh, ql, p);
-      ql = tk::add2(ql, pe);
-      two_sum2(ah, al, make_float2(fabsf(v), fabsf(w)));
-      fmx = fmaxf(fmx, fmaxf(v, w));
-      fmn = fminf(fmn, fminf(v, w));
+      two_sum(h0, l0, x);
+      const U p = vmul(x, x);
+      const U pe = vfma(x, x, vneg(p));                        // x^2 = p + pe exactly
+      two_sum(h1, l1, p);
+      l1 = vadd(l1, pe);
+      two_sum(h2, l2, vabs(x));
     } else {
       // d = x - mean = (s + e) - ml with s + e = x - mh exactly
-      float2 s_ = x, e = make_float2(0.f, 0.f);
-      two_sum2(s_, e, make_float2(-mh, -mh));
-      const float2 t = tk::add2(e, make_float2(-ml, -ml));
-      const float2 p = mul2(s_, s_);
-      const float2 pe = fma2(s_, s_, make_float2(-p.x, -p.y));
+      U s_ = x, e, m, two;
+      splat(e, 0.f);
+      splat(m, -mh);
+      two_sum(s_, e, m);
+      splat(m, -ml);
+      const U t = vadd(e, m);
+      const U p = vmul(s_, s_);
+      const U pe = vfma(s_, s_, vneg(p));
       // d^2 = p + pe + t (2 s + t); |t| can be a sizeable part of |s| when
       // the slice varies little around its mean, so t^2 stays
-      two_sum2(qh, ql, p);
-      ql = tk::add2(ql, fma2(fma2(s_, make_float2(2.f, 2.f), t), t, pe));
+      two_sum(h1, l1, p);
+      splat(two, 2.f);
+      l1 = vadd(l1, vfma(vfma(s_, two, t), t, pe));
     }
   }
-  // one element, into the first half
+  __device__ __forceinline__ void add2(float v, float w) {
+    if constexpr (W == 2) {
+      terms(make_float2(v, w), sh, sl, qh, ql, ah, al);
+      if (PASS == 0) {
+        fmx = fmaxf(fmx, fmaxf(v, w));
+        fmn = fminf(fmn, fminf(v, w));
+      }
+    } else {
+      add1(v);
+      add1(w);
+    }
+  }
+  // one element, into the first stream
   __device__ __forceinline__ void add1(float v) {
+    if constexpr (W == 2) terms(v, sh.x, sl.x, qh.x, ql.x, ah.x, al.x);
+    else terms(v, sh, sl, qh, ql, ah, al);
     if (PASS == 0) {
-      two_sum(sh.x, sl.x, v);
-      const float p = __fmul_rn(v, v);
-      const float pe = __fmaf_rn(v, v, -p);
-      two_sum(qh.x, ql.x, p);
-      ql.x = __fadd_rn(ql.x, pe);
-      two_sum(ah.x, al.x, fabsf(v));
       fmx = fmaxf(fmx, v);
       fmn = fminf(fmn, v);
-    } else {
-      float s_ = v, e = 0.f;
-      two_sum(s_, e, -mh);
-      const float t = __fsub_rn(e, ml);
-      const float p = __fmul_rn(s_, s_);
-      const float pe = __fmaf_rn(s_, s_, -p);
-      two_sum(qh.x, ql.x, p);
-      ql.x = __fadd_rn(ql.x, __fmaf_rn(__fmaf_rn(2.f, s_, t), t, pe));
     }
   }
-  // after every k <= 8 terms of a half: merge before a group exceeds kGroup
-  __device__ __forceinline__ void tick(int k) {
+  // after every k <= MOST terms of a stream: merge before a group exceeds kGroup
+  template <int MOST> __device__ __forceinline__ void tick(int k) {
     n += k;
-    if (n > kGroup - 8) merge();
+    if (n > kGroup - MOST) merge();
   }
   // (H, L) += (h, l) exactly up to the rounding of L, then renormalised so
   // that |L| <= ulp(H) / 2 (its later roundings stay at 2^-48 of H)
-  __device__ __forceinline__ static void merge_pair(float2& H, float2& L, float2 h, float2 l) {
-    two_sum2(H, L, h);
-    L = tk::add2(L, l);
-    float2 t = H, e = make_float2(0.f, 0.f);    // (t, e) = H + L exactly (TwoSum)
-    two_sum2(t, e, L);
+  template <typename U>
+  __device__ __forceinline__ static void merge_pair(U& H, U& L, U h, U l) {
+    two_sum(H, L, h);
+    L = vadd(L, l);
+    U t = H, e;                                 // (t, e) = H + L exactly (TwoSum)
+    splat(e, 0.f);
+    two_sum(t, e, L);
     H = t;
     L = e;
   }
   // level 1 -> level 2 every kGroup terms; level 2 -> FP64 every kGroups groups
   __device__ void merge() {
-    const float2 z = make_float2(0.f, 0.f);
     if (PASS == 0) {
       merge_pair(SH, SL, sh, sl);
       merge_pair(QH, QL, qh, ql);
       merge_pair(AH, AL, ah, al);
-      sh = sl = qh = ql = ah = al = z;
     } else {
       merge_pair(QH, QL, qh, ql);
-      qh = ql = z;
     }
+    clear1();
     n = 0;
     if (++g == kGroups) flush_groups();
   }
+  // A level-2 sum in FP64; of two streams the second is merged into the first by
+  // FP32 operations, as a group is (a conversion and an addition on the FP64 pipe take
+  // 128 cycles a warp, and a thread of a small tensor does little else).
+  __device__ static double total(float H, float L) { return (double)H + (double)L; }
   __device__ static double total(float2 H, float2 L) {
-    return ((double)H.x + (double)L.x) + ((double)H.y + (double)L.y);
+    merge_pair(H.x, L.x, H.y, L.y);
+    return total(H.x, L.x);
   }
   __device__ void flush_groups() {
-    const float2 z = make_float2(0.f, 0.f);
     if (PASS == 0) {
       s += total(SH, SL);
       s2 += total(QH, QL);
       sa += total(AH, AL);
-      SH = SL = QH = QL = AH = AL = z;
     } else {
       c2 += total(QH, QL);
-      QH = QL = z;
     }
+    clear2();
     g = 0;
   }
   // everything into the FP64 totals (before a reduction)
@@ -239,8 +263,8 @@ template <int PASS> struct Part<float, PASS> {
   }
 };
 
-template <typename T, int PASS>
-__device__ void to_global(double* acc, int64_t i, const Part<T, PASS>& p) {
+template <typename T, int PASS, int W>
+__device__ void to_global(double* acc, int64_t i, const Part<T, PASS, W>& p) {
   double* a = acc + i * kAcc;
   if (PASS == 0) {
     atomicAdd(a + 0, p.s);
@@ -254,8 +278,8 @@ __device__ void to_global(double* acc, int64_t i, const Part<T, PASS>& p) {
 }
 
 // Block reduction of the FP64 totals into thread 0 (all threads call it).
-template <typename T, int PASS>
-__device__ void block_reduce(Part<T, PASS>& p) {
+template <typename T, int PASS, int W>
+__device__ void block_reduce(Part<T, PASS, W>& p) {
   __shared__ double sh[4][kThreads / 32];
   __shared__ long long sm[2][kThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -299,7 +323,7 @@ __global__ void __launch_bounds__(kThreads) k_stats_rows(const T* __restrict__ x
   if (q >= P || c >= C) return;
   const int64_t i = q / L;
   const int64_t r0 = Rt * blockIdx.y / ncol, r1 = Rt * (blockIdx.y + 1) / ncol;
-  Part<T, PASS> p;
+  Part<T, PASS, 1> p;
   p.init(PASS ? mean[i] : 0.0);
   const int64_t step = (int64_t)C * P;
   const T* ptr = x + q + P * (r0 + c);
@@ -309,14 +333,14 @@ __global__ void __launch_bounds__(kThreads) k_stats_rows(const T* __restrict__ x
             e = __ldg(ptr + 3 * step);
     p.add2(a, b);
     p.add2(d, e);
-    p.tick(2);
+    p.template tick<4>(4);
   }
   for (; r < r1; r += C, ptr += step) {
     p.add1(__ldg(ptr));
-    p.tick(1);
+    p.template tick<1>(1);
   }
   p.flush();
-  if (r1 > r0) to_global(acc, i, p);
+  if (r0 + c < r1) to_global(acc, i, p);
 }
 
 // CTAs per SM in the grids of the runs kernels: several waves, as the SMs' shares
@@ -341,7 +365,7 @@ __global__ void __launch_bounds__(kThreads) k_stats_runs(const T* __restrict__ x
   if (u0 >= u1) return;
   int64_t cur = u0 / per_i, rest0 = u0 % per_i;
   int64_t i = cur, r = rest0 / nch, ch = rest0 % nch;
-  Part<T, PASS> p;
+  Part<T, PASS, 2> p;
   p.init(PASS ? mean[cur] : 0.0);
   for (int64_t u = u0; u < u1; ++u) {
     if (i != cur) {                       // uniform across the block
@@ -364,7 +388,7 @@ __global__ void __launch_bounds__(kThreads) k_stats_runs(const T* __restrict__ x
           for (int k = 0; k < U; ++k) q[k] = __ldg(reinterpret_cast<const float4*>(run + l + k * V * kThreads));
 #pragma unroll
           for (int k = 0; k < U; ++k) { p.add2(q[k].x, q[k].y); p.add2(q[k].z, q[k].w); }
-          p.tick(2 * U);
+          p.template tick<8>(2 * U);
         } else {
           double2 q[U];
 #pragma unroll
@@ -380,11 +404,11 @@ __global__ void __launch_bounds__(kThreads) k_stats_runs(const T* __restrict__ x
                 d = __ldg(run + l + 2 * kThreads), e = __ldg(run + l + 3 * kThreads);
         p.add2(a, b);
         p.add2(d, e);
-        p.tick(2);
+        p.template tick<8>(2);
       }
       for (; l < l1; l += kThreads) {
         p.add1(__ldg(run + l));
-        p.tick(1);
+        p.template tick<8>(1);
       }
     }
     if (++ch == nch) {
@@ -572,10 +596,15 @@ __global__ void k_params(const double* stats, int64_t I, int method, double* shi
   }
 }
 
-// rows-regime grid: (row blocks, column chunks) about 8 CTAs per SM
-void rows_grid(int64_t P, int64_t Rt, int num_sms, unsigned& gx, int& nc) {
+// rows-regime grid: (row blocks, column chunks) about 8 CTAs per SM; fewer where a
+// thread would have less than `per` elements (0: whatever it has).  The statistics take
+// 32: a thread ends with five atomics on one set of words per hyperslice, which otherwise
+// are the pass (standardizing 60,000 elements along 40 rows and back: 338 us with 1,216
+// chunks, 118 with 7; 1.1e6 along 100 186 and 123 us).
+void rows_grid(int64_t P, int64_t Rt, int num_sms, int per, unsigned& gx, int& nc) {
   const int64_t rb = P < kThreads ? 1 : (P + kThreads - 1) / kThreads;
   int64_t c = ((int64_t)num_sms * 8 + rb - 1) / rb;
+  if (per > 0) c = std::min(c, Rt / (per * (P < kThreads ? kThreads / P : 1)));
   if (c > Rt) c = Rt;
   if (c > 65535) c = 65535;
   gx = (unsigned)rb;
@@ -589,7 +618,7 @@ void stats_pass(const T* x, int64_t L, int64_t I, int64_t Rt, const double* mean
     const int64_t P = L * I;
     unsigned gx;
     int nc;
-    rows_grid(P, Rt, num_sms, gx, nc);
+    rows_grid(P, Rt, num_sms, 32, gx, nc);
     k_stats_rows<T, PASS><<<dim3(gx, (unsigned)nc), kThreads, 0, st>>>(x, L, P, Rt, nc, mean,
                                                                         acc);
   } else {
@@ -626,7 +655,7 @@ void apply_t(const T* x, int64_t L, int64_t I, int64_t Rt, const double* shift,
     const int64_t P = L * I;
     unsigned gx;
     int nc;
-    rows_grid(P, Rt, num_sms, gx, nc);
+    rows_grid(P, Rt, num_sms, 0, gx, nc);
     k_apply_rows<T, INV><<<dim3(gx, (unsigned)nc), kThreads, 0, st>>>(x, L, P, Rt, nc, shift,
                                                                        scale, y);
     return;
