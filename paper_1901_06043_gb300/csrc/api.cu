@@ -673,6 +673,32 @@ bool use_tridiag(const tucker_ctx* c, int n) {
   return n >= 1 && n <= 4096;
 }
 
+// Z^T Z of one problem into P.gram, for pass 0 or 1 of its Cholesky QR: the Gram of
+// the column-major view of Z (L = 1, I = R, Rt = n).  Pass 1 is wanted only where
+// pass 0 has set info[1] and not failed.  Up to 63 vectors the kernels look at the
+// word; above, where a Gram and its factor are a dozen launches or more, the host reads
+// it (*need = false: neither the Gram nor the factor was wanted, and none was made).
+tucker_status z_gram(tucker_ctx* c, const EigProblem& P, int pass, bool* need) {
+  const SlabView zv{1, (int64_t)P.R, (int64_t)P.n, 1};
+  *need = true;
+  const GramPlan ps = plan_gram_small(zv.L, zv.I, zv.Rt, c->num_sms, zv.L0);
+  if (pass > 0 && ps.nctas > 0) {
+    DevBuf scratch;
+    TK_TRY(dev_alloc(c, scratch, ps.scratch_bytes));
+    TK_CUDA(c, launch_gram_small(P.z, TUCKER_F64, zv.L, zv.I, zv.Rt, zv.L0, ps,
+                                 scratch.as<double>(), P.gram, c->stream, P.info + 1));
+    return TUCKER_OK;
+  }
+  if (pass > 0) {
+    int info[2] = {0, 0};
+    TK_CUDA(c, cudaMemcpyAsync(info, P.info, sizeof info, cudaMemcpyDeviceToHost, c->stream));
+    TK_TRY(sync(c));
+    *need = info[0] == 0 && info[1] != 0;
+    if (!*need) return TUCKER_OK;
+  }
+  return do_gram(c, P.z, TUCKER_F64, zv, TUCKER_PREC_FP64, P.gram, nullptr);
+}
+
 // All eigenvalues (descending, into w) and the leading R eigenvectors of S by
 // the tridiagonal solver (tridiag.cu); R from the cut at thr, or fixed_R > 0.
 // U is allocated here (I x R, column-major).  *failed: the Cholesky QR
@@ -737,12 +763,12 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   h.zoff = 0;
   TK_CUDA(c, cudaMemcpyAsync(pd, &h, sizeof(h), cudaMemcpyHostToDevice, st));
   TK_CUDA(c, launch_invit(pd, 1, Ri, st));
-  // Cholesky QR, twice (the second pass restores orthogonality to rounding
-  // when eigenvalues are clustered and the vectors are far from orthogonal).
-  // Z^T Z is the Gram of the column-major view of Z (L = 1, I = R, Rt = n).
-  const SlabView zv{1, (int64_t)Ri, (int64_t)n, 1};
+  // Cholesky QR, a second time where the first pass found the vectors far from
+  // orthogonal (clustered eigenvalues; info[1]).
   for (int pass = 0; pass < 2; ++pass) {
-    TK_TRY(do_gram(c, h.z, TUCKER_F64, zv, TUCKER_PREC_FP64, h.gram, nullptr));
+    bool need = true;
+    TK_TRY(z_gram(c, h, pass, &need));
+    if (!need) break;
     TK_CUDA(c, launch_cholqr(pd, &h, 1, pass, c->num_sms, st));
   }
   TK_CUDA(c, wy.join());
@@ -1699,18 +1725,26 @@ tucker_status tucker_sthosvd_batched(tucker_ctx* c, int count, const void* const
     }
     TK_CUDA(c, cudaMemcpyAsync(pd, h.data(), sizeof(EigProblem) * m, cudaMemcpyHostToDevice, st));
     TK_CUDA(c, launch_invit(pd, m, zoff, st));
+    // (the second pass of problems with R > 64 only where the first wants it, by the host)
+    std::vector<int> info(3 * m);
+    bool large = false;
+    for (int q = 0; q < m; ++q) large |= h[q].R > zgram_batched_max_r();
     for (int pass = 0; pass < 2; ++pass) {
       TK_CUDA(c, launch_zgram_batched(pd, m, pass, st));   // problems with R <= 64
+      if (pass > 0 && large) {
+        TK_CUDA(c, cudaMemcpyAsync(info.data(), info_d, 3 * sizeof(int) * m, cudaMemcpyDeviceToHost, st));
+        TK_TRY(sync(c));
+      }
       for (int q = 0; q < m; ++q)
-        if (h[q].R > zgram_batched_max_r()) {
+        if (h[q].R > zgram_batched_max_r() && (pass == 0 || (info[3 * q] == 0 && info[3 * q + 1]))) {
           const SlabView zv{1, (int64_t)h[q].R, (int64_t)h[q].n, 1};
           TK_TRY(do_gram(c, h[q].z, TUCKER_F64, zv, TUCKER_PREC_FP64, h[q].gram, nullptr));
         }
-      TK_CUDA(c, launch_cholqr(pd, h.data(), m, pass, c->num_sms, st));
+      TK_CUDA(c, launch_cholqr(pd, h.data(), m, pass, c->num_sms, st,
+                               pass > 0 && large ? info.data() : nullptr));
     }
     TK_CUDA(c, launch_wy(pd, nullptr, m, nmax, st));
     TK_CUDA(c, launch_backtransform(pd, m, zoff, nmax, st));
-    std::vector<int> info(3 * m);
     unsigned berr = 0;
     TK_CUDA(c, cudaMemcpyAsync(info.data(), info_d, 3 * sizeof(int) * m, cudaMemcpyDeviceToHost, st));
     TK_CUDA(c, cudaMemcpyAsync(&berr, berr_d, sizeof(unsigned), cudaMemcpyDeviceToHost, st));

@@ -33,7 +33,9 @@ constexpr int SPPT = (SMAXP + SNT - 1) / SNT;               // entries per threa
 
 template <typename TIn>
 __global__ void __launch_bounds__(SNT) k_gram_small(const TIn* __restrict__ y, KGeom g,
+                                                    const int* __restrict__ need,
                                                     double* __restrict__ part) {
+  if (need && *need == 0) return;
   __shared__ double ys[SBK][SMAXI + 2];   // odd row stride in doubles: the l-major staging spreads over banks
   const int I = (int)g.I;
   const int npair = I * (I + 1) / 2;
@@ -95,7 +97,8 @@ __global__ void __launch_bounds__(SNT) k_gram_small(const TIn* __restrict__ y, K
 // entry, lane l summing parts l, l + 32, ... in order, then a fixed butterfly
 // across the lanes (a chain of ~nparts / 32 FP64 additions instead of nparts).
 __global__ void k_gram_small_reduce(const double* __restrict__ part, int nparts, int I,
-                                    double* __restrict__ S) {
+                                    const int* __restrict__ need, double* __restrict__ S) {
+  if (need && *need == 0) return;
   const int npair = I * (I + 1) / 2;
   const int p = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
@@ -131,14 +134,14 @@ GramPlan plan_gram_small(int64_t L, int64_t I, int64_t Rt, int num_sms, int64_t 
 
 cudaError_t launch_gram_small(const void* y, tucker_dtype dt, int64_t L, int64_t I, int64_t Rt,
                               int64_t L0, const GramPlan& p, double* scratch, double* S,
-                              cudaStream_t st) {
+                              cudaStream_t st, const int* need) {
   const KGeom g = make_kgeom(L, I, Rt, SBK, L0);
   if (dt == TUCKER_F64)
-    k_gram_small<double><<<p.nctas, SNT, 0, st>>>((const double*)y, g, scratch);
+    k_gram_small<double><<<p.nctas, SNT, 0, st>>>((const double*)y, g, need, scratch);
   else
-    k_gram_small<float><<<p.nctas, SNT, 0, st>>>((const float*)y, g, scratch);
+    k_gram_small<float><<<p.nctas, SNT, 0, st>>>((const float*)y, g, need, scratch);
   const int npair = (int)(I * (I + 1) / 2);
-  k_gram_small_reduce<<<(npair + 7) / 8, 256, 0, st>>>(scratch, p.nctas, (int)I, S);
+  k_gram_small_reduce<<<(npair + 7) / 8, 256, 0, st>>>(scratch, p.nctas, (int)I, need, S);
   count_launches(2);
   return cudaGetLastError();
 }

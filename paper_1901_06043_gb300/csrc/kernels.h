@@ -96,11 +96,12 @@ cudaError_t launch_gram_f32(const float* y, int64_t L, int64_t I, int64_t Rt, in
                             const GramPlan& p, double* scratch, double* S, cudaStream_t st);
 
 // ---- Gram of a small mode (I < 64) in FP64 (products of FP32 inputs are
-// exact), for every precision; plan.nctas == 0 when it does not apply
+// exact), for every precision; plan.nctas == 0 when it does not apply.  need: a device
+// word; the kernels return at once where it is 0 (NULL: they run)
 GramPlan plan_gram_small(int64_t L, int64_t I, int64_t Rt, int num_sms, int64_t L0);
 cudaError_t launch_gram_small(const void* y, tucker_dtype dt, int64_t L, int64_t I, int64_t Rt,
                               int64_t L0, const GramPlan& p, double* scratch, double* S,
-                              cudaStream_t st);
+                              cudaStream_t st, const int* need = nullptr);
 
 // ---- SIMT TTM
 // a32_scratch: K * I floats for the FP32 copy of A (FP32 arithmetic), or NULL
@@ -192,9 +193,11 @@ cudaError_t launch_bisect(const EigProblem* probs_dev, int count, int nmax, int 
                           int num_sms, cudaStream_t st);
 cudaError_t launch_invit(const EigProblem* probs_dev, int count, int total_vectors, cudaStream_t st);
 // Cholesky QR of every problem's Z with its Gram in P.gram, pass 0 or 1 (pass 1
-// does nothing where pass 0 found the Gram near the identity: info[1] == 0)
+// does nothing where pass 0 found the Gram near the identity: info[1] == 0).  info: for
+// pass 1, the problems' info words on the host, or NULL; with it nothing is launched
+// for a problem with R > 64 that does not want the pass
 cudaError_t launch_cholqr(const EigProblem* probs_dev, const EigProblem* probs_host, int count,
-                          int pass, int num_sms, cudaStream_t st);
+                          int pass, int num_sms, cudaStream_t st, const int* info = nullptr);
 // T factors of the blocked back-transformation (after launch_tridiag; needed by
 // launch_backtransform): of the `count` problems, or of `one` (host) alone
 cudaError_t launch_wy(const EigProblem* probs_dev, const EigProblem* one, int count, int nmax,

@@ -1438,7 +1438,7 @@ cudaError_t launch_invit(const EigProblem* probs_dev, int count, int total_vecto
 }
 
 cudaError_t launch_cholqr(const EigProblem* probs_dev, const EigProblem* probs_host, int count,
-                          int pass, int num_sms, cudaStream_t st) {
+                          int pass, int num_sms, cudaStream_t st, const int* info) {
   int nmax = 0;
   for (int p = 0; p < count; ++p)
     if (probs_host[p].R <= CS) nmax = probs_host[p].n > nmax ? probs_host[p].n : nmax;
@@ -1449,7 +1449,7 @@ cudaError_t launch_cholqr(const EigProblem* probs_dev, const EigProblem* probs_h
   }
   for (int p = 0; p < count; ++p) {
     const int R = probs_host[p].R, n = probs_host[p].n;
-    if (R <= CS) continue;
+    if (R <= CS || (info && (info[3 * p] != 0 || info[3 * p + 1] == 0))) continue;
     const EigProblem* pd = probs_dev + p;
     if (pass == 0) {
       k_chol_far<<<(int)std::min<int64_t>(((int64_t)R * R + TNT - 1) / TNT, num_sms), TNT, 0, st>>>(pd);

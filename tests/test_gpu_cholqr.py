@@ -35,6 +35,27 @@ def test_vectors_are_orthonormal_eigenvectors(ctx, n, R, clustered):
     assert np.abs(S @ U - U * w[:R]).max() <= 1e-13 * n
 
 
+def test_second_pass_is_launched_only_where_needed(ctx):
+    """Above 64 vectors the second pass (its Gram and the factor's blocks) is not launched
+    for well separated eigenvalues."""
+    import torch
+    from paper_1901_06043_gb300 import tucker
+    n, R = 200, 97
+    rng = np.random.default_rng(0)
+    Q, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    counts = []
+    for lam in (np.linspace(2, 1, n), np.repeat(np.linspace(2, 1, n // 4), 4)):
+        S = (Q * lam) @ Q.T
+        St = torch.from_numpy((S + S.T) / 2).cuda()
+        before = tucker.kernel_launches()
+        _, U, _, _ = ctx.eig_trunc(St, R=R)
+        counts.append(tucker.kernel_launches() - before)
+        U = U.cpu().numpy()
+        assert np.abs(U.T @ U - np.eye(R)).max() <= 1e-13 * n
+    # two launches of the Gram, 3 * 3 + 1 of the four blocks' factor, one of the product
+    assert counts[0] + 12 <= counts[1]
+
+
 @pytest.mark.parametrize("n", [1, 2, 127, 128, 129, 1023, 1024, 1025, 2500])
 def test_rank_cut_sums_in_order(ctx, n):
     """Bitwise the sequential sum from the smallest value up, also across the
