@@ -667,7 +667,10 @@ __global__ void __launch_bounds__(TNT, sizeof(TC) == 4 ? 4 : 2)
   extern __shared__ __align__(16) unsigned char ttm_sm[];
   TIn* Ys = reinterpret_cast<TIn*>(ttm_sm);                         // COL: [2][MT][YP], else [2][TIC][MT]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t m0 = (int64_t)blockIdx.x * MT, k0 = (int64_t)blockIdx.y * KT;
+  // (tiles of outputs beyond the 65,535 that a grid's y counts go along z)
+  const int64_t m0 = (int64_t)blockIdx.x * MT;
+  const int64_t k0 = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * KT;
+  if (k0 >= K) return;
   const int nk = (int)min((int64_t)KT, K - k0);
 
   // entries of A for i0..: threads along whichever index is contiguous
@@ -1013,13 +1016,13 @@ static cudaError_t ttm_tile(const TIn* y, int64_t L, int64_t I, int64_t M, const
                             int64_t lda, int arow, const float* A32, TOut* z, int zt,
                             cudaStream_t st) {
   constexpr int WK = KT == 8 ? 2 : 4, MM = WK, MT = TNT;
-  const int64_t gx = (M + MT - 1) / MT;
-  if (gx > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+  const int64_t gx = (M + MT - 1) / MT, tiles = (K + KT - 1) / KT, gz = (tiles + 65534) / 65535;
+  if (gx > 0x7fffffffll || gz > 65535) return cudaErrorInvalidConfiguration;
   auto kern = k_ttm<TIn, TOut, TC, KT, WK, MM, COL>;
   cudaError_t e = allow_max_dyn_smem((const void*)kern);
   if (e != cudaSuccess) return e;
-  kern<<<dim3((unsigned)gx, (unsigned)((K + KT - 1) / KT)), TNT, ttm_smem<TIn, TC, KT, MT, COL>(), st>>>(
-      y, L, I, M, A, K, lda, arow, A32, z, zt);
+  const dim3 grid((unsigned)gx, (unsigned)((tiles + gz - 1) / gz), (unsigned)gz);
+  kern<<<grid, TNT, ttm_smem<TIn, TC, KT, MT, COL>(), st>>>(y, L, I, M, A, K, lda, arow, A32, z, zt);
   return cudaGetLastError();
 }
 

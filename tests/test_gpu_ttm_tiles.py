@@ -55,6 +55,25 @@ def test_ttm_tiles(ctx, dims, mode, K, prec):
             assert (np.abs(z - want) <= bound).all()
 
 
+@pytest.mark.parametrize("dims,mode", [((3, 4), 0), ((2, 3, 2), 1)])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_more_output_tiles_than_a_grid_dimension(ctx, dims, mode, prec):
+    """2.2 million outputs: 68,751 tiles of 32."""
+    K = 2200001
+    gen = torch.Generator("cuda").manual_seed(3)
+    dt = torch.float32 if prec == "fp32" else torch.float64
+    x = torch.randn(12, device="cuda", generator=gen, dtype=dt)
+    A = torch.randn(K, 3, device="cuda", generator=gen, dtype=torch.float64)
+    z = ctx.ttm(x, dims, mode, A, prec=prec).double()
+    U = x.double().reshape(tuple(reversed(dims)))
+    if mode == 0:
+        got, want, scale = z.reshape(4, K), U @ A.T, U.abs() @ A.abs().T
+    else:
+        got, want, scale = z.reshape(2, K, 2), A @ U, A.abs() @ U.abs()
+    u = 2.0 ** -24 if prec == "fp32" else 2.0 ** -53
+    assert bool(((got - want).abs() <= 6 * u * scale).all())
+
+
 @pytest.mark.parametrize("dims,mode,K", [((40, 128), 0, 17), ((500, 384), 0, 100), ((16, 33, 7), 1, 300),
                                          ((132, 54, 3), 1, 513), ((128, 5, 2), 1, 1)])
 @pytest.mark.parametrize("scale", [1e-25, 1.0, 1e12])
