@@ -61,7 +61,7 @@ typedef enum { TUCKER_F32 = 0, TUCKER_F64 = 1 } tucker_dtype;
  * threshold eps^2 ||X||^2 / N below that.  The result reports the kernel of
  * every step.
  *   FP64   : products and sums in FP64 (any input dtype); core in FP64.  From
- *            a size (csrc/digit64.cu: plan_gram_d64, ttm_d64_supported) Grams
+ *            a size (csrc/digit64.cu: plan_gram_d64, ttm_d64_chosen) Grams
  *            and TTMs are formed on the tensor cores from integer digits:
  *            each value as a 55-bit fixed-point number of its row (of a TTM:
  *            of its fibre, and of its row of the operator), so within 2^-55

@@ -837,7 +837,8 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
   // FP64: seven exact digits on the tensor cores from the size where they
   // beat the FP64 pipe (digit64.cu); out of their range (NaN, Inf, rows below
   // 2^-958): the FP64 pipe
-  if (prec == TUCKER_PREC_FP64 && !c->fp64_pipe && ttm_d64_supported(v.L, v.I, v.Rt, K)) {
+  if (prec == TUCKER_PREC_FP64 && !c->fp64_pipe &&
+      ttm_d64_chosen(v.L, v.I, v.Rt, K, c->num_sms)) {
     DevBuf scratch;
     TK_TRY(dev_alloc(c, scratch, ttm_d64_scratch_bytes(v.L, v.I, v.Rt, K)));
     TK_CUDA(c, launch_ttm_d64(y, ydt, v.L, v.I, v.Rt, A, K, lda, arow, z, zdt, zt, scratch.p,

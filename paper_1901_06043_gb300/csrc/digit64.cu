@@ -72,6 +72,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -106,11 +107,34 @@ constexpr int BAD_EXP = 0x7ff, MIN_EXP = 64;   // biased exponents of a row: bad
 constexpr int OUT_EXP = -2 * 1022 - 70;        // an entry is its sum times 2^(eb + eb' + OUT_EXP)
 // Work from which a step comes here.  Gram: I^2 K >= 2e7 (whole calls, I = 200:
 // 86 us on the FP64 pipe and 76 us here at 2e7; 66 and 75 us at 1e7; 235 and 89
-// us at 1e8).  TTM: a contraction of 64 or more (the FP64-pipe kernel takes ~1.1
-// us per i whatever the size: 163 us against 89 at I = 128, 96 against 86 at
-// I = 60), or 2 K I M >= 4e7 (I = 26: 95 and 87 us; 64 and 87 us at 2e7).
-constexpr double kDigit64MinGram = 2e7, kDigit64MinTtm = 4e7;
+// us at 1e8).
+constexpr double kDigit64MinGram = 2e7;
+// TTM: where the digits are the faster by the two models of a whole call below (us,
+// FP64 data, one wave being num_sms blocks), fitted to 720 calls with I from 8 to 500, K from
+// 4 to 200 and M from 300 to 4e5, column and row views: within 22 % (FP64 pipe), 20 %
+// (here, column views) and 33 % (row views).  On these calls the rule loses 0.5 % to the
+// better of the two, and 28 % at worst (26 x 24000 to 28, row view, 101 us there and 79
+// here).  Both sides, there and here: 64 x 1500 to 4 51 and 68, to 28 101 and 75; 200 x 1500 to 4 94
+// and 89; 16 x 1e5 to 16 83 and 108, to 28 132 and 113; 200 x 4e5 to 28 4248 and 808.
+//   A block of the pipe's kernel takes 0.31, 0.57 or 1.08 us per i for 8, 16 or more
+// outputs, a CTA here per item of 128 m and 64 outputs 2 (row views 1.6) us per stage of
+// 16 i and its drain; 1.2 ps per value are the exponent pass.
+//   And not below I = 64 and 2 K I M = 4e7, where the digits gain 22 us at most and a
+// value keeps fewer bits there.
+constexpr double kDigit64MinTtm = 4e7;
 constexpr int kDigit64MinTtmI = 64;
+inline double ceil_div(double a, double b) { return std::ceil(a / b); }
+double ttm_pipe_us(double M, double I, double K, double sms) {
+  const double per = ceil_div(K, ceil_div(K, 32.0));            // outputs per tile (simt.cu)
+  const double kt = per <= 8 ? 8 : per <= 16 ? 16 : per <= 24 ? 24 : 32;
+  const double blocks = ceil_div(M, 128.0) * ceil_div(K, kt);
+  return 30.0 + (kt == 8 ? 0.31 : kt == 16 ? 0.57 : 1.08) * I * ceil_div(blocks, sms);
+}
+double ttm_digit_us(double M, double I, double K, double sms, bool col) {
+  const double items = ceil_div(ceil_div(M, MT) * ceil_div(K, NT), sms), st = ceil_div(I, BK);
+  const double k = std::min(K, (double)NT);
+  return 62.0 + items * (col ? 2.0 * st + 3.0 + 0.1 * k : 1.6 * st + 4.0 + 0.04 * k) + 1.2e-6 * I * M;
+}
 // Modes below 64 (gram_small.cu otherwise, ~I^2 / 2 FP64 instructions per 32 k;
 // here ~0.6 ns a k whatever I, one padded tile): K (I^2 - 565) >= 6.5e7.  Whole calls
 // there and here: I = 28, K = 4e5 342 and 332 us (2e5 197 and 220); I = 40, 5e4 122 and
@@ -1013,9 +1037,15 @@ __global__ void __launch_bounds__(256) k_digit64_prep(const double* __restrict__
 
 int ttm_d64_supported(int64_t L, int64_t I, int64_t Rt, int64_t K) {
   return I >= 1 && I <= 65536 && K >= 1 && K <= 65536 && L >= 1 && Rt >= 1 &&
-         L * I < ((int64_t)1 << 31) &&
-         (I >= kDigit64MinTtmI ||
-          2.0 * (double)K * (double)I * (double)L * (double)Rt >= kDigit64MinTtm);
+         L * I < ((int64_t)1 << 31);
+}
+
+int ttm_d64_chosen(int64_t L, int64_t I, int64_t Rt, int64_t K, int num_sms) {
+  if (!ttm_d64_supported(L, I, Rt, K)) return 0;
+  const double M = (double)L * (double)Rt;
+  if (I < kDigit64MinTtmI && 2.0 * (double)K * (double)I * M < kDigit64MinTtm) return 0;
+  return ttm_digit_us(M, (double)I, (double)K, num_sms, L == 1) <
+         ttm_pipe_us(M, (double)I, (double)K, num_sms);
 }
 
 namespace {

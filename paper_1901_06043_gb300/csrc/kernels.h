@@ -57,7 +57,7 @@ cudaError_t launch_rowmax_slab(const float* y, int64_t L, int64_t I, int64_t Rt,
                                unsigned* rowmax_bits, cudaStream_t st);
 
 // ---- FP64 Gram and TTM on exact seven-digit tensor-core products
-// (digit64.cu).  plan.nctas == 0 / supported == 0 when the work is too small
+// (digit64.cu).  plan.nctas == 0 / chosen == 0 when the work is too small
 // (or I > 8192 for the Gram).  scratch: plan.scratch_bytes / ttm_d64_scratch_bytes,
 // holding two verdict words (*_verdict): [0] nonzero when an operand holds NaN, Inf or a
 // row below 2^-958, or (err NULL) the operator of a TTM a zero beside other values in a
@@ -70,6 +70,7 @@ cudaError_t launch_gram_d64(const void* y, tucker_dtype dt, int64_t L, int64_t I
                             const GramPlan& p, int num_sms, void* scratch, unsigned* err, double* S,
                             cudaStream_t st);
 int ttm_d64_supported(int64_t L, int64_t I, int64_t Rt, int64_t K);
+int ttm_d64_chosen(int64_t L, int64_t I, int64_t Rt, int64_t K, int num_sms);
 size_t ttm_d64_scratch_bytes(int64_t L, int64_t I, int64_t Rt, int64_t K);
 const unsigned* ttm_d64_verdict(int64_t L, int64_t I, int64_t Rt, int64_t K, const void* scratch);
 cudaError_t launch_ttm_d64(const void* y, tucker_dtype ydt, int64_t L, int64_t I, int64_t Rt,

@@ -78,8 +78,8 @@ def test_fp64_gram_on_digits(ctx, dims, mode, shift, dtype, spread):
     assert (np.abs(got - want) <= bound).all()
 
 
-TTMS = [  # dims, mode, K, shift
-    ((64, 129), 0, 1, 0), ((65, 128), 0, 64, 1), ((200, 401), 0, 65, 0), ((128, 127), 0, 28, 0),
+TTMS = [  # dims, mode, K, shift (the first is too small and stays on the FP64 pipe)
+    ((64, 129), 0, 1, 0), ((300, 129), 0, 1, 0), ((65, 128), 0, 64, 1), ((200, 401), 0, 65, 0), ((128, 127), 0, 28, 0),
     ((145, 300), 0, 33, 0), ((33, 64, 12), 1, 64, 0), ((4, 130, 70), 1, 129, 0),
     ((8, 130, 70), 1, 20, 1), ((7, 100, 31), 1, 17, 0), ((130, 16, 200), 1, 65, 0),
     ((3, 17, 33, 70), 2, 200, 0), ((40, 48, 64), 2, 54, 0), ((26, 9000), 0, 100, 0)]
@@ -192,6 +192,26 @@ def test_the_fp64_pipe_on_request(dims, mode):
     with pytest.raises(tucker.TuckerError):
         c.set_option(tucker.OPT_FP64_PIPE, 2)
     c.close()
+
+
+@pytest.mark.parametrize("dims,mode,K,digits", [((64, 1500), 0, 4, False), ((96, 6000), 0, 4, False),
+                                                ((10, 64, 150), 1, 16, False), ((16, 30000), 0, 64, False),
+                                                ((64, 1500), 0, 28, True), ((10, 64, 150), 1, 28, True),
+                                                ((200, 24000), 0, 4, True), ((16, 100000), 0, 28, True)])
+def test_ttm_takes_the_faster_kernel(ctx, dims, mode, K, digits):
+    """The FP64 pipe's kernel (one launch) or the digits (three), by the work of both."""
+    import torch
+    from paper_1901_06043_gb300 import tucker
+    x = torch.randn(int(np.prod(dims)), device="cuda", dtype=torch.float64)
+    A = torch.randn(K, dims[mode], device="cuda", dtype=torch.float64)
+    n0 = tucker.kernel_launches()
+    z = ctx.ttm(x, dims, mode, A, prec="fp64")
+    assert tucker.kernel_launches() - n0 == (3 if digits else 1)
+    X = x.cpu().numpy().reshape(dims, order="F")
+    want = np.tensordot(A.cpu().numpy(), X, (1, mode))
+    got = np.moveaxis(z.cpu().numpy().reshape([K if k == mode else d for k, d in enumerate(dims)],
+                                              order="F"), mode, 0)
+    assert np.abs(got - want).max() <= 1e-14 * dims[mode] * np.abs(want).max()
 
 
 def test_batched_tensors_with_tiny_slices(ctx):
