@@ -195,7 +195,7 @@ def test_the_fp64_pipe_on_request(dims, mode):
 
 
 @pytest.mark.parametrize("dims,mode,K,digits", [((64, 1500), 0, 4, False), ((96, 6000), 0, 4, False),
-                                                ((10, 64, 150), 1, 16, False), ((16, 30000), 0, 64, False),
+                                                ((10, 64, 150), 1, 16, False), ((16, 24000), 0, 64, False),
                                                 ((64, 1500), 0, 28, True), ((10, 64, 150), 1, 28, True),
                                                 ((200, 24000), 0, 4, True), ((16, 100000), 0, 28, True)])
 def test_ttm_takes_the_faster_kernel(ctx, dims, mode, K, digits):
