@@ -177,10 +177,11 @@ const char* tucker_last_error(const tucker_ctx* ctx);
  *                          (0, the default: the device's free memory plus
  *                          what the default memory pool holds unused).
  *                          tucker_sthosvd predicts its workspace from the
- *                          mode sizes before it starts (the Gram and
- *                          eigenvector matrices, the first Gram's split-K
- *                          scratch, the first TTM output at rank 1) and, once
- *                          each rank is cut, the TTM output; a prediction
+ *                          mode sizes before it starts (the largest Gram and
+ *                          eigensolver workspace, the first Gram's split-K
+ *                          scratch, the first TTM's output and scratch at rank
+ *                          1) and, once each rank is cut, the TTM's output and
+ *                          scratch; a prediction
  *                          above the figure returns TUCKER_ERR_OOM before
  *                          that step launches or allocates anything.
  *   TUCKER_OPT_GRAM_DIGITS digits per value of the exact-digit Gram (MIXED):

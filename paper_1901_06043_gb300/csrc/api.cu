@@ -579,6 +579,12 @@ tucker_status do_gram(tucker_ctx* c, const void* y, tucker_dtype dt, const SlabV
   return gram_once(c, y, dt, v, prec, S, kernel_used, maxabs, check, rowmax, ndig, kern, best);
 }
 
+// Scratch of the FP64 Gram on digits (0 where it is not taken).  The FP64 pipe may follow
+// it (values out of the digits' range), after it has given its scratch back.
+size_t digit_gram64_bytes(const tucker_ctx* c, const SlabView& v) {
+  return c->fp64_pipe ? 0 : plan_gram_d64(v.L, v.I, v.Rt, c->num_sms).scratch_bytes;
+}
+
 // Device bytes of the split-K scratch do_gram allocates for a view.
 size_t gram_scratch_bytes(const tucker_ctx* c, tucker_prec prec, tucker_dtype dt,
                           const SlabView& v) {
@@ -587,16 +593,13 @@ size_t gram_scratch_bytes(const tucker_ctx* c, tucker_prec prec, tucker_dtype dt
   if (kern == 2) return plan_gram_tc(v.L, v.I, v.Rt, c->num_sms).scratch_bytes;
   if (kern == 3)
     return std::max(plan_gram_small(v.L, v.I, v.Rt, c->num_sms, v.L0).scratch_bytes,
-                    plan_gram_d64(v.L, v.I, v.Rt, c->num_sms).scratch_bytes);
+                    digit_gram64_bytes(c, v));
   if (kern == 1 && dt == TUCKER_F32) {
     const GramPlan pc = plan_gram_f32(v.L, v.I, v.Rt, c->num_sms, v.L0);
     if (pc.ntiles > 0) return pc.scratch_bytes;
   }
-  if (kern == 0) {
-    const GramPlan pd = plan_gram_d64(v.L, v.I, v.Rt, c->num_sms);
-    if (pd.nctas > 0) return pd.scratch_bytes;
-  }
-  return plan_gram_simt(v.L, v.I, v.Rt, c->num_sms, v.L0).scratch_bytes;
+  const size_t pipe = plan_gram_simt(v.L, v.I, v.Rt, c->num_sms, v.L0).scratch_bytes;
+  return kern == 0 ? std::max(pipe, digit_gram64_bytes(c, v)) : pipe;
 }
 
 // Bytes a call may still allocate: with TUCKER_OPT_MEM_LIMIT set, that
@@ -673,6 +676,19 @@ bool use_tridiag(const tucker_ctx* c, int n) {
   return n >= 1 && n <= 4096;
 }
 
+// Workspace of do_eig_tri for an n x n matrix, without the R vectors': exchange words,
+// the copy that is reduced, the reflectors, d, e, tau and the T factors.
+size_t eig_tri_bytes(int n) {
+  return sizeof(double) * (eig_xch_doubles(n) + 2 * (size_t)n * n + 3 * (size_t)n + eig_wy_doubles(n)) +
+         sizeof(EigProblem) + 16;
+}
+
+// Device bytes the truncated eigensolve of an n x n Gram takes beside it, before the rank
+// (and so the vectors' share) is known.
+size_t eig_work_bytes(const tucker_ctx* c, int n) {
+  return use_tridiag(c, n) ? eig_tri_bytes(n) : sizeof(double) * (size_t)n * n + jacobi_work_bytes(n);
+}
+
 // Z^T Z of one problem into P.gram, for pass 0 or 1 of its Cholesky QR: the Gram of
 // the column-major view of Z (L = 1, I = R, Rt = n).  Pass 1 is wanted only where
 // pass 0 has set info[1] and not failed.  Up to 63 vectors the kernels look at the
@@ -710,9 +726,8 @@ tucker_status do_eig_tri(tucker_ctx* c, const double* S, int n, double thr, int 
   const size_t nn = (size_t)n * n;
   const size_t nwy = eig_wy_doubles(n);
   const size_t nxch = eig_xch_doubles(n);
-  const size_t ndbl = nxch + 2 * nn + 3 * (size_t)n + nwy;
   DevBuf work;
-  TK_TRY(dev_alloc(c, work, sizeof(double) * ndbl + sizeof(EigProblem) + 16));
+  TK_TRY(dev_alloc(c, work, eig_tri_bytes(n)));
   EigProblem h{};
   h.xch = work.as<double>();
   h.A = h.xch + nxch;
@@ -855,6 +870,17 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
   TK_CUDA(c, launch_ttm_simt(y, ydt, prec == TUCKER_PREC_FP64, v.L, v.I, v.Rt, A, K, lda, arow,
                              a32.as<float>(), z, zdt, c->stream, zt));
   return TUCKER_OK;
+}
+
+// Device bytes of the scratch do_ttm allocates for a view and K outputs.
+size_t ttm_scratch_bytes(const tucker_ctx* c, tucker_prec prec, const SlabView& v, int64_t K) {
+  if (prec == TUCKER_PREC_FP64)
+    return !c->fp64_pipe && ttm_d64_chosen(v.L, v.I, v.Rt, K, c->num_sms)
+               ? ttm_d64_scratch_bytes(v.L, v.I, v.Rt, K) : 0;
+  size_t b = sizeof(float) * (size_t)K * v.I;
+  if (ttm_tc_supported(v.L, v.I, v.Rt, K)) b = std::max(b, ttm_tc_scratch_bytes(v.I, K));
+  if (ttm_tc_row_supported(v.L, v.I, v.Rt, K)) b = std::max(b, ttm_tc_row_scratch_bytes(K));
+  return b;
 }
 
 void order_search(int N, const int64_t* R, const int64_t* K, int objective, int* out) {
@@ -1135,6 +1161,28 @@ struct StreamedMode0 {
   float ms_norm = 0.f, ms_gram0 = 0.f;
 };
 
+// What an ST-HOSVD holds in every mode: the Gram of the largest mode and the largest
+// eigensolve's workspace.
+static double fixed_bytes(const tucker_ctx* c, int ndim, const int64_t* dims) {
+  double imax = 0.0, eig = 0.0;
+  for (int k = 0; k < ndim; ++k) {
+    imax = std::max(imax, (double)dims[k]);
+    eig = std::max(eig, (double)eig_work_bytes(c, (int)dims[k]));
+  }
+  return 8.0 * imax * imax + eig;
+}
+
+// What its first mode needs at least: that, the Gram's split-K scratch, and the TTM's
+// output and scratch at rank 1.
+static double first_mode_bytes(const tucker_ctx* c, tucker_prec prec, tucker_dtype dt, int ndim,
+                               const int64_t* dims, const int* order) {
+  const tucker_dtype wdt = (prec == TUCKER_PREC_FP64) ? TUCKER_F64 : dt;
+  const SlabView v0 = slab_view(ndim, dims, order[0]);
+  return fixed_bytes(c, ndim, dims) + (double)gram_scratch_bytes(c, prec, dt, v0) +
+         (double)dtype_size(wdt) * (double)(numel(ndim, dims) / dims[order[0]]) +
+         (double)ttm_scratch_bytes(c, prec, v0, 1);
+}
+
 // Algorithm 1 on the device tensor x; pre != null: the norm (and maybe the
 // first Gram) come from a streamed input (tucker_sthosvd_host).
 static tucker_status sthosvd_impl(tucker_ctx* c, const void* x, tucker_dtype dt, int ndim,
@@ -1145,16 +1193,9 @@ static tucker_status sthosvd_impl(tucker_ctx* c, const void* x, tucker_dtype dt,
   for (int k = 0; k < ndim; ++k) imax = std::max(imax, dims[k]);
 
   const tucker_dtype wdt = (prec == TUCKER_PREC_FP64) ? TUCKER_F64 : dt;
-  // workspace the first mode needs at least (nothing is launched or
-  // allocated when it does not fit): the Gram and eigenvector matrices,
-  // the first Gram's split-K scratch and its TTM output at rank 1
-  const double ws_fixed = 16.0 * (double)imax * (double)imax;
-  {
-    const SlabView v0 = slab_view(ndim, dims, order[0]);
-    const double need0 = ws_fixed + (double)gram_scratch_bytes(c, prec, dt, v0) +
-                         (double)dtype_size(wdt) * (double)(numel(ndim, dims) / dims[order[0]]);
-    TK_TRY(predict_oom(c, need0, 0.0, "the first mode"));
-  }
+  // (nothing is launched or allocated when the first mode does not fit)
+  const double ws_fixed = fixed_bytes(c, ndim, dims);
+  TK_TRY(predict_oom(c, first_mode_bytes(c, prec, dt, ndim, dims, order), 0.0, "the first mode"));
 
   tucker_result* r = new tucker_result();
   memset(r, 0, sizeof(*r));
@@ -1210,7 +1251,6 @@ static tucker_status sthosvd_impl(tucker_ctx* c, const void* x, tucker_dtype dt,
 
   DevBuf S, V, ycur;
   TK_TRY(dev_alloc(c, S, sizeof(double) * imax * imax));
-  TK_TRY(dev_alloc(c, V, sizeof(double) * imax * imax));
   const void* y = x;
   tucker_dtype ydt = dt;
   int64_t cur[TUCKER_MAX_MODES];
@@ -1286,6 +1326,7 @@ static tucker_status sthosvd_impl(tucker_ctx* c, const void* x, tucker_dtype dt,
       r->eig_kernel[n] = 1;
     }
     if (!have) {
+      if (!V.p) TK_TRY(dev_alloc(c, V, sizeof(double) * imax * imax));
       es = do_eig(c, Sn, I, w.as<double>(), V.as<double>(), &sweeps);
       if (es != TUCKER_OK && es != TUCKER_ERR_EIG_NOCONV) return es;
       TK_TRY(do_cut(c, w.as<double>(), I, thr, fixed_R, &R, &disc));
@@ -1310,8 +1351,8 @@ static tucker_status sthosvd_impl(tucker_ctx* c, const void* x, tucker_dtype dt,
     {
       const double held = ws_fixed + held_factors +
                           (s > 0 ? (double)dtype_size(ydt) * (double)numel(ndim, cur) : 0.0);
-      TK_TRY(predict_oom(c, (double)dtype_size(wdt) * (double)numel(ndim, nd), held,
-                         "a TTM"));
+      TK_TRY(predict_oom(c, (double)dtype_size(wdt) * (double)numel(ndim, nd) +
+                                (double)ttm_scratch_bytes(c, prec, v, R), held, "a TTM"));
     }
     DevBuf z;
     TK_TRY(dev_alloc(c, z, dtype_size(wdt) * numel(ndim, nd)));
@@ -1384,15 +1425,12 @@ tucker_status tucker_sthosvd_host(tucker_ctx* c, const void* x_host, tucker_dtyp
   const int64_t nx = numel(ndim, dims);
   const size_t esz = dtype_size(dt);
   const int64_t I0 = dims[0];
-  int64_t imax = 0;
-  for (int k = 0; k < ndim; ++k) imax = std::max(imax, dims[k]);
-  // the device copy, then the first mode's workspace (as tucker_sthosvd)
+  // the device copy and (mode 0 first) the Grams of its pieces, then the first mode's
+  // workspace (as tucker_sthosvd)
   {
-    const tucker_dtype wdt = (prec == TUCKER_PREC_FP64) ? TUCKER_F64 : dt;
-    const SlabView v0 = slab_view(ndim, dims, order[0]);
-    const double need = (double)esz * (double)nx + 16.0 * (double)imax * (double)imax * 2.0 +
-                        (double)gram_scratch_bytes(c, prec, dt, v0) +
-                        (double)dtype_size(wdt) * (double)(nx / dims[order[0]]);
+    const double need = (double)esz * (double)nx +
+                        (order[0] == 0 ? 16.0 * (double)I0 * (double)I0 : 0.0) +
+                        first_mode_bytes(c, prec, dt, ndim, dims, order);
     TK_TRY(predict_oom(c, need, 0.0, "the host input's device copy"));
   }
   DevBuf xd;

@@ -112,6 +112,65 @@ def test_oom_predicted_before_a_ttm(ctx):
     ctx.set_option(tucker.OPT_MEM_LIMIT, 0)
 
 
+class PoolHigh:
+    """High-water mark of the device's default memory pool, where the library allocates."""
+    HIGH, CURRENT = 8, 7                 # CU_MEMPOOL_ATTR_USED_MEM_HIGH, _USED_MEM_CURRENT
+
+    def __init__(self):
+        import ctypes
+        self.ct, self.cu = ctypes, ctypes.CDLL("libcuda.so.1")
+        dev, self.pool = ctypes.c_int(), ctypes.c_void_p()
+        assert self.cu.cuDeviceGet(ctypes.byref(dev), torch.cuda.current_device()) == 0
+        assert self.cu.cuDeviceGetDefaultMemPool(ctypes.byref(self.pool), dev) == 0
+
+    def _attr(self, f, key, value=0):
+        v = self.ct.c_uint64(value)
+        assert f(self.pool, key, self.ct.byref(v)) == 0
+        return v.value
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        self._attr(self.cu.cuMemPoolSetAttribute, self.HIGH, 0)
+        self.base = self._attr(self.cu.cuMemPoolGetAttribute, self.CURRENT)
+        return self
+
+    def __exit__(self, *a):
+        torch.cuda.synchronize()
+        self.held = self._attr(self.cu.cuMemPoolGetAttribute, self.HIGH) - self.base
+
+
+# large modes (the eigensolver's workspace), a digit TTM with many fibres (its exponents),
+# a small mode with a long Gram (the digits' and the FP64 pipe's scratch)
+@pytest.mark.parametrize("dims,ranks", [((64, 64, 2000), (8, 8, 4)), ((1500, 30, 20), (9, 8, 7)),
+                                        ((64, 640, 500), (1, 1, 1)), ((40, 100, 900), (20, 2, 2))])
+def test_prediction_covers_what_a_call_holds(ctx, dims, ranks):
+    """The smallest limit under which a call runs is at least what it held at once, less
+    what depends on the rank: the vectors of the eigensolve, 6.25 n R + R^2 doubles."""
+    from paper_1901_06043_gb300 import tucker
+    x = torch.randn(int(np.prod(dims)), device="cuda", dtype=torch.float64)
+
+    def runs(limit):
+        ctx.set_option(tucker.OPT_MEM_LIMIT, limit)
+        try:
+            ctx.sthosvd(x, dims, ranks=ranks, prec="fp64").close()
+            return True
+        except tucker.TuckerError as e:
+            assert e.name == "OOM" and "predicted" in str(e), str(e)
+            return False
+
+    lo, hi = 1000.0, 8e9
+    assert not runs(lo) and runs(hi)
+    while hi - lo > 100.0:
+        mid = 0.5 * (lo + hi)
+        lo, hi = (lo, mid) if runs(mid) else (mid, hi)
+    with PoolHigh() as pool:
+        assert runs(hi)
+    ctx.set_option(tucker.OPT_MEM_LIMIT, 0)
+    vectors = 8 * max(6.25 * n * r + r * r for n, r in zip(dims, ranks))
+    # (allocations are rounded up to 512 bytes, some twenty at once)
+    assert pool.held <= hi + vectors + 32 * 512, (pool.held, hi)
+
+
 def test_rcp64_within_one_ulp():
     from paper_1901_06043_gb300 import tucker
     rng = np.random.default_rng(5)
