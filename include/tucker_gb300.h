@@ -233,6 +233,15 @@ int64_t tucker_autotune_entries(void);
 tucker_status tucker_selftest_rcp64(const double* x_dev, double* y_dev, int64_t n,
                                     void* stream);
 
+/* Diagnostics, as above: the FP64 square root of the Householder reduction (an
+ * FP32 estimate of 1/sqrt, one Goldschmidt step and a correction; within one
+ * ulp for x in [2^-1000, 2^1000]), and the conversion to FP32 by integer
+ * operations (to nearest, ties to even, as a cast). */
+tucker_status tucker_selftest_sqrt64(const double* x_dev, double* y_dev, int64_t n,
+                                     void* stream);
+tucker_status tucker_selftest_f64_to_f32(const double* x_dev, float* y_dev, int64_t n,
+                                         void* stream);
+
 /* ST-HOSVD, Algorithm 1 (Section 3.3).
  *   x_dev      input tensor (dtype, dims), read only.
  *   eps        relative accuracy; R_n = min{R in 1..I_n : sum_{i>=R} lambda_i

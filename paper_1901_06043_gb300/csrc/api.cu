@@ -2012,14 +2012,30 @@ long double sthosvd_order_cost(int N, const int64_t* I, const int64_t* R, const 
 
 }  // namespace
 
-tucker_status tucker_selftest_rcp64(const double* x_dev, double* y_dev, int64_t n,
-                                   void* stream) {
-  if (!x_dev || !y_dev || n < 0) return TUCKER_ERR_INVALID;
-  if (launch_rcp64_probe(x_dev, y_dev, n, (cudaStream_t)stream) != cudaSuccess) {
+static tucker_status probe_status(cudaError_t e, void* stream) {
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return TUCKER_ERR_CUDA;
   }
   return cudaStreamSynchronize((cudaStream_t)stream) == cudaSuccess ? TUCKER_OK : TUCKER_ERR_CUDA;
+}
+
+tucker_status tucker_selftest_rcp64(const double* x_dev, double* y_dev, int64_t n,
+                                   void* stream) {
+  if (!x_dev || !y_dev || n < 0) return TUCKER_ERR_INVALID;
+  return probe_status(launch_rcp64_probe(x_dev, y_dev, n, (cudaStream_t)stream), stream);
+}
+
+tucker_status tucker_selftest_sqrt64(const double* x_dev, double* y_dev, int64_t n,
+                                     void* stream) {
+  if (!x_dev || !y_dev || n < 0) return TUCKER_ERR_INVALID;
+  return probe_status(launch_sqrt64_probe(x_dev, y_dev, n, (cudaStream_t)stream), stream);
+}
+
+tucker_status tucker_selftest_f64_to_f32(const double* x_dev, float* y_dev, int64_t n,
+                                         void* stream) {
+  if (!x_dev || !y_dev || n < 0) return TUCKER_ERR_INVALID;
+  return probe_status(launch_f64_to_f32_probe(x_dev, y_dev, n, (cudaStream_t)stream), stream);
 }
 
 tucker_status tucker_sthosvd_order(int ndim, const int64_t* dims, const int64_t* ranks,

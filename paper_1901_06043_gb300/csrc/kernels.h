@@ -187,8 +187,11 @@ inline size_t eig_xch_doubles(int n) { return 8 * (size_t)n + 2; }
 cudaError_t launch_tridiag(const EigProblem* probs_dev, EigProblem* probs_host, int count,
                            const double* S, unsigned* err, cudaStream_t st,
                            unsigned long long poll_limit);
-// y[i] = the tridiagonal solver's FP64 reciprocal of x[i] (diagnostics)
+// y[i] = the tridiagonal solver's FP64 reciprocal or square root of x[i], or x[i] in FP32
+// by f64_to_f32 (diagnostics)
 cudaError_t launch_rcp64_probe(const double* x, double* y, int64_t n, cudaStream_t st);
+cudaError_t launch_sqrt64_probe(const double* x, double* y, int64_t n, cudaStream_t st);
+cudaError_t launch_f64_to_f32_probe(const double* x, float* y, int64_t n, cudaStream_t st);
 // total_eigs: the sum of n over the problems (sets the lanes per eigenvalue)
 cudaError_t launch_bisect(const EigProblem* probs_dev, int count, int nmax, int total_eigs,
                           int num_sms, cudaStream_t st);

@@ -675,9 +675,14 @@ __device__ __forceinline__ double hash_unit(uint32_t i, uint32_t j) {
   return __hiloint2double((int)(0x3ff00000u | (h & 0x800fffffu)), (int)(h * 0x9E3779B1u));
 }
 
-__global__ void k_rcp64_probe(const double* x, double* y, int64_t n) {
+// OP 0: rcp64, 1: sqrt64, 2: f64_to_f32
+template <int OP, typename TOut>
+__global__ void k_scalar_probe(const double* x, TOut* y, int64_t n) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = rcp64(x[i]);
+  if (i >= n) return;
+  if constexpr (OP == 0) y[i] = rcp64(x[i]);
+  else if constexpr (OP == 1) y[i] = sqrt64(x[i]);
+  else y[i] = f64_to_f32(x[i]);
 }
 
 __global__ void __launch_bounds__(32) k_invit(const EigProblem* probs, int nprob, int total) {
@@ -1496,10 +1501,20 @@ cudaError_t launch_backtransform(const EigProblem* probs_dev, int count, int tot
   return cudaGetLastError();
 }
 
-cudaError_t launch_rcp64_probe(const double* x, double* y, int64_t n, cudaStream_t st) {
-  if (n > 0) k_rcp64_probe<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, y, n);
+template <int OP, typename TOut>
+static cudaError_t scalar_probe(const double* x, TOut* y, int64_t n, cudaStream_t st) {
+  if (n > 0) k_scalar_probe<OP, TOut><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, y, n);
   count_launches(n > 0 ? 1 : 0);
   return cudaGetLastError();
+}
+cudaError_t launch_rcp64_probe(const double* x, double* y, int64_t n, cudaStream_t st) {
+  return scalar_probe<0>(x, y, n, st);
+}
+cudaError_t launch_sqrt64_probe(const double* x, double* y, int64_t n, cudaStream_t st) {
+  return scalar_probe<1>(x, y, n, st);
+}
+cudaError_t launch_f64_to_f32_probe(const double* x, float* y, int64_t n, cudaStream_t st) {
+  return scalar_probe<2>(x, y, n, st);
 }
 
 }  // namespace tk

@@ -32,7 +32,8 @@ EXPORTS = ["tucker_create", "tucker_destroy", "tucker_last_error", "tucker_set_o
            "tucker_eig", "tucker_eig_trunc", "tucker_rank_cut", "tucker_ttm",
            "tucker_kernel_launches", "tucker_gram_noalloc", "tucker_hosvd",
            "tucker_sthosvd_order", "tucker_slice_stats", "tucker_slice_transform",
-           "tucker_preprocess", "tucker_selftest_rcp64", "tucker_autotune_entries",
+           "tucker_preprocess", "tucker_selftest_rcp64", "tucker_selftest_sqrt64",
+           "tucker_selftest_f64_to_f32", "tucker_autotune_entries",
            "tucker_sthosvd_host"]
 STATS = ("mean", "std", "max", "min", "norm1", "norm2")
 PRE_METHOD = {"standardize": 0, "max": 1}
@@ -120,7 +121,8 @@ def lib():
                                    ctypes.POINTER(ctypes.POINTER(CResult))]
         L.tucker_sthosvd_host.argtypes = L.tucker_sthosvd.argtypes
         L.tucker_sthosvd_order.argtypes = [c_int, i64p, i64p, ctypes.POINTER(c_int)]
-        L.tucker_selftest_rcp64.argtypes = [vp, vp, ctypes.c_int64, vp]
+        for name in ("rcp64", "sqrt64", "f64_to_f32"):
+            getattr(L, "tucker_selftest_" + name).argtypes = [vp, vp, ctypes.c_int64, vp]
         L.tucker_slice_stats.argtypes = [vp, vp, c_int, c_int, i64p, c_int, vp]
         L.tucker_slice_transform.argtypes = [vp, vp, c_int, c_int, i64p, c_int, vp, vp, c_int, vp]
         L.tucker_preprocess.argtypes = [vp, vp, c_int, c_int, i64p, c_int, c_int, vp, vp, vp]
@@ -551,19 +553,34 @@ def sthosvd_order(dims, ranks):
     return tuple(out[k] for k in range(N))
 
 
-def selftest_rcp64(x):
-    """The tridiagonal eigensolver's FP64 reciprocal of every entry of the
-    FP64 device tensor x (diagnostics)."""
+def _selftest(name, x, out_dtype):
     import torch
     _check_dev(x, "x")
     if x.dtype != torch.float64:
         raise ValueError("x must be float64")
-    y = torch.empty_like(x)
-    st = lib().tucker_selftest_rcp64(ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(y.data_ptr()),
-                                     x.numel(), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    y = torch.empty_like(x, dtype=out_dtype)
+    st = getattr(lib(), name)(ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(y.data_ptr()),
+                              x.numel(), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
     if st != 0:
-        raise TuckerError(st, "tucker_selftest_rcp64")
+        raise TuckerError(st, name)
     return y
+
+
+def selftest_rcp64(x):
+    """The tridiagonal eigensolver's FP64 reciprocal of every entry of the
+    FP64 device tensor x (diagnostics)."""
+    return _selftest("tucker_selftest_rcp64", x, x.dtype)
+
+
+def selftest_sqrt64(x):
+    """Its FP64 square root (x in [2^-1000, 2^1000])."""
+    return _selftest("tucker_selftest_sqrt64", x, x.dtype)
+
+
+def selftest_f64_to_f32(x):
+    """The kernels' conversion of FP64 values to FP32."""
+    import torch
+    return _selftest("tucker_selftest_f64_to_f32", x, torch.float32)
 
 
 def autotune_entries():

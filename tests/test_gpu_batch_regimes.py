@@ -1,7 +1,8 @@
 """The batched truncated eigensolve where its launches differ most: as many tensors as
 SMs or more, so that every team is one CTA (rows in shared memory up to 123, else in
 global memory; one lane per eigenvalue in the bisection), with small and large modes in
-one launch.  Ranks and eigenvalues against the same tensor by itself."""
+one launch; fewer tensors, with a team behind a barrier (above 640 rows) beside teams that
+exchange words.  Ranks and eigenvalues against the same tensor by itself."""
 import numpy as np
 import pytest
 
@@ -52,3 +53,34 @@ def test_teams_of_one_with_small_and_large_modes(ctx):
     rest = [3, 100, 123, 124, 300]
     sizes = [2350, 123, 700] + [rest[k % 5] for k in range(sms() - 2)]
     check(ctx, sizes, 500)
+
+
+def test_a_team_behind_a_barrier_beside_teams_with_words(ctx):
+    """100 tensors: 1000 rows in a team of some 30 CTAs, 640 and 641 beside it, the small
+    ones mostly in teams of one."""
+    sizes = [1000, 640, 641, 124, 123] + [20 + k for k in range(95)]
+    check(ctx, sizes, 900)
+
+
+def test_large_ranks_in_a_batch(ctx):
+    """More than 64 vectors (blocks of 32, the second pass chosen on the host) beside fewer;
+    well separated and clustered eigenvalues in one batch."""
+    rng = np.random.default_rng(11)
+    xs, dims = [], []
+    for n, clustered in ((150, False), (150, True), (90, True), (40, False)):
+        d = (n, 180, 2)
+        Q = np.linalg.qr(rng.standard_normal((n, n)))[0]
+        P = np.linalg.qr(rng.standard_normal((360, n)))[0]
+        s = np.linspace(2, 1, n)
+        if clustered:
+            s = s[(np.arange(n) // 5) * 5]
+        xs.append(torch.from_numpy(np.reshape((Q * s) @ P.T, -1, order="F").copy()).cuda())
+        dims.append(d)
+    many = ctx.sthosvd_batched(xs, dims, eps=0.1, prec="fp64")
+    for x, d, r in zip(xs, dims, many):
+        U = r.factors[0].cpu().numpy()
+        R = r.ranks[0]
+        assert U.shape == (d[0], R) and (d[0] < 90 or R > 64)
+        assert np.abs(U.T @ U - np.eye(R)).max() <= 1e-13 * d[0]
+        assert float((r.reconstruct() - x).norm()) <= 0.1 * float(x.norm())
+        r.close()

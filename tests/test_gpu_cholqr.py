@@ -72,13 +72,15 @@ def test_rank_cut_sums_in_order(ctx, n):
         assert (R, d) == (want, tail[want])
 
 
-@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 16, 17, 31, 47, 64, 129, 153, 304, 305, 610])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 16, 17, 31, 47, 64, 129, 153, 304, 305, 610,
+                               640, 641, 1000])
 @pytest.mark.parametrize("kind", ["dense", "diagonal", "split", "tiny", "huge"])
 def test_eigenvalues_and_vectors_over_sizes(ctx, n, kind):
-    """Every width of the multisection (one to four warps per eigenvalue, down
-    to one lane in batches), the two-ended inverse iteration at odd and even
-    sizes, exact zeros on T's off-diagonal and matrices near the ends of the
-    exponent range."""
+    """The widths of the multisection that one matrix takes (four warps per eigenvalue to
+    16 lanes; narrower ones in test_gpu_batch_regimes.py), the two-ended inverse
+    iteration at odd and even sizes, both exchanges of the reduction (words up to 640
+    rows, a barrier above), exact zeros on T's off-diagonal and matrices near the ends of
+    the exponent range."""
     import torch
     rng = np.random.default_rng(n)
     S = rng.standard_normal((n, n)) * 10.0 ** rng.uniform(-3, 0, n)

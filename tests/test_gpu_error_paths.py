@@ -187,3 +187,41 @@ def test_rcp64_within_one_ulp():
     ulp = np.spacing(np.abs(want[fin]))
     err = np.abs(y[fin] - want[fin])
     assert np.all(err <= ulp), np.max(err / ulp)
+
+
+def test_sqrt64_within_one_ulp():
+    """Over the exponents of its range, odd and even, and squares of whole numbers."""
+    from paper_1901_06043_gb300 import tucker
+    rng = np.random.default_rng(6)
+    e = rng.integers(-1000, 1000, 200000)
+    x = np.ldexp(rng.uniform(1.0, 2.0, e.size), e)
+    x = np.concatenate([x, np.arange(1.0, 2000.0) ** 2, np.ldexp(1.0, np.arange(-1000, 1001)),
+                        np.nextafter(np.ldexp(1.0, np.arange(-999, 1001)), 0.0)])
+    y = tucker.selftest_sqrt64(torch.from_numpy(x).cuda()).cpu().numpy()
+    want = np.sqrt(x)
+    assert np.all(np.abs(y - want) <= np.spacing(want)), np.max(np.abs(y - want) / np.spacing(want))
+
+
+def test_f64_to_f32_rounds_as_a_cast():
+    """Ties to even and one bit on either side of them, the ends of FP32's normal range
+    and beyond, zeros, denormals, infinities and NaN."""
+    from paper_1901_06043_gb300 import tucker
+    rng = np.random.default_rng(7)
+    e = rng.integers(-160, 140, 200000)
+    x = np.ldexp(rng.uniform(1.0, 2.0, e.size), e)
+    m = rng.integers(1 << 23, 1 << 24, 20000).astype(np.float64)
+    m = np.concatenate([m, [2.0 ** 23, 2.0 ** 24 - 1]])
+    ties = np.concatenate([(m + 0.5 + d) * s for d in (-2.0 ** -29, 0.0, 2.0 ** -29)
+                           for s in 2.0 ** np.arange(-175, 106, 7)])
+    f = np.finfo(np.float32)
+    ends = np.array([0.0, float(f.tiny), float(f.max), 5e-324, 1e-310, 1e-45, 7e-46, 1e300, np.inf, np.nan])
+    ends = np.concatenate([ends, np.nextafter(ends, np.inf), np.nextafter(ends, 0.0),
+                           float(f.max) * (1 + 2.0 ** -25) * np.array([1 - 2.0 ** -50, 1.0, 1 + 2.0 ** -50])])
+    x = np.concatenate([x, ties, ends])
+    x = np.concatenate([x, -x])
+    y = tucker.selftest_f64_to_f32(torch.from_numpy(x).cuda()).cpu().numpy()
+    with np.errstate(all="ignore"):
+        want = x.astype(np.float32)
+    nan = np.isnan(want)
+    assert np.array_equal(np.isnan(y), nan)
+    assert np.array_equal(y[~nan].view(np.uint32), want[~nan].view(np.uint32))
