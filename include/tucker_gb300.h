@@ -76,7 +76,7 @@ typedef enum { TUCKER_F32 = 0, TUCKER_F64 = 1 } tucker_dtype;
  *            values of one row meet small values of the other.  TTMs with an
  *            operator that has zeros beside other values (selections,
  *            differences) therefore stay on the FP64 pipe, and
- *            TUCKER_OPT_FP64_PIPE keeps every step there.  An operand with
+ *            TUCKER_OPT_FP64_KERNEL keeps every step there.  An operand with
  *            NaN, Inf or a row below 2^-958 takes the FP64 pipe (in a batch,
  *            a row below 2^-958 counts in units of 2^-1013, and the
  *            operators are the factors).
@@ -200,12 +200,13 @@ const char* tucker_last_error(const tucker_ctx* ctx);
  *   TUCKER_OPT_HOST_CHUNK  bytes per piece in which tucker_sthosvd_host copies
  *                          its input (rounded to whole mode-0 columns, four at
  *                          a time); default 2^30, at least 1.
- *   TUCKER_OPT_FP64_PIPE   1: every Gram and TTM of precision FP64, and the
- *                          FP64 Grams of the others, multiplies and adds FP64
- *                          values on the FP64 pipe whatever its size (entries
- *                          to the rounding of FP64 sums; 3 to 30 times the
- *                          time of large steps).  0 (default): integer digits
- *                          from a size (see FP64). */
+ *   TUCKER_OPT_FP64_KERNEL the kernels of Gram and TTM in precision FP64, and of
+ *                          the FP64 Grams of the others: 0 (default) integer
+ *                          digits from a size (see FP64), 1 the FP64 pipe
+ *                          whatever the size (values multiplied and added in
+ *                          FP64: entries to the rounding of FP64 sums, 3 to
+ *                          30 times the time of large steps), 2 as 0, and
+ *                          digits for TTMs of every size. */
 #define TUCKER_OPT_TIMING 1
 #define TUCKER_OPT_MAX_SWEEPS 2
 #define TUCKER_OPT_JACOBI_TOL 3
@@ -215,7 +216,7 @@ const char* tucker_last_error(const tucker_ctx* ctx);
 #define TUCKER_OPT_GRAM_DIGITS 7
 #define TUCKER_OPT_AUTOTUNE 8
 #define TUCKER_OPT_HOST_CHUNK 9
-#define TUCKER_OPT_FP64_PIPE 10
+#define TUCKER_OPT_FP64_KERNEL 10
 tucker_status tucker_set_option(tucker_ctx* ctx, int key, double value);
 
 /* Diagnostics: number of device kernels this library has launched in the

@@ -55,7 +55,7 @@ struct tucker_ctx {
   unsigned long long barrier_polls = 1ull << 24;   // grid-barrier poll limit of the eigensolvers
   double mem_limit = 0.0;        // bytes assumed available to a call (0: ask the device)
   int gram_digits = 0;           // digits of the exact-digit Gram: 0 auto, 2 or 3
-  int fp64_pipe = 0;             // 1: no FP64 step on the integer digits (digit64.cu)
+  int fp64_kernel = 0;           // 0 by size, 1 FP64 pipe, 2 integer digits (digit64.cu) for every TTM
   int autotune = 0;              // 1: split-K of the Gram kernels chosen by timing
   double host_chunk = 1073741824.0;   // bytes per piece of tucker_sthosvd_host's copy
   std::string err;
@@ -458,7 +458,7 @@ tucker_status gram_once(tucker_ctx* c, const void* y, tucker_dtype dt, const Sla
     }
     return TUCKER_OK;
   }
-  if ((kern == 0 || kern == 3) && !c->fp64_pipe) {
+  if ((kern == 0 || kern == 3) && c->fp64_kernel != 1) {
     // FP64 products: seven exact digits on the tensor cores from the size
     // where they beat the FP64 pipe (digit64.cu); out of their range (NaN,
     // Inf, rows below 2^-958): the FP64 pipe
@@ -534,7 +534,7 @@ tucker_status do_gram(tucker_ctx* c, const void* y, tucker_dtype dt, const SlabV
     return gram_once(c, y, dt, v, prec, S, kernel_used, maxabs, check, rowmax, ndig, kern,
                      c->num_sms);
   const std::array<int64_t, 7> key{c->device, kern, v.L, v.I, v.Rt, (int64_t)dt,
-                                   kern == 5 ? ndig : (kern == 0 || kern == 3 ? c->fp64_pipe : 0)};
+                                   kern == 5 ? ndig : (kern == 0 || kern == 3 ? c->fp64_kernel == 1 : 0)};
   int best = 0;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -582,7 +582,7 @@ tucker_status do_gram(tucker_ctx* c, const void* y, tucker_dtype dt, const SlabV
 // Scratch of the FP64 Gram on digits (0 where it is not taken).  The FP64 pipe may follow
 // it (values out of the digits' range), after it has given its scratch back.
 size_t digit_gram64_bytes(const tucker_ctx* c, const SlabView& v) {
-  return c->fp64_pipe ? 0 : plan_gram_d64(v.L, v.I, v.Rt, c->num_sms).scratch_bytes;
+  return c->fp64_kernel == 1 ? 0 : plan_gram_d64(v.L, v.I, v.Rt, c->num_sms).scratch_bytes;
 }
 
 // Device bytes of the split-K scratch do_gram allocates for a view.
@@ -804,6 +804,12 @@ tucker_status do_cut(tucker_ctx* c, const double* w, int n, double thr, int fixe
   return sync(c);
 }
 
+// Whether an FP64 TTM with K outputs runs on integer digits.
+bool ttm_on_digits(const tucker_ctx* c, const SlabView& v, int64_t K) {
+  if (c->fp64_kernel == 2) return ttm_d64_supported(v.L, v.I, v.Rt, K);
+  return c->fp64_kernel == 0 && ttm_d64_chosen(v.L, v.I, v.Rt, K, c->num_sms);
+}
+
 // ymax: max|y| if the caller knows it (e.g. from the norm pass), else <= 0.
 // check = false: as do_gram, for the tensor-core TTM's error word (d_words[9]).
 // zt (column-mode views): Z written transposed, slab fastest (the new mode
@@ -851,9 +857,8 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
   }
   // FP64: seven exact digits on the tensor cores from the size where they
   // beat the FP64 pipe (digit64.cu); out of their range (NaN, Inf, rows below
-  // 2^-958): the FP64 pipe
-  if (prec == TUCKER_PREC_FP64 && !c->fp64_pipe &&
-      ttm_d64_chosen(v.L, v.I, v.Rt, K, c->num_sms)) {
+  // 2^-958) and for operators with zeros beside other values: the FP64 pipe
+  if (prec == TUCKER_PREC_FP64 && ttm_on_digits(c, v, K)) {
     DevBuf scratch;
     TK_TRY(dev_alloc(c, scratch, ttm_d64_scratch_bytes(v.L, v.I, v.Rt, K)));
     TK_CUDA(c, launch_ttm_d64(y, ydt, v.L, v.I, v.Rt, A, K, lda, arow, z, zdt, zt, scratch.p,
@@ -875,8 +880,7 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
 // Device bytes of the scratch do_ttm allocates for a view and K outputs.
 size_t ttm_scratch_bytes(const tucker_ctx* c, tucker_prec prec, const SlabView& v, int64_t K) {
   if (prec == TUCKER_PREC_FP64)
-    return !c->fp64_pipe && ttm_d64_chosen(v.L, v.I, v.Rt, K, c->num_sms)
-               ? ttm_d64_scratch_bytes(v.L, v.I, v.Rt, K) : 0;
+    return ttm_on_digits(c, v, K) ? ttm_d64_scratch_bytes(v.L, v.I, v.Rt, K) : 0;
   size_t b = sizeof(float) * (size_t)K * v.I;
   if (ttm_tc_supported(v.L, v.I, v.Rt, K)) b = std::max(b, ttm_tc_scratch_bytes(v.I, K));
   if (ttm_tc_row_supported(v.L, v.I, v.Rt, K)) b = std::max(b, ttm_tc_row_scratch_bytes(K));
@@ -994,9 +998,10 @@ tucker_status tucker_set_option(tucker_ctx* c, int key, double value) {
         return set_err(c, TUCKER_ERR_INVALID, "eigensolver must be 0 (auto), 1 or 2");
       c->eig_solver = (int)value;
       return TUCKER_OK;
-    case TUCKER_OPT_FP64_PIPE:
-      if (value != 0.0 && value != 1.0) return set_err(c, TUCKER_ERR_INVALID, "FP64 pipe must be 0 or 1");
-      c->fp64_pipe = (int)value;
+    case TUCKER_OPT_FP64_KERNEL:
+      if (value != 0.0 && value != 1.0 && value != 2.0)
+        return set_err(c, TUCKER_ERR_INVALID, "FP64 kernel must be 0 (by size), 1 or 2");
+      c->fp64_kernel = (int)value;
       return TUCKER_OK;
     case TUCKER_OPT_AUTOTUNE:
       if (value != 0.0 && value != 1.0) return set_err(c, TUCKER_ERR_INVALID, "autotune must be 0 or 1");

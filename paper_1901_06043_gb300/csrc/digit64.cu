@@ -32,7 +32,7 @@
 // |x_i|_1), where an FP64 sum is off by 2^-53 of each of its partial sums.
 // Against the rows' norms that is no more than an FP64 sum has; against the entry
 // itself it is more where the large values of one row meet small ones of the other
-// (a value 2^-40 of its row's largest keeps 15 bits).  Hence TUCKER_OPT_FP64_PIPE, and
+// (a value 2^-40 of its row's largest keeps 15 bits).  Hence TUCKER_OPT_FP64_KERNEL, and
 // a TTM whose operator has a zero beside other values in a row (it may be there to leave
 // out a fibre's large values: selections, differences) is computed on the FP64 pipe.
 //   NaN, Inf, or a row whose largest magnitude is below 2^-958 (its exponents

@@ -22,7 +22,8 @@ F32, F64 = 0, 1
 PREC = {"fp64": 0, "fp32": 1, "mixed": 2, "tensor": 3}
 OPT_TIMING, OPT_MAX_SWEEPS, OPT_JACOBI_TOL, OPT_EIG_SOLVER = 1, 2, 3, 4
 OPT_BARRIER_POLLS, OPT_MEM_LIMIT, OPT_GRAM_DIGITS, OPT_AUTOTUNE = 5, 6, 7, 8
-OPT_HOST_CHUNK, OPT_FP64_PIPE = 9, 10
+OPT_HOST_CHUNK, OPT_FP64_KERNEL = 9, 10
+FP64_KERNEL = {"auto": 0, "pipe": 1, "digits": 2}
 EIG_SOLVER = {"auto": 0, "jacobi": 1, "tridiag": 2}
 
 EXPORTS = ["tucker_create", "tucker_destroy", "tucker_last_error", "tucker_set_option",

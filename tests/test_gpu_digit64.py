@@ -16,8 +16,10 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture(scope="module")
 def ctx():
+    """Digits for TTMs of every size (small ones are faster on the FP64 pipe)."""
     from paper_1901_06043_gb300 import tucker
     c = tucker.Context()
+    c.set_option(tucker.OPT_FP64_KERNEL, tucker.FP64_KERNEL["digits"])
     yield c
     c.close()
 
@@ -78,8 +80,8 @@ def test_fp64_gram_on_digits(ctx, dims, mode, shift, dtype, spread):
     assert (np.abs(got - want) <= bound).all()
 
 
-TTMS = [  # dims, mode, K, shift (the first is too small and stays on the FP64 pipe)
-    ((64, 129), 0, 1, 0), ((300, 129), 0, 1, 0), ((65, 128), 0, 64, 1), ((200, 401), 0, 65, 0), ((128, 127), 0, 28, 0),
+TTMS = [  # dims, mode, K, shift
+    ((64, 129), 0, 1, 0), ((65, 128), 0, 64, 1), ((200, 401), 0, 65, 0), ((128, 127), 0, 28, 0),
     ((145, 300), 0, 33, 0), ((33, 64, 12), 1, 64, 0), ((4, 130, 70), 1, 129, 0),
     ((8, 130, 70), 1, 20, 1), ((7, 100, 31), 1, 17, 0), ((130, 16, 200), 1, 65, 0),
     ((3, 17, 33, 70), 2, 200, 0), ((40, 48, 64), 2, 54, 0), ((26, 9000), 0, 100, 0)]
@@ -169,12 +171,12 @@ def test_operators_with_zeros_keep_small_entries(ctx, what, arow):
 
 @pytest.mark.parametrize("dims,mode", [((96, 4000), 0), ((5, 96, 900), 1), ((40, 70000), 0)])
 def test_the_fp64_pipe_on_request(dims, mode):
-    """TUCKER_OPT_FP64_PIPE: entries to the rounding of FP64 sums, n 2^-53 sum |x| |y|,
+    """TUCKER_OPT_FP64_KERNEL: entries to the rounding of FP64 sums, n 2^-53 sum |x| |y|,
     where rows differ by 40 binary digits within themselves."""
     import torch
     from paper_1901_06043_gb300 import tucker
     c = tucker.Context()
-    c.set_option(tucker.OPT_FP64_PIPE, 1)
+    c.set_option(tucker.OPT_FP64_KERNEL, tucker.FP64_KERNEL["pipe"])
     I, K = dims[mode], int(np.prod(dims)) // dims[mode]
     U = graded(K, I, 6).T                       # rows graded along the columns
     full = np.moveaxis(U.reshape([I] + [d for k, d in enumerate(dims) if k != mode], order="F"), 0, mode)
@@ -190,7 +192,7 @@ def test_the_fp64_pipe_on_request(dims, mode):
     assert (np.abs(unfold(z, zd, mode) - A.astype(np.longdouble) @ L)
             <= (I + 1) * 2.0 ** -53 * (np.abs(A) @ np.abs(U))).all()
     with pytest.raises(tucker.TuckerError):
-        c.set_option(tucker.OPT_FP64_PIPE, 2)
+        c.set_option(tucker.OPT_FP64_KERNEL, 3)
     c.close()
 
 
@@ -198,11 +200,12 @@ def test_the_fp64_pipe_on_request(dims, mode):
                                                 ((10, 64, 150), 1, 16, False), ((16, 24000), 0, 64, False),
                                                 ((64, 1500), 0, 28, True), ((10, 64, 150), 1, 28, True),
                                                 ((200, 24000), 0, 4, True), ((16, 100000), 0, 28, True)])
-def test_ttm_takes_the_faster_kernel(ctx, dims, mode, K, digits):
+def test_ttm_takes_the_faster_kernel(dims, mode, K, digits):
     """The FP64 pipe's kernel (one launch) or the digits (three), by the work of both."""
     import torch
     from paper_1901_06043_gb300 import tucker
     x = torch.randn(int(np.prod(dims)), device="cuda", dtype=torch.float64)
+    ctx = tucker.Context()
     A = torch.randn(K, dims[mode], device="cuda", dtype=torch.float64)
     n0 = tucker.kernel_launches()
     z = ctx.ttm(x, dims, mode, A, prec="fp64")
@@ -213,6 +216,7 @@ def test_ttm_takes_the_faster_kernel(ctx, dims, mode, K, digits):
                                               order="F"), mode, 0)
     assert np.abs(got - want).max() <= 1e-14 * dims[mode] * np.abs(want).max()
 
+    ctx.close()
 
 def test_batched_tensors_with_tiny_slices(ctx):
     """A batch does not wait for the verdict on each step; a slice below the digits' range
