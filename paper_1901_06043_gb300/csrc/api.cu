@@ -873,7 +873,7 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
   if (prec != TUCKER_PREC_FP64 && (double)v.L * (double)v.Rt * (double)K >= 16777216.0)
     TK_TRY(dev_alloc(c, a32, sizeof(float) * (size_t)K * v.I));
   TK_CUDA(c, launch_ttm_simt(y, ydt, prec == TUCKER_PREC_FP64, v.L, v.I, v.Rt, A, K, lda, arow,
-                             a32.as<float>(), z, zdt, c->stream, zt));
+                             a32.as<float>(), z, zdt, c->num_sms, c->stream, zt));
   return TUCKER_OK;
 }
 

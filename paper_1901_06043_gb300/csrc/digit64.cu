@@ -111,22 +111,21 @@ constexpr int OUT_EXP = -2 * 1022 - 70;        // an entry is its sum times 2^(e
 constexpr double kDigit64MinGram = 2e7;
 // TTM: where the digits are the faster by the two models of a whole call below (us,
 // FP64 data, one wave being num_sms blocks), fitted to 720 calls with I from 8 to 500, K from
-// 4 to 200 and M from 300 to 4e5, column and row views: within 22 % (FP64 pipe), 20 %
-// (here, column views) and 33 % (row views).  On these calls the rule loses 0.5 % to the
-// better of the two, and 28 % at worst (26 x 24000 to 28, row view, 101 us there and 79
-// here).  Both sides, there and here: 64 x 1500 to 4 51 and 68, to 28 101 and 75; 200 x 1500 to 4 94
-// and 89; 16 x 1e5 to 16 83 and 108, to 28 132 and 113; 200 x 4e5 to 28 4248 and 808.
+// 4 to 200 and M from 300 to 4e5, column and row views: within 26 % (FP64 pipe and here, column
+// views) and 35 % (row views).  On these calls the rule loses 0.3 % to the better of the two,
+// and 31 % at worst (26 x 24000 to 28, row view, 103 us there and 78 here).  Both sides, there
+// and here: 64 x 1500 to 4 52 and 71, to 28 52 and 78; 200 x 1500 to 28 95 and 94; 16 x 1e5
+// to 16 84 and 107, to 28 135 and 114; 200 x 4e5 to 28 4242 and 807.
 //   A block of the pipe's kernel takes 0.31, 0.57 or 1.08 us per i for 8, 16 or more
 // outputs, a CTA here per item of 128 m and 64 outputs 2 (row views 1.6) us per stage of
 // 16 i and its drain; 1.2 ps per value are the exponent pass.
-//   And not below I = 64 and 2 K I M = 4e7, where the digits gain 22 us at most and a
+//   And not below I = 64 and 2 K I M = 4e7, where the digits gain 25 us at most and a
 // value keeps fewer bits there.
 constexpr double kDigit64MinTtm = 4e7;
 constexpr int kDigit64MinTtmI = 64;
 inline double ceil_div(double a, double b) { return std::ceil(a / b); }
-double ttm_pipe_us(double M, double I, double K, double sms) {
-  const double per = ceil_div(K, ceil_div(K, 32.0));            // outputs per tile (simt.cu)
-  const double kt = per <= 8 ? 8 : per <= 16 ? 16 : per <= 24 ? 24 : 32;
+double ttm_pipe_us(double M, double I, double K, int sms) {
+  const int kt = ttm_tile_outputs((int64_t)M, (int64_t)K, sms);
   const double blocks = ceil_div(M, 128.0) * ceil_div(K, kt);
   return 30.0 + (kt == 8 ? 0.31 : kt == 16 ? 0.57 : 1.08) * I * ceil_div(blocks, sms);
 }

@@ -109,8 +109,10 @@ cudaError_t launch_gram_small(const void* y, tucker_dtype dt, int64_t L, int64_t
 // zt (column mode only): Z written transposed, z[slab + Rt k] (the new mode last)
 cudaError_t launch_ttm_simt(const void* y, tucker_dtype ydt, bool fp64, int64_t L, int64_t I,
                             int64_t Rt, const double* A, int64_t K, int64_t lda, int a_rowmajor,
-                            float* a32_scratch, void* z, tucker_dtype zdt, cudaStream_t st,
-                            bool zt = false);
+                            float* a32_scratch, void* z, tucker_dtype zdt, int num_sms,
+                            cudaStream_t st, bool zt = false);
+// outputs per tile (of 128 m) that it takes
+int ttm_tile_outputs(int64_t M, int64_t K, int num_sms);
 
 // ---- tensor-core (tcgen05) Gram and TTM on the FP16 hi/lo split
 struct TcGramPlan {

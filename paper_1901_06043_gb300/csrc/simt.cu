@@ -627,9 +627,8 @@ cudaError_t launch_gram_simt(const void* y, tucker_dtype dt, bool fp64, int64_t 
 // ------------------------------------------------------------------- TTM
 //
 // Z (K x M) = A (K x I) * Y (I x M), M = the (l, r) pairs of the slab view, l
-// fastest.  A block of four warps owns MT m and KT outputs, KT = 8, 16, 24 or 32, the
-// smallest that divides K into tiles of at most 32 (few outputs are what a
-// truncation leaves).  WK warps share the outputs and 4 / WK the m; a thread owns MM
+// fastest.  A block of four warps owns MT m and KT outputs, KT = 8, 16, 24 or 32
+// (ttm_tile_outputs; few outputs are what a truncation leaves).  WK warps share the outputs and 4 / WK the m; a thread owns MM
 // m (lane + 32 j) and KK = KT / WK outputs of each.  The sums run over i in order.
 //   Stages of 32 i, two in turn, through registers a quarter at a time between the
 // products (16-byte accesses where the view allows).  L > 1: Y as it lies, m fastest.
@@ -895,7 +894,8 @@ __global__ void __launch_bounds__(TNT, sizeof(TC) == 4 ? 4 : 2)
 constexpr int TT = 64;    // output tile (k and m)
 constexpr int TBI = 16;   // contraction step
 
-// FP32 arithmetic on FP64 input or output (a 64 x 64 tile per block).
+// FP32 arithmetic on FP64 input or output, and FP32 row views of few rows and many
+// outputs (ttm_wide_tiles): a 64 x 64 tile per block.
 // Z (K x M) = A (K x I) * Y (I x M), M = the (r, l) pairs of the slab view.
 // Row mode (L > 1): an m-tile is 64 consecutive l of one slab.  Column mode
 // (L == 1): an m-tile is 64 consecutive slabs; zt writes Z transposed
@@ -1028,25 +1028,49 @@ static cudaError_t ttm_tile(const TIn* y, int64_t L, int64_t I, int64_t M, const
 
 template <typename TIn, typename TOut, typename TC>
 static cudaError_t ttm_new(const void* y, int64_t L, int64_t I, int64_t Rt, const double* A, int64_t K,
-                           int64_t lda, int arow, const float* A32, void* z, int zt,
+                           int64_t lda, int arow, const float* A32, void* z, int zt, int num_sms,
                            cudaStream_t st) {
-  const int64_t nt = (K + 31) / 32, per = (K + nt - 1) / nt;       // outputs per tile
+  const int kt = ttm_tile_outputs(L * Rt, K, num_sms);
   auto tile = [&](auto KT) {
     return L == 1 ? ttm_tile<TIn, TOut, TC, decltype(KT)::value, true>(
                         (const TIn*)y, L, I, Rt, A, K, lda, arow, A32, (TOut*)z, zt, st)
                   : ttm_tile<TIn, TOut, TC, decltype(KT)::value, false>(
                         (const TIn*)y, L, I, L * Rt, A, K, lda, arow, A32, (TOut*)z, zt, st);
   };
-  if (per <= 8) return tile(std::integral_constant<int, 8>());
-  if (per <= 16) return tile(std::integral_constant<int, 16>());
-  if (per <= 24) return tile(std::integral_constant<int, 24>());
+  if (kt == 8) return tile(std::integral_constant<int, 8>());
+  if (kt == 16) return tile(std::integral_constant<int, 16>());
+  if (kt == 24) return tile(std::integral_constant<int, 24>());
   return tile(std::integral_constant<int, 32>());
+}
+
+// The smallest tile that divides K into tiles of at most 32; smaller ones while the grid
+// still leaves half the SMs idle (a block's time grows with its outputs: 0.31, 0.57 and 1.08 us
+// per i in FP64 for 8, 16 and 24 or 32): FP32 row view 300 x 3000 to 32 72 -> 49 us, FP64
+// 64 x 1500 to 28 101 -> 52.
+int ttm_tile_outputs(int64_t M, int64_t K, int num_sms) {
+  const int64_t nt = (K + 31) / 32, per = (K + nt - 1) / nt;
+  int kt = per <= 8 ? 8 : per <= 16 ? 16 : per <= 24 ? 24 : 32;
+  while (kt > 8 && 2 * ((M + TNT - 1) / TNT) * ((K + kt - 1) / kt) <= num_sms) kt = kt > 16 ? 16 : 8;
+  return kt;
+}
+
+// FP32 row views with more than 32 outputs whose I leaves half of k_ttm's last stage of 32
+// unused, up to 16 rows, or 33 to 48 where the view allows no 16-byte loads: the 64 x 64 tiles
+// of k_ttm_simt (stages of 16), where at least half of their entries are used.  k_ttm and
+// there: 25000 x 12 x 10 to 310 235 and 190 us, x 16 to 50 76 and 61, x 16 to 33 67 and 60,
+// x 17 to 310 254 and 274; 24999 x 48 x 10 to 50 118 and 103, 25000 x 48 x 10 to 310 435 and
+// 431; 52 x 12 x 5000 to 65 89 and 106.
+static bool ttm_wide_tiles(const void* y, int64_t L, int64_t I, int64_t K) {
+  const int64_t l = (L + TT - 1) / TT, k = (K + TT - 1) / TT;
+  const bool vec = L % 4 == 0 && ((uintptr_t)y & 15) == 0;
+  return L > 1 && K > 32 && k <= 65535 && (I <= 16 || (!vec && I > 32 && I <= 48)) &&
+         2 * (double)L * (double)K >= (double)(l * TT) * (double)(k * TT);
 }
 
 cudaError_t launch_ttm_simt(const void* y, tucker_dtype ydt, bool fp64, int64_t L, int64_t I,
                             int64_t Rt, const double* A, int64_t K, int64_t lda, int a_rowmajor,
-                            float* a32_scratch, void* z, tucker_dtype zdt, cudaStream_t st,
-                            bool zt) {
+                            float* a32_scratch, void* z, tucker_dtype zdt, int num_sms,
+                            cudaStream_t st, bool zt) {
   if (zt && L != 1) return cudaErrorInvalidValue;
   if (L * Rt <= 0 || K <= 0) return cudaSuccess;
   const float* A32 = nullptr;
@@ -1060,16 +1084,19 @@ cudaError_t launch_ttm_simt(const void* y, tucker_dtype ydt, bool fp64, int64_t 
   count_launches(1);
   const bool yd = ydt == TUCKER_F64, zd = zdt == TUCKER_F64;
   if (fp64) {
-    if (yd) return zd ? ttm_new<double, double, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st)
-                      : ttm_new<double, float, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st);
-    return zd ? ttm_new<float, double, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st)
-              : ttm_new<float, float, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st);
+    if (yd) return zd ? ttm_new<double, double, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, num_sms, st)
+                      : ttm_new<double, float, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, num_sms, st);
+    return zd ? ttm_new<float, double, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, num_sms, st)
+              : ttm_new<float, float, double>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, num_sms, st);
   }
-  if (!yd && !zd) return ttm_new<float, float, float>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, st);
   const int64_t nLT = L == 1 ? 1 : (L + TT - 1) / TT, nMT = L == 1 ? (Rt + TT - 1) / TT : Rt * nLT;
+  if (!yd && !zd && !(ttm_wide_tiles(y, L, I, K) && nMT <= 0x7fffffffll))
+    return ttm_new<float, float, float>(y, L, I, Rt, A, K, lda, a_rowmajor, A32, z, zt, num_sms, st);
   if (nMT > 0x7fffffffll) return cudaErrorInvalidConfiguration;
   const dim3 grid((unsigned)nMT, (unsigned)((K + TT - 1) / TT));
-  if (yd && zd)
+  if (!yd && !zd)
+    k_ttm_simt<float, float, float><<<grid, 256, 0, st>>>((const float*)y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, (float*)z, zt);
+  else if (yd && zd)
     k_ttm_simt<double, double, float><<<grid, 256, 0, st>>>((const double*)y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, (double*)z, zt);
   else if (yd)
     k_ttm_simt<double, float, float><<<grid, 256, 0, st>>>((const double*)y, L, I, Rt, nLT, A, K, lda, a_rowmajor, A32, (float*)z, zt);

@@ -198,14 +198,15 @@ def test_the_fp64_pipe_on_request(dims, mode):
 
 @pytest.mark.parametrize("dims,mode,K,digits", [((64, 1500), 0, 4, False), ((96, 6000), 0, 4, False),
                                                 ((10, 64, 150), 1, 16, False), ((16, 24000), 0, 64, False),
-                                                ((64, 1500), 0, 28, True), ((10, 64, 150), 1, 28, True),
+                                                ((64, 1500), 0, 28, False), ((10, 64, 150), 1, 28, False),
+                                                ((64, 24000), 0, 28, True), ((300, 64, 80), 1, 28, True),
                                                 ((200, 24000), 0, 4, True), ((16, 100000), 0, 28, True)])
 def test_ttm_takes_the_faster_kernel(dims, mode, K, digits):
     """The FP64 pipe's kernel (one launch) or the digits (three), by the work of both."""
     import torch
     from paper_1901_06043_gb300 import tucker
-    x = torch.randn(int(np.prod(dims)), device="cuda", dtype=torch.float64)
     ctx = tucker.Context()
+    x = torch.randn(int(np.prod(dims)), device="cuda", dtype=torch.float64)
     A = torch.randn(K, dims[mode], device="cuda", dtype=torch.float64)
     n0 = tucker.kernel_launches()
     z = ctx.ttm(x, dims, mode, A, prec="fp64")
@@ -215,8 +216,8 @@ def test_ttm_takes_the_faster_kernel(dims, mode, K, digits):
     got = np.moveaxis(z.cpu().numpy().reshape([K if k == mode else d for k, d in enumerate(dims)],
                                               order="F"), mode, 0)
     assert np.abs(got - want).max() <= 1e-14 * dims[mode] * np.abs(want).max()
-
     ctx.close()
+
 
 def test_batched_tensors_with_tiny_slices(ctx):
     """A batch does not wait for the verdict on each step; a slice below the digits' range

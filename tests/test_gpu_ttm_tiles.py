@@ -55,6 +55,25 @@ def test_ttm_tiles(ctx, dims, mode, K, prec):
             assert (np.abs(z - want) <= bound).all()
 
 
+@pytest.mark.parametrize("dims", [(51, 12, 40), (64, 16, 3), (65, 16, 7), (128, 17, 9), (2999, 7, 5), (31, 16, 33),
+                                  (51, 33, 40), (65, 48, 7), (65, 49, 7), (64, 40, 9)])
+@pytest.mark.parametrize("K", [32, 33, 63, 64, 65, 130])
+def test_row_views_of_few_rows(ctx, dims, K):
+    """FP32 row views around the lines between the 64 x 64 tiles (at most 16 rows, or 33 to 48
+    without 16-byte loads, more than 32 outputs, half of the tiles' entries used) and the
+    narrower ones; bound as above."""
+    rng = np.random.default_rng(K + dims[0])
+    x = rng.standard_normal(dims).astype(np.float32)
+    A = rng.standard_normal((K, dims[1]))
+    want = np.einsum("ki,lir->lkr", A, x.astype(np.float64))
+    scale = np.einsum("ki,lir->lkr", np.abs(A), np.abs(x).astype(np.float64))
+    xt = torch.from_numpy(x.reshape(-1, order="F").copy()).cuda()
+    for At in (torch.from_numpy(A).cuda(), torch.from_numpy(A.T.copy()).cuda().t()):
+        z = ctx.ttm(xt, dims, 1, At, prec="fp32").double().cpu().numpy()
+        z = z.reshape((dims[0], K, dims[2]), order="F")
+        assert (np.abs(z - want) <= (dims[1] + 3) * 2.0 ** -24 * scale).all()
+
+
 @pytest.mark.parametrize("dims,mode", [((3, 4), 0), ((2, 3, 2), 1)])
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 def test_more_output_tiles_than_a_grid_dimension(ctx, dims, mode, prec):
