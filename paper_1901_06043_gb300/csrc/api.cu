@@ -818,7 +818,9 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
                      const double* A, int64_t K, int64_t lda, int arow, tucker_prec prec, void* z,
                      tucker_dtype zdt, int* kernel_used, double ymax = -1.0, bool check = true,
                      bool zt = false) {
-  // (the split scale needs max|y|: without it and without host syncs, SIMT)
+  // The tensor-core TTMs' split scale needs max|y|.  Where the caller does not know it, a
+  // norm pass leaves it in d_small[1], whose words all side streams of a batch share: a
+  // caller that runs on those (check = false) and does not know it keeps the FP32 pipe.
   const bool tc = (prec == TUCKER_PREC_MIXED || prec == TUCKER_PREC_TENSOR) && ydt == TUCKER_F32 &&
                   zdt == TUCKER_F32 && (((uintptr_t)y) & 15) == 0 && (check || ymax >= 0.0) &&
                   (!zt || (((uintptr_t)z) & 15) == 0) && ttm_tc_supported(v.L, v.I, v.Rt, K);
@@ -835,10 +837,7 @@ tucker_status do_ttm(tucker_ctx* c, const void* y, tucker_dtype ydt, const SlabV
     return check ? ttm_verdict(c, ymax_d != nullptr) : TUCKER_OK;
   }
   // row-mode views with a short contraction (I <= 64: the reconstruction's
-  // expansions) on the tensor cores, l as the MMA's M.  Its split scale needs
-  // max|y|: a caller that runs without host syncs (check = false, the batched
-  // path on side streams) and does not know it keeps the SIMT TTM rather than
-  // pay a synchronizing norm pass.
+  // expansions) on the tensor cores, l as the MMA's M
   const bool tc_row = !zt && (check || ymax >= 0.0) &&
                       (prec == TUCKER_PREC_MIXED || prec == TUCKER_PREC_TENSOR) &&
                       ydt == TUCKER_F32 && zdt == TUCKER_F32 && (((uintptr_t)y) & 15) == 0 &&
