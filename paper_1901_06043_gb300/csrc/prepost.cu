@@ -597,10 +597,11 @@ __global__ void k_params(const double* stats, int64_t I, int method, double* shi
 }
 
 // rows-regime grid: (row blocks, column chunks) about 8 CTAs per SM; fewer where a
-// thread would have less than `per` elements (0: whatever it has).  The statistics take
+// thread would have less than `per` elements (0: whatever it has).  FP32 statistics take
 // 32: a thread ends with five atomics on one set of words per hyperslice, which otherwise
 // are the pass (standardizing 60,000 elements along 40 rows and back: 338 us with 1,216
-// chunks, 118 with 7; 1.1e6 along 100 186 and 123 us).
+// chunks, 118 with 7; 1.1e6 along 100 186 and 123 us).  FP64 statistics keep their chunks,
+// in whose order their sums are rounded.
 void rows_grid(int64_t P, int64_t Rt, int num_sms, int per, unsigned& gx, int& nc) {
   const int64_t rb = P < kThreads ? 1 : (P + kThreads - 1) / kThreads;
   int64_t c = ((int64_t)num_sms * 8 + rb - 1) / rb;
@@ -618,7 +619,7 @@ void stats_pass(const T* x, int64_t L, int64_t I, int64_t Rt, const double* mean
     const int64_t P = L * I;
     unsigned gx;
     int nc;
-    rows_grid(P, Rt, num_sms, 32, gx, nc);
+    rows_grid(P, Rt, num_sms, sizeof(T) == 4 ? 32 : 0, gx, nc);
     k_stats_rows<T, PASS><<<dim3(gx, (unsigned)nc), kThreads, 0, st>>>(x, L, P, Rt, nc, mean,
                                                                         acc);
   } else {
